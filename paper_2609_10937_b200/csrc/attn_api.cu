@@ -895,21 +895,43 @@ int softmax_launch(const void* s, void* pout, long long rows, int cols, float sc
   const int nvec = cols / 8;                        // 16-byte vectors per row
   const __nv_bfloat16* sp = static_cast<const __nv_bfloat16*>(s);
   __nv_bfloat16* pp = static_cast<__nv_bfloat16*>(pout);
-  const dim3 grid((unsigned)rows);
-  // threads x vectors per thread >= nvec.  Small blocks (128 or 256 threads, the row in up to 8 -- for the widest
-  // rows 32 -- vectors per thread): several rows are then in flight per SM in different phases (load, reduce, store),
-  // which one large block per row does not give (measured: 1024-thread blocks reach half the bandwidth).
-  if (nvec <= 128) gemm::softmax_rows_kernel<1, 128><<<grid, 128, 0, stream>>>(sp, pp, cols, scale_log2);
-  else if (nvec <= 256) gemm::softmax_rows_kernel<2, 128><<<grid, 128, 0, stream>>>(sp, pp, cols, scale_log2);
-  else if (nvec <= 512) gemm::softmax_rows_kernel<4, 128><<<grid, 128, 0, stream>>>(sp, pp, cols, scale_log2);
-  else if (nvec <= 1024) gemm::softmax_rows_kernel<4, 256><<<grid, 256, 0, stream>>>(sp, pp, cols, scale_log2);
-  else if (nvec <= 2048) gemm::softmax_rows_kernel<8, 256><<<grid, 256, 0, stream>>>(sp, pp, cols, scale_log2);
+  DeviceState* st = nullptr;
+  int rc = device_state(&st);
+  if (rc != ATTN_OK) return rc;
+  const int sms = st->desc.num_units;
+  // Up to 128 vectors a row: a warp per row (half a warp below 17 vectors), at most 16 CTAs of four warps per SM.
+  auto launch_warp = [&](auto kern, int rows_per_warp) {
+    const long long ctas = (rows + 4 * rows_per_warp - 1) / (4 * rows_per_warp);
+    kern<<<(unsigned)std::min(ctas, 16LL * sms), 128, 0, stream>>>(sp, pp, rows, cols, scale_log2);
+  };
+  // Longer rows: a CTA per row, as few warps as hold it at VPT vectors a thread (5000 columns on 160 threads: 18.6 us for
+  // 5000 rows, on 256 threads 24.8).
+  auto launch_row = [&](auto kern, int threads) { kern<<<(unsigned)rows, threads, 0, stream>>>(sp, pp, cols, scale_log2); };
+#define SOFTMAX_ROW_CASE(VPT_, THREADS_) else if (nvec <= VPT_ * THREADS_) launch_row(gemm::softmax_rows_kernel<VPT_, THREADS_>, THREADS_)
+  if (nvec <= 16) launch_warp(gemm::softmax_rows_warp_kernel<1, 16, 1>, 2);
+  else if (nvec <= 32) launch_warp(gemm::softmax_rows_warp_kernel<1, 32, 1>, 1);
+  else if (nvec <= 64) launch_warp(gemm::softmax_rows_warp_kernel<2, 32, 1>, 1);
+  else if (nvec <= 96) launch_warp(gemm::softmax_rows_warp_kernel<3, 32, 1>, 1);
+  else if (nvec <= 128) launch_warp(gemm::softmax_rows_warp_kernel<4, 32, 1>, 1);
+  SOFTMAX_ROW_CASE(2, 96);
+  SOFTMAX_ROW_CASE(2, 128);
+  SOFTMAX_ROW_CASE(4, 96);
+  SOFTMAX_ROW_CASE(4, 128);
+  SOFTMAX_ROW_CASE(4, 160);
+  SOFTMAX_ROW_CASE(4, 192);
+  SOFTMAX_ROW_CASE(4, 224);
+  SOFTMAX_ROW_CASE(4, 256);
+  SOFTMAX_ROW_CASE(8, 160);
+  SOFTMAX_ROW_CASE(8, 192);
+  SOFTMAX_ROW_CASE(8, 224);
+  SOFTMAX_ROW_CASE(8, 256);
   else {
     // wider than the registers of one block hold: the row is staged in shared memory (2 bytes per column)
     auto kern = gemm::softmax_rows_staged_kernel<256>;
     ATTN_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 65536));
-    kern<<<grid, 256, cols * 2, stream>>>(sp, pp, cols, scale_log2);
+    kern<<<(unsigned)rows, 256, cols * 2, stream>>>(sp, pp, cols, scale_log2);
   }
+#undef SOFTMAX_ROW_CASE
   ATTN_CUDA_TRY(cudaGetLastError());
   ++t_launch_count;
   return ATTN_OK;

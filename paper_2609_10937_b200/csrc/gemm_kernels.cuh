@@ -6,7 +6,8 @@
 //                 (A tile, B tile) stages -> one MMA-issuing thread (tcgen05.mma, two 128-row
 //                 sub-tiles x 256 columns accumulated in tensor memory) -> eight epilogue warps
 //                 (tensor memory -> bf16 -> shared-memory staging -> TMA store).
-//   softmax_rows_kernel  one CTA per row, the row held in registers: one read, one write.
+//   softmax_rows_warp_kernel    short rows: one warp (or half of one) per row, no barrier.
+//   softmax_rows_kernel         longer rows: one CTA per row, the row held in registers.
 //   softmax_rows_staged_kernel  the same for rows too wide for registers: staged in shared memory.
 //
 // Every device-side wait is bounded (see attn_kernels.cuh).
@@ -494,93 +495,178 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant
 }
 
 // ---------------------------------------------------------------------------
-// Row softmax of scale * S, bf16 in and out (in place allowed).  One CTA of THREADS threads per row; thread t
-// holds VPT vectors of 8 consecutive columns (vector v covers columns (v * THREADS + t) * 8 ...).  Each thread keeps
-// the running statistics (m, d) of its columns; partials are merged with
-//   (m1, d1) (+) (m2, d2) = (max(m1, m2), d1 2^(m1 - m) + d2 2^(m2 - m))
-// first across the warp by shuffles, then across warps through shared memory.
+// Row softmax of scale * S, bf16 in and out (in place allowed).  Statistics are merged with
+//   (m1, d1) (+) (m2, d2) = (max(m1, m2), d1 2^(m1 - m) + d2 2^(m2 - m)).
 // ---------------------------------------------------------------------------
 
-__device__ __forceinline__ void merge_md(float& m, float& d, float m2, float d2) {
-  const float mn = fmaxf(m, m2);
-  // a side with no element yet has m = -inf and d = 0: its term is 0, not NaN
-  const float t1 = (m == -INFINITY) ? 0.f : d * exp2f(m - mn);
-  const float t2 = (m2 == -INFINITY) ? 0.f : d2 * exp2f(m2 - mn);
-  m = mn;
-  d = t1 + t2;
+// Sum of one warp's (or 16-lane group's) values; every lane gets it.
+template <int LANES>
+__device__ __forceinline__ float group_sum(float d) {
+#pragma unroll
+  for (int off = LANES / 2; off > 0; off >>= 1) d += __shfl_xor_sync(0xffffffffu, d, off);
+  return d;
+}
+// Maximum of packed bf16 pairs over the group; every lane gets it, as fp32.
+template <int LANES>
+__device__ __forceinline__ float group_max(uint32_t mx2) {
+#pragma unroll
+  for (int off = LANES / 2; off > 0; off >>= 1) mx2 = max_bf16x2(mx2, __shfl_xor_sync(0xffffffffu, mx2, off));
+  return fmaxf(__uint_as_float(mx2 << 16), __uint_as_float(mx2 & 0xFFFF0000u));
+}
+constexpr uint32_t kNegInfPair = 0xFF80FF80u;               // (-inf, -inf) in bf16: weight 0, never the maximum
+__device__ __forceinline__ uint32_t max_of(const uint4& q, uint32_t mx2) {
+  return max_bf16x2(max_bf16x2(mx2, q.x), max_bf16x2(max_bf16x2(q.y, q.z), q.w));
+}
+// 2^(x * scale - m) of a packed bf16 pair
+__device__ __forceinline__ uint64_t exp_pair(uint32_t w, uint64_t scale2, uint64_t negm2) {
+  const uint64_t t = fma_f32x2(pack_f32x2(__uint_as_float(w << 16), __uint_as_float(w & 0xFFFF0000u)), scale2, negm2);
+  float t0, t1;
+  unpack_f32x2(t, t0, t1);
+  return pack_f32x2(ex2_approx(t0), ex2_approx(t1));
+}
+__device__ __forceinline__ uint32_t scaled_pair(uint64_t x, uint64_t f2) {
+  float a0, a1;
+  unpack_f32x2(mul_f32x2(x, f2), a0, a1);
+  return pack_bf16x2(a0, a1);
 }
 
+// Short rows (up to 128 vectors of 8 columns).  A row belongs to LANES lanes of one warp, lane l holding vectors
+// l, l + LANES, ... (VPT of them), so a row needs no barrier; a warp works on R * 32 / LANES rows at a time and loads
+// its next rows before it works on these.  Bound by HBM.  One CTA of 128 threads per row spent its time on starting CTAs
+// and on the barrier (nearly half its threads without a vector at 520 columns): 32768 x 520 took 34.3 us, here 13.8
+// (4.9 TB/s); 131072 x 128 119 us, here 14.4; 65536 x 1024 71 us, here 43.0 (6.2 TB/s).
+template <int VPT, int LANES, int R>
+__global__ void __launch_bounds__(128)
+softmax_rows_warp_kernel(const __nv_bfloat16* s, __nv_bfloat16* pout, long long rows, int cols, float scale_log2) {
+  constexpr int kRowsPerGroup = 32 / LANES;
+  constexpr int kRowsPerWarp = R * kRowsPerGroup;
+  const int l = threadIdx.x % LANES;
+  const int nvec = cols / 8;
+  const long long stride = (long long)gridDim.x * 4 * kRowsPerWarp;
+  // row r of this lane's group: first + r * kRowsPerGroup
+  long long first = ((long long)blockIdx.x * 4 + (threadIdx.x >> 5)) * kRowsPerWarp + (threadIdx.x & 31) / LANES;
+  auto load = [&](uint4 (&w)[R][VPT], long long row0) {
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const long long row = row0 + r * kRowsPerGroup;
+      const uint4* src = reinterpret_cast<const uint4*>(s + row * cols);
+#pragma unroll
+      for (int v = 0; v < VPT; ++v) {
+        const int idx = v * LANES + l;
+        w[r][v] = make_uint4(kNegInfPair, kNegInfPair, kNegInfPair, kNegInfPair);
+        if (row < rows && idx < nvec) w[r][v] = src[idx];
+      }
+    }
+  };
+  const uint64_t scale2 = pack_f32x2(scale_log2, scale_log2);
+  uint4 w[R][VPT];
+  load(w, first);
+  // (the bound is the same for a warp's lanes: its first row)
+  for (long long lead = first - (threadIdx.x & 31) / LANES; lead < rows; lead += stride, first += stride) {
+    uint4 next[R][VPT];
+    load(next, first + stride);
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      uint32_t mx2 = kNegInfPair;
+#pragma unroll
+      for (int v = 0; v < VPT; ++v) mx2 = max_of(w[r][v], mx2);
+      const float m = group_max<LANES>(mx2) * scale_log2;    // scale > 0 keeps the order
+      const float neg_m = (m == -INFINITY) ? 0.f : -m;
+      const uint64_t negm2 = pack_f32x2(neg_m, neg_m);
+      uint64_t x[VPT][4];
+      uint64_t d2 = 0ull;
+#pragma unroll
+      for (int v = 0; v < VPT; ++v) {
+        x[v][0] = exp_pair(w[r][v].x, scale2, negm2);
+        x[v][1] = exp_pair(w[r][v].y, scale2, negm2);
+        x[v][2] = exp_pair(w[r][v].z, scale2, negm2);
+        x[v][3] = exp_pair(w[r][v].w, scale2, negm2);
+        d2 = add_f32x2(d2, add_f32x2(add_f32x2(x[v][0], x[v][1]), add_f32x2(x[v][2], x[v][3])));
+      }
+      float d0, d1;
+      unpack_f32x2(d2, d0, d1);
+      const float d = group_sum<LANES>(d0 + d1);
+      const float f = (m == -INFINITY && d == 0.f) ? 0.f : 1.0f / d;     // a row without an element: weights 0, not NaN
+      const uint64_t f2 = pack_f32x2(f, f);
+      const long long row = first + r * kRowsPerGroup;
+      uint4* dst = reinterpret_cast<uint4*>(pout + row * cols);
+#pragma unroll
+      for (int v = 0; v < VPT; ++v) {
+        const int idx = v * LANES + l;
+        if (row < rows && idx < nvec)
+          dst[idx] = make_uint4(scaled_pair(x[v][0], f2), scaled_pair(x[v][1], f2), scaled_pair(x[v][2], f2), scaled_pair(x[v][3], f2));
+      }
+    }
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+#pragma unroll
+      for (int v = 0; v < VPT; ++v) w[r][v] = next[r][v];
+  }
+}
+
+// Longer rows: one CTA per row, thread t holding VPT vectors t, t + THREADS, ...; the launcher takes the fewest whole
+// warps that hold the row.  The exponentials (one per element) are taken relative to the maximum of the warp or, from four
+// vectors a thread, of the thread (waiting for the warp's costs 5-14 % there, at two vectors it saves 8-13 %) and rescaled
+// once the warps' (m, d) have met in shared memory, behind the row's only barrier.
+// (The register bounds keep 1280 threads per SM at four vectors and 768 at eight: rows in flight are what the kernel lives
+// on -- with 59 registers instead of 48, four vectors a thread are 7 % slower.  8192 x 8192: 41.8 us = 6.4 TB/s, 43.7 with
+// the pairwise (m, d) merge in every shuffle step that stood here before; 4096 x 16384: 42.0 us against 48.4.)
 template <int VPT, int THREADS>
-__global__ void __launch_bounds__(THREADS)
+__global__ void __launch_bounds__(THREADS, VPT < 4 ? 1 : (VPT == 4 ? 1280 : 768) / THREADS)
 softmax_rows_kernel(const __nv_bfloat16* s, __nv_bfloat16* pout, int cols, float scale_log2) {
-  __shared__ float sm_m[THREADS / 32], sm_d[THREADS / 32];
+  __shared__ float2 part[THREADS / 32];                     // per warp: (m, d)
   const size_t row = blockIdx.x;
   const uint4* src = reinterpret_cast<const uint4*>(s + row * (size_t)cols);
   uint4* dst = reinterpret_cast<uint4*>(pout + row * (size_t)cols);
   const int nvec = cols / 8;
-  // Pass 1 on the packed bf16 words: load, running maximum per lane pair (scale > 0 keeps the order).
-  uint32_t w[VPT][4];
-  uint32_t mx2 = 0xFF80FF80u;                               // (-inf, -inf) in bf16
+  uint4 w[VPT];
 #pragma unroll
   for (int v = 0; v < VPT; ++v) {
     const int idx = v * THREADS + threadIdx.x;
-    if (idx < nvec) {
-      const uint4 q = src[idx];
-      w[v][0] = q.x; w[v][1] = q.y; w[v][2] = q.z; w[v][3] = q.w;
-#pragma unroll
-      for (int e = 0; e < 4; ++e) mx2 = max_bf16x2(mx2, w[v][e]);
-    } else {
-#pragma unroll
-      for (int e = 0; e < 4; ++e) w[v][e] = 0xFF80FF80u;    // -inf: weight 0
-    }
+    w[v] = make_uint4(kNegInfPair, kNegInfPair, kNegInfPair, kNegInfPair);
+    if (idx < nvec) w[v] = src[idx];
   }
-  float m = fmaxf(__uint_as_float(mx2 << 16), __uint_as_float(mx2 & 0xFFFF0000u)) * scale_log2;
-  // this thread's statistics; the exponentials are kept (relative to the thread's own maximum) and only
-  // rescaled once the row's maximum is known: one exponential per element
-  const float m_own = m;
+  uint32_t mx2 = kNegInfPair;
+#pragma unroll
+  for (int v = 0; v < VPT; ++v) mx2 = max_of(w[v], mx2);
+  // scale > 0 keeps the order
+  const float m = group_max<32>(mx2) * scale_log2;
+  const float m_own = VPT < 4 ? m : fmaxf(__uint_as_float(mx2 << 16), __uint_as_float(mx2 & 0xFFFF0000u)) * scale_log2;
   const float neg_m = (m_own == -INFINITY) ? 0.f : -m_own;
   const uint64_t scale2 = pack_f32x2(scale_log2, scale_log2), negm2 = pack_f32x2(neg_m, neg_m);
   uint64_t x[VPT][4];
   uint64_t d2 = 0ull;
 #pragma unroll
   for (int v = 0; v < VPT; ++v) {
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const uint64_t t = fma_f32x2(pack_f32x2(__uint_as_float(w[v][e] << 16), __uint_as_float(w[v][e] & 0xFFFF0000u)), scale2, negm2);
-      float t0, t1;
-      unpack_f32x2(t, t0, t1);
-      x[v][e] = pack_f32x2(ex2_approx(t0), ex2_approx(t1));
-      d2 = add_f32x2(d2, x[v][e]);
-    }
+    x[v][0] = exp_pair(w[v].x, scale2, negm2);
+    x[v][1] = exp_pair(w[v].y, scale2, negm2);
+    x[v][2] = exp_pair(w[v].z, scale2, negm2);
+    x[v][3] = exp_pair(w[v].w, scale2, negm2);
+    d2 = add_f32x2(d2, add_f32x2(add_f32x2(x[v][0], x[v][1]), add_f32x2(x[v][2], x[v][3])));
   }
   float d0, d1;
   unpack_f32x2(d2, d0, d1);
-  float d = d0 + d1;
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) {
-    const float m2 = __shfl_xor_sync(0xffffffffu, m, off), dd = __shfl_xor_sync(0xffffffffu, d, off);
-    merge_md(m, d, m2, dd);
-  }
-  if ((threadIdx.x & 31) == 0) { sm_m[threadIdx.x >> 5] = m; sm_d[threadIdx.x >> 5] = d; }
+  const float own = d0 + d1;
+  // (a thread without an element: its term is 0)
+  const float d = group_sum<32>(VPT < 4 ? own : (m_own == -INFINITY && own == 0.f) ? 0.f : own * exp2f(m_own - m));
+  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = make_float2(m, d);
   __syncthreads();
-  float mr = sm_m[0], dr = sm_d[0];
+  float mr = -INFINITY;
 #pragma unroll
-  for (int k = 1; k < THREADS / 32; ++k) merge_md(mr, dr, sm_m[k], sm_d[k]);
-  const float f = (m_own == -INFINITY) ? 0.f : exp2f(m_own - mr) / dr;
+  for (int k = 0; k < THREADS / 32; ++k) mr = fmaxf(mr, part[k].x);
+  float dr = 0.f;
+#pragma unroll
+  for (int k = 0; k < THREADS / 32; ++k) {
+    const float2 p = part[k];
+    if (p.x != -INFINITY || p.y != 0.f) dr += p.y * exp2f(p.x - mr);       // a warp without an element: its term is 0
+  }
+  const float f = (mr == -INFINITY && dr == 0.f) ? 0.f : exp2f(m_own - mr) / dr;
   const uint64_t f2 = pack_f32x2(f, f);
 #pragma unroll
   for (int v = 0; v < VPT; ++v) {
     const int idx = v * THREADS + threadIdx.x;
-    if (idx < nvec) {
-      uint32_t o[4];
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        float a0, a1;
-        unpack_f32x2(mul_f32x2(x[v][e], f2), a0, a1);
-        o[e] = pack_bf16x2(a0, a1);
-      }
-      dst[idx] = make_uint4(o[0], o[1], o[2], o[3]);
-    }
+    if (idx < nvec)
+      dst[idx] = make_uint4(scaled_pair(x[v][0], f2), scaled_pair(x[v][1], f2), scaled_pair(x[v][2], f2), scaled_pair(x[v][3], f2));
   }
 }
 

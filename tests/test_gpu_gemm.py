@@ -127,6 +127,32 @@ def test_row_softmax_matches_oracle(env, rows, cols):
     assert torch.equal(p2, p)
 
 
+@pytest.mark.parametrize("cols", [8, 128, 136, 256, 264, 512, 520, 768, 776, 1024, 1032, 1536, 2048, 2056, 3080, 4096, 5128,
+                                  6152, 7176, 8192, 8200, 10248, 12296, 14344, 16384])
+@pytest.mark.parametrize("rows", [1, 37, 9475])
+def test_row_softmax_at_the_edges_of_every_row_layout(env, rows, cols):
+    """Both sides of every width at which the kernel or its threads change, one row, a ragged number of rows, and more rows
+    than the persistent grid of the short-row kernel has warps; rows of -inf give zeros, a -inf half leaves the other half."""
+    torch, go, binding = env
+    if rows * cols > 1 << 25:
+        rows = 301
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(rows * 131 + cols)
+    s = (torch.randn((rows, cols), generator=gen, device="cuda") * 6.0).to(torch.bfloat16)
+    if rows > 1:
+        s[1] = -math.inf
+        s[rows - 1, : cols // 2] = -math.inf
+        s[rows // 2, cols - 1] = 300.0                            # a dominant last column
+    p = binding.softmax_rows(s, 0.37)
+    ref = torch.softmax(s.double() * float(np.float32(0.37)), dim=-1)
+    if rows > 1:
+        ref[1] = 0.0
+    # bf16 keeps 8 significant bits: half a unit in the last place is at most 2^-8 of the value.  The fp32 part stays below
+    # 2^-13: the exponent, up to 300 * 0.37 * log2 e = 160 in magnitude, carries 160 * 2^-24 = 2^-16.7 twice.
+    assert ((p.double() - ref).abs() <= ref * (2.0 ** -8 + 2.0 ** -13) + 1e-37).all()
+    assert torch.equal(binding.softmax_rows(s, 0.37, out=s), p)      # in place
+
+
 @pytest.mark.parametrize("B,H,L,d", [(1, 1, 256, 64), (1, 2, 1024, 128), (2, 2, 520, 64), (1, 1, 4096, 128), (1, 1, 16384, 128)])
 def test_unfused_attention_matches_its_oracle_and_the_fused_kernel(env, B, H, L, d):
     torch, go, binding = env
