@@ -14,6 +14,7 @@
 #include "attn.h"
 #include "attn_kernels.cuh"
 #include "attn_plan_internal.h"
+#include "decode_kernels.cuh"
 #include "gemm.h"
 #include "gemm_kernels.cuh"
 
@@ -79,6 +80,7 @@ struct DeviceState {
   bool arch_checked = false;
   bool arch_ok = false;
   attn_hw_desc desc;
+  int decode_clusters[5] = {};   // [i]: clusters of 2^i CTAs of the decode kernel that fit at once, + 1 (0 = not asked yet); guarded by g_mu
   int resident[2][9] = {};     // [causal][k]: clusters of k CTAs that fit at once, + 1 (0 = not asked yet); guarded by g_mu
 };
 DeviceState g_dev[kMaxDevices];
@@ -272,6 +274,114 @@ int launch_fwd(const void* q, const void* k, const void* v, void* o, int B, int 
   return ATTN_OK;
 }
 
+// Few query rows against many keys (decode_kernels.cuh).
+template <int D, int MT, bool HALF>
+int launch_decode(const void* q, const void* k, const void* v, void* o, int BH, int Lq, int Lk, int cluster_k, unsigned int* status,
+                  cudaStream_t stream) {
+  constexpr int kSlab = attn::decode_slab_keys(D);
+  CUtensorMap tk, tv;
+  int rc;
+  if ((rc = make_tmap(&tk, k, BH, Lk, D, kSlab)) != ATTN_OK) return rc;
+  if ((rc = make_tmap(&tv, v, BH, Lk, D, kSlab)) != ATTN_OK) return rc;
+  attn::DecodeParams p;
+  p.q = static_cast<const __nv_bfloat16*>(q);
+  p.o = static_cast<__nv_bfloat16*>(o);
+  p.Lq = Lq;
+  p.Lk = Lk;
+  p.cluster_k = cluster_k;
+  p.scale_log2 = (float)(1.4426950408889634 / std::sqrt((double)D));
+  p.status = status;
+  auto kern = attn::attn_decode_kernel<D, MT, HALF>;
+  constexpr int smem = attn::decode_smem_total<MT>();
+  ATTN_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  if (cluster_k > 8) ATTN_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(BH * cluster_k));
+  cfg.blockDim = dim3(32 * attn::kDecodeWarps);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = cluster_k;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  ATTN_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, tk, tv, p));
+  t_cluster_size = cluster_k > 1 ? cluster_k : 0;
+  t_launch_count = 1;
+  return ATTN_OK;
+}
+
+// Clusters of k CTAs of the decode kernel that the device holds at once (0: none, or k CTAs are not allowed).
+int resident_decode_clusters(int k) {
+  auto kern = attn::attn_decode_kernel<128, 1, true>;
+  constexpr int smem = attn::decode_smem_total<1>();
+  int n = 0;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)k);
+  cfg.blockDim = dim3(32 * attn::kDecodeWarps);
+  cfg.dynamicSmemBytes = smem;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = k;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
+      (k > 8 && cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) ||
+      cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return 0;
+  }
+  return n;
+}
+
+// CTAs per head: a power of two (other cluster sizes leave SMs of a GPC unused).  Unit of the estimate: the time a CTA
+// takes per slab when all slots are busy and HBM is the bound.  A CTA's start and end cost about 10 such units, k / 2 more
+// for the cluster's barriers and merge; a partly full wave runs faster in proportion, down to 0.55, where a CTA with an SM to
+// itself is bound by its own warps.  The slots are those the device reports for clusters of k: a cluster that has to wait for
+// a second wave costs as much as a whole one.  Measured (us for k = 1 / 2 / 4 / 8): 256 heads x 4096 keys, d = 128:
+// 83 / 81 / 87 / 101; 128 x 16384: 177 / 164 / 158 / 169; 32 x 4096: 39 / 22.5 / 15.0 / 15.2; 256 x 300: 9.2 / 14.5 / 21.4 /
+// 39.5; k = 8 / 16: 8 x 16384: 24.2 / 18.0, 15 x 16384: 25.9 / 36.6.
+int decode_split(int BH, int Lk, int d, const int (&clusters)[5]) {
+  const int slabs = (Lk + attn::decode_slab_keys(d) - 1) / attn::decode_slab_keys(d);
+  int best = 1;
+  double best_cost = 0.0;
+  for (int i = 0, k = 1; k <= attn::kDecodeMaxSplit; ++i, k *= 2) {
+    if (k > 1 && (clusters[i] == 0 || slabs < attn::kDecodeWarps * k)) break;      // at least one slab per warp
+    const double per_cta = (double)((slabs + k - 1) / k), ends = 10.0 + 0.5 * k;
+    const double waves = (double)BH / std::max(1, clusters[i]), full = std::floor(waves), part = waves - full;
+    const double cost = full * (per_cta + ends) + (part > 0.0 ? per_cta * std::max(part, 0.55) + ends : 0.0);
+    if (k == 1 || cost < best_cost) { best = k; best_cost = cost; }
+  }
+  return best;
+}
+
+int dispatch_decode(const void* q, const void* k, const void* v, void* o, int BH, int Lq, int Lk, int d, unsigned int* status,
+                    DeviceState* st, cudaStream_t s) {
+  int clusters[5];
+  {
+    std::lock_guard<std::mutex> lk(g_mu);
+    for (int i = 0; i < 5; ++i) {
+      if (st->decode_clusters[i] == 0) st->decode_clusters[i] = resident_decode_clusters(1 << i) + 1;
+      clusters[i] = st->decode_clusters[i] - 1;
+    }
+  }
+  const int ck = decode_split(BH, Lk, d, clusters);
+#define DECODE_CASE(D_)                                                                                          \
+  if (d == D_) {                                                                                                 \
+    if (Lq <= 8) return launch_decode<D_, 1, true>(q, k, v, o, BH, Lq, Lk, ck, status, s);                       \
+    if (Lq <= 16) return launch_decode<D_, 1, false>(q, k, v, o, BH, Lq, Lk, ck, status, s);                     \
+    return launch_decode<D_, 2, false>(q, k, v, o, BH, Lq, Lk, ck, status, s);                                   \
+  }
+  DECODE_CASE(64)
+  DECODE_CASE(128)
+#undef DECODE_CASE
+  return ATTN_ERR_UNSUPPORTED_SHAPE;
+}
+
 int dispatch_fwd(const void* q, const void* k, const void* v, void* o, int B, int H, int L, int d,
                  const attn_tiles& t, float* ws, unsigned int* status, DeviceState* st, cudaStream_t s, int Lk = 0,
                  bool may_overlap = false) {
@@ -289,6 +399,15 @@ int dispatch_fwd(const void* q, const void* k, const void* v, void* o, int B, in
   ATTN_CASE(64, 64, 1)
 #undef ATTN_CASE
   return ATTN_ERR_BAD_TILES;
+}
+
+// Calls that the decode kernel takes over from the tiled one.  Up to 16 rows (at d = 64 up to 32) it is faster at every size
+// measured (1.2-4.9 times).  17 to 32 rows at d = 128 keep its warps as busy as HBM: there only where the tiled kernel would
+// run whole tiles in waves over more than a thousand keys (24 rows, us tiled / decode: 192 heads x 8192 keys 201 / 145,
+// 192 x 2048 56 / 47; below that 128 x 2048 30.6 / 31.2, 128 x 512 13.4 / 17.1).
+bool decode_rows(int Lq, int Lk, int d, const attn_tiles& t, int sms) {
+  if (Lq <= 16 || (d == 64 && Lq <= 32)) return true;
+  return Lq <= 32 && t.tiles > sms && t.ctas == t.tiles && Lk >= 1024;
 }
 
 // A plan needs the workspace unless every CTA owns exactly one whole Q tile.
@@ -367,6 +486,8 @@ int forward_impl(const void* q, const void* k, const void* v, void* o, int B, in
       ws = static_cast<float*>(st->ws);
     }
   }
+  if (!ovr && !plan_desc && !call_ws && Lk != L && decode_rows(L, Lk, d, t, st->desc.num_units))
+    return dispatch_decode(q, k, v, o, B * H, L, Lk, d, nullptr, st, static_cast<cudaStream_t>(cuda_stream));
   return dispatch_fwd(q, k, v, o, B, H, L, d, t, ws, call_ws ? call_ws->status : nullptr, st,
                       static_cast<cudaStream_t>(cuda_stream), Lk, call_ws != nullptr);
 }
@@ -899,7 +1020,8 @@ int softmax_launch(const void* s, void* pout, long long rows, int cols, float sc
   int rc = device_state(&st);
   if (rc != ATTN_OK) return rc;
   const int sms = st->desc.num_units;
-  // Up to 128 vectors a row: a warp per row (half a warp below 17 vectors), at most 16 CTAs of four warps per SM.
+  // Up to 128 vectors a row: a warp per row (half a warp below 17 vectors), at most 16 CTAs of four warps per SM
+  // (65536 x 1024: 43.2 us, 8 CTAs 47.9; one CTA per row is slower at every width up to here).
   auto launch_warp = [&](auto kern, int rows_per_warp) {
     const long long ctas = (rows + 4 * rows_per_warp - 1) / (4 * rows_per_warp);
     kern<<<(unsigned)std::min(ctas, 16LL * sms), 128, 0, stream>>>(sp, pp, rows, cols, scale_log2);

@@ -1,0 +1,311 @@
+// sm_100a kernel for few query rows against many keys (decoding steps): O = softmax(Q K^T / sqrt(d)) V for at most
+// 16 * MT rows per head.
+//
+// Every key and value is read once and used by a handful of rows: the kernel is bound by HBM, not by the tensor pipe, and
+// what matters is that every SM has loads in flight all the time.  Hence no tensor memory and no roles: two CTAs of four
+// warps per SM, and every warp is a pipeline of its own -- it takes every fourth slab of its CTA's keys (8 KB: K and V rows
+// of 16 keys at d = 128, of 32 at d = 64), brings its slabs in by TMA through a private ring of kDecodeStages, and runs the
+// online softmax on them with the small matrix instruction (mma.m16n8k16), whose 16 rows are all that such a call has.  No
+// warp waits for another one before its keys are done.  The k CTAs of a head form a thread-block cluster: the warps'
+// partial (m, l, O) are merged first in the CTA, then through distributed shared memory, so no workspace is involved.
+#pragma once
+
+#include "attn_kernels.cuh"
+
+namespace attn {
+
+constexpr int kDecodeWarps = 4;
+constexpr int kDecodeStages = 3;           // 24 KB per warp, 192 KB of loads in flight per SM
+constexpr int kDecodeSlabBytes = 8192;
+constexpr int kDecodeMaxSplit = 16;        // CTAs per head (one cluster; above 8 only where the device allows it)
+enum : uint32_t { kRoleDecode = 9 };
+__host__ __device__ constexpr int decode_slab_keys(int d) { return kDecodeSlabBytes / (4 * d); }   // K and V, bf16
+
+struct DecodeParams {
+  const __nv_bfloat16* q;
+  __nv_bfloat16* o;
+  int Lq, Lk;
+  int cluster_k;           // CTAs per head
+  float scale_log2;        // log2(e) / sqrt(d)
+  unsigned int* status;    // as in FwdParams
+};
+
+template <int MT>
+struct DecodeMisc {
+  uint64_t full[kDecodeWarps][kDecodeStages];
+  float warp_m[kDecodeWarps][16 * MT], warp_l[kDecodeWarps][16 * MT];
+  float m[16 * MT], l[16 * MT];            // of the CTA; read by the other CTAs of the cluster
+  AbortCell abort;
+};
+template <int MT>
+__host__ __device__ constexpr int decode_smem_total() {
+  return kDecodeWarps * kDecodeStages * kDecodeSlabBytes + (int)sizeof(DecodeMisc<MT>);
+}
+
+__device__ __forceinline__ void ldmatrix4(uint32_t addr, uint32_t (&r)[4]) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
+}
+__device__ __forceinline__ void ldmatrix4_trans(uint32_t addr, uint32_t (&r)[4]) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
+}
+__device__ __forceinline__ void mma_16x8x16(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+  asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+               : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+               : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+__device__ __forceinline__ float4 ld_peer_f4(uint32_t peer_addr) {
+  float4 v;
+  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(peer_addr) : "memory");
+  return v;
+}
+__device__ __forceinline__ float ld_peer_f1(uint32_t peer_addr) {
+  float v;
+  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(peer_addr) : "memory");
+  return v;
+}
+// Weight of a part with reference m_part under the common reference m (a part without keys: -inf, weight 0).
+__device__ __forceinline__ float part_weight(float m_part, float m) { return m_part == -INFINITY ? 0.f : exp2f(m_part - m); }
+
+// HALF: at most 8 rows, so the accumulators' second eight rows hold nothing.
+template <int D, int MT, bool HALF>
+__global__ void __launch_bounds__(32 * kDecodeWarps, 2)
+attn_decode_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v, const DecodeParams p) {
+  static_assert(!HALF || MT == 1, "eight rows");
+  constexpr int kSlab = decode_slab_keys(D);
+  constexpr int KP = kSlab / 16;                      // 16-key groups of a slab
+  constexpr int kHalfBytes = kDecodeSlabBytes / 2;    // K, then V: [D / 64][kSlab][64] with 128-byte swizzle
+  constexpr int RH = HALF ? 1 : 2;                    // row halves (g, g + 8) that hold something
+  extern __shared__ __align__(1024) uint8_t smem_raw[];
+  const uint32_t smem_base = smem_u32(smem_raw);
+  DecodeMisc<MT>* misc = reinterpret_cast<DecodeMisc<MT>*>(smem_raw + kDecodeWarps * kDecodeStages * kDecodeSlabBytes);
+  volatile int* abort_flag = &misc->abort.flag;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int g = lane >> 2, t = lane & 3;              // row and column pair of this lane in an accumulator
+  const int k = p.cluster_k, head = blockIdx.x / k, rank = blockIdx.x % k;
+
+  if (threadIdx.x == 0) {
+    abort_cell_init(&misc->abort, p.status);
+    if (smem_base & 1023u) {                          // swizzled slabs need 1024-byte alignment
+      report_timeout(wait_info(kRoleDecode, 0, 0xFFFF), abort_flag);
+      misc->abort.flag = 1;
+    }
+    for (int w = 0; w < kDecodeWarps; ++w)
+      for (int s = 0; s < kDecodeStages; ++s) mbar_init(smem_u32(&misc->full[w][s]), 1);
+    fence_mbar_init();
+    prefetch_tmap(&tm_k);
+    prefetch_tmap(&tm_v);
+  }
+  __syncthreads();
+
+  // this CTA's slabs of the head's keys, every fourth of them this warp's
+  const int slabs = (p.Lk + kSlab - 1) / kSlab;
+  const int s_lo = (int)((long long)slabs * rank / k), s_hi = (int)((long long)slabs * (rank + 1) / k);
+  const int n = *abort_flag ? 0 : (s_hi - s_lo - warp + kDecodeWarps - 1) / kDecodeWarps;
+  const uint32_t ring = smem_base + warp * (kDecodeStages * kDecodeSlabBytes);
+  auto issue = [&](int it, int stage) {
+    const uint32_t dst = ring + stage * kDecodeSlabBytes, bar = smem_u32(&misc->full[warp][stage]);
+    const int key0 = (s_lo + warp + it * kDecodeWarps) * kSlab;
+    mbar_arrive_expect_tx(bar, kDecodeSlabBytes);
+#pragma unroll
+    for (int c = 0; c < D / 64; ++c) tma_load_3d(dst + c * (kSlab * 128), &tm_k, c * 64, key0, head, bar);
+#pragma unroll
+    for (int c = 0; c < D / 64; ++c) tma_load_3d(dst + kHalfBytes + c * (kSlab * 128), &tm_v, c * 64, key0, head, bar);
+  };
+  if (lane == 0)
+    for (int i = 0; i < kDecodeStages && i < n; ++i) issue(i, i);
+
+  // Q as A fragments; rows past Lq are zero
+  uint32_t qa[MT][D / 16][4];
+#pragma unroll
+  for (int mt = 0; mt < MT; ++mt)
+#pragma unroll
+    for (int kk = 0; kk < D / 16; ++kk)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const int row = mt * 16 + g + (e & 1) * 8, col = kk * 16 + t * 2 + (e >> 1) * 8;
+        qa[mt][kk][e] = 0u;
+        if (row < p.Lq && (!HALF || (e & 1) == 0))
+          qa[mt][kk][e] = *reinterpret_cast<const uint32_t*>(p.q + ((size_t)head * p.Lq + row) * D + col);
+      }
+  float acc[MT][D / 8][4];
+  float m_run[MT][2], l_run[MT][2];
+#pragma unroll
+  for (int mt = 0; mt < MT; ++mt) {
+#pragma unroll
+    for (int j = 0; j < D / 8; ++j)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) acc[mt][j][e] = 0.f;
+    m_run[mt][0] = m_run[mt][1] = -INFINITY;
+    l_run[mt][0] = l_run[mt][1] = 0.f;
+  }
+  // ldmatrix rows of this lane: matrix mi, row r of it
+  const int mi = lane >> 3, r = lane & 7;
+  const uint32_t k_row = (uint32_t)((mi >> 1) * 8 + r) * 128, v_row = (uint32_t)((mi & 1) * 8 + r) * 128;
+  int stage = 0;
+  uint32_t phase = 0;
+  for (int it = 0; it < n; ++it) {
+    if (!wait_bar_warp(smem_u32(&misc->full[warp][stage]), phase, abort_flag, wait_info(kRoleDecode, kBarKvFull, it))) break;
+    const uint32_t k_smem = ring + stage * kDecodeSlabBytes, v_smem = k_smem + kHalfBytes;
+    float s[MT][2 * KP][4];
+#pragma unroll
+    for (int mt = 0; mt < MT; ++mt)
+#pragma unroll
+      for (int j = 0; j < 2 * KP; ++j)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) s[mt][j][e] = 0.f;
+#pragma unroll
+    for (int kk = 0; kk < D / 16; ++kk)
+#pragma unroll
+      for (int kp = 0; kp < KP; ++kp) {
+        uint32_t b[4];
+        ldmatrix4(k_smem + (kk / 4) * (kSlab * 128) + kp * 2048 + k_row + (uint32_t)((((kk & 3) * 2 + (mi & 1)) ^ r) * 16), b);
+#pragma unroll
+        for (int mt = 0; mt < MT; ++mt) {
+          mma_16x8x16(s[mt][2 * kp], qa[mt][kk], b[0], b[1]);
+          mma_16x8x16(s[mt][2 * kp + 1], qa[mt][kk], b[2], b[3]);
+        }
+      }
+    // keys past the end of the sequence (zero-filled by TMA): score -inf
+    const int left = p.Lk - (s_lo + warp + it * kDecodeWarps) * kSlab;
+    if (left < kSlab) {
+#pragma unroll
+      for (int j = 0; j < 2 * KP; ++j)
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+          if (j * 8 + t * 2 + (e & 1) >= left)
+#pragma unroll
+            for (int mt = 0; mt < MT; ++mt) s[mt][j][e] = -INFINITY;
+    }
+    uint32_t pa[MT][KP][4];
+#pragma unroll
+    for (int mt = 0; mt < MT; ++mt) {
+      float alpha[2] = {1.f, 1.f};
+#pragma unroll
+      for (int h = 0; h < RH; ++h) {
+        float mx = fmaxf(s[mt][0][2 * h], s[mt][0][2 * h + 1]);
+#pragma unroll
+        for (int j = 1; j < 2 * KP; ++j) mx = max3(mx, s[mt][j][2 * h], s[mt][j][2 * h + 1]);
+        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
+        const float m_new = fmaxf(m_run[mt][h], mx * p.scale_log2);
+        const float ref = m_new == -INFINITY ? 0.f : m_new;     // no admissible score yet: weights 0, not NaN
+        alpha[h] = ex2_approx(m_run[mt][h] - ref);
+        m_run[mt][h] = m_new;
+        float sum = 0.f;
+#pragma unroll
+        for (int j = 0; j < 2 * KP; ++j) {
+          const float e0 = ex2_approx(fmaf(s[mt][j][2 * h], p.scale_log2, -ref));
+          const float e1 = ex2_approx(fmaf(s[mt][j][2 * h + 1], p.scale_log2, -ref));
+          sum += e0 + e1;
+          pa[mt][j / 2][(j & 1) * 2 + h] = pack_bf16x2(e0, e1);
+        }
+        l_run[mt][h] = l_run[mt][h] * alpha[h] + sum;           // this lane's share; the row's four lanes meet at the end
+      }
+      if (HALF) {
+#pragma unroll
+        for (int kp = 0; kp < KP; ++kp) pa[mt][kp][1] = pa[mt][kp][3] = 0u;
+      }
+      if (__any_sync(0xffffffffu, alpha[0] != 1.f || alpha[1] != 1.f)) {
+#pragma unroll
+        for (int j = 0; j < D / 8; ++j) {
+          acc[mt][j][0] *= alpha[0];
+          acc[mt][j][1] *= alpha[0];
+          if (!HALF) {
+            acc[mt][j][2] *= alpha[1];
+            acc[mt][j][3] *= alpha[1];
+          }
+        }
+      }
+    }
+#pragma unroll
+    for (int kp = 0; kp < KP; ++kp)
+#pragma unroll
+      for (int np = 0; np < D / 16; ++np) {
+        uint32_t b[4];
+        ldmatrix4_trans(v_smem + (np / 4) * (kSlab * 128) + kp * 2048 + v_row + (uint32_t)((((np & 3) * 2 + (mi >> 1)) ^ r) * 16), b);
+#pragma unroll
+        for (int mt = 0; mt < MT; ++mt) {
+          mma_16x8x16(acc[mt][2 * np], pa[mt][kp], b[0], b[1]);
+          mma_16x8x16(acc[mt][2 * np + 1], pa[mt][kp], b[2], b[3]);
+        }
+      }
+    __syncwarp();                                               // every lane has read the slab
+    if (lane == 0 && it + kDecodeStages < n) issue(it + kDecodeStages, stage);
+    if (++stage == kDecodeStages) { stage = 0; phase ^= 1u; }
+  }
+  if (*abort_flag) {                                            // a copy still in flight must land before the CTA exits
+    const long long t0 = clock64();
+    while (clock64() - t0 < 2000000LL) {}
+  }
+  __syncthreads();                                              // the rings are dead: they hold the partial results now
+
+  float* part = reinterpret_cast<float*>(smem_raw);             // [warp][row][D], then the CTA's own [row][D]
+  float* cta_o = part + kDecodeWarps * 16 * MT * D;
+#pragma unroll
+  for (int mt = 0; mt < MT; ++mt)
+#pragma unroll
+    for (int h = 0; h < RH; ++h) {
+      const int row = mt * 16 + h * 8 + g;
+      float l = l_run[mt][h];
+      l += __shfl_xor_sync(0xffffffffu, l, 1);
+      l += __shfl_xor_sync(0xffffffffu, l, 2);
+      if (row < p.Lq) {
+        if (t == 0) { misc->warp_m[warp][row] = m_run[mt][h]; misc->warp_l[warp][row] = l; }
+        float* dst = part + ((size_t)warp * 16 * MT + row) * D + t * 2;
+#pragma unroll
+        for (int j = 0; j < D / 8; ++j) *reinterpret_cast<float2*>(dst + j * 8) = make_float2(acc[mt][j][2 * h], acc[mt][j][2 * h + 1]);
+      }
+    }
+  __syncthreads();
+  const int units = p.Lq * (D / 4);                             // four columns of a row
+  for (int u = threadIdx.x; u < units; u += 32 * kDecodeWarps) {
+    const int row = u / (D / 4);
+    float m = -INFINITY;
+#pragma unroll
+    for (int w = 0; w < kDecodeWarps; ++w) m = fmaxf(m, misc->warp_m[w][row]);
+    float4 o4 = make_float4(0.f, 0.f, 0.f, 0.f);
+    float l = 0.f;
+#pragma unroll
+    for (int w = 0; w < kDecodeWarps; ++w) {
+      const float f = part_weight(misc->warp_m[w][row], m);
+      const float4 v = reinterpret_cast<const float4*>(part + (size_t)w * 16 * MT * D)[u];
+      l += f * misc->warp_l[w][row];
+      o4.x += f * v.x; o4.y += f * v.y; o4.z += f * v.z; o4.w += f * v.w;
+    }
+    reinterpret_cast<float4*>(cta_o)[u] = o4;
+    if (u % (D / 4) == 0) { misc->m[row] = m; misc->l[row] = l; }
+  }
+  if (k > 1) cluster_sync_release();
+  else __syncthreads();
+  // every CTA finishes its share of the head's output
+  const uint32_t o_addr = smem_u32(cta_o), m_addr = smem_u32(misc->m), l_addr = smem_u32(misc->l);
+  const int u_hi = (int)((long long)units * (rank + 1) / k);
+  for (int u = (int)((long long)units * rank / k) + threadIdx.x; u < u_hi; u += 32 * kDecodeWarps) {
+    const int row = u / (D / 4);
+    float m_q[kDecodeMaxSplit];
+    float m = -INFINITY;
+#pragma unroll
+    for (int q = 0; q < kDecodeMaxSplit; ++q) {
+      m_q[q] = q < k ? ld_peer_f1(map_to_cta(m_addr + row * 4, q)) : -INFINITY;
+      m = fmaxf(m, m_q[q]);
+    }
+    float4 o4 = make_float4(0.f, 0.f, 0.f, 0.f);
+    float l = 0.f;
+#pragma unroll
+    for (int q = 0; q < kDecodeMaxSplit; ++q) {                 // ascending key order
+      if (q >= k) break;
+      const float f = part_weight(m_q[q], m);
+      const float4 v = ld_peer_f4(map_to_cta(o_addr + u * 16, q));
+      l += f * ld_peer_f1(map_to_cta(l_addr + row * 4, q));
+      o4.x += f * v.x; o4.y += f * v.y; o4.z += f * v.z; o4.w += f * v.w;
+    }
+    const float inv = 1.0f / l;
+    *reinterpret_cast<uint2*>(p.o + (size_t)head * p.Lq * D + (size_t)u * 4) =
+        make_uint2(pack_bf16x2(o4.x * inv, o4.y * inv), pack_bf16x2(o4.z * inv, o4.w * inv));
+  }
+  if (k > 1) cluster_sync_release();                            // no CTA leaves while a peer may still read its part
+}
+
+}  // namespace attn

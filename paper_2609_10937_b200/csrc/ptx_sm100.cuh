@@ -297,6 +297,11 @@ __device__ __forceinline__ void tma_load_3d_pair(uint32_t dst_smem, const CUtens
 // fence.mbarrier_init.release.cluster)
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+// Barrier of the whole cluster that also makes this CTA's shared-memory writes visible to its peers.
+__device__ __forceinline__ void cluster_sync_release() {
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  cluster_wait();
+}
 // Address of the same shared-memory location in CTA `rank` of this cluster.
 __device__ __forceinline__ uint32_t map_to_cta(uint32_t smem_addr, uint32_t rank) {
   uint32_t r;

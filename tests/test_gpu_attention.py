@@ -795,3 +795,27 @@ def test_very_long_single_head(env, L, d):
     assert len(rows) >= 256
     _run_and_compare(env, case, binding.forward, rows=rows)
     _run_and_compare(env, case, lambda q, k, v: binding.forward(q, k, v, causal=True), rows=rows[::4], causal=True)
+
+
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("B,H,Lq,Lk", [
+    (1, 1, 1, 256), (1, 1, 8, 255), (1, 3, 9, 257), (2, 5, 16, 1), (1, 2, 16, 15), (1, 2, 3, 17), (3, 1, 5, 4097),
+    (1, 40, 2, 700), (8, 32, 1, 64), (4, 40, 1, 300), (1, 1, 1, 16384), (1, 5, 7, 9000), (2, 16, 15, 2048), (8, 40, 4, 500),
+    (1, 7, 17, 1000), (1, 150, 24, 1030), (5, 33, 32, 1025), (1, 2, 32, 33)])
+def test_few_query_rows_against_many_keys(env, B, H, Lq, Lk, d):
+    """Calls with at most 32 query rows: both sides of 8, 16 and 32 rows, of one slab of keys per warp, of every split of a
+    head (1 to 16 CTAs) and more heads than CTAs fit at once; NaN-filled output, every element against the oracle."""
+    torch, orc, binding = env
+    rng = np.random.default_rng([B, H, Lq, Lk, d, 3])
+    bits = lambda *shape: synth.f32_to_bf16_bits((rng.standard_normal(shape) * 1.5).astype(np.float32))
+    q, k, v = bits(B * H, Lq, d), bits(B * H, Lk, d), bits(B * H, Lk, d)
+    out = torch.full((B, H, Lq, d), float("nan"), dtype=torch.bfloat16, device="cuda")
+    dev = [to_cuda_bf16(x).view(B, H, -1, d) for x in (q, k, v)]
+    binding.forward_qk(*dev, out)
+    torch.cuda.synchronize()
+    assert binding.last_device_status()[0] == 0
+    qd, kd, vd = (x.double() for x in dev)
+    ref = (torch.softmax(qd @ kd.transpose(2, 3) / d ** 0.5, dim=-1) @ vd).cpu().numpy()
+    assert_close(to_host_f64(out).reshape(ref.shape), ref, f"{B} {H} {Lq} {Lk} {d}")
+    again = binding.forward_qk(*dev)
+    assert torch.equal(again.view(torch.int16), out.view(torch.int16))
