@@ -239,6 +239,8 @@ int attn_status_read(uint32_t *status_dev, void *workspace, void *cuda_stream, u
  * operator is the case Lq == Lk; a block of query rows of a longer sequence is the case
  * q = Q + r0 * d, Lq = rows in the block (what attn_forward_host uses to overlap copies with
  * compute).  attn_plan_qk is the derivation for it (tiles from Lq, key steps from Lk).
+ * Few rows (up to 16; up to 32 at d = 64 and for many long heads) with Lq != Lk run in a kernel of their own that streams
+ * the keys; the CTAs of a head are then one cluster (attn_last_cluster_size) and no workspace is touched.
  * Errors as attn_forward.
  */
 int attn_plan_qk(const attn_hw_desc *desc, int B, int H, int Lq, int Lk, int d, attn_tiles *out);
@@ -251,6 +253,7 @@ int attn_forward_qk(const void *q, const void *k, const void *v, void *o,
  * that masked elements are -inf, never zero, Section "Online Softmax", applied to
  * a triangular mask; the paper itself evaluates non-causal attention only).
  * Key steps wholly after a Q tile's last row are skipped, not computed and masked.
+ * Where it is faster, a plan of equal ranges is executed as whole tiles, longest first (the tiles then need no merge).
  * Always needs a registered workspace (attn_workspace_bytes of attn_plan_ex(...,1,...)).
  */
 int attn_forward_causal(const void *q, const void *k, const void *v, void *o,

@@ -17,6 +17,7 @@
 #include "decode_kernels.cuh"
 #include "gemm.h"
 #include "gemm_kernels.cuh"
+#include "tiles_kernel.cuh"
 
 namespace {
 
@@ -382,10 +383,62 @@ int dispatch_decode(const void* q, const void* k, const void* v, void* o, int BH
   return ATTN_ERR_UNSUPPORTED_SHAPE;
 }
 
+// Causal attention as whole Q tiles, one CTA each (tiles_kernel.cuh).
+template <int D>
+int launch_causal_tiles(const void* q, const void* k, const void* v, void* o, int BH, int L, int local_mem, unsigned int* status,
+                        DeviceState* st, cudaStream_t stream) {
+  using SM = attn::TilesSmem<D>;
+  CUtensorMap tq, tk, tv, to;
+  int rc;
+  if ((rc = make_tmap(&tq, q, BH, L, D, attn::kSub)) != ATTN_OK) return rc;
+  if ((rc = make_tmap(&tk, k, BH, L, D, 128)) != ATTN_OK) return rc;
+  if ((rc = make_tmap(&tv, v, BH, L, D, 128)) != ATTN_OK) return rc;
+  if ((rc = make_tmap(&to, o, BH, L, D, 32)) != ATTN_OK) return rc;    // every warp stores its own 32 rows
+  attn::TilesParams p;
+  p.L = L;
+  p.q_tiles = (L + 2 * attn::kSub - 1) / (2 * attn::kSub);
+  p.heads = BH;
+  // Heads dealt out together: equal groups whose K and V take at most a third of the cache (32 heads of 8192, d = 128: 220 MB
+  // read from DRAM in groups of ten, 828 MB with 148 ranges that each walk a head of their own).  Equal, because a short
+  // last group would start its longest tiles when most CTAs have run dry.
+  const long long at_most = std::max(1LL, st->desc.cache_bytes / (3 * 4LL * L * D));
+  const long long groups = (BH + at_most - 1) / at_most;
+  p.group_heads = (int)((BH + groups - 1) / groups);
+  p.stages = std::min(attn::kMaxStages, (local_mem - SM::total(0)) / SM::kStageBytes);
+  p.scale_log2 = (float)(1.4426950408889634 / std::sqrt((double)D));
+  p.status = status;
+  const int smem = SM::total(p.stages);
+  auto kern = attn::attn_causal_tiles_kernel<D>;
+  ATTN_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  kern<<<(unsigned)(BH * p.q_tiles), 512, smem, stream>>>(tq, tk, tv, to, p);
+  ATTN_CUDA_TRY(cudaGetLastError());
+  t_cluster_size = 0;
+  t_launch_count = 1;
+  return ATTN_OK;
+}
+
+// Whether a causal plan of equal ranges runs as whole tiles instead.  Longest first, whole tiles take the longest tile's steps
+// or an even share of all steps, one more per tile, whichever is more; 5 for the start and the end.  Measured (us, ranges /
+// whole tiles): 128 heads x 4096, d = 128 625 / 501; 32 x 1111, d = 64 36 / 20; 16 x 4096, d = 128 88 / 66; where the longest
+// tile decides, ranges stay: 8 x 4096 55 / (33 steps of 2) 66.  (Four ring stages: the MMA warp looks that far ahead.)
+bool causal_whole_tiles(const attn_tiles& t, int BH, int L, int d, int local_mem, int sms) {
+  if (!t.causal || t.n_q != 2 || t.tile_kv != 128) return false;
+  if (local_mem < (d == 64 ? attn::TilesSmem<64>::total(4) : attn::TilesSmem<128>::total(4))) return false;
+  if (t.ctas % t.tiles == 0 && t.ctas > t.tiles) return false;      // clusters that share out each tile's own steps
+  const int steps = (L + 127) / 128;
+  const long long units = BH * attn_internal::head_units((L + 255) / 256, steps, 2, 1);
+  const long long even = (units + t.tiles + sms - 1) / sms;
+  return std::max<long long>(steps, even) + 5 <= t.cost_steps;
+}
+
 int dispatch_fwd(const void* q, const void* k, const void* v, void* o, int B, int H, int L, int d,
                  const attn_tiles& t, float* ws, unsigned int* status, DeviceState* st, cudaStream_t s, int Lk = 0,
-                 bool may_overlap = false) {
+                 bool may_overlap = false, const attn_hw_desc* own_plan_of = nullptr) {
   if (Lk == 0) Lk = L;
+  // (a plan made here, not one that a caller has changed)
+  if (own_plan_of && Lk == L && causal_whole_tiles(t, B * H, L, d, own_plan_of->local_mem_bytes, st->desc.num_units))
+    return d == 128 ? launch_causal_tiles<128>(q, k, v, o, B * H, L, own_plan_of->local_mem_bytes, status, st, s)
+                    : launch_causal_tiles<64>(q, k, v, o, B * H, L, own_plan_of->local_mem_bytes, status, st, s);
 #define ATTN_CASE(D_, TKV_, NQ_) \
   if (d == D_ && t.tile_kv == TKV_ && t.n_q == NQ_) \
     return launch_fwd<D_, TKV_, NQ_>(q, k, v, o, B, H, L, Lk, t, ws, status, st, s, may_overlap);
@@ -489,7 +542,7 @@ int forward_impl(const void* q, const void* k, const void* v, void* o, int B, in
   if (!ovr && !plan_desc && !call_ws && Lk != L && decode_rows(L, Lk, d, t, st->desc.num_units))
     return dispatch_decode(q, k, v, o, B * H, L, Lk, d, nullptr, st, static_cast<cudaStream_t>(cuda_stream));
   return dispatch_fwd(q, k, v, o, B, H, L, d, t, ws, call_ws ? call_ws->status : nullptr, st,
-                      static_cast<cudaStream_t>(cuda_stream), Lk, call_ws != nullptr);
+                      static_cast<cudaStream_t>(cuda_stream), Lk, call_ws != nullptr, ovr ? nullptr : &desc);
 }
 
 template <int D, int TKV>

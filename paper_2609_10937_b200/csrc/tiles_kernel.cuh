@@ -1,0 +1,641 @@
+// attn_causal_tiles_kernel: the fused attention step loop of attn_kernels.cuh for causal grids in which every Q tile is worked on
+// by one CTA from its first key to its last (nothing to merge).
+//
+// What it has over attn_fwd_kernel is a pipeline that does not stop between tiles.  There, the softmax warps finish a tile
+// themselves: they wait for its last product, normalise and store, and only then start on the next tile's scores -- about
+// 5.7 us per tile on the causal shapes, as much as three key steps.  Here
+//   * the correction warpgroup finishes a tile (tensor memory -> bf16 -> TMA store) while the softmax warps are already on the
+//     next tile's first scores: the MMA warp issues a sub-tile's first product of the next tile in the very slot in which it
+//     would have issued that sub-tile's next step, so a change of tile looks like one more step to every role;
+//   * the two sub-tiles of a tile have step counts of their own: causal sub-tile 0 does not run the last key step, which lies
+//     wholly after its rows, and a sub-tile past the end of the sequence does not run at all;
+//   * CTAs take their next tile from the hardware's queue of CTAs not yet started (clusterlaunchcontrol.try_cancel), one
+//     tile ahead, so that unequal (causal) tiles even out without a counter in memory: the tiles are launched longest first
+//     within groups of heads whose K and V stay in L2.
+// Roles, barriers and the arithmetic of a step are those of attn_fwd_kernel (128-key tiles, two sub-tiles of 128 rows).
+#pragma once
+
+#include "attn_kernels.cuh"
+
+namespace attn {
+
+struct TilesParams {
+  int L;                   // query rows and keys per head
+  int q_tiles;             // Q tiles per head = ceil(L / 256)
+  int heads;               // B * H
+  int group_heads;         // heads whose tiles are dealt out together, longest first
+  int stages;              // ring depth
+  float scale_log2;        // log2(e) / sqrt(d)
+  unsigned int* status;    // as in FwdParams
+};
+
+template <int D>
+struct TilesSmem {
+  static constexpr int kQBufs = D == 64 ? 2 : 1;                 // Q tiles in shared memory
+  static constexpr int kSubBytes = kSub * D * 2;
+  static constexpr int kQBytes = kQBufs * 2 * kSubBytes;
+  static constexpr int kStageBytes = 128 * D * 2;
+  static constexpr int kOutBytes = 8 * 4096;                     // two [32 rows][64 columns] bf16 chunks per correction warp
+  static constexpr int kMiscBytes = D == 64 ? 4096 : 3072;
+  __host__ __device__ static constexpr int total(int stages) { return kQBytes + stages * kStageBytes + kOutBytes + kMiscBytes; }
+};
+
+constexpr int kSchedReaders = 14;          // warps that read a tile's index: 8 softmax, 4 correction, MMA, TMA
+template <int D>
+struct TilesMisc {
+  // d = 64 stores a step's factor before it knows that the factor of the step before has been read
+  static constexpr int kAlphaBufs = D == 64 ? 2 : 1;
+  float alpha[2][kAlphaBufs][kSub];        // [sub-tile][step mod kAlphaBufs][row] rescale factor
+  float inv[2][kSub];                      // [sub-tile][row] 1 / denominator of a finished tile
+  uint4 sched[2];              // answers of try_cancel (16 bytes each)
+  uint64_t sched_full[2], sched_empty[2];
+  uint64_t q_full[2][2], q_empty[2][2];    // [sub-tile][buffer]
+  uint64_t kv_full[kMaxStages], kv_empty[kMaxStages];
+  uint64_t s_full[2], s_free[2], p_full[2], p_half[2], o_full[2], alpha_full[2], fin_full[2];
+  AbortCell abort;
+  uint32_t tmem_slot;
+};
+static_assert(sizeof(TilesMisc<64>) <= TilesSmem<64>::kMiscBytes && sizeof(TilesMisc<128>) <= TilesSmem<128>::kMiscBytes, "misc region too large");
+
+// Asks for the index of a CTA of this grid that has not been started; the 16-byte answer is counted on `bar`.
+__device__ __forceinline__ void clc_try_cancel(uint32_t answer_smem, uint32_t bar) {
+  asm volatile("clusterlaunchcontrol.try_cancel.async.shared::cta.mbarrier::complete_tx::bytes.b128 [%0], [%1];"
+               ::"r"(answer_smem), "r"(bar) : "memory");
+}
+// The CTA index in an answer, or -1: none left.
+__device__ __forceinline__ int clc_answer(uint32_t answer_smem) {
+  int got, x;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t.reg .b128 a;\n\t"
+      "ld.shared.b128 a, [%2];\n\t"
+      "clusterlaunchcontrol.query_cancel.is_canceled.pred.b128 p, a;\n\t"
+      "selp.s32 %0, 1, 0, p;\n\t"
+      "mov.b32 %1, 0;\n\t"
+      "@p clusterlaunchcontrol.query_cancel.get_first_ctaid::x.b32.b128 %1, a;\n\t}"
+      : "=r"(got), "=r"(x) : "r"(answer_smem) : "memory");
+  return got ? x : -1;
+}
+
+// A tile: its head, first row and the key steps of its two sub-tiles (n[1] is n[0], n[0] + 1 or 0; n[0] > 0).
+struct TileWork {
+  int bh, q_row0, n0, n1;
+  __device__ __forceinline__ int steps(int i) const { return i ? n1 : n0; }
+  __device__ __forceinline__ int steps() const { return n1 > n0 ? n1 : n0; }
+};
+__device__ __forceinline__ TileWork tile_work(int index, const TilesParams& p) {
+  TileWork w;
+  const int per_group = p.group_heads * p.q_tiles;
+  const int group = index / per_group, r = index - group * per_group;
+  const int first = group * p.group_heads;
+  const int n = p.heads - first < p.group_heads ? p.heads - first : p.group_heads;
+  const int q = p.q_tiles - 1 - r / n;
+  w.bh = first + r % n;
+  w.q_row0 = q * 2 * kSub;
+  // a sub-tile's last key step is the one that holds its own rows
+  w.n0 = 2 * q + 1;
+  w.n1 = w.q_row0 + kSub >= p.L ? 0 : 2 * q + 2;
+  return w;
+}
+
+template <int D>
+__global__ void __launch_bounds__(512, 1)
+attn_causal_tiles_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
+                  const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_o, const TilesParams p) {
+  constexpr int TKV = 128, NCH = TKV / 32, KCH = D / 64;
+  constexpr bool kSplitP = D == 64;                   // P in tensor-memory columns of its own (see attn_fwd_kernel)
+  constexpr int O_COL0 = 2 * TKV, P_COL0 = 2 * (TKV + D);
+  constexpr int kPoly = kPolyPairsPer8;
+  using SM = TilesSmem<D>;
+  constexpr int QB = SM::kQBufs;
+
+  extern __shared__ __align__(1024) uint8_t smem_raw[];
+  const uint32_t smem_base = smem_u32(smem_raw);
+  const uint32_t ring_smem = smem_base + SM::kQBytes;
+  const uint32_t out_smem = ring_smem + p.stages * SM::kStageBytes;
+  using Misc = TilesMisc<D>;
+  Misc* const misc = reinterpret_cast<Misc*>(smem_raw + SM::kQBytes + p.stages * SM::kStageBytes + SM::kOutBytes);
+  volatile int* abort_flag = &misc->abort.flag;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+
+  if (threadIdx.x == 0) {
+    abort_cell_init(&misc->abort, p.status);
+    if (smem_base & 1023u) {                          // swizzled tiles need 1024-byte alignment
+      note_timeout(wait_info(kRoleLoad, 0, 0xFFFF), &misc->abort.flag);
+    }
+    for (int s = 0; s < kMaxStages; ++s) {
+      mbar_init(smem_u32(&misc->kv_full[s]), 1);
+      mbar_init(smem_u32(&misc->kv_empty[s]), 1);
+    }
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(smem_u32(&misc->sched_full[i]), 1);
+      mbar_init(smem_u32(&misc->sched_empty[i]), kSchedReaders);
+      for (int b = 0; b < 2; ++b) {
+        mbar_init(smem_u32(&misc->q_full[i][b]), 1);
+        mbar_init(smem_u32(&misc->q_empty[i][b]), 1);
+      }
+      mbar_init(smem_u32(&misc->s_full[i]), 1);
+      mbar_init(smem_u32(&misc->s_free[i]), kSub);
+      mbar_init(smem_u32(&misc->p_full[i]), 2 * kSub);          // softmax rows + correction rows
+      mbar_init(smem_u32(&misc->p_half[i]), kSub);
+      mbar_init(smem_u32(&misc->o_full[i]), 1);
+      mbar_init(smem_u32(&misc->alpha_full[i]), kSub);
+      mbar_init(smem_u32(&misc->fin_full[i]), kSub);
+    }
+    fence_mbar_init();
+    prefetch_tmap(&tm_q);
+    prefetch_tmap(&tm_k);
+    prefetch_tmap(&tm_v);
+    prefetch_tmap(&tm_o);
+  }
+  if (warp == 15) {
+    tmem_alloc(smem_u32(&misc->tmem_slot), 512);
+    tmem_relinquish();
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem_base = misc->tmem_slot;
+  const bool run = *const_cast<volatile int*>(&misc->abort.flag) == 0;
+
+  // Index of this CTA's tile number `s` (s >= 1; tile 0 is blockIdx.x), -1 after the last, -2 if a wait expired.  Every
+  // role's warp calls it once per s, with all lanes.
+  auto next_tile = [&](int s, uint32_t role) __attribute__((always_inline)) -> int {
+    const int slot = s & 1;
+    if (!wait_quiet_warp(smem_u32(&misc->sched_full[slot]), ((s - 1) >> 1) & 1, abort_flag, wait_info(role, kBarSync, s))) return -2;
+    const int x = clc_answer(smem_u32(&misc->sched[slot]));
+    fence_proxy_async_smem();                         // the answer has been read: the next one may be written there
+    __syncwarp();
+    if (lane == 0) mbar_arrive(smem_u32(&misc->sched_empty[slot]));
+    return x;
+  };
+
+  if (warp < 8) {
+    // ===================================================== softmax warpgroup
+    setmaxnreg_inc<192>();
+    const int i = warp >> 2;
+    const int row = (warp & 3) * 32 + lane;
+    const uint32_t lane_base = tmem_base + ((uint32_t)((warp & 3) * 32) << 16);
+    const uint32_t s_tmem = lane_base + i * TKV;
+    const uint32_t p_tmem = kSplitP ? lane_base + P_COL0 + i * (TKV / 2) : s_tmem;   // else P aliases the front of S
+    const uint32_t bar_s = smem_u32(&misc->s_full[i]);
+    const uint32_t bar_p = smem_u32(&misc->p_full[i]);
+    const uint32_t bar_h = smem_u32(&misc->p_half[i]);
+    const uint32_t bar_a = smem_u32(&misc->alpha_full[i]);
+    const float scale = p.scale_log2;
+    const ExpConsts ek = make_exp_consts(scale);
+    bool ok = run;
+    uint32_t g = 0;                                    // steps of this sub-tile over all tiles
+    int tile = blockIdx.x;
+    for (int seq = 1; ok && tile >= 0; ++seq) {
+      const TileWork w = tile_work(tile, p);
+      const int n = w.steps(i);
+      if (n > 0) {
+        float m_run = -INFINITY, delta = 0.f;
+        const uint32_t g_seg0 = g;                     // this tile's first step
+        // One key step.  The masked variant (the causal diagonal) is compiled separately so that
+        // the common step pays nothing for it; `lim` is the last key column the thread's row may attend to.
+        auto softmax_step = [&](auto mask_tag, int lim) __attribute__((always_inline)) -> bool {
+          constexpr bool kMasked = decltype(mask_tag)::value;
+          if (!wait_quiet_warp(bar_s, g & 1, abort_flag, wait_info(kRoleSoftmax, kBarSFull, g))) return false;
+          tc_fence_after();
+          uint32_t s[TKV];
+          // load the row in two halves: the maximum of the first half is taken while the second is in flight
+#pragma unroll
+          for (int c = 0; c < NCH / 2; ++c) tmem_ld32_nowait(s_tmem + c * 32, *reinterpret_cast<uint32_t(*)[32]>(&s[c * 32]));
+#pragma unroll
+          for (int c = 0; c < NCH / 2; ++c) tmem_ld_fence(*reinterpret_cast<uint32_t(*)[32]>(&s[c * 32]));
+#pragma unroll
+          for (int c = NCH / 2; c < NCH; ++c) tmem_ld32_nowait(s_tmem + c * 32, *reinterpret_cast<uint32_t(*)[32]>(&s[c * 32]));
+          // keys after the query's position: score -inf, never zero
+          if constexpr (kMasked) {
+#pragma unroll
+            for (int k = 0; k < TKV / 2; ++k)
+              if (k > lim) s[k] = 0xFF800000u;
+          }
+          const float mx_a = fmaxf(fmaxf(chain_max<0, TKV / 8>(s), chain_max<TKV / 8, TKV / 4>(s)),
+                                   fmaxf(chain_max<TKV / 4, 3 * TKV / 8>(s), chain_max<3 * TKV / 8, TKV / 2>(s)));
+#pragma unroll
+          for (int c = NCH / 2; c < NCH; ++c) tmem_ld_fence(*reinterpret_cast<uint32_t(*)[32]>(&s[c * 32]));
+          if constexpr (kSplitP) {
+            tc_fence_before();
+            mbar_arrive(smem_u32(&misc->s_free[i]));   // the scores are in registers: the buffer may be overwritten
+          }
+          if constexpr (kMasked) {
+#pragma unroll
+            for (int k = TKV / 2; k < TKV; ++k)
+              if (k > lim) s[k] = 0xFF800000u;
+          }
+          const float mx_b = fmaxf(fmaxf(chain_max<TKV / 2, 5 * TKV / 8>(s), chain_max<5 * TKV / 8, 3 * TKV / 4>(s)),
+                                   fmaxf(chain_max<3 * TKV / 4, 7 * TKV / 8>(s), chain_max<7 * TKV / 8, TKV>(s)));
+          const float mx = fmaxf(mx_a, mx_b);
+          // lazy rescale, as in attn_fwd_kernel
+          const float m_cand = kMasked ? fmaxf(fmaxf(m_run, mx * scale), -1e30f) : fmaxf(m_run, mx * scale);
+          const float gap = m_cand - m_run;
+          const float shrink = ex2_approx(-gap);
+          const bool move = (gap > kRescaleThreshold) || (gap > 0.f && kDominanceFactor > delta * shrink);
+          const float m_new = move ? m_cand : m_run;
+          const float alpha = move ? shrink : 1.0f;
+          misc->alpha[i][g % Misc::kAlphaBufs][row] = alpha;
+          if constexpr (kSplitP) {
+            // P's columns must have been read by the previous step's P V, and every arrival of this step must come after
+            // it (attn_fwd_kernel says why); a tile's first step is covered by the wait at the end of the tile before
+            if (g != g_seg0) {
+              if (!wait_quiet_warp(smem_u32(&misc->o_full[i]), (g - 1) & 1, abort_flag, wait_info(kRoleSoftmax, kBarOFull, 0x4000 | g))) return false;
+              tc_fence_after();
+            }
+          }
+          mbar_arrive(bar_a);
+          const uint64_t neg_m2 = pack_f32x2(-m_new, -m_new);
+          uint64_t sum_a = 0ull, sum_b = 0ull;         // packed (0.f, 0.f)
+          uint32_t pk[16];
+          // first half of the row: the second product may start on it while the rest is computed
+#pragma unroll
+          for (int c = 0; c < NCH / 2; ++c) {
+            exp_chunk<kPoly>(&s[c * 32], ek, neg_m2, sum_a, pk);
+            tmem_st16(p_tmem + c * 16, pk);
+          }
+          uint32_t pk2[16];
+          exp_chunk<kPoly>(&s[(NCH / 2) * 32], ek, neg_m2, sum_b, pk2);
+          tmem_wait_st();
+          tc_fence_before();
+          mbar_arrive(bar_p);
+          tmem_st16(p_tmem + (NCH / 2) * 16, pk2);
+#pragma unroll
+          for (int c = NCH / 2 + 1; c < NCH; ++c) {
+            exp_chunk<kPoly>(&s[c * 32], ek, neg_m2, sum_b, pk);
+            tmem_st16(p_tmem + c * 16, pk);
+          }
+          float sa0, sa1, sb0, sb1;
+          unpack_f32x2(sum_a, sa0, sa1);
+          unpack_f32x2(sum_b, sb0, sb1);
+          delta = delta * alpha + ((sa0 + sa1) + (sb0 + sb1));
+          m_run = m_new;
+          tmem_wait_st();
+          tc_fence_before();
+          mbar_arrive(bar_h);
+          return true;
+        };
+        for (int jj = 0; ok && jj < n; ++jj, ++g) {
+          // Only the last step needs a mask: the diagonal, which starts at the sub-tile's first row and ends, in a ragged
+          // last key tile, before the padding for every row of the sequence.
+          if (jj == n - 1) ok = softmax_step(MaskTag<true>{}, row);
+          else ok = softmax_step(MaskTag<false>{}, TKV - 1);
+        }
+        if (!ok) break;
+        // The denominators go to the correction warpgroup, which finishes the tile.  Its arrival on p_full of a tile's first
+        // step says that it has read those of the tile before; from two steps on, the second step's scores come after it.  A
+        // tile of one step waits for its only product instead, and so does d = 64 always (see softmax_step).
+        if (kSplitP || n == 1) {
+          ok = wait_quiet_warp(smem_u32(&misc->o_full[i]), (g - 1) & 1, abort_flag, wait_info(kRoleSoftmax, kBarOFull, g));
+          if (!ok) break;
+          tc_fence_after();
+        }
+        misc->inv[i][row] = 1.0f / delta;
+        mbar_arrive(smem_u32(&misc->fin_full[i]));
+      }
+      tile = next_tile(seq, kRoleSoftmax);
+    }
+  } else if (warp < 12) {
+    // ================================================== correction warpgroup
+    setmaxnreg_dec<64>();
+    const int wq = warp & 3, row = wq * 32 + lane;
+    const uint32_t lane_base = tmem_base + ((uint32_t)(wq * 32) << 16);
+    const uint32_t stage_w = out_smem + wq * 8192;     // this warp's two staging chunks
+    bool ok = run;
+    // steps of the sub-tiles; in bit i: sub-tile i's finished tiles mod 2, whether one waits for its epilogue (arrays would be
+    // indexed at run time and live in local memory)
+    uint32_t g0 = 0, g1 = 0, fin = 0, pending = 0, chunk_ctr = 0;
+    int out_bh = 0, out_row0 = 0;                      // of the finished tile
+    // A tile's end: normalise this warp's 32 rows of sub-tile i, 64 columns at a time through its two staging chunks in turn.
+    auto finish = [&](int i) __attribute__((always_inline)) -> bool {
+      if (!wait_quiet_warp(smem_u32(&misc->fin_full[i]), (fin >> i) & 1, abort_flag, wait_info(kRoleCorrection, kBarAlpha, 0x8000))) return false;
+      const float inv = misc->inv[i][row];
+      fin ^= 1u << i;
+      if (!wait_quiet_warp(smem_u32(&misc->o_full[i]), ((i ? g1 : g0) - 1) & 1, abort_flag, wait_info(kRoleCorrection, kBarOFull, 0x8000))) return false;
+      tc_fence_after();
+      const uint32_t o_tmem = lane_base + O_COL0 + i * D;
+#pragma unroll 1
+      for (int h = 0; h < KCH; ++h, ++chunk_ctr) {
+        const uint32_t dst = stage_w + (chunk_ctr & 1) * 4096;
+        // the store that last read this chunk (two chunks ago) must have finished reading it
+        if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
+        __syncwarp();
+#pragma unroll 1
+        for (int c = 0; c < 2; ++c) {
+          uint32_t r[32];
+          float v[32];
+          tmem_ld32(o_tmem + h * 64 + c * 32, r);
+#pragma unroll
+          for (int k = 0; k < 32; ++k) v[k] = __uint_as_float(r[k]) * inv;
+          stage_row_chunk(dst, c, lane, v);
+        }
+        fence_proxy_async_smem();
+        __syncwarp();
+        if (lane == 0) {                               // (rows past the end of the sequence are clipped by the tensor map)
+          tma_store_3d(&tm_o, dst, h * 64, out_row0 + i * kSub + wq * 32, out_bh);
+          tma_store_commit();
+        }
+      }
+      tc_fence_before();                               // O has been read: this thread's next arrival on p_full says so
+      pending &= ~(1u << i);
+      return true;
+    };
+    int tile = blockIdx.x;
+    for (int seq = 1; ok && tile >= 0; ++seq) {
+      const TileWork w = tile_work(tile, p);
+      const int n = w.steps();
+      for (int j = 0; ok && j < n; ++j) {
+#pragma unroll 1
+        for (int i = 0; i < 2; ++i) {
+          if (j == 0 && ((pending >> i) & 1) && !finish(i)) { ok = false; break; }
+          if (j >= (i ? w.n1 : w.n0)) continue;
+          const uint32_t gi = i ? g1 : g0;
+          if (!wait_quiet_warp(smem_u32(&misc->alpha_full[i]), gi & 1, abort_flag, wait_info(kRoleCorrection, kBarAlpha, j))) { ok = false; break; }
+          const float a = misc->alpha[i][gi % Misc::kAlphaBufs][row];
+          if (j > 0) {                                 // a tile's first step starts O afresh
+            const bool need = __any_sync(0xffffffffu, a != 1.0f);
+            if (need) {
+              if (!wait_quiet_warp(smem_u32(&misc->o_full[i]), (gi - 1) & 1, abort_flag, wait_info(kRoleCorrection, kBarOFull, j))) { ok = false; break; }
+              tc_fence_after();
+              const uint32_t o_tmem = lane_base + O_COL0 + i * D;
+              // (16 columns at a time: 32 make this role spill)
+#pragma unroll 1
+              for (int c = 0; c < D / 16; ++c) {
+                uint32_t r[16];
+                tmem_ld16(o_tmem + c * 16, r);
+#pragma unroll
+                for (int k = 0; k < 16; ++k) r[k] = __float_as_uint(__uint_as_float(r[k]) * a);
+                tmem_st16(o_tmem + c * 16, r);
+              }
+              tmem_wait_st();
+            }
+            tc_fence_before();
+          }
+          mbar_arrive(smem_u32(&misc->p_full[i]));
+          if (i) ++g1; else ++g0;
+        }
+      }
+      if (!ok) break;
+      pending = (w.n0 > 0 ? 1u : 0u) | (w.n1 > 0 ? 2u : 0u);
+      out_bh = w.bh;
+      out_row0 = w.q_row0;
+      tile = next_tile(seq, kRoleCorrection);
+    }
+#pragma unroll 1
+    for (int i = 0; i < 2; ++i)
+      if (ok && tile == -1 && ((pending >> i) & 1)) ok = finish(i);
+    if (lane == 0) tma_store_wait_read();              // shared memory is read by the stores until here
+    __syncwarp();
+  } else if (warp == 12) {
+    // ============================================================ MMA issuer (the whole warp walks the loop, one lane issues)
+    setmaxnreg_dec<64>();
+    bool ok = run;
+    // (no arrays indexed at run time here: they would live in local memory, whose latency this warp passes on to every step)
+    uint32_t gp = 0;                                   // bit i: steps of sub-tile i whose P V has been issued, mod 2
+    uint32_t uses = 0;                                 // bits 8 i, 8 i + 1: Q loads of sub-tile i that have been read, mod 4
+    int vs = 1 % p.stages;                             // ring position of V_j
+    uint32_t vph = 0;
+    auto wait = [&](uint64_t* bar, uint32_t parity, uint32_t id, uint32_t tag) __attribute__((always_inline)) -> bool {
+      if (!wait_quiet_warp(smem_u32(bar), parity, abort_flag, wait_info(kRoleMma, id, tag))) { ok = false; return false; }
+      tc_fence_after();
+      return true;
+    };
+    // A product S_i = Q_i K^T that is ready to be issued: its operands have arrived.
+    struct Scores { int st, b; bool go, last, release; };
+    // Waits for the operands: the K tile at ring position st and, for the first product of a tile, its Q.  last: no later
+    // step reads this Q; release: no other sub-tile reads this K tile any more.
+    auto ready = [&](int i, int st, uint32_t ph, bool first, bool last, bool release) __attribute__((always_inline)) -> Scores {
+      Scores sc = {st, 0, false, last, release};
+      if (!wait(&misc->kv_full[st], ph, kBarKvFull, i)) return sc;
+      if (first) {
+        const uint32_t u = uses >> (8 * i);
+        if (!wait(&misc->q_full[i][QB == 2 ? u & 1 : 0], QB == 2 ? (u >> 1) & 1 : u & 1, kBarQ, i)) return sc;
+        uses = (uses & ~(3u << (8 * i))) | (((u + 1) & 3u) << (8 * i));
+      }
+      sc.b = QB == 2 ? ((uses >> (8 * i)) + 1) & 1 : 0;           // the buffer of the load read last
+      sc.go = true;
+      return sc;
+    };
+    // (one lane)
+    auto issue_scores = [&](int i, const Scores& sc) __attribute__((always_inline)) {
+      issue_qk<D, TKV>(tmem_base + i * TKV, smem_base + (sc.b * 2 + i) * SM::kSubBytes, ring_smem + sc.st * SM::kStageBytes);
+      umma_commit(smem_u32(&misc->s_full[i]));
+      if (sc.release) umma_commit(smem_u32(&misc->kv_empty[sc.st]));
+      if (sc.last) umma_commit(smem_u32(&misc->q_empty[i][sc.b]));
+    };
+    auto scores = [&](int i, const Scores& sc) __attribute__((always_inline)) {
+      if (sc.go && elect_one()) issue_scores(i, sc);
+      __syncwarp();
+    };
+    auto p_times_v = [&](int i, int j, bool second) __attribute__((always_inline)) {       // (one lane)
+      const uint32_t o = tmem_base + O_COL0 + i * D, pt = kSplitP ? tmem_base + P_COL0 + i * (TKV / 2) : tmem_base + i * TKV;
+      const uint32_t v = ring_smem + vs * SM::kStageBytes;
+      if (!second) issue_pv<D, TKV>(o, pt, v, j > 0, TKV * 128, 1024, 0, TKV / 32);
+      else {
+        issue_pv<D, TKV>(o, pt, v, true, TKV * 128, 1024, TKV / 32, TKV / 16);
+        umma_commit(smem_u32(&misc->o_full[i]));
+      }
+    };
+    int tile = blockIdx.x;
+    int n0, n1, m0 = 0, m1 = 0;                        // steps of the two sub-tiles in this tile and the next
+    {
+      const TileWork w = tile_work(tile, p);
+      n0 = w.n0;
+      n1 = w.n1;
+    }
+    if (ok) {
+      // the first tile's first scores; at d = 64 sub-tile 1's follow half a step later (below), which sets up the offset
+      // between the two softmax warpgroups that the rest of the walk keeps
+      scores(0, ready(0, 0, 0, true, n0 == 1, n1 == 0));
+      if (ok && !kSplitP && n1 > 0) scores(1, ready(1, 0, 0, true, n1 == 1, true));
+    }
+    bool defer = kSplitP && n1 > 0, ahead = false;     // (d = 64) ahead: sub-tile 0's next step has been issued
+    for (int seq = 1; ok && tile >= 0; ++seq) {
+      const int n = n1 > n0 ? n1 : n0;
+      int next = -3;                                   // not asked yet
+      // The product that follows step j of sub-tile i: its next step, or its first step of the next tile.
+      auto next_scores = [&](int i, int j) __attribute__((always_inline)) -> Scores {
+        const Scores none = {0, 0, false, false, false};
+        const int ni = i ? n1 : n0;
+        int items = 1, left = ni - j - 1, other = n1;  // ring items from V_j to the K tile; steps left with this Q; (release)
+        const bool first = left <= 0;
+        if (first) {
+          if (j != (ni > 0 ? ni - 1 : n - 1)) return none;
+          if (next == -3) {
+            next = next_tile(seq, kRoleMma);
+            if (next == -2) { ok = false; return none; }
+            if (next >= 0) {
+              const TileWork w = tile_work(next, p);
+              m0 = w.n0;
+              m1 = w.n1;
+            }
+          }
+          left = i ? m1 : m0;
+          if (next < 0 || left == 0) return none;
+          items = 2 * (n - j) - 1;                     // K_0 of the next tile
+          other = m1;
+        }
+        int st = vs + items;
+        uint32_t ph = vph;
+        if (st >= p.stages) { st -= p.stages; ph ^= 1u; }
+        return ready(i, st, ph, first, left == 1, i == 1 || other == 0);
+      };
+      for (int j = 0; ok && j < n; ++j) {
+        if constexpr (kSplitP) {
+          // Nothing ties the two sub-tiles to each other here, and left alone their softmax warpgroups end up in the same
+          // phase of the step (both at the exponentials, then neither).  So sub-tile 1's scores are held back until
+          // sub-tile 0 has its row maxima of that step: half a step behind.
+          if (j < n0) {
+            if (!wait(&misc->s_free[0], gp & 1, kBarPFull, 0x100)) break;
+            const Scores sc = next_scores(0, j);
+            scores(0, sc);
+            ahead = sc.go;
+            if (!ok || !wait(&misc->kv_full[vs], vph, kBarKvFull, 0x102) || !wait(&misc->p_full[0], gp & 1, kBarPFull, 0x103)) break;
+            if (elect_one()) p_times_v(0, j, false);
+            __syncwarp();
+          }
+          if (defer) {
+            defer = false;
+            scores(1, ready(1, 0, 0, true, n1 == 1, true));
+            if (!ok) break;
+          }
+          if (j < n1 && !wait(&misc->s_free[1], (gp >> 1) & 1, kBarPFull, 0x105)) break;
+          scores(1, next_scores(1, j));
+          if (!ok) break;
+          if (j < n0) {
+            if (!wait(&misc->p_half[0], gp & 1, kBarPFull, 0x106)) break;
+            if (elect_one()) p_times_v(0, j, true);
+            __syncwarp();
+            gp ^= 1u;
+          }
+          if (j < n1) {
+            if (j >= n0 && !wait(&misc->kv_full[vs], vph, kBarKvFull, 0x107)) break;
+            if (!wait(&misc->p_full[1], (gp >> 1) & 1, kBarPFull, 0x108)) break;
+            if (elect_one()) p_times_v(1, j, false);
+            __syncwarp();
+            if (!wait(&misc->p_half[1], (gp >> 1) & 1, kBarPFull, 0x109)) break;
+            if (elect_one()) p_times_v(1, j, true);
+            __syncwarp();
+            gp ^= 2u;
+          }
+        } else {
+          if (!wait(&misc->kv_full[vs], vph, kBarKvFull, 0x10A)) break;
+#pragma unroll 1
+          for (int i = 0; i < 2; ++i) {
+            const int ni = i ? n1 : n0;
+            {
+              if (j < ni) {
+                if (!wait(&misc->p_full[i], (gp >> i) & 1, kBarPFull, i)) break;
+                if (elect_one()) p_times_v(i, j, false);
+                __syncwarp();
+                if (!wait(&misc->p_half[i], (gp >> i) & 1, kBarPFull, 0x8000 | i)) break;
+                if (elect_one()) p_times_v(i, j, true);
+                __syncwarp();
+                gp ^= 1u << i;
+              }
+              scores(i, next_scores(i, j));
+              if (!ok) break;
+            }
+          }
+          if (!ok) break;
+        }
+        if (elect_one()) umma_commit(smem_u32(&misc->kv_empty[vs]));
+        __syncwarp();
+        vs += 2;
+        if (vs >= p.stages) { vs -= p.stages; vph ^= 1u; }
+      }
+      if (!ok) break;
+      tile = next;
+      n0 = m0;
+      n1 = m1;
+    }
+  } else if (warp == 13) {
+    // ================================================== TMA producer, and the requests for the next tile
+    setmaxnreg_dec<64>();
+    bool ok = run;
+    int stage = 0, issued = 0, asked = 0;              // asked: requests made
+    uint32_t phase = 0;
+    uint32_t q_loads0 = 0, q_loads1 = 0;
+    // (the waits are taken by the whole warp, the copies issued by one lane)
+    auto load_kv = [&](const CUtensorMap* tm, int kv_row, int bh) __attribute__((always_inline)) -> bool {
+      if (!wait_quiet_warp(smem_u32(&misc->kv_empty[stage]), phase ^ 1u, abort_flag, wait_info(kRoleLoad, kBarKvEmpty, issued))) return false;
+      if (elect_one()) {
+        const uint32_t bar = smem_u32(&misc->kv_full[stage]), dst = ring_smem + stage * SM::kStageBytes;
+        mbar_arrive_expect_tx(bar, SM::kStageBytes);
+#pragma unroll
+        for (int c = 0; c < KCH; ++c) tma_load_3d(dst + c * (TKV * 128), tm, c * 64, kv_row, bh, bar);
+      }
+      __syncwarp();
+      ++issued;
+      if (++stage == p.stages) { stage = 0; phase ^= 1u; }
+      return true;
+    };
+    auto load_q = [&](int i, const TileWork& w) __attribute__((always_inline)) -> bool {
+      const uint32_t u = i ? q_loads1 : q_loads0, b = u % QB;
+      if (u >= QB && !wait_quiet_warp(smem_u32(&misc->q_empty[i][b]), (u / QB - 1) & 1, abort_flag, wait_info(kRoleLoad, kBarQ, u))) return false;
+      if (elect_one()) {
+        const uint32_t bar = smem_u32(&misc->q_full[i][b]), dst = smem_base + (b * 2 + i) * SM::kSubBytes;
+        mbar_arrive_expect_tx(bar, SM::kSubBytes);
+#pragma unroll
+        for (int c = 0; c < KCH; ++c) tma_load_3d(dst + c * (kSub * 128), &tm_q, c * 64, w.q_row0 + i * kSub, w.bh, bar);
+      }
+      __syncwarp();
+      if (i) ++q_loads1; else ++q_loads0;
+      return true;
+    };
+    int tile = blockIdx.x;
+    for (int seq = 1; ok && tile >= 0; ++seq) {
+      const TileWork w = tile_work(tile, p);
+      const int n = w.steps();
+      // the first product needs K_0 and Q of sub-tile 0; the first tile's Q buffer is free at once
+      if (seq == 1) ok = load_q(0, w);
+      if (ok) ok = load_kv(&tm_k, 0, w.bh);
+      if (ok && seq > 1) ok = load_q(0, w);
+      if (ok && w.n1 > 0) ok = load_q(1, w);
+      for (int j = 0; ok && j < n; ++j) {
+        if (j > 0) ok = load_kv(&tm_k, j * TKV, w.bh);
+        if (ok && j == n - 1) {
+          // Ask for the tile after this one, into the slot that held the tile before this one -- as late as the answer is
+          // sure to be back in time (a ring's depth ahead of the MMA warp): a tile asked for early would be tied to this
+          // CTA while others run dry.
+          if (seq >= 3)
+            ok = wait_quiet_warp(smem_u32(&misc->sched_empty[seq & 1]), ((seq - 3) >> 1) & 1, abort_flag, wait_info(kRoleLoad, kBarSync, seq));
+          if (!ok) break;
+          if (elect_one()) {
+            mbar_arrive_expect_tx(smem_u32(&misc->sched_full[seq & 1]), 16);
+            clc_try_cancel(smem_u32(&misc->sched[seq & 1]), smem_u32(&misc->sched_full[seq & 1]));
+          }
+          __syncwarp();
+          asked = seq;
+        }
+        if (ok) ok = load_kv(&tm_v, j * TKV, w.bh);
+      }
+      if (!ok) break;
+      tile = next_tile(seq, kRoleLoad);
+    }
+    if (tile == -2) ok = false;
+    if (!ok && lane == 0) {
+      // Drain: every copy started here must land before the CTA may exit, and so must an answer still on its way.
+      auto drain = [&](uint64_t* bar, uint32_t parity) {
+        const long long t0 = clock64();
+        while (!mbar_try_wait(smem_u32(bar), parity) && clock64() - t0 < kWaitLimitCycles) {}
+      };
+      for (int t = issued > p.stages ? issued - p.stages : 0; t < issued; ++t)
+        drain(&misc->kv_full[t % p.stages], (uint32_t)(t / p.stages) & 1u);
+      for (int i = 0; i < 2; ++i)
+        for (uint32_t q = i ? q_loads1 : q_loads0, u = q > (uint32_t)QB ? q - QB : 0; u < q; ++u) drain(&misc->q_full[i][u % QB], (u / QB) & 1);
+      if (asked > 0) drain(&misc->sched_full[asked & 1], ((asked - 1) >> 1) & 1);
+    }
+  } else {
+    setmaxnreg_dec<64>();
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 15) {
+    tc_fence_after();
+    tmem_dealloc(tmem_base, 512);
+  }
+  if (threadIdx.x == 0) report_abort(&misc->abort);
+}
+
+}  // namespace attn

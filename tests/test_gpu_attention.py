@@ -819,3 +819,33 @@ def test_few_query_rows_against_many_keys(env, B, H, Lq, Lk, d):
     assert_close(to_host_f64(out).reshape(ref.shape), ref, f"{B} {H} {Lq} {Lk} {d}")
     again = binding.forward_qk(*dev)
     assert torch.equal(again.view(torch.int16), out.view(torch.int16))
+
+
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("B,H,L", [(1, 150, 129), (2, 80, 200), (1, 300, 256), (1, 200, 257), (4, 40, 384), (1, 160, 385),
+                                   (1, 152, 640), (2, 20, 1111), (3, 50, 900), (1, 64, 2048), (1, 33, 1793)])
+def test_causal_whole_tiles_match_the_reference(env, B, H, L, d):
+    """Causal shapes with more tiles than the equal ranges are good for: both sides of a sub-tile and of a tile in the
+    length (last sub-tile absent, of one row, full), tiles of one key step, one and many tiles per CTA, group boundaries.
+    NaN-filled output, every element against fp64, the same bits again."""
+    torch, orc, binding = env
+    rng = np.random.default_rng([B, H, L, d, 5])
+    dev = [to_cuda_bf16(synth.f32_to_bf16_bits((rng.standard_normal((B * H, L, d)) * 1.5).astype(np.float32))).view(B, H, L, d)
+           for _ in range(3)]
+    out = torch.full((B, H, L, d), float("nan"), dtype=torch.bfloat16, device="cuda")
+    binding.forward(*dev, out, causal=True)
+    torch.cuda.synchronize()
+    assert binding.last_device_status()[0] == 0 and binding.last_cluster_size() == 0
+    # Bound per element: bf16 keeps 8 significant bits, so a rounding moves a value by at most 2^-8 of it.  Rounded are the
+    # weights (at most 2^-8 sum p |v| in all; the exponentials' own error, 2^-13, likewise) and the output (2^-8 |o|).
+    keep = torch.ones((L, L), dtype=torch.bool, device="cuda").tril()
+    q, k, v, o = (x.view(B * H, L, d) for x in (*dev, out))
+    for h in range(0, B * H, 16):
+        s = (q[h:h + 16].double() @ k[h:h + 16].double().transpose(1, 2) / d ** 0.5).masked_fill(~keep, -math.inf)
+        p, vd = torch.softmax(s, dim=-1), v[h:h + 16].double()
+        ref, spread = p @ vd, p @ vd.abs()
+        assert ((o[h:h + 16].double() - ref).abs() <= (2.0 ** -8 + 2.0 ** -13) * spread + 2.0 ** -8 * ref.abs() + 1e-6).all(), h
+        assert float((o[h:h + 16].double() - ref).norm() / ref.norm()) <= 5e-3, h
+    for _ in range(3):
+        again = binding.forward(*dev, causal=True)
+        assert torch.equal(again.view(torch.int16), out.view(torch.int16))
