@@ -185,12 +185,37 @@ def ensure_workspace(device_index: int, nbytes: int) -> None:
     _workspaces[device_index] = buf
 
 
+def _call(dev, where, fn, *args, workspace=None):
+    """One library call with device `dev` current.  `workspace()` gives the bytes that the call's plan asks for; it is
+    asked only when the library says that what is registered is too small, so that the usual call derives its plan once."""
+    import torch
+
+    if torch.cuda.current_device() != dev:
+        with torch.cuda.device(dev):
+            return _call(dev, where, fn, *args, workspace=workspace)
+    rc = fn(*args)
+    if rc == ERR_NEED_WORKSPACE and workspace is not None:
+        ensure_workspace(dev, workspace())
+        rc = fn(*args)
+    if rc != ATTN_OK:
+        raise AttnError(rc, where)
+
+
+def _stream(dev: int) -> int:
+    """Handle of the current stream of a device."""
+    import torch
+
+    return torch._C._cuda_getCurrentRawStream(dev)
+
+
 def _prep(q, k, v, o):
     import torch
 
-    if q.dtype != torch.bfloat16 or k.dtype != torch.bfloat16 or v.dtype != torch.bfloat16:
+    bf16 = torch.bfloat16
+    if q.dtype != bf16 or k.dtype != bf16 or v.dtype != bf16:
         raise TypeError("q, k, v must be torch.bfloat16")
-    if q.dim() != 4 or q.shape != k.shape or q.shape != v.shape:
+    shape = q.shape
+    if len(shape) != 4 or shape != k.shape or shape != v.shape:
         raise ValueError("q, k, v must share the shape [B, H, L, d]")
     if not (q.is_cuda and k.is_cuda and v.is_cuda):
         raise ValueError("q, k, v must be CUDA tensors (there is no CPU path)")
@@ -200,26 +225,19 @@ def _prep(q, k, v, o):
         o = torch.empty_like(q)
     elif o.shape != q.shape or o.dtype != torch.bfloat16 or not o.is_contiguous() or o.device != q.device:
         raise ValueError("o must match q in shape, dtype, device and be contiguous")
-    B, H, L, d = (int(x) for x in q.shape)
-    dev = q.device.index if q.device.index is not None else torch.cuda.current_device()
-    stream = torch.cuda.current_stream(q.device).cuda_stream
-    return o, B, H, L, d, dev, stream
+    B, H, L, d = shape
+    dev = q.get_device()
+    return o, B, H, L, d, dev, _stream(dev)
 
 
 def forward(q, k, v, o=None, causal=False):
     """O = softmax(Q K^T / sqrt(d)) V with the closed-form default tiles (asynchronous).
 
     causal=True: row i attends to keys 0..i only."""
-    import torch
-
     o, B, H, L, d, dev, stream = _prep(q, k, v, o)
-    with torch.cuda.device(dev):
-        t = plan(_device_desc(dev), B, H, L, d, causal)
-        if t.feasible:
-            ensure_workspace(dev, workspace_bytes(t, B, H, L, d))
-        fn = lib().attn_forward_causal if causal else lib().attn_forward
-        _check(fn(q.data_ptr(), k.data_ptr(), v.data_ptr(), o.data_ptr(), B, H, L, d, stream),
-               "attn_forward_causal" if causal else "attn_forward")
+    fn, where = (lib().attn_forward_causal, "attn_forward_causal") if causal else (lib().attn_forward, "attn_forward")
+    _call(dev, where, fn, q.data_ptr(), k.data_ptr(), v.data_ptr(), o.data_ptr(), B, H, L, d, stream,
+          workspace=lambda: workspace_bytes(plan(_device_desc(dev), B, H, L, d, causal), B, H, L, d))
     return o
 
 
@@ -304,19 +322,16 @@ def forward_qk(q, k, v, o=None):
     for name, x in (("q", q), ("k", k), ("v", v)):
         if x.dtype != torch.bfloat16 or not x.is_cuda or not x.is_contiguous() or x.dim() != 4:
             raise ValueError(f"{name} must be a contiguous CUDA bfloat16 tensor [B, H, L, d]")
-    B, H, Lq, d = (int(x) for x in q.shape)
-    Lk = int(k.shape[2])
-    if tuple(k.shape) != (B, H, Lk, d) or tuple(v.shape) != (B, H, Lk, d):
+    B, H, Lq, d = q.shape
+    Lk = k.shape[2]
+    if k.shape != (B, H, Lk, d) or v.shape != (B, H, Lk, d):
         raise ValueError("k and v must be [B, H, Lk, d] with q's B, H and d")
     if o is None:
         o = torch.empty_like(q)
-    dev = q.device.index if q.device.index is not None else torch.cuda.current_device()
-    with torch.cuda.device(dev):
-        t = plan_qk(_device_desc(dev), B, H, Lq, Lk, d)
-        ensure_workspace(dev, workspace_bytes(t, B, H, Lq, d))
-        stream = torch.cuda.current_stream(q.device).cuda_stream
-        _check(lib().attn_forward_qk(q.data_ptr(), k.data_ptr(), v.data_ptr(), o.data_ptr(), B, H, Lq, Lk, d, stream),
-               "attn_forward_qk")
+    dev = q.get_device()
+    _call(dev, "attn_forward_qk", lib().attn_forward_qk, q.data_ptr(), k.data_ptr(), v.data_ptr(), o.data_ptr(),
+          B, H, Lq, Lk, d, _stream(dev),
+          workspace=lambda: workspace_bytes(plan_qk(_device_desc(dev), B, H, Lq, Lk, d), B, H, Lq, d))
     return o
 
 
@@ -410,11 +425,12 @@ def gemm_plan(desc: AttnHwDesc, batch: int, M: int, N: int, K: int) -> GemmTiles
 
 
 def _mat(x, name):
+    """(batch, rows, columns) of a matrix operand."""
     import torch
 
     if x.dtype != torch.bfloat16 or not x.is_cuda or not x.is_contiguous() or x.dim() not in (2, 3):
         raise ValueError(f"{name} must be a contiguous CUDA bfloat16 tensor of 2 or 3 dimensions")
-    return x if x.dim() == 3 else x.unsqueeze(0)
+    return x.shape if x.dim() == 3 else (1, *x.shape)
 
 
 def gemm(a, b, c=None, *, b_layout="kn", cta_pair=0, tile_n=0, tail_split=0):
@@ -424,31 +440,30 @@ def gemm(a, b, c=None, *, b_layout="kn", cta_pair=0, tile_n=0, tail_split=0):
     tiles (tile sweep only; 0 keeps them)."""
     import torch
 
-    a3, b3 = _mat(a, "a"), _mat(b, "b")
-    batch, M, K = (int(x) for x in a3.shape)
+    batch, M, K = _mat(a, "a")
+    b_batch, rows, cols = _mat(b, "b")
     if b_layout == "kn":
-        kb, N = int(b3.shape[1]), int(b3.shape[2])
+        kb, N = rows, cols
     elif b_layout == "nk":
-        N, kb = int(b3.shape[1]), int(b3.shape[2])
+        N, kb = rows, cols
     else:
         raise ValueError("b_layout is 'kn' or 'nk'")
-    if kb != K or int(b3.shape[0]) != batch:
+    if kb != K or b_batch != batch:
         raise ValueError("a and b do not agree in batch or K")
     if c is None:
         c = torch.empty((batch, M, N) if a.dim() == 3 else (M, N), dtype=torch.bfloat16, device=a.device)
     elif c.dtype != torch.bfloat16 or not c.is_contiguous() or c.numel() != batch * M * N or c.device != a.device:
         raise ValueError("c must be a contiguous bfloat16 tensor of batch*M*N elements on a's device")
-    dev = a.device.index if a.device.index is not None else torch.cuda.current_device()
-    with torch.cuda.device(dev):
-        stream = torch.cuda.current_stream(a.device).cuda_stream
-        if cta_pair or tile_n or tail_split:
-            ov = GemmTiles()
-            ov.cta_pair, ov.tile_n, ov.tail_split = int(cta_pair), int(tile_n), int(tail_split)
-            _check(lib().gemm_forward_tiles(a.data_ptr(), b.data_ptr(), c.data_ptr(), batch, M, N, K,
-                                            0 if b_layout == "kn" else 1, ctypes.byref(ov), stream), "gemm_forward_tiles")
-        else:
-            _check(lib().gemm_forward(a.data_ptr(), b.data_ptr(), c.data_ptr(), batch, M, N, K,
-                                      0 if b_layout == "kn" else 1, stream), "gemm_forward")
+    dev = a.get_device()
+    layout = 0 if b_layout == "kn" else 1
+    if cta_pair or tile_n or tail_split:
+        ov = GemmTiles()
+        ov.cta_pair, ov.tile_n, ov.tail_split = int(cta_pair), int(tile_n), int(tail_split)
+        _call(dev, "gemm_forward_tiles", lib().gemm_forward_tiles, a.data_ptr(), b.data_ptr(), c.data_ptr(), batch, M, N, K,
+              layout, ctypes.byref(ov), _stream(dev))
+    else:
+        _call(dev, "gemm_forward", lib().gemm_forward, a.data_ptr(), b.data_ptr(), c.data_ptr(), batch, M, N, K, layout,
+              _stream(dev))
     return c
 
 
@@ -464,11 +479,9 @@ def softmax_rows(s, scale: float, out=None):
         raise ValueError("out must match s")
     cols = int(s.shape[-1])
     rows = s.numel() // cols
-    dev = s.device.index if s.device.index is not None else torch.cuda.current_device()
-    with torch.cuda.device(dev):
-        stream = torch.cuda.current_stream(s.device).cuda_stream
-        _check(lib().softmax_rows_forward(s.data_ptr(), out.data_ptr(), rows, cols, float(scale), stream),
-               "softmax_rows_forward")
+    dev = s.get_device()
+    _call(dev, "softmax_rows_forward", lib().softmax_rows_forward, s.data_ptr(), out.data_ptr(), rows, cols, float(scale),
+          _stream(dev))
     return out
 
 

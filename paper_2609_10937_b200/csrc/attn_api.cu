@@ -10,6 +10,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <mutex>
+#include <unordered_map>
 
 #include "attn.h"
 #include "attn_kernels.cuh"
@@ -103,6 +104,27 @@ int device_state(DeviceState** out) {
   return s.arch_ok ? ATTN_OK : ATTN_ERR_WRONG_ARCH;
 }
 
+// Dynamic shared memory a kernel may use on the current device, raised when a launch needs more than any before it (asking
+// the driver every time took about as long as the launch itself).
+int allow_smem(const void* kern, int bytes) {
+  static std::mutex mu;
+  static std::unordered_map<const void*, int> allowed[kMaxDevices];
+  int dev = 0;
+  ATTN_CUDA_TRY(cudaGetDevice(&dev));
+  if (dev < 0 || dev >= kMaxDevices) return ATTN_ERR_INVALID_ARG;
+  std::lock_guard<std::mutex> lk(mu);
+  int& have = allowed[dev][kern];
+  if (have >= bytes) return ATTN_OK;
+  ATTN_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+  have = bytes;
+  return ATTN_OK;
+}
+#define ATTN_ALLOW_SMEM(kern, bytes)                                                 \
+  do {                                                                               \
+    const int rc__ = allow_smem(reinterpret_cast<const void*>(kern), bytes);         \
+    if (rc__ != ATTN_OK) return rc__;                                                \
+  } while (0)
+
 bool overlaps(const void* a, size_t na, const void* b, size_t nb) {
   const uintptr_t a0 = (uintptr_t)a, b0 = (uintptr_t)b;
   return a0 < b0 + nb && b0 < a0 + na;
@@ -172,7 +194,7 @@ int launch_fwd(const void* q, const void* k, const void* v, void* o, int B, int 
   const bool eager = !p.causal && t.ctas > t.tiles && t.ctas % t.tiles == 0 && grid <= sms;
   const bool wait_roles_ok = !may_overlap;
   auto launch = [&](auto kern) -> int {
-    ATTN_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    ATTN_ALLOW_SMEM(kern, smem);
     kern<<<grid, 512, smem, stream>>>(tq, tk, tv, to, p);
     return ATTN_OK;
   };
@@ -184,8 +206,8 @@ int launch_fwd(const void* q, const void* k, const void* v, void* o, int B, int 
   p.cluster_k = 0;
   t_cluster_size = 0;
   auto launch_eager = [&](auto kern, auto kern_cluster) -> int {
-    ATTN_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    ATTN_CUDA_TRY(cudaFuncSetAttribute(kern_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    ATTN_ALLOW_SMEM(kern, smem);
+    ATTN_ALLOW_SMEM(kern_cluster, smem);
     const int kk = t.ctas / t.tiles;
     const size_t landing = (size_t)((4 * NQ + kk - 1) / kk) * (kk - 1) * (32 * D * 4 + 256);
     if (kk >= 2 && kk <= 8 && landing <= (size_t)t.kv_stages * SM::kStageBytes) {
@@ -230,7 +252,7 @@ int launch_fwd(const void* q, const void* k, const void* v, void* o, int B, int 
   if (p.causal && ck >= 2 && ck <= 4 && p.ratio >= 2 && c_landing <= (size_t)t.kv_stages * SM::kStageBytes) {
     // causal, ck CTAs per tile as one cluster: each a share of the tile's own key steps (the only way to run this grid)
     auto kern = attn::attn_fwd_kernel<D, TKV, NQ, true, true, true>;
-    ATTN_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    ATTN_ALLOW_SMEM(kern, smem);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(512);
@@ -294,7 +316,7 @@ int launch_decode(const void* q, const void* k, const void* v, void* o, int BH, 
   p.status = status;
   auto kern = attn::attn_decode_kernel<D, MT, HALF>;
   constexpr int smem = attn::decode_smem_total<MT>();
-  ATTN_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  ATTN_ALLOW_SMEM(kern, smem);
   if (cluster_k > 8) ATTN_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(BH * cluster_k));
@@ -409,7 +431,7 @@ int launch_causal_tiles(const void* q, const void* k, const void* v, void* o, in
   p.status = status;
   const int smem = SM::total(p.stages);
   auto kern = attn::attn_causal_tiles_kernel<D>;
-  ATTN_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  ATTN_ALLOW_SMEM(kern, smem);
   kern<<<(unsigned)(BH * p.q_tiles), 512, smem, stream>>>(tq, tk, tv, to, p);
   ATTN_CUDA_TRY(cudaGetLastError());
   t_cluster_size = 0;
@@ -556,7 +578,7 @@ int launch_simple(const void* q, const void* k, const void* v, void* o, int B, i
   if ((rc = make_tmap(&tv, v, BH, L, D, TKV)) != ATTN_OK) return rc;
   const int smem = attn::kSub * D * 2 + 2 * TKV * D * 2 + 1024;
   auto kern = attn::attn_fwd_simple_kernel<D, TKV>;
-  ATTN_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  ATTN_ALLOW_SMEM(kern, smem);
   const float scale_log2 = (float)(1.4426950408889634 / std::sqrt((double)D));
   dim3 grid((L + attn::kSub - 1) / attn::kSub, BH);
   kern<<<grid, 128, smem, stream>>>(tq, tk, tv, reinterpret_cast<__nv_bfloat16*>(o), L, scale_log2, scores_out);
@@ -1026,7 +1048,7 @@ int gemm_launch(const void* a, const void* b, void* c, int batch, int M, int N, 
     p.tail_tiles = t.tail_split;
     const int smem = gemm::pair_smem_total(t.stages, t.tile_n);
     auto launch_pair = [&](auto kernel) -> int {
-      ATTN_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+      ATTN_ALLOW_SMEM(kernel, smem);
       cudaLaunchConfig_t cfg = {};
       cfg.gridDim = dim3((unsigned)t.ctas);
       cfg.blockDim = dim3(gemm::kPairThreads);
@@ -1047,7 +1069,7 @@ int gemm_launch(const void* a, const void* b, void* c, int batch, int M, int N, 
   } else {
     const int smem = gemm::smem_total(t.stages, t.tile_n);
     auto launch = [&](auto kernel) -> int {
-      ATTN_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+      ATTN_ALLOW_SMEM(kernel, smem);
       kernel<<<t.ctas, gemm::kThreads, smem, stream>>>(ta, tb, tc, p);
       return ATTN_OK;
     };
@@ -1103,7 +1125,7 @@ int softmax_launch(const void* s, void* pout, long long rows, int cols, float sc
   else {
     // wider than the registers of one block hold: the row is staged in shared memory (2 bytes per column)
     auto kern = gemm::softmax_rows_staged_kernel<256>;
-    ATTN_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 65536));
+    ATTN_ALLOW_SMEM(kern, 65536);
     kern<<<(unsigned)rows, 256, cols * 2, stream>>>(sp, pp, cols, scale_log2);
   }
 #undef SOFTMAX_ROW_CASE
