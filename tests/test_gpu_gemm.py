@@ -110,6 +110,15 @@ def test_matrix_product_full_size_sampled(env):
     _check_product(env, 1, 4096, 4096, 4096, "kn", seed=2, rows_per_batch=48)
 
 
+@pytest.mark.parametrize("layout", ["kn", "nk"])
+@pytest.mark.parametrize("batch,M,N,K", [(1, 64, 64, 8192), (1, 1, 8, 2048), (1, 129, 136, 1000), (2, 128, 128, 512), (1, 700, 200, 3000),
+                                         (4, 500, 520, 264), (1, 1000, 1000, 1000), (1, 1500, 1400, 72), (1, 100, 8000, 2000)])
+def test_products_with_few_output_tiles(env, batch, M, N, K, layout):
+    """Outputs of at most one 128 x 128 tile per SM: one tile and many, rows and columns past the end of the last, K split over
+    1 to 8 CTAs with a ragged last step, more and fewer steps than the ring has stages."""
+    _check_product(env, batch, M, N, K, layout, seed=M + N + K)
+
+
 @pytest.mark.parametrize("rows,cols", [(4, 8), (7, 256), (33, 2048), (5, 2056), (3, 16384), (2, 32768), (9, 1000),
                                        (3, 16392), (2, 20000), (5, 32760)])   # the last three: staged in shared memory
 def test_row_softmax_matches_oracle(env, rows, cols):
