@@ -74,13 +74,16 @@ int gemm_plan(const attn_hw_desc *desc, int batch, int M, int N, int K, gemm_til
  * b_layout 1: b is [batch][N][K] (C = A B^T).  c: [batch][M][N].  Any M, N >= 1;
  * K, N (and for b_layout 0 also N as the row length of b) must be multiples of 8
  * so that every row starts 16-byte aligned.  c must not overlap a or b.
+ * Runs the tiles of gemm_plan, except for an output of at most one 128 x 128 tile per compute unit whose plan has
+ * larger tiles: that one runs as one 128 x 128 tile per CTA.  Every kernel sums the K products of an element in the
+ * same order, so an element's bits do not depend on the tiles, on the batch or on the other rows and columns.
  * Errors: ATTN_ERR_INVALID_ARG, ATTN_ERR_UNSUPPORTED_SHAPE, ATTN_ERR_MISALIGNED,
  * ATTN_ERR_ALIASING, ATTN_ERR_WRONG_ARCH, ATTN_ERR_INFEASIBLE_PLAN, ATTN_ERR_CUDA.
  */
 int gemm_forward(const void *a, const void *b, void *c, int batch, int M, int N, int K, int b_layout,
                  void *cuda_stream);
 
-/* Same with tile fields overridden (tile sweep only; 0 keeps the closed-form value): cta_pair = 1 runs the
+/* Same with the tiles of gemm_plan at every size and with fields overridden (tile sweep only; 0 keeps the closed-form value): cta_pair = 1 runs the
  * lone-CTA tiling where the closed form takes pairs, cta_pair = 2 insists on pairs; tile_n (128 | 256) narrows a
  * pair's tile; tail_split < 0 keeps whole tiles in the last wave.  ATTN_ERR_BAD_TILES if the combination was not compiled or does not fit. */
 int gemm_forward_tiles(const void *a, const void *b, void *c, int batch, int M, int N, int K, int b_layout,

@@ -981,23 +981,14 @@ int make_tmap_mat(CUtensorMap* m, const void* base, int batch, int rows, int col
   return make_tmap(m, base, batch, rows, cols, box_rows);
 }
 
-// CTAs per 128 x 128 tile of gemm_split_kernel, or 0: the plan's tiles are better.  Estimates in microseconds, from the loads
-// of a K step (32 KB into one SM: 0.27) or the products of one (256 x 256 per pair: 0.39; 128 x 256 per lone CTA: 0.39) and
-// 2 for a kernel's ends, 1.5 more for a cluster's barriers and exchange.  Only grids of one wave: beyond that the plan's
-// larger tiles load less per product.
-int gemm_split(int batch, int M, int N, int K, const gemm_tiles& t, int sms) {
+// Products that gemm_small_kernel takes over from the plan's kernels: at most one 128 x 128 tile per SM, where the plan's tile
+// is larger.  There it is faster at every size measured (1.2 to 1.6 times where the plan has lone CTAs, 1.0 to 1.3 times where
+// it has pairs; K = 64 to 8192).  A plan of 128 x 128 tiles keeps its kernel: launched as clusters of one, this one took 14.6 us
+// against 13.5 at 16384 x 128 x 2048 and 37.5 against 34.5 at 128 x 128 x 8192.  K is never shared out between CTAs: an element's
+// sum would depend on how many tiles stand beside it.
+bool gemm_small(int batch, int M, int N, const gemm_tiles& t, int sms) {
   const long long tiles = (long long)batch * ((M + 127) / 128) * ((N + 127) / 128);
-  const int steps = (K + gemm::kTileK - 1) / gemm::kTileK;
-  if (tiles > sms) return 0;
-  const int units = t.cta_pair == 2 ? t.ctas / 2 : t.ctas;
-  double best_cost = ((t.tiles + units - 1) / units) * steps * 0.39 + 2.0;
-  int best = 0;
-  for (int k = 1; k <= gemm::kSplitMaxK; k *= 2) {
-    if (tiles * k > sms || steps < 4 * k) break;
-    const double cost = ((steps + k - 1) / k) * 0.27 + 2.0 + (k > 1 ? 1.5 : 0.0);
-    if (cost < best_cost) { best = k; best_cost = cost; }
-  }
-  return best;
+  return tiles <= sms && (t.tile_m > 128 || t.tile_n > 128);
 }
 
 int gemm_launch(const void* a, const void* b, void* c, int batch, int M, int N, int K, int b_layout, cudaStream_t stream,
@@ -1036,7 +1027,7 @@ int gemm_launch(const void* a, const void* b, void* c, int batch, int M, int N, 
   if (!t.feasible || (t.n_sub != 1 && t.n_sub != 2) || t.tile_m != t.n_sub * attn::kSub || (t.tile_n != 128 && t.tile_n != 256) ||
       t.tile_k != gemm::kTileK || t.stages > gemm::kMaxStages || t.stages < 2)
     return ATTN_ERR_INFEASIBLE_PLAN;
-  if (const int split = ovr ? 0 : gemm_split(batch, M, N, K, t, st->desc.num_units)) {
+  if (!ovr && gemm_small(batch, M, N, t, st->desc.num_units)) {
     CUtensorMap ta, tb;
     if ((rc = make_tmap_mat(&ta, a, batch, M, K, 128)) != ATTN_OK) return rc;
     if (b_layout == 0) rc = make_tmap_mat(&tb, b, batch, K, N, gemm::kTileK);
@@ -1047,27 +1038,16 @@ int gemm_launch(const void* a, const void* b, void* c, int batch, int M, int N, 
     p.m_tiles = (M + 127) / 128;
     p.n_tiles = (N + 127) / 128;
     p.k_steps = (K + gemm::kTileK - 1) / gemm::kTileK;
-    p.stages = std::min(gemm::kMaxStages, (st->desc.local_mem_bytes - gemm::kMiscBytes) / gemm::kSplitStageBytes);
-    const int tiles = batch * p.m_tiles * p.n_tiles, smem = gemm::split_smem_total(p.stages);
-    auto launch_split = [&](auto kernel) -> int {
+    p.stages = std::min(gemm::kMaxStages, (st->desc.local_mem_bytes - gemm::kMiscBytes) / gemm::kSmallStageBytes);
+    const int tiles = batch * p.m_tiles * p.n_tiles, smem = gemm::small_smem_total(p.stages);
+    auto launch_small = [&](auto kernel) -> int {
       ATTN_ALLOW_SMEM(kernel, smem);
-      cudaLaunchConfig_t cfg = {};
-      cfg.gridDim = dim3((unsigned)(tiles * split));
-      cfg.blockDim = dim3(gemm::kThreads);
-      cfg.dynamicSmemBytes = smem;
-      cfg.stream = stream;
-      cudaLaunchAttribute attr[1];
-      attr[0].id = cudaLaunchAttributeClusterDimension;
-      attr[0].val.clusterDim.x = split;
-      attr[0].val.clusterDim.y = 1;
-      attr[0].val.clusterDim.z = 1;
-      cfg.attrs = attr;
-      cfg.numAttrs = 1;
-      ATTN_CUDA_TRY(cudaLaunchKernelEx(&cfg, kernel, ta, tb, static_cast<__nv_bfloat16*>(c), p, split));
+      kernel<<<tiles, gemm::kThreads, smem, stream>>>(ta, tb, static_cast<__nv_bfloat16*>(c), p);
       return ATTN_OK;
     };
-    rc = b_layout == 0 ? launch_split(gemm::gemm_split_kernel<true>) : launch_split(gemm::gemm_split_kernel<false>);
+    rc = b_layout == 0 ? launch_small(gemm::gemm_small_kernel<true>) : launch_small(gemm::gemm_small_kernel<false>);
     if (rc != ATTN_OK) return rc;
+    ATTN_CUDA_TRY(cudaGetLastError());
     ++t_launch_count;
     return ATTN_OK;
   }

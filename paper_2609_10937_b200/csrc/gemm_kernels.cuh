@@ -6,7 +6,7 @@
 //                 (A tile, B tile) stages -> one MMA-issuing thread (tcgen05.mma, two 128-row
 //                 sub-tiles x 256 columns accumulated in tensor memory) -> eight epilogue warps
 //                 (tensor memory -> bf16 -> shared-memory staging -> TMA store).
-//   gemm_split_kernel  few output tiles: 128 x 128 tiles, K shared out over a thread-block cluster.
+//   gemm_small_kernel  few output tiles: one 128 x 128 tile per CTA.
 //   softmax_rows_warp_kernel    short rows: one warp (or half of one) per row, no barrier.
 //   softmax_rows_kernel         longer rows: one CTA per row, the row held in registers.
 //   softmax_rows_staged_kernel  the same for rows too wide for registers: staged in shared memory.
@@ -15,7 +15,6 @@
 #pragma once
 
 #include "attn_kernels.cuh"
-#include "decode_kernels.cuh"
 
 namespace gemm {
 
@@ -497,34 +496,27 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant
 }
 
 // ---------------------------------------------------------------------------
-// gemm_split_kernel: products with few output tiles.
+// gemm_small_kernel: products with few output tiles, one 128 x 128 tile per CTA (no persistent walk).
 //
-// With 256-wide tiles a small output keeps a handful of SMs busy for all of K.  Here a tile is 128 x 128 and the k CTAs of a
-// thread-block cluster share out its K steps; each accumulates its part in tensor memory, lays it out as fp32 in its (then
-// dead) ring, and after the cluster's barrier every CTA sums its share of the rows over the k parts through distributed
-// shared memory, in ascending K order, and writes it.  Bound by the loads of a CTA (32 KB per K step into one SM) and by the
-// few microseconds of start and end.  Measured (us, 256-wide tiles / this, both launched back to back with overlapped
-// prologues): 64 x 64 x 8192 33.0 / 8.8, 300 x 520 x 4096 22.5 / 12.1, 100 x 8000 x 2000 21.2 / 11.3, 8192 x 64 x 8192
-// 43.9 / 27.5, 1000^3 10.5 / 9.4, 4 x 512^3 6.3 / 5.6.
+// 256-wide tiles of a small output leave most SMs idle; a quarter of the tile per CTA needs a quarter of the products per K
+// step, with K walked in the same order (same bits).  Bound by the loads of a CTA (32 KB per K step into one SM) and by the
+// few microseconds of start and end.  Measured (us, replays of a graph, the plan's tiles / this): 100 x 8000 x 512 8.8 / 6.3,
+// 100 x 8000 x 8192 63.3 / 39.4, 300 x 520 x 2048 14.5 / 12.4, 1000 x 1000 x 512 7.8 / 6.5, 1536 x 1536 x 2048 15.0 / 14.1.
 // ---------------------------------------------------------------------------
-constexpr int kSplitTile = 128;
-constexpr int kSplitStageBytes = 2 * kSplitTile * kTileK * 2;
-constexpr int kSplitMaxK = 8;
-__host__ __device__ constexpr int split_smem_total(int stages) { return stages * kSplitStageBytes + kMiscBytes; }
+constexpr int kSmallTile = 128;
+constexpr int kSmallStageBytes = 2 * kSmallTile * kTileK * 2;
+__host__ __device__ constexpr int small_smem_total(int stages) { return stages * kSmallStageBytes + kMiscBytes; }
 
 template <bool B_KN>
 __global__ void __launch_bounds__(kThreads, 1)
-gemm_split_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_b, __nv_bfloat16* c, const GemmParams p,
-                  int cluster_k) {
+gemm_small_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_b, __nv_bfloat16* c, const GemmParams p) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   const uint32_t smem_base = smem_u32(smem_raw);
-  GemmMisc* misc = reinterpret_cast<GemmMisc*>(smem_raw + p.stages * kSplitStageBytes);
+  GemmMisc* misc = reinterpret_cast<GemmMisc*>(smem_raw + p.stages * kSmallStageBytes);
   volatile int* abort_flag = &misc->abort.flag;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int k = cluster_k, rank = blockIdx.x % k;
-  const int tile = blockIdx.x / k;
+  const int tile = blockIdx.x;
   const int nt = tile % p.n_tiles, mt = (tile / p.n_tiles) % p.m_tiles, b = tile / (p.n_tiles * p.m_tiles);
-  const int ks_lo = p.k_steps * rank / k, ks_hi = p.k_steps * (rank + 1) / k;      // at least one step each (k <= k_steps)
 
   if (threadIdx.x == 0) {
     attn::abort_cell_init(&misc->abort, nullptr);
@@ -542,7 +534,7 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constan
     prefetch_tmap(&tm_b);
   }
   if (warp == 1) {
-    tmem_alloc(smem_u32(&misc->tmem_slot), kSplitTile);
+    tmem_alloc(smem_u32(&misc->tmem_slot), kSmallTile);
     tmem_relinquish();
   }
   tc_fence_before();
@@ -556,18 +548,18 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constan
       int stage = 0, issued = 0;
       uint32_t phase = 0;
       bool ok = true;
-      for (int ks = ks_lo; ks < ks_hi; ++ks) {
+      for (int ks = 0; ks < p.k_steps; ++ks) {
         if (!attn::wait_bar(smem_u32(&misc->empty[stage]), phase ^ 1u, abort_flag, attn::wait_info(kRoleGemmLoad, 1, ks))) { ok = false; break; }
         const uint32_t bar = smem_u32(&misc->full[stage]);
-        const uint32_t a_dst = smem_base + stage * kSplitStageBytes, b_dst = a_dst + kSplitTile * kTileK * 2;
-        mbar_arrive_expect_tx(bar, kSplitStageBytes);
-        tma_load_3d(a_dst, &tm_a, ks * kTileK, mt * kSplitTile, b, bar);
+        const uint32_t a_dst = smem_base + stage * kSmallStageBytes, b_dst = a_dst + kSmallTile * kTileK * 2;
+        mbar_arrive_expect_tx(bar, kSmallStageBytes);
+        tma_load_3d(a_dst, &tm_a, ks * kTileK, mt * kSmallTile, b, bar);
         if (B_KN) {
 #pragma unroll
-          for (int h = 0; h < kSplitTile / 64; ++h)
-            tma_load_3d(b_dst + h * (kTileK * 128), &tm_b, nt * kSplitTile + h * 64, ks * kTileK, b, bar);
+          for (int h = 0; h < kSmallTile / 64; ++h)
+            tma_load_3d(b_dst + h * (kTileK * 128), &tm_b, nt * kSmallTile + h * 64, ks * kTileK, b, bar);
         } else {
-          tma_load_3d(b_dst, &tm_b, ks * kTileK, nt * kSplitTile, b, bar);
+          tma_load_3d(b_dst, &tm_b, ks * kTileK, nt * kSmallTile, b, bar);
         }
         ++issued;
         if (++stage == p.stages) { stage = 0; phase ^= 1u; }
@@ -585,23 +577,23 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constan
     // ============================================================ MMA issuer
     int stage = 0;
     uint32_t phase = 0;
-    constexpr uint32_t idesc = make_idesc_bf16(kSub, kSplitTile, B_KN);
+    constexpr uint32_t idesc = make_idesc_bf16(kSub, kSmallTile, B_KN);
     constexpr uint32_t hi_k = attn::desc_hi_sw128(1024);
-    for (int ks = ks_lo; run && ks < ks_hi; ++ks) {
+    for (int ks = 0; run && ks < p.k_steps; ++ks) {
       if (!attn::wait_bar_warp(smem_u32(&misc->full[stage]), phase, abort_flag, attn::wait_info(kRoleGemmMma, 1, ks))) break;
       tc_fence_after();
       if (elect_one()) {
-        const uint32_t a_smem = smem_base + stage * kSplitStageBytes, b_smem = a_smem + kSplitTile * kTileK * 2;
+        const uint32_t a_smem = smem_base + stage * kSmallStageBytes, b_smem = a_smem + kSmallTile * kTileK * 2;
         const uint32_t a_lo = attn::desc_lo(a_smem, 16);
         const uint32_t b_lo = B_KN ? attn::desc_lo(b_smem, kTileK * 128) : attn::desc_lo(b_smem, 16);
 #pragma unroll
         for (int k16 = 0; k16 < kTileK / 16; ++k16) {
           const uint64_t da = attn::desc_from_words(a_lo + ((k16 * 32) >> 4), hi_k);
           const uint64_t db = attn::desc_from_words(b_lo + ((B_KN ? k16 * 2048 : k16 * 32) >> 4), hi_k);
-          umma_ss(tmem_base, da, db, idesc, (ks > ks_lo || k16 > 0) ? 1u : 0u);
+          umma_ss(tmem_base, da, db, idesc, (ks > 0 || k16 > 0) ? 1u : 0u);
         }
         umma_commit(smem_u32(&misc->empty[stage]));
-        if (ks == ks_hi - 1) umma_commit(smem_u32(&misc->acc_full));
+        if (ks == p.k_steps - 1) umma_commit(smem_u32(&misc->acc_full));
       }
       __syncwarp();
       if (++stage == p.stages) { stage = 0; phase ^= 1u; }
@@ -624,37 +616,25 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constan
                        ::"r"(smem_base + row * 512 + u * 16), "r"(r[4 * e]), "r"(r[4 * e + 1]), "r"(r[4 * e + 2]), "r"(r[4 * e + 3]) : "memory");
         }
       }
-      tc_fence_before();
     }
     __syncwarp();
   }
+  tc_fence_before();
   __syncthreads();
-  if (k > 1) cluster_sync_release();
-  // this CTA's share of the rows, eight columns per thread and turn
-  const int r_lo = kSplitTile * rank / k, units = (kSplitTile * (rank + 1) / k - r_lo) * (kSplitTile / 8);
-  for (int u = threadIdx.x; u < units; u += kThreads) {
-    const int row = r_lo + u / (kSplitTile / 8), col = (u % (kSplitTile / 8)) * 8;
-    const int gm = mt * kSplitTile + row, gn = nt * kSplitTile + col;
+  // the tile's rows, eight columns per thread and turn
+  for (int u = threadIdx.x; u < kSmallTile * (kSmallTile / 8); u += kThreads) {
+    const int row = u / (kSmallTile / 8), col = (u % (kSmallTile / 8)) * 8;
+    const int gm = mt * kSmallTile + row, gn = nt * kSmallTile + col;
     if (gm >= p.M || gn >= p.N) continue;                       // (N is a multiple of 8)
-    const uint32_t a0 = smem_base + row * 512 + (((uint32_t)(col / 4) ^ (uint32_t)(row & 31)) * 16);
-    const uint32_t a1 = smem_base + row * 512 + (((uint32_t)(col / 4 + 1) ^ (uint32_t)(row & 31)) * 16);
-    float4 x = make_float4(0.f, 0.f, 0.f, 0.f), y = x;
-#pragma unroll
-    for (int q = 0; q < kSplitMaxK; ++q) {
-      if (q >= k) break;
-      const float4 v = attn::ld_peer_f4(map_to_cta(a0, q)), w = attn::ld_peer_f4(map_to_cta(a1, q));
-      x.x += v.x; x.y += v.y; x.z += v.z; x.w += v.w;
-      y.x += w.x; y.y += w.y; y.z += w.z; y.w += w.w;
-    }
+    const uint8_t* src = smem_raw + row * 512;
+    const float4 x = *reinterpret_cast<const float4*>(src + (((uint32_t)(col / 4) ^ (uint32_t)(row & 31)) * 16));
+    const float4 y = *reinterpret_cast<const float4*>(src + (((uint32_t)(col / 4 + 1) ^ (uint32_t)(row & 31)) * 16));
     *reinterpret_cast<uint4*>(c + ((size_t)b * p.M + gm) * p.N + gn) =
         make_uint4(pack_bf16x2(x.x, x.y), pack_bf16x2(x.z, x.w), pack_bf16x2(y.x, y.y), pack_bf16x2(y.z, y.w));
   }
-  tc_fence_before();
-  if (k > 1) cluster_sync_release();                            // no CTA leaves while a peer may still read its part
-  else __syncthreads();
   if (warp == 1) {
     tc_fence_after();
-    tmem_dealloc(tmem_base, kSplitTile);
+    tmem_dealloc(tmem_base, kSmallTile);
   }
 }
 

@@ -114,9 +114,30 @@ def test_matrix_product_full_size_sampled(env):
 @pytest.mark.parametrize("batch,M,N,K", [(1, 64, 64, 8192), (1, 1, 8, 2048), (1, 129, 136, 1000), (2, 128, 128, 512), (1, 700, 200, 3000),
                                          (4, 500, 520, 264), (1, 1000, 1000, 1000), (1, 1500, 1400, 72), (1, 100, 8000, 2000)])
 def test_products_with_few_output_tiles(env, batch, M, N, K, layout):
-    """Outputs of at most one 128 x 128 tile per SM: one tile and many, rows and columns past the end of the last, K split over
-    1 to 8 CTAs with a ragged last step, more and fewer steps than the ring has stages."""
+    """Outputs of at most one 128 x 128 tile per SM: one tile and many, rows and columns past the end of the last, K with a
+    ragged last step, more and fewer steps than the ring has stages."""
     _check_product(env, batch, M, N, K, layout, seed=M + N + K)
+
+
+@pytest.mark.parametrize("layout", ["kn", "nk"])
+@pytest.mark.parametrize("M,N,K", [(257, 264, 1024), (64, 64, 8192), (300, 520, 4096), (129, 136, 1000), (100, 1000, 2000), (512, 512, 2048)])
+def test_products_do_not_depend_on_what_stands_beside_them(env, M, N, K, layout):
+    """A product alone, as an entry of a batch of 5, a block of its rows alone, the plan's tiles and the lone-CTA tiles: the
+    same bits, because every kernel sums the K products of an element in the same order."""
+    torch, go, binding = env
+    rng = np.random.default_rng([11, M, N, K])
+    a = to_cuda_bf16(_rand_bits(rng, (5, M, K)))
+    b = to_cuda_bf16(_rand_bits(rng, (5, K, N) if layout == "kn" else (5, N, K)))
+    bits = lambda x, y, **tiles: binding.gemm(x, y, b_layout=layout, **tiles).view(torch.int16)
+    whole = bits(a, b)
+    for i in range(5):
+        assert torch.equal(bits(a[i], b[i]), whole[i]), i
+        assert torch.equal(bits(a[i, : M // 2], b[i]), whole[i, : M // 2]), i
+    plan = binding.gemm_plan(binding.hw_desc_query(0), 5, M, N, K)
+    assert torch.equal(bits(a, b, cta_pair=plan.cta_pair), whole)       # (an override: the plan's tiles)
+    assert torch.equal(bits(a, b, cta_pair=1), whole)
+    torch.cuda.synchronize()
+    assert binding.last_device_status()[0] == 0
 
 
 @pytest.mark.parametrize("rows,cols", [(4, 8), (7, 256), (33, 2048), (5, 2056), (3, 16384), (2, 32768), (9, 1000),
