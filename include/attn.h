@@ -253,7 +253,8 @@ int attn_forward_qk(const void *q, const void *k, const void *v, void *o,
  * that masked elements are -inf, never zero, Section "Online Softmax", applied to
  * a triangular mask; the paper itself evaluates non-causal attention only).
  * Key steps wholly after a Q tile's last row are skipped, not computed and masked.
- * Where it is faster, a plan of equal ranges is executed as whole tiles, longest first (the tiles then need no merge).
+ * Where it is faster, the device's own plan of equal ranges is executed as whole tiles, longest first (the tiles then need no
+ * merge); attn_forward_desc and attn_forward_tiles launch the grid of their plan.
  * Always needs a registered workspace (attn_workspace_bytes of attn_plan_ex(...,1,...)).
  */
 int attn_forward_causal(const void *q, const void *k, const void *v, void *o,
@@ -391,6 +392,22 @@ int attn_last_launch_count(void);
  * uniform key split of k CTAs per Q tile and those were launched as one cluster each (their
  * partial results then travel through distributed shared memory), 0 otherwise. */
 int attn_last_cluster_size(void);
+
+/* The kernel of the last launch that a call on this thread made (of its last one where it made several), and the number
+ * of CTAs it was launched with. */
+enum attn_kernel {
+  ATTN_KERNEL_NONE = 0,
+  ATTN_KERNEL_TILED = 1,         /* the fused kernel with the plan's grid                        */
+  ATTN_KERNEL_CAUSAL_TILES = 2,  /* causal, one CTA per Q tile                                   */
+  ATTN_KERNEL_FEW_ROWS = 3,      /* few query rows against many keys                             */
+  ATTN_KERNEL_SIMPLE = 4,        /* attn_forward_simple                                          */
+  ATTN_KERNEL_GEMM = 5,          /* matrix product, lone CTAs                                    */
+  ATTN_KERNEL_GEMM_PAIR = 6,     /* matrix product, CTA pairs                                    */
+  ATTN_KERNEL_GEMM_SMALL = 7,    /* matrix product, one 128 x 128 tile per CTA                   */
+  ATTN_KERNEL_SOFTMAX = 8        /* row softmax                                                  */
+};
+int attn_last_kernel(void);
+int attn_last_grid(void);
 
 /* Static description of a status code; never NULL. */
 const char *attn_status_string(int status);

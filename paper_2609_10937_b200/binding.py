@@ -18,13 +18,15 @@ ATTN_OK = 0
 ERR_INVALID_ARG, ERR_UNSUPPORTED_SHAPE, ERR_MISALIGNED, ERR_ALIASING = -1, -2, -3, -4
 ERR_INFEASIBLE_PLAN, ERR_WRONG_ARCH, ERR_NEED_WORKSPACE, ERR_CUDA = -5, -6, -7, -8
 ERR_DEVICE_TIMEOUT, ERR_BAD_TILES, ERR_SCRATCH_LIMIT = -9, -10, -11
+(KERNEL_NONE, KERNEL_TILED, KERNEL_CAUSAL_TILES, KERNEL_FEW_ROWS, KERNEL_SIMPLE, KERNEL_GEMM, KERNEL_GEMM_PAIR, KERNEL_GEMM_SMALL,
+ KERNEL_SOFTMAX) = range(9)
 BIND_NAMES = ("none", "smem", "tmem", "reg", "atom", "shape")
 
 EXPORTED_SYMBOLS = (
     "attn_hw_desc_b200", "attn_hw_desc_query", "attn_plan", "attn_plan_ex", "attn_workspace_bytes",
     "attn_set_workspace", "attn_workspace_init", "attn_forward_ws", "attn_status_read", "attn_forward", "attn_forward_causal", "attn_forward_tiles", "attn_forward_simple", "attn_forward_host", "attn_forward_host_workspace_bytes", "attn_forward_static_scratch", "attn_forward_desc", "attn_plan_qk", "attn_forward_qk",
     "attn_last_device_status", "attn_selftest_wait_expiry", "attn_selftest_wait_expiry_to",
-    "attn_last_launch_count", "attn_last_cluster_size", "attn_status_string", "attn_last_cuda_error",
+    "attn_last_launch_count", "attn_last_cluster_size", "attn_last_kernel", "attn_last_grid", "attn_status_string", "attn_last_cuda_error",
     "gemm_plan", "gemm_forward", "gemm_forward_tiles", "softmax_rows_forward", "attn_forward_unfused",
 )
 
@@ -109,6 +111,8 @@ def lib() -> ctypes.CDLL:
         L.attn_selftest_wait_expiry_to.argtypes = [vp, vp]
         L.attn_last_launch_count.argtypes = []
         L.attn_last_cluster_size.argtypes = []
+        L.attn_last_kernel.argtypes = []
+        L.attn_last_grid.argtypes = []
         L.attn_status_string.argtypes = [i32]
         L.attn_status_string.restype = ctypes.c_char_p
         L.attn_last_cuda_error.argtypes = []
@@ -415,6 +419,16 @@ def last_launch_count() -> int:
 def last_cluster_size() -> int:
     """CTAs per thread-block cluster of the last fused launch (0: launched without clusters)."""
     return int(lib().attn_last_cluster_size())
+
+
+def last_kernel() -> int:
+    """Kernel of the last launch on this thread (KERNEL_...)."""
+    return int(lib().attn_last_kernel())
+
+
+def last_grid() -> int:
+    """CTAs of the last launch on this thread."""
+    return int(lib().attn_last_grid())
 
 
 # ----------------------------------------------------------------- unfused path

@@ -25,6 +25,8 @@ namespace {
 thread_local char t_cuda_error[256] = "";
 thread_local int t_launch_count = 0;
 thread_local int t_cluster_size = 0;   // CTAs per thread-block cluster of the last fused launch (0: no clusters)
+thread_local int t_kernel = ATTN_KERNEL_NONE, t_grid = 0;   // the last launch and its CTAs
+void launched(int kernel, long long ctas) { t_kernel = kernel; t_grid = (int)ctas; }
 
 int cuda_fail(cudaError_t e, const char* what) {
   std::snprintf(t_cuda_error, sizeof t_cuda_error, "%s: %s", what, cudaGetErrorString(e));
@@ -294,6 +296,7 @@ int launch_fwd(const void* q, const void* k, const void* v, void* o, int B, int 
   if (rc != ATTN_OK) return rc;
   ATTN_CUDA_TRY(cudaGetLastError());
   t_launch_count = 1;
+  launched(ATTN_KERNEL_TILED, grid);
   return ATTN_OK;
 }
 
@@ -333,6 +336,7 @@ int launch_decode(const void* q, const void* k, const void* v, void* o, int BH, 
   ATTN_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, tk, tv, p));
   t_cluster_size = cluster_k > 1 ? cluster_k : 0;
   t_launch_count = 1;
+  launched(ATTN_KERNEL_FEW_ROWS, (long long)BH * cluster_k);
   return ATTN_OK;
 }
 
@@ -407,8 +411,8 @@ int dispatch_decode(const void* q, const void* k, const void* v, void* o, int BH
 
 // Causal attention as whole Q tiles, one CTA each (tiles_kernel.cuh).
 template <int D>
-int launch_causal_tiles(const void* q, const void* k, const void* v, void* o, int BH, int L, int local_mem, unsigned int* status,
-                        DeviceState* st, cudaStream_t stream) {
+int launch_causal_tiles(const void* q, const void* k, const void* v, void* o, int BH, int L, unsigned int* status, DeviceState* st,
+                        cudaStream_t stream) {
   using SM = attn::TilesSmem<D>;
   CUtensorMap tq, tk, tv, to;
   int rc;
@@ -426,7 +430,7 @@ int launch_causal_tiles(const void* q, const void* k, const void* v, void* o, in
   const long long at_most = std::max(1LL, st->desc.cache_bytes / (3 * 4LL * L * D));
   const long long groups = (BH + at_most - 1) / at_most;
   p.group_heads = (int)((BH + groups - 1) / groups);
-  p.stages = std::min(attn::kMaxStages, (local_mem - SM::total(0)) / SM::kStageBytes);
+  p.stages = std::min(attn::kMaxStages, (st->desc.local_mem_bytes - SM::total(0)) / SM::kStageBytes);
   p.scale_log2 = (float)(1.4426950408889634 / std::sqrt((double)D));
   p.status = status;
   const int smem = SM::total(p.stages);
@@ -436,6 +440,7 @@ int launch_causal_tiles(const void* q, const void* k, const void* v, void* o, in
   ATTN_CUDA_TRY(cudaGetLastError());
   t_cluster_size = 0;
   t_launch_count = 1;
+  launched(ATTN_KERNEL_CAUSAL_TILES, (long long)BH * p.q_tiles);
   return ATTN_OK;
 }
 
@@ -455,12 +460,12 @@ bool causal_whole_tiles(const attn_tiles& t, int BH, int L, int d, int local_mem
 
 int dispatch_fwd(const void* q, const void* k, const void* v, void* o, int B, int H, int L, int d,
                  const attn_tiles& t, float* ws, unsigned int* status, DeviceState* st, cudaStream_t s, int Lk = 0,
-                 bool may_overlap = false, const attn_hw_desc* own_plan_of = nullptr) {
+                 bool may_overlap = false, bool own_plan = false) {
   if (Lk == 0) Lk = L;
-  // (a plan made here, not one that a caller has changed)
-  if (own_plan_of && Lk == L && causal_whole_tiles(t, B * H, L, d, own_plan_of->local_mem_bytes, st->desc.num_units))
-    return d == 128 ? launch_causal_tiles<128>(q, k, v, o, B * H, L, own_plan_of->local_mem_bytes, status, st, s)
-                    : launch_causal_tiles<64>(q, k, v, o, B * H, L, own_plan_of->local_mem_bytes, status, st, s);
+  // own_plan: the device's own, with no field changed and from no caller's descriptor -- those say how many CTAs run
+  if (own_plan && Lk == L && causal_whole_tiles(t, B * H, L, d, st->desc.local_mem_bytes, st->desc.num_units))
+    return d == 128 ? launch_causal_tiles<128>(q, k, v, o, B * H, L, status, st, s)
+                    : launch_causal_tiles<64>(q, k, v, o, B * H, L, status, st, s);
 #define ATTN_CASE(D_, TKV_, NQ_) \
   if (d == D_ && t.tile_kv == TKV_ && t.n_q == NQ_) \
     return launch_fwd<D_, TKV_, NQ_>(q, k, v, o, B, H, L, Lk, t, ws, status, st, s, may_overlap);
@@ -564,7 +569,7 @@ int forward_impl(const void* q, const void* k, const void* v, void* o, int B, in
   if (!ovr && !plan_desc && !call_ws && Lk != L && decode_rows(L, Lk, d, t, st->desc.num_units))
     return dispatch_decode(q, k, v, o, B * H, L, Lk, d, nullptr, st, static_cast<cudaStream_t>(cuda_stream));
   return dispatch_fwd(q, k, v, o, B, H, L, d, t, ws, call_ws ? call_ws->status : nullptr, st,
-                      static_cast<cudaStream_t>(cuda_stream), Lk, call_ws != nullptr, ovr ? nullptr : &desc);
+                      static_cast<cudaStream_t>(cuda_stream), Lk, call_ws != nullptr, !ovr && !plan_desc);
 }
 
 template <int D, int TKV>
@@ -584,6 +589,7 @@ int launch_simple(const void* q, const void* k, const void* v, void* o, int B, i
   kern<<<grid, 128, smem, stream>>>(tq, tk, tv, reinterpret_cast<__nv_bfloat16*>(o), L, scale_log2, scores_out);
   ATTN_CUDA_TRY(cudaGetLastError());
   t_launch_count = 1;
+  launched(ATTN_KERNEL_SIMPLE, (long long)grid.x * grid.y);
   return ATTN_OK;
 }
 
@@ -950,6 +956,8 @@ extern "C" int attn_last_device_status(void* cuda_stream, uint32_t* detail) {
 
 extern "C" int attn_last_launch_count(void) { return t_launch_count; }
 extern "C" int attn_last_cluster_size(void) { return t_cluster_size; }
+extern "C" int attn_last_kernel(void) { return t_kernel; }
+extern "C" int attn_last_grid(void) { return t_grid; }
 
 extern "C" const char* attn_last_cuda_error(void) { return t_cuda_error; }
 
@@ -1049,6 +1057,7 @@ int gemm_launch(const void* a, const void* b, void* c, int batch, int M, int N, 
     if (rc != ATTN_OK) return rc;
     ATTN_CUDA_TRY(cudaGetLastError());
     ++t_launch_count;
+    launched(ATTN_KERNEL_GEMM_SMALL, tiles);
     return ATTN_OK;
   }
   CUtensorMap ta, tb, tc;
@@ -1113,6 +1122,7 @@ int gemm_launch(const void* a, const void* b, void* c, int batch, int M, int N, 
   if (rc != ATTN_OK) return rc;
   ATTN_CUDA_TRY(cudaGetLastError());
   ++t_launch_count;
+  launched(pair ? ATTN_KERNEL_GEMM_PAIR : ATTN_KERNEL_GEMM, t.ctas);
   return ATTN_OK;
 }
 
@@ -1129,11 +1139,12 @@ int softmax_launch(const void* s, void* pout, long long rows, int cols, float sc
   int rc = device_state(&st);
   if (rc != ATTN_OK) return rc;
   const int sms = st->desc.num_units;
+  long long ctas = rows;
   // Up to 128 vectors a row: a warp per row (half a warp below 17 vectors), at most 16 CTAs of four warps per SM
   // (65536 x 1024: 43.2 us, 8 CTAs 47.9; one CTA per row is slower at every width up to here).
   auto launch_warp = [&](auto kern, int rows_per_warp) {
-    const long long ctas = (rows + 4 * rows_per_warp - 1) / (4 * rows_per_warp);
-    kern<<<(unsigned)std::min(ctas, 16LL * sms), 128, 0, stream>>>(sp, pp, rows, cols, scale_log2);
+    ctas = std::min((rows + 4 * rows_per_warp - 1) / (4 * rows_per_warp), 16LL * sms);
+    kern<<<(unsigned)ctas, 128, 0, stream>>>(sp, pp, rows, cols, scale_log2);
   };
   // Longer rows: a CTA per row, as few warps as hold it at VPT vectors a thread (5000 columns on 160 threads: 18.6 us for
   // 5000 rows, on 256 threads 24.8).
@@ -1165,6 +1176,7 @@ int softmax_launch(const void* s, void* pout, long long rows, int cols, float sc
 #undef SOFTMAX_ROW_CASE
   ATTN_CUDA_TRY(cudaGetLastError());
   ++t_launch_count;
+  launched(ATTN_KERNEL_SOFTMAX, ctas);
   return ATTN_OK;
 }
 

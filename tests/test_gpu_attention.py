@@ -539,6 +539,23 @@ def test_changed_cost_constants_change_the_grid_and_the_launch_follows(env):
     assert binding.last_cluster_size() == 0
 
 
+@pytest.mark.parametrize("B,H,L,d,units", [(1, 2, 4096, 128, 16), (1, 12, 2048, 64, 40), (2, 40, 300, 64, 100)])
+def test_causal_launch_stays_inside_the_descriptors_machine(env, B, H, L, d, units):
+    """attn_forward_desc, causal, with fewer compute units than Q tiles: the launch is the plan's, no more CTAs than the
+    descriptor has units, also at shapes that the device's own plan would run as one CTA per Q tile; and so it is when only
+    the cost constants differ."""
+    torch, _, binding = env
+    case = _case("desc_causal", B, H, L, d)
+    rows = synth.sample_rows(L) if L > 1024 else None
+    for field, value in (("num_units", units), ("ovh_causal_ranges", 60)):
+        desc = binding.hw_desc_query(0)
+        setattr(desc, field, value)
+        plan = binding.plan(desc, B, H, L, d, causal=True)
+        assert plan.feasible and plan.ctas <= desc.num_units
+        _run_and_compare(env, case, lambda a, b, c: binding.forward_desc(desc, a, b, c, causal=True), rows=rows, causal=True)
+        assert (binding.last_kernel(), binding.last_grid()) == (binding.KERNEL_TILED, plan.ctas), (field, plan.ctas)
+
+
 def test_uniform_split_larger_than_the_machine_is_merged_by_the_last_finisher(env):
     """Fixed merge roles make a merging warp wait for the other CTAs of its tile, so they need every CTA resident.  A
     uniform split with more CTAs than SMs (an override; the closed form never asks for one) runs the instantiation in
