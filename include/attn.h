@@ -384,6 +384,10 @@ int attn_selftest_wait_expiry(void *cuda_stream);
 /* The same with the record going to four caller-owned DEVICE words (as attn_forward_ws's status_dev; NULL: the
  * device-wide record): shows that an expiry is attributed to the launch whose status words were given. */
 int attn_selftest_wait_expiry_to(uint32_t *status_dev, void *cuda_stream);
+/* The same for the wait whose expiry is noted and reported by one thread at the end of the kernel (the causal kernel's), with a
+ * copy under way that has to land first: detail[1] as above if it did, step 0 in it if not.  Takes twice the limit, about
+ * a second. */
+int attn_selftest_quiet_expiry_to(uint32_t *status_dev, void *cuda_stream);
 
 /* Number of kernels the last attn_forward* call on this thread launched. */
 int attn_last_launch_count(void);

@@ -920,16 +920,56 @@ __global__ void wait_expiry_selftest_kernel(unsigned int* status) {
   (void)attn::wait_bar_warp(sm100::smem_u32(&bar), 0, &abort_cell.flag,
                             attn::wait_info(attn::kRoleSimple, attn::kBarSync, ATTN_SELFTEST_STEP));
 }
+
+// The other way out of a wait: a warp with a copy under way waits with wait_quiet on a barrier that nothing arrives at, drains
+// its copy, and one thread reports.  The reported step is ATTN_SELFTEST_STEP only if the copy had landed when its drain
+// ended, and a drain of the barrier that nothing arrives at gave up.
+__device__ __align__(16) uint32_t g_selftest_words[4] = {0x11, 0x22, 0x33, 0x44};
+__global__ void quiet_expiry_selftest_kernel(unsigned int* status) {
+  __shared__ uint64_t bar, copy_bar;
+  __shared__ __align__(16) uint32_t words[4];
+  __shared__ attn::AbortCell abort_cell;
+  if (threadIdx.x == 0) {
+    attn::abort_cell_init(&abort_cell, status);
+    sm100::mbar_init(sm100::smem_u32(&bar), 1);
+    sm100::mbar_init(sm100::smem_u32(&copy_bar), 1);
+    sm100::fence_mbar_init();
+    sm100::mbar_arrive_expect_tx(sm100::smem_u32(&copy_bar), sizeof words);
+    sm100::bulk_load(sm100::smem_u32(words), g_selftest_words, sizeof words, sm100::smem_u32(&copy_bar));
+  }
+  __syncthreads();
+  const bool arrived = attn::wait_quiet_warp(sm100::smem_u32(&bar), 0, &abort_cell.flag,
+                                             attn::wait_info(attn::kRoleSimple, attn::kBarSync, ATTN_SELFTEST_STEP));
+  if (!arrived && threadIdx.x == 0) {
+    bool good = attn::drain_bar(sm100::smem_u32(&copy_bar), 0);
+    for (int i = 0; i < 4; ++i) good = good && words[i] == g_selftest_words[i];
+    good = good && !attn::drain_bar(sm100::smem_u32(&bar), 0);
+    if (!good) abort_cell.info = attn::wait_info(attn::kRoleSimple, attn::kBarSync, 0);
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) attn::report_abort(&abort_cell);
+}
 }  // namespace
 
-extern "C" int attn_selftest_wait_expiry_to(uint32_t* status_dev, void* cuda_stream) {
+namespace {
+template <class Kernel>
+int launch_selftest(Kernel kern, uint32_t* status_dev, void* cuda_stream) {
   if (status_dev && ((uintptr_t)status_dev & 15u)) return ATTN_ERR_MISALIGNED;
   DeviceState* st = nullptr;
   int rc = device_state(&st);
   if (rc != ATTN_OK) return rc;
-  wait_expiry_selftest_kernel<<<1, 32, 0, static_cast<cudaStream_t>(cuda_stream)>>>(status_dev);
+  kern<<<1, 32, 0, static_cast<cudaStream_t>(cuda_stream)>>>(status_dev);
   ATTN_CUDA_TRY(cudaGetLastError());
   return ATTN_OK;
+}
+}  // namespace
+
+extern "C" int attn_selftest_wait_expiry_to(uint32_t* status_dev, void* cuda_stream) {
+  return launch_selftest(wait_expiry_selftest_kernel, status_dev, cuda_stream);
+}
+
+extern "C" int attn_selftest_quiet_expiry_to(uint32_t* status_dev, void* cuda_stream) {
+  return launch_selftest(quiet_expiry_selftest_kernel, status_dev, cuda_stream);
 }
 
 extern "C" int attn_selftest_wait_expiry(void* cuda_stream) { return attn_selftest_wait_expiry_to(nullptr, cuda_stream); }

@@ -114,6 +114,14 @@ __device__ __forceinline__ bool wait_quiet(uint32_t bar, uint32_t parity, volati
 __device__ __forceinline__ bool wait_quiet_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag, uint32_t info) {
   return __all_sync(0xffffffffu, wait_quiet(bar, parity, abort_flag, info) ? 1 : 0) != 0;
 }
+// On the way out of an expired wait: a copy that is under way must land before its memory is used again or the CTA exits.
+// Bounded like the waits; false if it has not landed.
+__device__ __forceinline__ bool drain_bar(uint32_t bar, uint32_t parity) {
+  const long long t0 = clock64();
+  while (!mbar_try_wait(bar, parity))
+    if (clock64() - t0 > kWaitLimitCycles) return false;
+  return true;
+}
 // By one thread, when every thread of the CTA is past its last wait.
 __device__ __forceinline__ void report_abort(const AbortCell* c) {
   if (c->flag == 0) return;

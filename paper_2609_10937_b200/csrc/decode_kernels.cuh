@@ -20,6 +20,10 @@ constexpr int kDecodeSlabBytes = 8192;
 constexpr int kDecodeMaxSplit = 16;        // CTAs per head (one cluster; above 8 only where the device allows it)
 enum : uint32_t { kRoleDecode = 9 };
 __host__ __device__ constexpr int decode_slab_keys(int d) { return kDecodeSlabBytes / (4 * d); }   // K and V, bf16
+// While a warp waits for slab `it` of its n, the slabs it has started and not yet waited for are it ... (this) - 1.
+__host__ __device__ constexpr int decode_started(int it, int n) { return it + kDecodeStages < n ? it + kDecodeStages : n; }
+static_assert(decode_started(0, 1) == 1 && decode_started(0, kDecodeStages) == kDecodeStages && decode_started(0, 9) == kDecodeStages &&
+              decode_started(5, 9) == 5 + kDecodeStages && decode_started(7, 9) == 9 && decode_started(8, 9) == 9, "slabs under way");
 
 struct DecodeParams {
   const __nv_bfloat16* q;
@@ -145,7 +149,8 @@ attn_decode_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_consta
   const uint32_t k_row = (uint32_t)((mi >> 1) * 8 + r) * 128, v_row = (uint32_t)((mi & 1) * 8 + r) * 128;
   int stage = 0;
   uint32_t phase = 0;
-  for (int it = 0; it < n; ++it) {
+  int it = 0;
+  for (; it < n; ++it) {
     if (!wait_bar_warp(smem_u32(&misc->full[warp][stage]), phase, abort_flag, wait_info(kRoleDecode, kBarKvFull, it))) break;
     const uint32_t k_smem = ring + stage * kDecodeSlabBytes, v_smem = k_smem + kHalfBytes;
     float s[MT][2 * KP][4];
@@ -235,10 +240,8 @@ attn_decode_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_consta
     if (lane == 0 && it + kDecodeStages < n) issue(it + kDecodeStages, stage);
     if (++stage == kDecodeStages) { stage = 0; phase ^= 1u; }
   }
-  if (*abort_flag) {                                            // a copy still in flight must land before the CTA exits
-    const long long t0 = clock64();
-    while (clock64() - t0 < 2000000LL) {}
-  }
+  if (it < n && lane == 0)                                      // a wait gave up
+    for (int u = it; u < decode_started(it, n); ++u) drain_bar(smem_u32(&misc->full[warp][u % kDecodeStages]), (uint32_t)(u / kDecodeStages) & 1u);
   __syncthreads();                                              // the rings are dead: they hold the partial results now
 
   float* part = reinterpret_cast<float*>(smem_raw);             // [warp][row][D], then the CTA's own [row][D]

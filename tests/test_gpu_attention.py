@@ -649,6 +649,29 @@ def test_bounded_wait_expiry_is_recorded_in_the_callers_status_words(env):
     assert torch.equal(out.view(torch.int16), want.view(torch.int16))
 
 
+@pytest.mark.parametrize("own_status", [False, True])
+def test_quietly_expired_wait_drains_its_copies_and_is_reported(env, own_status):
+    """The wait of the causal kernel and the drain of the few-row kernel: the self-test's warp gives up on a barrier nothing
+    arrives at, finds the copy it had under way landed, gives up draining the silent barrier too, and reports at its end, in the
+    caller's status words or in the device-wide record.  Both kernels then compute as before."""
+    torch, _, binding = env
+    assert binding.last_device_status()[0] == 0
+    status = torch.zeros(4, dtype=torch.int32, device="cuda")
+    stream = torch.cuda.current_stream().cuda_stream
+    assert binding.lib().attn_selftest_quiet_expiry_to(status.data_ptr() if own_status else None, stream) == 0
+    code, detail = binding.status_read(status, None) if own_status else binding.last_device_status()
+    assert code == binding.ERR_DEVICE_TIMEOUT
+    assert detail[0] == 1 and detail[1] == (5 << 24) | (10 << 16) | 0x7E57 and detail[2] == 0
+    assert binding.last_device_status()[0] == 0 and binding.status_read(status, None) == (0, [0, 0, 0, 0])
+    case = _case("after_quiet_expiry", 1, 160, 257, 64)
+    _run_and_compare(env, case, lambda a, b, c: binding.forward(a, b, c, causal=True), causal=True)
+    assert binding.last_kernel() == binding.KERNEL_CAUSAL_TILES
+    q, k, v = (torch.randn(1, 2, n, 64, device="cuda").to(torch.bfloat16) for n in (1, 500, 500))
+    ref = torch.softmax(q.double() @ k.double().transpose(2, 3) / 8, dim=-1) @ v.double()
+    assert_close(to_host_f64(binding.forward_qk(q, k, v)).reshape(ref.shape), ref.cpu().numpy())
+    assert binding.last_kernel() == binding.KERNEL_FEW_ROWS and binding.last_device_status()[0] == 0
+
+
 @pytest.mark.parametrize("B,H,L,d,causal", [(2, 40, 2048, 64, False), (4, 32, 8192, 64, False), (1, 8, 2048, 64, False),
                                             (2, 40, 2048, 128, False), (2, 40, 2048, 64, True)])
 def test_many_launches_no_wait_expires_and_the_bits_repeat(env, B, H, L, d, causal):
