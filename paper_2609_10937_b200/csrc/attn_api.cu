@@ -106,19 +106,32 @@ int device_state(DeviceState** out) {
   return s.arch_ok ? ATTN_OK : ATTN_ERR_WRONG_ARCH;
 }
 
-// Dynamic shared memory a kernel may use on the current device, raised when a launch needs more than any before it (asking
-// the driver every time took about as long as the launch itself).
+// Number of the current context, unlike any other of the process; 0 if none is current yet.
+unsigned long long current_context() {
+  using GetIdFn = CUresult (*)(CUcontext, unsigned long long*);
+  static const GetIdFn fn = [] {
+    void* p = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPoint("cuCtxGetId", &p, cudaEnableDefault, &q) != cudaSuccess || q != cudaDriverEntryPointSuccess) p = nullptr;
+    return reinterpret_cast<GetIdFn>(p);
+  }();
+  unsigned long long id = 0;
+  return fn && fn(nullptr, &id) == CUDA_SUCCESS ? id : 0;
+}
+
+// Dynamic shared memory a kernel may use, raised when a launch needs more than the last one that raised it (asking the driver
+// every time took about as long as the launch itself).  The allowance belongs to the context: it is asked for again in a
+// context other than the one it was last asked for in (several contexts on a device; cudaDeviceReset).
 int allow_smem(const void* kern, int bytes) {
+  struct Allowed { unsigned long long context; int bytes; };
   static std::mutex mu;
-  static std::unordered_map<const void*, int> allowed[kMaxDevices];
-  int dev = 0;
-  ATTN_CUDA_TRY(cudaGetDevice(&dev));
-  if (dev < 0 || dev >= kMaxDevices) return ATTN_ERR_INVALID_ARG;
+  static std::unordered_map<const void*, Allowed> allowed;
+  const unsigned long long context = current_context();
   std::lock_guard<std::mutex> lk(mu);
-  int& have = allowed[dev][kern];
-  if (have >= bytes) return ATTN_OK;
+  Allowed& have = allowed[kern];
+  if (context != 0 && have.context == context && have.bytes >= bytes) return ATTN_OK;
   ATTN_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
-  have = bytes;
+  have = {context, bytes};
   return ATTN_OK;
 }
 #define ATTN_ALLOW_SMEM(kern, bytes)                                                 \

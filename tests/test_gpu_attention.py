@@ -696,6 +696,60 @@ def test_many_launches_no_wait_expires_and_the_bits_repeat(env, B, H, L, d, caus
             assert torch.equal(out.view(torch.int16), first.view(torch.int16)), f"launch {it} differs from the first"
 
 
+_RESET_CHILD = """
+import ctypes, sys
+import numpy as np
+rt, lib = ctypes.CDLL("libcudart.so.12"), ctypes.CDLL(sys.argv[1])
+vp, i32, size = ctypes.c_void_p, ctypes.c_int, ctypes.c_size_t
+lib.attn_last_cuda_error.restype = ctypes.c_char_p
+
+def dev(nbytes, host=None):
+    p = vp()
+    assert rt.cudaMalloc(ctypes.byref(p), size(nbytes)) == 0
+    if host is not None:
+        assert rt.cudaMemcpy(p, host.ctypes.data_as(vp), size(nbytes), 1) == 0
+    return p
+
+def call(fn, sizes, tail):
+    # inputs of the given sizes (bf16 values, the last one the output), then the call's other arguments
+    rng = np.random.default_rng(3)
+    ins = [(rng.standard_normal(n).astype(np.float32).view(np.uint32) >> 16).astype(np.uint16) for n in sizes[:-1]]
+    ptrs = [dev(2 * n, h) for n, h in zip(sizes, ins)] + [dev(2 * sizes[-1])]
+    rc = getattr(lib, fn)(*ptrs, *tail, vp(None))
+    assert rc == 0, (fn, rc, lib.attn_last_cuda_error())
+    assert rt.cudaDeviceSynchronize() == 0
+    out = np.zeros(sizes[-1], np.uint16)
+    assert rt.cudaMemcpy(out.ctypes.data_as(vp), ptrs[-1], size(2 * sizes[-1]), 2) == 0
+    return out
+
+def all_calls():
+    assert lib.attn_set_workspace(0, dev(64 << 20), size(64 << 20)) == 0
+    n, m = 2 * 512 * 128, 160 * 257 * 64
+    return [call("attn_forward", [n] * 4, [i32(x) for x in (1, 2, 512, 128)]),
+            call("attn_forward_causal", [m] * 4, [i32(x) for x in (1, 160, 257, 64)]),
+            call("attn_forward_qk", [256, n, n, 256], [i32(x) for x in (1, 2, 1, 512, 128)]),
+            call("gemm_forward", [1000 * 64, 1000 * 64, 1000 * 1000], [i32(x) for x in (1, 1000, 1000, 64, 1)]),
+            call("gemm_forward", [4096 * 320, 768 * 320, 4096 * 768], [i32(x) for x in (1, 4096, 768, 320, 1)]),
+            call("softmax_rows_forward", [3 * 32768] * 2, [ctypes.c_longlong(3), i32(32768), ctypes.c_float(0.5)])]
+
+first = all_calls()
+assert rt.cudaDeviceReset() == 0
+assert all((a == b).all() for a, b in zip(first, all_calls()))
+print("same")
+"""
+
+
+def test_calls_go_on_in_a_new_context(env):
+    """A program that resets the device between two calls (its context ends, and with it what a kernel was allowed in it) gets
+    the same results after it has registered a workspace again.  In a process of its own: the reset ends its context only."""
+    import subprocess
+    import sys
+
+    _, _, binding = env
+    r = subprocess.run([sys.executable, "-c", _RESET_CHILD, str(binding.LIB_PATH)], capture_output=True, text=True, timeout=120)
+    assert r.returncode == 0 and r.stdout.strip() == "same", r.stdout + r.stderr
+
+
 def test_descriptor_of_a_larger_machine_is_refused(env):
     torch, _, binding = env
     desc = binding.hw_desc_query(0)
