@@ -239,7 +239,7 @@ int attn_status_read(uint32_t *status_dev, void *workspace, void *cuda_stream, u
  * operator is the case Lq == Lk; a block of query rows of a longer sequence is the case
  * q = Q + r0 * d, Lq = rows in the block (what attn_forward_host uses to overlap copies with
  * compute).  attn_plan_qk is the derivation for it (tiles from Lq, key steps from Lk).
- * Few rows (up to 16; up to 32 at d = 64 and for many long heads) with Lq != Lk run in a kernel of their own that streams
+ * Few rows (up to 16; up to 32 at d = 64, and at d = 128 where many long heads would leave compute units idle) with Lq != Lk run in a kernel of their own that streams
  * the keys; the CTAs of a head are then one cluster (attn_last_cluster_size) and no workspace is touched.
  * Errors as attn_forward.
  */

@@ -494,13 +494,16 @@ int dispatch_fwd(const void* q, const void* k, const void* v, void* o, int B, in
   return ATTN_ERR_BAD_TILES;
 }
 
-// Calls that the decode kernel takes over from the tiled one.  Up to 16 rows (at d = 64 up to 32) it is faster at every size
-// measured (1.2-4.9 times).  17 to 32 rows at d = 128 keep its warps as busy as HBM: there only where the tiled kernel would
-// run whole tiles in waves over more than a thousand keys (24 rows, us tiled / decode: 192 heads x 8192 keys 201 / 145,
-// 192 x 2048 56 / 47; below that 128 x 2048 30.6 / 31.2, 128 x 512 13.4 / 17.1).
+// Calls that the decode kernel takes over from the tiled one.  Up to 16 rows (at d = 64 up to 32) it is as fast or faster at every
+// size measured (1.0-5 times).  17 to 32 rows at d = 128 keep its warps as busy as HBM: there only where the tiled kernel would
+// run whole tiles in waves and leave an eighth of their slots empty, in an even number of waves (two of them are one of the
+// decode kernel's, which has two CTAs per SM), over 750 keys a wave or more (us tiled / decode, 24 rows: 192 heads x 2048 keys
+// 55.7 / 49.6, 256 x 4096 103 / 88; 32 rows: 256 x 1500 48.5 / 44.5, 500 x 3000 158 / 140).  On the other side, 32 rows:
+// 256 x 1280 39.8 / 40.0, 296 x 4096 103 / 110, 350 x 1280 57 / 74, 444 x 1024 48 / 65.
 bool decode_rows(int Lq, int Lk, int d, const attn_tiles& t, int sms) {
   if (Lq <= 16 || (d == 64 && Lq <= 32)) return true;
-  return Lq <= 32 && t.tiles > sms && t.ctas == t.tiles && Lk >= 1024;
+  const long long waves = (t.tiles + sms - 1) / sms;
+  return Lq <= 32 && t.ctas == t.tiles && waves % 2 == 0 && 8LL * t.tiles <= 7LL * waves * sms && Lk >= 750LL * waves;
 }
 
 // A plan needs the workspace unless every CTA owns exactly one whole Q tile.

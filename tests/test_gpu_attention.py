@@ -915,6 +915,26 @@ def test_few_query_rows_against_many_keys(env, B, H, Lq, Lk, d):
     assert torch.equal(again.view(torch.int16), out.view(torch.int16))
 
 
+@pytest.mark.parametrize("heads,Lq,Lk,few", [(192, 17, 1500, True), (259, 32, 2049, True), (260, 32, 2048, False), (192, 24, 1499, False),
+                                              (444, 32, 1024, False), (350, 28, 1280, False), (148, 17, 2048, False),
+                                              (518, 25, 3000, True), (519, 25, 3000, False), (500, 25, 2999, False)])
+def test_seventeen_to_thirty_two_rows_at_d128_on_both_sides_of_the_rule(env, heads, Lq, Lk, few):
+    """17 to 32 rows at d = 128 run in the few-row kernel only where the tiled kernel has an even number of waves, no more than seven
+    eighths full, over at least 750 keys a wave: outside, the tiled kernel is as fast or faster.  Every element against fp64."""
+    torch, _, binding = env
+    assert binding.hw_desc_query(0).num_units == 148
+    gen = torch.Generator(device="cuda").manual_seed(heads + Lq + Lk)
+    q, k, v = (torch.randn(1, heads, n, 128, generator=gen, device="cuda").to(torch.bfloat16) for n in (Lq, Lk, Lk))
+    out = binding.forward_qk(q, k, v, torch.full_like(q, float("nan")))
+    assert binding.last_kernel() == (binding.KERNEL_FEW_ROWS if few else binding.KERNEL_TILED)
+    torch.cuda.synchronize()
+    assert binding.last_device_status()[0] == 0
+    for h in range(0, heads, 32):
+        qd, kd, vd = (x[:, h:h + 32].double() for x in (q, k, v))
+        ref = (torch.softmax(qd @ kd.transpose(2, 3) / 128 ** 0.5, dim=-1) @ vd).cpu().numpy()
+        assert_close(to_host_f64(out[:, h:h + 32]).reshape(ref.shape), ref, f"{heads} {Lq} {Lk} {h}")
+
+
 @pytest.mark.parametrize("d", [64, 128])
 @pytest.mark.parametrize("B,H,L", [(1, 150, 129), (2, 80, 200), (1, 300, 256), (1, 200, 257), (4, 40, 384), (1, 160, 385),
                                    (1, 152, 640), (2, 20, 1111), (3, 50, 900), (1, 64, 2048), (1, 33, 1793)])
