@@ -437,8 +437,8 @@ int launch_causal_tiles(const void* q, const void* k, const void* v, void* o, in
   p.L = L;
   p.q_tiles = (L + 2 * attn::kSub - 1) / (2 * attn::kSub);
   p.heads = BH;
-  // Heads dealt out together: equal groups whose K and V take at most a third of the cache (32 heads of 8192, d = 128: 220 MB
-  // read from DRAM in groups of ten, 828 MB with 148 ranges that each walk a head of their own).  Equal, because a short
+  // Heads dealt out together: equal groups whose K and V take at most a third of the cache (32 heads of 8192, d = 128: 202 MB
+  // read from DRAM in groups of eight, 830 MB with 148 ranges that each walk a head of their own).  Equal, because a short
   // last group would start its longest tiles when most CTAs have run dry.
   const long long at_most = std::max(1LL, st->desc.cache_bytes / (3 * 4LL * L * D));
   const long long groups = (BH + at_most - 1) / at_most;
@@ -1047,8 +1047,8 @@ int make_tmap_mat(CUtensorMap* m, const void* base, int batch, int rows, int col
 
 // Products that gemm_small_kernel takes over from the plan's kernels: at most one 128 x 128 tile per SM, where the plan's tile
 // is larger.  There it is faster at every size measured (1.2 to 1.6 times where the plan has lone CTAs, 1.0 to 1.3 times where
-// it has pairs; K = 64 to 8192).  A plan of 128 x 128 tiles keeps its kernel: launched as clusters of one, this one took 14.6 us
-// against 13.5 at 16384 x 128 x 2048 and 37.5 against 34.5 at 128 x 128 x 8192.  K is never shared out between CTAs: an element's
+// it has pairs; K = 64 to 8192).  A plan of 128 x 128 tiles keeps its kernel: there neither is faster at every size (us, plan /
+// this, operands in the cache: 16384 x 128 x 2048 13.7 / 14.6, 128 x 128 x 8192 34.3 / 36.6, 16384 x 128 x 16384 98 / 88).  K is never shared out between CTAs: an element's
 // sum would depend on how many tiles stand beside it.
 bool gemm_small(int batch, int M, int N, const gemm_tiles& t, int sms) {
   const long long tiles = (long long)batch * ((M + 127) / 128) * ((N + 127) / 128);
@@ -1202,15 +1202,15 @@ int softmax_launch(const void* s, void* pout, long long rows, int cols, float sc
     ctas = std::min((rows + 4 * rows_per_warp - 1) / (4 * rows_per_warp), 16LL * sms);
     kern<<<(unsigned)ctas, 128, 0, stream>>>(sp, pp, rows, cols, scale_log2);
   };
-  // Longer rows: a CTA per row, as few warps as hold it at VPT vectors a thread (5000 columns on 160 threads: 18.6 us for
-  // 5000 rows, on 256 threads 24.8).
+  // Longer rows: a CTA per row, as few warps as hold it at VPT vectors a thread (5000 columns on 160 threads: 16.9 us for
+  // 5000 rows; a kernel with 256 threads for every row of 4104 to 8192 columns took 24.6).
   auto launch_row = [&](auto kern, int threads) { kern<<<(unsigned)rows, threads, 0, stream>>>(sp, pp, cols, scale_log2); };
 #define SOFTMAX_ROW_CASE(VPT_, THREADS_) else if (nvec <= VPT_ * THREADS_) launch_row(gemm::softmax_rows_kernel<VPT_, THREADS_>, THREADS_)
-  if (nvec <= 16) launch_warp(gemm::softmax_rows_warp_kernel<1, 16, 1>, 2);
-  else if (nvec <= 32) launch_warp(gemm::softmax_rows_warp_kernel<1, 32, 1>, 1);
-  else if (nvec <= 64) launch_warp(gemm::softmax_rows_warp_kernel<2, 32, 1>, 1);
-  else if (nvec <= 96) launch_warp(gemm::softmax_rows_warp_kernel<3, 32, 1>, 1);
-  else if (nvec <= 128) launch_warp(gemm::softmax_rows_warp_kernel<4, 32, 1>, 1);
+  if (nvec <= 16) launch_warp(gemm::softmax_rows_warp_kernel<1, 16>, 2);
+  else if (nvec <= 32) launch_warp(gemm::softmax_rows_warp_kernel<1, 32>, 1);
+  else if (nvec <= 64) launch_warp(gemm::softmax_rows_warp_kernel<2, 32>, 1);
+  else if (nvec <= 96) launch_warp(gemm::softmax_rows_warp_kernel<3, 32>, 1);
+  else if (nvec <= 128) launch_warp(gemm::softmax_rows_warp_kernel<4, 32>, 1);
   SOFTMAX_ROW_CASE(2, 96);
   SOFTMAX_ROW_CASE(2, 128);
   SOFTMAX_ROW_CASE(4, 96);

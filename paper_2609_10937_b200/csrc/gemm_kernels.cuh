@@ -675,76 +675,64 @@ __device__ __forceinline__ uint32_t scaled_pair(uint64_t x, uint64_t f2) {
 }
 
 // Short rows (up to 128 vectors of 8 columns).  A row belongs to LANES lanes of one warp, lane l holding vectors
-// l, l + LANES, ... (VPT of them), so a row needs no barrier; a warp works on R * 32 / LANES rows at a time and loads
-// its next rows before it works on these.  Bound by HBM.  One CTA of 128 threads per row spent its time on starting CTAs
-// and on the barrier (nearly half its threads without a vector at 520 columns): 32768 x 520 took 34.3 us, here 13.8
-// (4.9 TB/s); 131072 x 128 119 us, here 14.4; 65536 x 1024 71 us, here 43.0 (6.2 TB/s).
-template <int VPT, int LANES, int R>
+// l, l + LANES, ... (VPT of them), so a row needs no barrier; a warp works on 32 / LANES rows at a time and loads its next
+// rows before it works on these.  Bound by HBM.  One CTA of 128 threads per row spent its time on starting CTAs
+// and on the barrier (nearly half its threads without a vector at 520 columns): 32768 x 520 took 34.8 us, here 13.5
+// (5.0 TB/s); 131072 x 128 119 us, here 14.6; 65536 x 1024 72 us, here 44.4 (6.0 TB/s).
+template <int VPT, int LANES>
 __global__ void __launch_bounds__(128)
 softmax_rows_warp_kernel(const __nv_bfloat16* s, __nv_bfloat16* pout, long long rows, int cols, float scale_log2) {
-  constexpr int kRowsPerGroup = 32 / LANES;
-  constexpr int kRowsPerWarp = R * kRowsPerGroup;
+  constexpr int kRowsPerWarp = 32 / LANES;
   const int l = threadIdx.x % LANES;
   const int nvec = cols / 8;
   const long long stride = (long long)gridDim.x * 4 * kRowsPerWarp;
-  // row r of this lane's group: first + r * kRowsPerGroup
-  long long first = ((long long)blockIdx.x * 4 + (threadIdx.x >> 5)) * kRowsPerWarp + (threadIdx.x & 31) / LANES;
-  auto load = [&](uint4 (&w)[R][VPT], long long row0) {
+  long long row = ((long long)blockIdx.x * 4 + (threadIdx.x >> 5)) * kRowsPerWarp + (threadIdx.x & 31) / LANES;
+  auto load = [&](uint4 (&w)[VPT], long long row) {
+    const uint4* src = reinterpret_cast<const uint4*>(s + row * cols);
 #pragma unroll
-    for (int r = 0; r < R; ++r) {
-      const long long row = row0 + r * kRowsPerGroup;
-      const uint4* src = reinterpret_cast<const uint4*>(s + row * cols);
-#pragma unroll
-      for (int v = 0; v < VPT; ++v) {
-        const int idx = v * LANES + l;
-        w[r][v] = make_uint4(kNegInfPair, kNegInfPair, kNegInfPair, kNegInfPair);
-        if (row < rows && idx < nvec) w[r][v] = src[idx];
-      }
+    for (int v = 0; v < VPT; ++v) {
+      const int idx = v * LANES + l;
+      w[v] = make_uint4(kNegInfPair, kNegInfPair, kNegInfPair, kNegInfPair);
+      if (row < rows && idx < nvec) w[v] = src[idx];
     }
   };
   const uint64_t scale2 = pack_f32x2(scale_log2, scale_log2);
-  uint4 w[R][VPT];
-  load(w, first);
+  uint4 w[VPT];
+  load(w, row);
   // (the bound is the same for a warp's lanes: its first row)
-  for (long long lead = first - (threadIdx.x & 31) / LANES; lead < rows; lead += stride, first += stride) {
-    uint4 next[R][VPT];
-    load(next, first + stride);
+  for (long long lead = row - (threadIdx.x & 31) / LANES; lead < rows; lead += stride, row += stride) {
+    uint4 next[VPT];
+    load(next, row + stride);
+    uint32_t mx2 = kNegInfPair;
 #pragma unroll
-    for (int r = 0; r < R; ++r) {
-      uint32_t mx2 = kNegInfPair;
+    for (int v = 0; v < VPT; ++v) mx2 = max_of(w[v], mx2);
+    const float m = group_max<LANES>(mx2) * scale_log2;      // scale > 0 keeps the order
+    const float neg_m = (m == -INFINITY) ? 0.f : -m;
+    const uint64_t negm2 = pack_f32x2(neg_m, neg_m);
+    uint64_t x[VPT][4];
+    uint64_t d2 = 0ull;
 #pragma unroll
-      for (int v = 0; v < VPT; ++v) mx2 = max_of(w[r][v], mx2);
-      const float m = group_max<LANES>(mx2) * scale_log2;    // scale > 0 keeps the order
-      const float neg_m = (m == -INFINITY) ? 0.f : -m;
-      const uint64_t negm2 = pack_f32x2(neg_m, neg_m);
-      uint64_t x[VPT][4];
-      uint64_t d2 = 0ull;
+    for (int v = 0; v < VPT; ++v) {
+      x[v][0] = exp_pair(w[v].x, scale2, negm2);
+      x[v][1] = exp_pair(w[v].y, scale2, negm2);
+      x[v][2] = exp_pair(w[v].z, scale2, negm2);
+      x[v][3] = exp_pair(w[v].w, scale2, negm2);
+      d2 = add_f32x2(d2, add_f32x2(add_f32x2(x[v][0], x[v][1]), add_f32x2(x[v][2], x[v][3])));
+    }
+    float d0, d1;
+    unpack_f32x2(d2, d0, d1);
+    const float d = group_sum<LANES>(d0 + d1);
+    const float f = (m == -INFINITY && d == 0.f) ? 0.f : 1.0f / d;       // a row without an element: weights 0, not NaN
+    const uint64_t f2 = pack_f32x2(f, f);
+    uint4* dst = reinterpret_cast<uint4*>(pout + row * cols);
 #pragma unroll
-      for (int v = 0; v < VPT; ++v) {
-        x[v][0] = exp_pair(w[r][v].x, scale2, negm2);
-        x[v][1] = exp_pair(w[r][v].y, scale2, negm2);
-        x[v][2] = exp_pair(w[r][v].z, scale2, negm2);
-        x[v][3] = exp_pair(w[r][v].w, scale2, negm2);
-        d2 = add_f32x2(d2, add_f32x2(add_f32x2(x[v][0], x[v][1]), add_f32x2(x[v][2], x[v][3])));
-      }
-      float d0, d1;
-      unpack_f32x2(d2, d0, d1);
-      const float d = group_sum<LANES>(d0 + d1);
-      const float f = (m == -INFINITY && d == 0.f) ? 0.f : 1.0f / d;     // a row without an element: weights 0, not NaN
-      const uint64_t f2 = pack_f32x2(f, f);
-      const long long row = first + r * kRowsPerGroup;
-      uint4* dst = reinterpret_cast<uint4*>(pout + row * cols);
-#pragma unroll
-      for (int v = 0; v < VPT; ++v) {
-        const int idx = v * LANES + l;
-        if (row < rows && idx < nvec)
-          dst[idx] = make_uint4(scaled_pair(x[v][0], f2), scaled_pair(x[v][1], f2), scaled_pair(x[v][2], f2), scaled_pair(x[v][3], f2));
-      }
+    for (int v = 0; v < VPT; ++v) {
+      const int idx = v * LANES + l;
+      if (row < rows && idx < nvec)
+        dst[idx] = make_uint4(scaled_pair(x[v][0], f2), scaled_pair(x[v][1], f2), scaled_pair(x[v][2], f2), scaled_pair(x[v][3], f2));
     }
 #pragma unroll
-    for (int r = 0; r < R; ++r)
-#pragma unroll
-      for (int v = 0; v < VPT; ++v) w[r][v] = next[r][v];
+    for (int v = 0; v < VPT; ++v) w[v] = next[v];
   }
 }
 
@@ -752,9 +740,10 @@ softmax_rows_warp_kernel(const __nv_bfloat16* s, __nv_bfloat16* pout, long long 
 // warps that hold the row.  The exponentials (one per element) are taken relative to the maximum of the warp or, from four
 // vectors a thread, of the thread (waiting for the warp's costs 5-14 % there, at two vectors it saves 8-13 %) and rescaled
 // once the warps' (m, d) have met in shared memory, behind the row's only barrier.
-// (The register bounds keep 1280 threads per SM at four vectors and 768 at eight: rows in flight are what the kernel lives
-// on -- with 59 registers instead of 48, four vectors a thread are 7 % slower.  8192 x 8192: 41.8 us = 6.4 TB/s, 43.7 with
-// the pairwise (m, d) merge in every shuffle step that stood here before; 4096 x 16384: 42.0 us against 48.4.)
+// (The register bounds keep 1120 to 1280 threads per SM at four vectors -- 48 registers, 56 at 192 and 224 threads -- and 640 to
+// 768 at eight: rows in flight are what the kernel lives on -- with 59 registers instead of 48, 128 threads of four vectors
+// are 7 % slower.  <4, 256> and eight vectors on 192 threads or more spill 12 to 24 bytes for it.  8192 x 8192: 42.8 us = 6.3 TB/s, 44.2 with
+// the pairwise (m, d) merge in every shuffle step that stood here before; 4096 x 16384: 43.4 us against 48.8.)
 template <int VPT, int THREADS>
 __global__ void __launch_bounds__(THREADS, VPT < 4 ? 1 : (VPT == 4 ? 1280 : 768) / THREADS)
 softmax_rows_kernel(const __nv_bfloat16* s, __nv_bfloat16* pout, int cols, float scale_log2) {

@@ -449,7 +449,7 @@ attn_causal_tiles_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
       scores(0, ready(0, 0, 0, true, n0 == 1, n1 == 0));
       if (ok && !kSplitP && n1 > 0) scores(1, ready(1, 0, 0, true, n1 == 1, true));
     }
-    bool defer = kSplitP && n1 > 0, ahead = false;     // (d = 64) ahead: sub-tile 0's next step has been issued
+    bool defer = kSplitP && n1 > 0;                    // (d = 64) sub-tile 1's first scores are still to come
     for (int seq = 1; ok && tile >= 0; ++seq) {
       const int n = n1 > n0 ? n1 : n0;
       int next = -3;                                   // not asked yet
@@ -483,13 +483,11 @@ attn_causal_tiles_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
       for (int j = 0; ok && j < n; ++j) {
         if constexpr (kSplitP) {
           // Nothing ties the two sub-tiles to each other here, and left alone their softmax warpgroups end up in the same
-          // phase of the step (both at the exponentials, then neither).  So sub-tile 1's scores are held back until
-          // sub-tile 0 has its row maxima of that step: half a step behind.
+          // phase of the step (both at the exponentials, then neither).  So sub-tile 1's scores are issued behind the first
+          // half of sub-tile 0's P of the step: half a step behind.
           if (j < n0) {
             if (!wait(&misc->s_free[0], gp & 1, kBarPFull, 0x100)) break;
-            const Scores sc = next_scores(0, j);
-            scores(0, sc);
-            ahead = sc.go;
+            scores(0, next_scores(0, j));
             if (!ok || !wait(&misc->kv_full[vs], vph, kBarKvFull, 0x102) || !wait(&misc->p_full[0], gp & 1, kBarPFull, 0x103)) break;
             if (elect_one()) p_times_v(0, j, false);
             __syncwarp();
