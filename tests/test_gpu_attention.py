@@ -774,7 +774,7 @@ def test_persistent_grid_with_ragged_lengths(env, B, H, L, d):
 
 def test_random_shapes_every_grid_mode_agrees_with_an_unsplit_run(env):
     """Seeded random shapes, causal and not: whatever grid the plan picks (one CTA per tile, clusters of 2 to 8,
-    equal ranges, persistent), the output equals that of a launch that shares no Q tile between CTAs, up to the
+    equal ranges, persistent, causal whole tiles), the output equals that of a launch that shares no Q tile between CTAs, up to the
     merge's rounding; the modes met are counted so that a change of the plan that stops exercising one shows."""
     torch, _, binding = env
     import random
@@ -792,15 +792,16 @@ def test_random_shapes_every_grid_mode_agrees_with_an_unsplit_run(env):
         q, k, v = (torch.randn(B, H, L, d, device="cuda", generator=g).mul_(1.3).to(torch.bfloat16) for _ in range(3))
         t = binding.plan(desc, B, H, L, d, causal=causal)
         o = binding.forward(q, k, v, causal=causal)
-        cl = binding.last_cluster_size()
+        cl, kernel = binding.last_cluster_size(), binding.last_kernel()
         ref = binding.forward_tiles(q, k, v, ctas=1 if causal else t.tiles, causal=causal)
         torch.cuda.synchronize()
         assert binding.last_device_status()[0] == 0, (B, H, L, d, causal)
         assert bool(torch.isfinite(o.float()).all())
         assert float((o.float() - ref.float()).abs().max()) <= 2e-2, (B, H, L, d, causal, t.ctas, t.tiles, cl)
-        mode = ("causal " if causal else "") + ("cluster" if cl else "tiles" if t.ctas == t.tiles else "ranges")
+        mode = ("causal " if causal else "") + ("cluster" if cl else "whole tiles" if kernel == binding.KERNEL_CAUSAL_TILES else
+                                                "tiles" if t.ctas == t.tiles else "ranges")
         modes[mode] = modes.get(mode, 0) + 1
-    assert all(modes.get(m, 0) >= 3 for m in ("cluster", "tiles", "ranges", "causal cluster", "causal ranges")), modes
+    assert all(modes.get(m, 0) >= 3 for m in ("cluster", "tiles", "ranges", "causal cluster", "causal ranges", "causal whole tiles")), modes
 
 
 @pytest.mark.parametrize("B,H,Lq,Lk,d", [(1, 2, 300, 1408, 128), (2, 3, 1000, 2500, 64), (1, 1, 4096, 16384, 128),
@@ -897,8 +898,8 @@ def test_very_long_single_head(env, L, d):
     (1, 40, 2, 700), (8, 32, 1, 64), (4, 40, 1, 300), (1, 1, 1, 16384), (1, 5, 7, 9000), (2, 16, 15, 2048), (8, 40, 4, 500),
     (1, 7, 17, 1000), (1, 150, 24, 1030), (5, 33, 32, 1025), (1, 2, 32, 33)])
 def test_few_query_rows_against_many_keys(env, B, H, Lq, Lk, d):
-    """Calls with at most 32 query rows: both sides of 8, 16 and 32 rows, of one slab of keys per warp, of every split of a
-    head (1 to 16 CTAs) and more heads than CTAs fit at once; NaN-filled output, every element against the oracle."""
+    """Calls with at most 32 query rows: both sides of 8, 16 and 32 rows, of one slab of keys per warp, and more heads than
+    CTAs fit at once; NaN-filled output, every element against the oracle."""
     torch, orc, binding = env
     rng = np.random.default_rng([B, H, Lq, Lk, d, 3])
     bits = lambda *shape: synth.f32_to_bf16_bits((rng.standard_normal(shape) * 1.5).astype(np.float32))
@@ -906,6 +907,8 @@ def test_few_query_rows_against_many_keys(env, B, H, Lq, Lk, d):
     out = torch.full((B, H, Lq, d), float("nan"), dtype=torch.bfloat16, device="cuda")
     dev = [to_cuda_bf16(x).view(B, H, -1, d) for x in (q, k, v)]
     binding.forward_qk(*dev, out)
+    # 17 to 32 rows at d = 128 stay with the tiled kernel at these shapes
+    assert binding.last_kernel() == (binding.KERNEL_FEW_ROWS if Lq <= 16 or d == 64 else binding.KERNEL_TILED)
     torch.cuda.synchronize()
     assert binding.last_device_status()[0] == 0
     qd, kd, vd = (x.double() for x in dev)
@@ -935,6 +938,30 @@ def test_seventeen_to_thirty_two_rows_at_d128_on_both_sides_of_the_rule(env, hea
         assert_close(to_host_f64(out[:, h:h + 32]).reshape(ref.shape), ref, f"{heads} {Lq} {Lk} {h}")
 
 
+def test_few_row_kernel_in_every_split_of_a_head(env):
+    """The few-row kernel with a head on 1, 2, 4, 8 and 16 CTAs (one row, d = 128), and with two row groups a warp at d = 128; every
+    element against fp64, the same bits again."""
+    torch, _, binding = env
+    splits = set()
+    for heads, Lq, Lk in [(256, 1, 300), (128, 1, 4096), (64, 1, 8192), (15, 1, 16384), (8, 1, 16384), (192, 24, 2048)]:
+        gen = torch.Generator(device="cuda").manual_seed(heads + Lq + Lk)
+        q, k, v = (torch.randn(1, heads, n, 128, generator=gen, device="cuda").to(torch.bfloat16) for n in (Lq, Lk, Lk))
+        out = torch.full_like(q, float("nan"))
+        binding.forward_qk(q, k, v, out)
+        assert binding.last_kernel() == binding.KERNEL_FEW_ROWS, (heads, Lq, Lk)
+        split = binding.last_grid() // heads
+        assert binding.last_cluster_size() == (split if split > 1 else 0)
+        splits.add(split)
+        torch.cuda.synchronize()
+        assert binding.last_device_status()[0] == 0
+        for h in range(0, heads, 32):
+            qd, kd, vd = (x[:, h:h + 32].double() for x in (q, k, v))
+            ref = (torch.softmax(qd @ kd.transpose(2, 3) / 128 ** 0.5, dim=-1) @ vd).cpu().numpy()
+            assert_close(to_host_f64(out[:, h:h + 32]).reshape(ref.shape), ref, f"{heads} {Lq} {Lk} {h}")
+        assert torch.equal(binding.forward_qk(q, k, v).view(torch.int16), out.view(torch.int16))
+    assert splits == {1, 2, 4, 8, 16}, splits
+
+
 @pytest.mark.parametrize("d", [64, 128])
 @pytest.mark.parametrize("B,H,L", [(1, 150, 129), (2, 80, 200), (1, 300, 256), (1, 200, 257), (4, 40, 384), (1, 160, 385),
                                    (1, 152, 640), (2, 20, 1111), (3, 50, 900), (1, 64, 2048), (1, 33, 1793)])
@@ -950,6 +977,7 @@ def test_causal_whole_tiles_match_the_reference(env, B, H, L, d):
     binding.forward(*dev, out, causal=True)
     torch.cuda.synchronize()
     assert binding.last_device_status()[0] == 0 and binding.last_cluster_size() == 0
+    assert (binding.last_kernel(), binding.last_grid()) == (binding.KERNEL_CAUSAL_TILES, B * H * -(-L // 256))
     # Bound per element: bf16 keeps 8 significant bits, so a rounding moves a value by at most 2^-8 of it.  Rounded are the
     # weights (at most 2^-8 sum p |v| in all; the exponentials' own error, 2^-13, likewise) and the output (2^-8 |o|).
     keep = torch.ones((L, L), dtype=torch.bool, device="cuda").tril()

@@ -72,7 +72,7 @@ def test_cta_pairs_and_lone_ctas_agree_with_the_oracle_and_each_other(env, layou
     assert binding.gemm_plan(desc, batch, M, N, K).cta_pair == 2
     if M >= 1280 and N > 4000:
         assert binding.gemm_plan(desc, batch, M, N, K).tail_split > 0
-    _check_product(env, batch, M, N, K, layout, seed=4, rows_per_batch=300)                 # closed-form default: pairs
+    _check_product(env, batch, M, N, K, layout, seed=4, rows_per_batch=300)                 # pairs, or one 128 x 128 tile per CTA
     _check_product(env, batch, M, N, K, layout, seed=4, rows_per_batch=300, cta_pair=1)
     _check_product(env, batch, M, N, K, layout, seed=4, rows_per_batch=300, cta_pair=2, tile_n=128)
     _check_product(env, batch, M, N, K, layout, seed=4, rows_per_batch=300, tail_split=-1)   # whole tiles in the last wave
@@ -115,8 +115,14 @@ def test_matrix_product_full_size_sampled(env):
                                          (4, 500, 520, 264), (1, 1000, 1000, 1000), (1, 1500, 1400, 72), (1, 100, 8000, 2000)])
 def test_products_with_few_output_tiles(env, batch, M, N, K, layout):
     """Outputs of at most one 128 x 128 tile per SM: one tile and many, rows and columns past the end of the last, K with a
-    ragged last step, more and fewer steps than the ring has stages."""
+    ragged last step, more and fewer steps than the ring has stages.  Those whose plan has larger tiles run as one such tile per
+    CTA, the others with the plan's."""
+    torch, _, binding = env
     _check_product(env, batch, M, N, K, layout, seed=M + N + K)
+    small = N > 128                                  # (128 columns or fewer: the plan's tile is 128 x 128)
+    assert binding.last_kernel() == (binding.KERNEL_GEMM_SMALL if small else binding.KERNEL_GEMM)
+    if small:
+        assert binding.last_grid() == batch * -(-M // 128) * -(-N // 128)
 
 
 @pytest.mark.parametrize("layout", ["kn", "nk"])
