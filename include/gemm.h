@@ -96,7 +96,7 @@ int gemm_forward_tiles(const void *a, const void *b, void *c, int batch, int M, 
  * memory when it has more than 16384 columns.  scale must be positive and finite
  * (the row maximum is taken on the unscaled scores, which a positive scale keeps
  * in order): ATTN_ERR_INVALID_ARG otherwise.
- * Errors: ATTN_ERR_INVALID_ARG, ATTN_ERR_UNSUPPORTED_SHAPE, ATTN_ERR_MISALIGNED, ATTN_ERR_CUDA.
+ * Errors: ATTN_ERR_INVALID_ARG, ATTN_ERR_UNSUPPORTED_SHAPE, ATTN_ERR_MISALIGNED, ATTN_ERR_WRONG_ARCH, ATTN_ERR_CUDA.
  */
 int softmax_rows_forward(const void *s, void *p, long long rows, int cols, float scale, void *cuda_stream);
 
