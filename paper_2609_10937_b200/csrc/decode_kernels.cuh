@@ -69,8 +69,10 @@ __device__ __forceinline__ float ld_peer_f1(uint32_t peer_addr) {
   asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(peer_addr) : "memory");
   return v;
 }
-// Weight of a part with reference m_part under the common reference m (a part without keys: -inf, weight 0).
-__device__ __forceinline__ float part_weight(float m_part, float m) { return m_part == -INFINITY ? 0.f : exp2f(m_part - m); }
+// Weight of a part with reference score m_part under the common reference m (a part without keys: -inf, weight 0).
+__device__ __forceinline__ float part_weight(float m_part, float m, float scale_log2) {
+  return m_part == -INFINITY ? 0.f : exp2f((m_part - m) * scale_log2);
+}
 
 // HALF: at most 8 rows, so the accumulators' second eight rows hold nothing.
 template <int D, int MT, bool HALF>
@@ -194,15 +196,18 @@ attn_decode_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_consta
         for (int j = 1; j < 2 * KP; ++j) mx = max3(mx, s[mt][j][2 * h], s[mt][j][2 * h + 1]);
         mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
         mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
-        const float m_new = fmaxf(m_run[mt][h], mx * p.scale_log2);
+        // References are scores, not scaled ones, and are subtracted before the scale: the largest score's weight is 1 at any
+        // magnitude.  fma(s, scale, -max * scale) leaves the product's rounding, which from scores of 2^24 on is no small number
+        // (a single score of 1e20 gave a row of NaN).
+        const float m_new = fmaxf(m_run[mt][h], mx);
         const float ref = m_new == -INFINITY ? 0.f : m_new;     // no admissible score yet: weights 0, not NaN
-        alpha[h] = ex2_approx(m_run[mt][h] - ref);
+        alpha[h] = ex2_approx((m_run[mt][h] - ref) * p.scale_log2);
         m_run[mt][h] = m_new;
         float sum = 0.f;
 #pragma unroll
         for (int j = 0; j < 2 * KP; ++j) {
-          const float e0 = ex2_approx(fmaf(s[mt][j][2 * h], p.scale_log2, -ref));
-          const float e1 = ex2_approx(fmaf(s[mt][j][2 * h + 1], p.scale_log2, -ref));
+          const float e0 = ex2_approx((s[mt][j][2 * h] - ref) * p.scale_log2);
+          const float e1 = ex2_approx((s[mt][j][2 * h + 1] - ref) * p.scale_log2);
           sum += e0 + e1;
           pa[mt][j / 2][(j & 1) * 2 + h] = pack_bf16x2(e0, e1);
         }
@@ -272,7 +277,7 @@ attn_decode_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_consta
     float l = 0.f;
 #pragma unroll
     for (int w = 0; w < kDecodeWarps; ++w) {
-      const float f = part_weight(misc->warp_m[w][row], m);
+      const float f = part_weight(misc->warp_m[w][row], m, p.scale_log2);
       const float4 v = reinterpret_cast<const float4*>(part + (size_t)w * 16 * MT * D)[u];
       l += f * misc->warp_l[w][row];
       o4.x += f * v.x; o4.y += f * v.y; o4.z += f * v.z; o4.w += f * v.w;
@@ -299,7 +304,7 @@ attn_decode_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_consta
 #pragma unroll
     for (int q = 0; q < kDecodeMaxSplit; ++q) {                 // ascending key order
       if (q >= k) break;
-      const float f = part_weight(m_q[q], m);
+      const float f = part_weight(m_q[q], m, p.scale_log2);
       const float4 v = ld_peer_f4(map_to_cta(o_addr + u * 16, q));
       l += f * ld_peer_f1(map_to_cta(l_addr + row * 4, q));
       o4.x += f * v.x; o4.y += f * v.y; o4.z += f * v.z; o4.w += f * v.w;

@@ -938,6 +938,33 @@ def test_seventeen_to_thirty_two_rows_at_d128_on_both_sides_of_the_rule(env, hea
         assert_close(to_host_f64(out[:, h:h + 32]).reshape(ref.shape), ref, f"{heads} {Lq} {Lk} {h}")
 
 
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("big", [3e4, 1e20, -1e20])
+@pytest.mark.parametrize("heads,Lq,Lk", [(2, 1, 300), (2, 16, 4096), (3, 9, 70), (160, 7, 500), (192, 24, 2048)])
+def test_few_row_kernel_with_scores_of_any_magnitude(env, heads, Lq, Lk, d, big):
+    """One key, a stretch of keys or all of them with a huge component: scores up to 1e20 in size take the weights that they have,
+    the largest one 1, whichever warp or CTA holds them; every element against fp64."""
+    torch, _, binding = env
+    for where in (slice(Lk // 2, Lk // 2 + 1), slice(Lk - 1, Lk), slice(0, Lk // 2), slice(0, Lk)):
+        gen = torch.Generator(device="cuda").manual_seed(heads + Lq + Lk)
+        q, k, v = (torch.randn(1, heads, n, d, generator=gen, device="cuda").to(torch.bfloat16) for n in (Lq, Lk, Lk))
+        k[:, :, where, 3] = big
+        if where == slice(0, Lk):
+            k[:, :, Lk // 3, 3] *= 1.25                      # equal huge components leave the small ones below fp32's last bit
+        out = binding.forward_qk(q, k, v, torch.full_like(q, float("nan")))
+        assert binding.last_kernel() == binding.KERNEL_FEW_ROWS
+        s = q.double() @ k.double().transpose(2, 3) / d ** 0.5
+        ref = torch.softmax(s, dim=-1) @ v.double()
+        # rows whose weights hang on differences below fp32's resolution of such scores have no value to compare with
+        top = s.topk(2, dim=-1).values
+        sure = ((top[..., 0] - top[..., 1]) > 2.0 ** -20 * top.abs().amax(-1)) | (s.abs().amax(-1) < 100)
+        assert bool(torch.isfinite(out).all()), where
+        err = ((out.double() - ref).abs().amax(-1) * sure).max()
+        assert float(err) <= 2e-2, (where, float(err))
+        torch.cuda.synchronize()
+        assert binding.last_device_status()[0] == 0
+
+
 def test_few_row_kernel_in_every_split_of_a_head(env):
     """The few-row kernel with a head on 1, 2, 4, 8 and 16 CTAs (one row, d = 128), and with two row groups a warp at d = 128; every
     element against fp64, the same bits again."""
