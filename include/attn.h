@@ -408,7 +408,8 @@ enum attn_kernel {
   ATTN_KERNEL_GEMM = 5,          /* matrix product, lone CTAs                                    */
   ATTN_KERNEL_GEMM_PAIR = 6,     /* matrix product, CTA pairs                                    */
   ATTN_KERNEL_GEMM_SMALL = 7,    /* matrix product, one 128 x 128 tile per CTA                   */
-  ATTN_KERNEL_SOFTMAX = 8        /* row softmax                                                  */
+  ATTN_KERNEL_SOFTMAX = 8,       /* row softmax                                                  */
+  ATTN_KERNEL_NARROW_TILES = 9   /* d = 64, not causal, one CTA per Q tile                       */
 };
 int attn_last_kernel(void);
 int attn_last_grid(void);

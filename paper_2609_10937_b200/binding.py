@@ -19,7 +19,7 @@ ERR_INVALID_ARG, ERR_UNSUPPORTED_SHAPE, ERR_MISALIGNED, ERR_ALIASING = -1, -2, -
 ERR_INFEASIBLE_PLAN, ERR_WRONG_ARCH, ERR_NEED_WORKSPACE, ERR_CUDA = -5, -6, -7, -8
 ERR_DEVICE_TIMEOUT, ERR_BAD_TILES, ERR_SCRATCH_LIMIT = -9, -10, -11
 (KERNEL_NONE, KERNEL_TILED, KERNEL_CAUSAL_TILES, KERNEL_FEW_ROWS, KERNEL_SIMPLE, KERNEL_GEMM, KERNEL_GEMM_PAIR, KERNEL_GEMM_SMALL,
- KERNEL_SOFTMAX) = range(9)
+ KERNEL_SOFTMAX, KERNEL_NARROW_TILES) = range(10)
 BIND_NAMES = ("none", "smem", "tmem", "reg", "atom", "shape")
 
 EXPORTED_SYMBOLS = (

@@ -19,6 +19,7 @@
 #include "gemm.h"
 #include "gemm_kernels.cuh"
 #include "tiles_kernel.cuh"
+#include "narrow_kernel.cuh"
 
 namespace {
 
@@ -422,11 +423,11 @@ int dispatch_decode(const void* q, const void* k, const void* v, void* o, int BH
   return ATTN_ERR_UNSUPPORTED_SHAPE;
 }
 
-// Causal attention as whole Q tiles, one CTA each (tiles_kernel.cuh).
-template <int D>
+// Causal attention at d = 128 as whole Q tiles, one CTA each (tiles_kernel.cuh).
 int launch_causal_tiles(const void* q, const void* k, const void* v, void* o, int BH, int L, unsigned int* status, DeviceState* st,
                         cudaStream_t stream) {
-  using SM = attn::TilesSmem<D>;
+  using SM = attn::TilesSmem;
+  constexpr int D = 128;
   CUtensorMap tq, tk, tv, to;
   int rc;
   if ((rc = make_tmap(&tq, q, BH, L, D, attn::kSub)) != ATTN_OK) return rc;
@@ -447,7 +448,7 @@ int launch_causal_tiles(const void* q, const void* k, const void* v, void* o, in
   p.scale_log2 = (float)(1.4426950408889634 / std::sqrt((double)D));
   p.status = status;
   const int smem = SM::total(p.stages);
-  auto kern = attn::attn_causal_tiles_kernel<D>;
+  auto kern = attn::attn_causal_tiles_kernel;
   ATTN_ALLOW_SMEM(kern, smem);
   kern<<<(unsigned)(BH * p.q_tiles), 512, smem, stream>>>(tq, tk, tv, to, p);
   ATTN_CUDA_TRY(cudaGetLastError());
@@ -457,18 +458,63 @@ int launch_causal_tiles(const void* q, const void* k, const void* v, void* o, in
   return ATTN_OK;
 }
 
+// d = 64 as whole Q tiles, one CTA each (narrow_kernel.cuh).
+template <bool CAUSAL>
+int launch_narrow(const void* q, const void* k, const void* v, void* o, int BH, int Lq, int Lk, unsigned int* status, DeviceState* st,
+                  cudaStream_t stream) {
+  using SM = attn::NarrowSmem;
+  CUtensorMap tq, tk, tv, to;
+  int rc;
+  if ((rc = make_tmap(&tq, q, BH, Lq, 64, attn::kSub)) != ATTN_OK) return rc;
+  if ((rc = make_tmap(&tk, k, BH, Lk, 64, 128)) != ATTN_OK) return rc;
+  if ((rc = make_tmap(&tv, v, BH, Lk, 64, 128)) != ATTN_OK) return rc;
+  if ((rc = make_tmap(&to, o, BH, Lq, 64, 32)) != ATTN_OK) return rc;    // every warp stores its own 32 rows
+  attn::NarrowParams p;
+  p.Lq = Lq;
+  p.Lk = Lk;
+  p.q_tiles = (Lq + 2 * attn::kSub - 1) / (2 * attn::kSub);
+  p.n_steps = (Lk + 127) / 128;
+  p.heads = BH;
+  // (causal: groups of heads as in launch_causal_tiles)
+  const long long at_most = std::max(1LL, st->desc.cache_bytes / (3 * 4LL * Lk * 64));
+  const long long groups = (BH + at_most - 1) / at_most;
+  p.group_heads = (int)((BH + groups - 1) / groups);
+  p.stages = std::min(attn::kMaxStages, (st->desc.local_mem_bytes - SM::total(0)) / SM::kStageBytes);
+  p.scale_log2 = (float)(1.4426950408889634 / std::sqrt(64.0));
+  p.status = status;
+  const int smem = SM::total(p.stages);
+  auto kern = attn::attn_narrow_kernel<CAUSAL>;
+  ATTN_ALLOW_SMEM(kern, smem);
+  kern<<<(unsigned)(BH * p.q_tiles), attn::kNarrowThreads, smem, stream>>>(tq, tk, tv, to, p);
+  ATTN_CUDA_TRY(cudaGetLastError());
+  t_cluster_size = 0;
+  t_launch_count = 1;
+  launched(CAUSAL ? ATTN_KERNEL_CAUSAL_TILES : ATTN_KERNEL_NARROW_TILES, (long long)BH * p.q_tiles);
+  return ATTN_OK;
+}
+
 // Whether a causal plan of equal ranges runs as whole tiles instead.  Longest first, whole tiles take the longest tile's steps
 // or an even share of all steps, one more per tile, whichever is more; 5 for the start and the end.  Measured (us, ranges /
 // whole tiles): 128 heads x 4096, d = 128 625 / 501; 32 x 1111, d = 64 36 / 20; 16 x 4096, d = 128 88 / 66; where the longest
 // tile decides, ranges stay: 8 x 4096 55 / (33 steps of 2) 66.  (Four ring stages: the MMA warp looks that far ahead.)
 bool causal_whole_tiles(const attn_tiles& t, int BH, int L, int d, int local_mem, int sms) {
   if (!t.causal || t.n_q != 2 || t.tile_kv != 128) return false;
-  if (local_mem < (d == 64 ? attn::TilesSmem<64>::total(4) : attn::TilesSmem<128>::total(4))) return false;
+  if (local_mem < (d == 64 ? attn::NarrowSmem::total(4) : attn::TilesSmem::total(4))) return false;
   if (t.ctas % t.tiles == 0 && t.ctas > t.tiles) return false;      // clusters that share out each tile's own steps
   const int steps = (L + 127) / 128;
   const long long units = BH * attn_internal::head_units((L + 255) / 256, steps, 2, 1);
   const long long even = (units + t.tiles + sms - 1) / sms;
   return std::max<long long>(steps, even) + 5 <= t.cost_steps;
+}
+
+// Whether a non-causal plan at d = 64 runs as whole tiles of narrow_kernel.cuh: at three waves of tiles or more whose last one
+// leaves at most a tenth of all slots empty.  Measured (us in a loop, attn_fwd_kernel / narrow): 128 heads x 8192 2890 / 2797,
+// 128 x 4096 747 / 727, 256 x 1000 120 / 115; on the other side 128 x 1024 (3.46 waves) 61.7 / 62.6, 18 x 4096 (1.95) 107 / 109,
+// 10 x 8192 (2.16) 222 / 290, 32 x 2048 (0.86) 57 / 62.
+bool narrow_tiles(const attn_tiles& t, int d, int local_mem, int sms) {
+  if (d != 64 || t.causal || t.n_q != 2 || t.tile_kv != 128 || local_mem < attn::NarrowSmem::total(4)) return false;
+  const long long slots = (long long)((t.tiles + sms - 1) / sms) * sms;
+  return t.tiles >= 3 * sms && 10 * slots <= 11LL * t.tiles;
 }
 
 int dispatch_fwd(const void* q, const void* k, const void* v, void* o, int B, int H, int L, int d,
@@ -477,8 +523,10 @@ int dispatch_fwd(const void* q, const void* k, const void* v, void* o, int B, in
   if (Lk == 0) Lk = L;
   // own_plan: the device's own, with no field changed and from no caller's descriptor -- those say how many CTAs run
   if (own_plan && Lk == L && causal_whole_tiles(t, B * H, L, d, st->desc.local_mem_bytes, st->desc.num_units))
-    return d == 128 ? launch_causal_tiles<128>(q, k, v, o, B * H, L, status, st, s)
-                    : launch_causal_tiles<64>(q, k, v, o, B * H, L, status, st, s);
+    return d == 128 ? launch_causal_tiles(q, k, v, o, B * H, L, status, st, s)
+                    : launch_narrow<true>(q, k, v, o, B * H, L, L, status, st, s);
+  if (own_plan && narrow_tiles(t, d, st->desc.local_mem_bytes, st->desc.num_units))
+    return launch_narrow<false>(q, k, v, o, B * H, L, Lk, status, st, s);
 #define ATTN_CASE(D_, TKV_, NQ_) \
   if (d == D_ && t.tile_kv == TKV_ && t.n_q == NQ_) \
     return launch_fwd<D_, TKV_, NQ_>(q, k, v, o, B, H, L, Lk, t, ws, status, st, s, may_overlap);

@@ -1,0 +1,473 @@
+// attn_narrow_kernel: fused attention for d = 64 in which every Q tile is worked on by one CTA from its first key to its last
+// (nothing to merge between CTAs), causal or not.
+//
+// At d = 64 the step is bound by the softmax warps' instructions: 256 x 128 exponentials, maxima, conversions and sums take a
+// scheduler partition about 1930 cycles however they are written (2040 beside the matrix products), the products 1300.
+// attn_fwd_kernel gives a partition two softmax warps of 128 scores a row and takes 2800 cycles a step.  Here it has four, of
+// 64 scores a row: a tile of 256 query rows is worked on as four streams, two sub-tiles of 128 rows times the two halves of
+// every 128-key tile.  A stream has its own scores, reference, denominator and accumulator in tensor memory (4 x (64 + 64)
+// columns: all 512; P overwrites the front of its scores) and its own softmax warpgroup; the two streams of a sub-tile meet
+// when the tile is finished, in the epilogue warpgroup, which reads both accumulators.  2600 cycles a step.  In a loop (us,
+// before / this kernel): causal 128 heads x 8192 1667 / 1474, 128 x 4096 491 / 388, 128 x 2048 144 / 115, 256 x 300 31.2 / 24.6,
+// 32 x 1111 22.5 / 20.8; not causal 128 x 8192 2890 / 2797, where the power limit takes back most of it.
+//   * One barrier each way per step: scores ready (commit of Q K^T, which also says that the stream's P V of the step before
+//     is complete) and P ready.  A softmax warp whose reference moved rescales its accumulator itself: that is rare, and
+//     no other warp has to be asked.
+//   * Every stream has an MMA warp of its own, which issues P V of a step and then Q K^T of the stream's next step: what is in
+//     flight for one stream runs under the exponentials of the other three.  One MMA warp that served the streams in turn took
+//     800 cycles a turn, waits and instruction issue together, and bound the step at 3200 cycles.
+//   * Tiles come from the hardware's queue of CTAs not yet started, and the epilogue of a tile runs under the next one, as in
+//     attn_causal_tiles_kernel.
+#pragma once
+
+#include "tiles_kernel.cuh"
+
+namespace attn {
+
+struct NarrowParams {
+  int Lq, Lk;              // query rows and keys per head
+  int q_tiles;             // Q tiles per head = ceil(Lq / 256)
+  int n_steps;             // key steps per head = ceil(Lk / 128)
+  int heads;               // B * H
+  int group_heads;         // causal: heads whose tiles are dealt out together, longest first
+  int stages;              // ring depth
+  float scale_log2;        // log2(e) / sqrt(d)
+  unsigned int* status;    // as in FwdParams
+};
+
+struct NarrowSmem {
+  static constexpr int kSubBytes = kSub * 128;                   // one sub-tile of Q
+  static constexpr int kQBytes = 2 * 2 * kSubBytes;              // two tiles
+  static constexpr int kStageBytes = 128 * 128;
+  static constexpr int kOutBytes = 8 * 4096;                     // two [32 rows][64 columns] bf16 chunks per epilogue warp
+  static constexpr int kMiscBytes = 9216;
+  __host__ __device__ static constexpr int total(int stages) { return kQBytes + stages * kStageBytes + kOutBytes + kMiscBytes; }
+};
+// 16 softmax warps, 4 epilogue, 4 MMA, TMA, tensor-memory allocation, 2 idle.  Registers: 896 x 72 at launch, then 512 x 96 and
+// 384 x 40.
+constexpr int kNarrowThreads = 896;
+constexpr int kNarrowSchedReaders = 25;    // warps that read a tile's index: all but the last three
+
+struct NarrowMisc {
+  float2 stat[2][4][kSub];                 // [the sub-tile's tiles mod 2][stream][row] reference and denominator of a finished tile
+  uint4 sched[2];                          // answers of try_cancel (16 bytes each)
+  uint64_t sched_full[2], sched_empty[2];
+  uint64_t q_full[2][2], q_empty[2][2];    // [sub-tile][buffer]
+  uint64_t kv_full[kMaxStages], kv_empty[kMaxStages];
+  uint64_t s_full[4], p_full[4];           // per stream
+  uint64_t fin_full[4];                    // per stream
+  uint64_t o_full[2], o_free[2];           // per sub-tile
+  AbortCell abort;
+  uint32_t tmem_slot;
+};
+static_assert(sizeof(NarrowMisc) <= NarrowSmem::kMiscBytes, "misc region too large");
+
+template <bool CAUSAL>
+__device__ __forceinline__ TileWork narrow_work(int index, const NarrowParams& p) {
+  TileWork w;
+  if constexpr (CAUSAL) {
+    const int per_group = p.group_heads * p.q_tiles;
+    const int group = index / per_group, r = index - group * per_group;
+    const int first = group * p.group_heads;
+    const int n = p.heads - first < p.group_heads ? p.heads - first : p.group_heads;
+    const int q = p.q_tiles - 1 - r / n;
+    w.bh = first + r % n;
+    w.q_row0 = q * 2 * kSub;
+    w.n0 = 2 * q + 1;                      // a sub-tile's last key step is the one that holds its own rows
+    w.n1 = w.q_row0 + kSub >= p.Lq ? 0 : 2 * q + 2;
+  } else {
+    w.bh = index / p.q_tiles;
+    w.q_row0 = (index - w.bh * p.q_tiles) * 2 * kSub;
+    w.n0 = p.n_steps;
+    w.n1 = w.q_row0 + kSub >= p.Lq ? 0 : p.n_steps;
+  }
+  return w;
+}
+
+template <bool CAUSAL>
+__global__ void __launch_bounds__(kNarrowThreads, 1)
+attn_narrow_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
+                   const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_o, const NarrowParams p) {
+  constexpr int D = 64, TKV = 128, HKV = TKV / 2;     // a stream takes one half of every key tile
+  constexpr int O_COL0 = 4 * HKV;
+  constexpr int kPoly = kPolyPairsPer8;
+  using SM = NarrowSmem;
+
+  extern __shared__ __align__(1024) uint8_t smem_raw[];
+  const uint32_t smem_base = smem_u32(smem_raw);
+  const uint32_t ring_smem = smem_base + SM::kQBytes;
+  const uint32_t out_smem = ring_smem + p.stages * SM::kStageBytes;
+  NarrowMisc* const misc = reinterpret_cast<NarrowMisc*>(smem_raw + SM::kQBytes + p.stages * SM::kStageBytes + SM::kOutBytes);
+  volatile int* abort_flag = &misc->abort.flag;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+
+  if (threadIdx.x == 0) {
+    abort_cell_init(&misc->abort, p.status);
+    if (smem_base & 1023u) note_timeout(wait_info(kRoleLoad, 0, 0xFFFF), &misc->abort.flag);   // swizzled tiles need 1024-byte alignment
+    for (int s = 0; s < kMaxStages; ++s) {
+      mbar_init(smem_u32(&misc->kv_full[s]), 1);
+      mbar_init(smem_u32(&misc->kv_empty[s]), 4);                 // the four streams
+    }
+    for (int i = 0; i < 4; ++i) {
+      mbar_init(smem_u32(&misc->s_full[i]), 1);
+      mbar_init(smem_u32(&misc->p_full[i]), kSub);
+      mbar_init(smem_u32(&misc->fin_full[i]), kSub);
+    }
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(smem_u32(&misc->sched_full[i]), 1);
+      mbar_init(smem_u32(&misc->sched_empty[i]), kNarrowSchedReaders);
+      for (int b = 0; b < 2; ++b) {
+        mbar_init(smem_u32(&misc->q_full[i][b]), 1);
+        mbar_init(smem_u32(&misc->q_empty[i][b]), 2);             // the sub-tile's two streams
+      }
+      mbar_init(smem_u32(&misc->o_full[i]), 2);
+      mbar_init(smem_u32(&misc->o_free[i]), kSub);
+    }
+    fence_mbar_init();
+    prefetch_tmap(&tm_q);
+    prefetch_tmap(&tm_k);
+    prefetch_tmap(&tm_v);
+    prefetch_tmap(&tm_o);
+  }
+  if (warp == 25) {
+    tmem_alloc(smem_u32(&misc->tmem_slot), 512);
+    tmem_relinquish();
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem_base = misc->tmem_slot;
+  const bool run = *const_cast<volatile int*>(&misc->abort.flag) == 0;
+
+  // Index of this CTA's tile number `s` (s >= 1; tile 0 is blockIdx.x), -1 after the last, -2 if a wait expired.  Every
+  // role's warp calls it once per s, with all lanes.
+  auto next_tile = [&](int s, uint32_t role) __attribute__((always_inline)) -> int {
+    const int slot = s & 1;
+    if (!wait_quiet_warp(smem_u32(&misc->sched_full[slot]), ((s - 1) >> 1) & 1, abort_flag, wait_info(role, kBarSync, s))) return -2;
+    const int x = clc_answer(smem_u32(&misc->sched[slot]));
+    fence_proxy_async_smem();                         // the answer has been read: the next one may be written there
+    __syncwarp();
+    if (lane == 0) mbar_arrive(smem_u32(&misc->sched_empty[slot]));
+    return x;
+  };
+
+  if (warp < 16) {
+    // ===================================================== softmax warpgroup of one stream
+    setmaxnreg_inc<96>();
+    const int st = warp >> 2, i = st >> 1, half = st & 1;
+    const int row = (warp & 3) * 32 + lane;
+    const uint32_t lane_base = tmem_base + ((uint32_t)((warp & 3) * 32) << 16);
+    const uint32_t s_tmem = lane_base + st * HKV;      // P goes to the front of it
+    const uint32_t bar_s = smem_u32(&misc->s_full[st]);
+    const uint32_t bar_p = smem_u32(&misc->p_full[st]);
+    const float scale = p.scale_log2;
+    const ExpConsts ek = make_exp_consts(scale);
+    const int kv_tail = CAUSAL ? 0 : p.Lk & (TKV - 1);
+    bool ok = run;
+    uint32_t g = 0, done = 0;                          // steps of this stream over all tiles; finished tiles
+    int tile = blockIdx.x;
+    for (int seq = 1; ok && tile >= 0; ++seq) {
+      const TileWork w = narrow_work<CAUSAL>(tile, p);
+      const int n = w.steps(i);
+      if (n > 0) {
+        float m_run = -INFINITY, delta = 0.f;
+        // One key step.  The masked variant (the causal diagonal, a ragged last key tile) is compiled separately so that the
+        // common step pays nothing for it; `lim` is the last key column of this half the thread's row may attend to.
+        auto softmax_step = [&](auto mask_tag, int lim, bool first, bool last) __attribute__((always_inline)) -> bool {
+          constexpr bool kMasked = decltype(mask_tag)::value;
+          if (!wait_quiet_warp(bar_s, g & 1, abort_flag, wait_info(kRoleSoftmax, kBarSFull, g))) return false;
+          tc_fence_after();
+          uint32_t s[HKV];
+          // load the row in two halves: the maximum of the first half is taken while the second is in flight
+          tmem_ld32_nowait(s_tmem, *reinterpret_cast<uint32_t(*)[32]>(&s[0]));
+          tmem_ld_fence(*reinterpret_cast<uint32_t(*)[32]>(&s[0]));
+          tmem_ld32_nowait(s_tmem + 32, *reinterpret_cast<uint32_t(*)[32]>(&s[32]));
+          // keys past the end or after the query's position: score -inf, never zero
+          if constexpr (kMasked) {
+#pragma unroll
+            for (int k = 0; k < HKV / 2; ++k)
+              if (k > lim) s[k] = 0xFF800000u;
+          }
+          const float mx_a = fmaxf(chain_max<0, HKV / 4>(s), chain_max<HKV / 4, HKV / 2>(s));
+          tmem_ld_fence(*reinterpret_cast<uint32_t(*)[32]>(&s[32]));
+          if constexpr (kMasked) {
+#pragma unroll
+            for (int k = HKV / 2; k < HKV; ++k)
+              if (k > lim) s[k] = 0xFF800000u;
+          }
+          const float mx = max3(mx_a, chain_max<HKV / 2, 3 * HKV / 4>(s), chain_max<3 * HKV / 4, HKV>(s));
+          // Lazy rescale, as in attn_fwd_kernel.  The reference is finite from the first step on, also where a stream's
+          // half of the keys holds none that the row may attend to.
+          const float m_cand = max3(m_run, mx * scale, -1e30f);
+          const float gap = m_cand - m_run;
+          const float shrink = ex2_approx(-gap);
+          const bool move = (gap > kRescaleThreshold) || (gap > 0.f && kDominanceFactor > delta * shrink);
+          const float alpha = move ? shrink : 1.0f;
+          m_run = move ? m_cand : m_run;
+          // The step before is complete (see s_full), so the accumulator may be rescaled here; P V of this step waits for P.
+          if (!first && __any_sync(0xffffffffu, move)) {
+            const uint32_t o_tmem = lane_base + O_COL0 + st * D;
+#pragma unroll 1
+            for (int c = 0; c < D / 16; ++c) {
+              uint32_t r[16];
+              tmem_ld16(o_tmem + c * 16, r);
+#pragma unroll
+              for (int k = 0; k < 16; ++k) r[k] = __float_as_uint(__uint_as_float(r[k]) * alpha);
+              tmem_st16(o_tmem + c * 16, r);
+            }
+          }
+          const uint64_t neg_m2 = pack_f32x2(-m_run, -m_run);
+          uint64_t sum2 = 0ull;                        // packed (0.f, 0.f)
+          uint32_t pk[16];
+          exp_chunk<kPoly>(&s[0], ek, neg_m2, sum2, pk);
+          tmem_st16(s_tmem, pk);
+          uint32_t pk2[16];
+          exp_chunk<kPoly>(&s[32], ek, neg_m2, sum2, pk2);
+          tmem_st16(s_tmem + 16, pk2);
+          float sum0, sum1;
+          unpack_f32x2(sum2, sum0, sum1);
+          delta = delta * alpha + (sum0 + sum1);
+          if (last) {
+            // The epilogue warpgroup finishes the tile.  It has read what stood here two tiles ago: this tile's first scores
+            // came after the first P V of the tile before, which waited for that (o_free).  The arrival stands before the one
+            // on p_full: a thread that is a tile ahead has seen scores that came after every thread's p_full, so it cannot
+            // make its next arrival here before a slow thread has made this one.
+            // (A tile of one step: its only scores did not wait for the epilogue of the tile before, which may still be
+            // waiting for that tile's arrivals here.)
+            if (first && done > 0 && !wait_quiet_warp(smem_u32(&misc->o_free[i]), (done - 1) & 1, abort_flag, wait_info(kRoleSoftmax, kBarOFull, g))) return false;
+            misc->stat[done & 1][st][row] = make_float2(m_run, delta);
+            mbar_arrive(smem_u32(&misc->fin_full[st]));
+          }
+          tmem_wait_st();
+          tc_fence_before();
+          mbar_arrive(bar_p);
+          return true;
+        };
+        for (int jj = 0; ok && jj < n; ++jj, ++g) {
+          // Only the last step may need a mask: the causal diagonal, which starts at the sub-tile's first row and ends, in a
+          // ragged last key tile, before the padding for every row of the sequence; else a ragged last key tile.
+          const bool last = jj == n - 1;
+          if (last && (CAUSAL || kv_tail != 0)) ok = softmax_step(MaskTag<true>{}, (CAUSAL ? row : kv_tail - 1) - half * HKV, jj == 0, true);
+          else ok = softmax_step(MaskTag<false>{}, HKV - 1, jj == 0, !CAUSAL && last);
+        }
+        if (!ok) break;
+        ++done;
+      }
+      tile = next_tile(seq, kRoleSoftmax);
+    }
+  } else if (warp < 20) {
+    // ================================================== epilogue warpgroup
+    setmaxnreg_dec<40>();
+    const int wq = warp & 3, row = wq * 32 + lane;
+    const uint32_t lane_base = tmem_base + ((uint32_t)(wq * 32) << 16);
+    const uint32_t stage_w = out_smem + wq * 8192;     // this warp's two staging chunks
+    bool ok = run;
+    uint32_t fin = 0, chunk_ctr = 0;                   // bit i: finished tiles of sub-tile i, mod 2
+    int tile = blockIdx.x;
+    for (int seq = 1; ok && tile >= 0; ++seq) {
+      const TileWork w = narrow_work<CAUSAL>(tile, p);
+#pragma unroll 1
+      for (int i = 0; ok && i < 2; ++i) {
+        if (w.steps(i) == 0) continue;
+        const uint32_t ph = (fin >> i) & 1;
+        fin ^= 1u << i;
+        if (!wait_quiet_warp(smem_u32(&misc->fin_full[2 * i]), ph, abort_flag, wait_info(kRoleCorrection, kBarAlpha, 2 * i)) ||
+            !wait_quiet_warp(smem_u32(&misc->fin_full[2 * i + 1]), ph, abort_flag, wait_info(kRoleCorrection, kBarAlpha, 2 * i + 1))) { ok = false; break; }
+        // the two streams' parts on the common reference, normalised
+        const float2 a = misc->stat[ph][2 * i][row], b = misc->stat[ph][2 * i + 1][row];
+        const float m = fmaxf(a.x, b.x);
+        float wa = ex2_approx(a.x - m), wb = ex2_approx(b.x - m);
+        const float inv = 1.0f / (a.y * wa + b.y * wb);
+        wa *= inv;
+        wb *= inv;
+        if (!wait_quiet_warp(smem_u32(&misc->o_full[i]), ph, abort_flag, wait_info(kRoleCorrection, kBarOFull, i))) { ok = false; break; }
+        tc_fence_after();
+        const uint32_t o_tmem = lane_base + O_COL0 + 2 * i * D;
+        const uint32_t dst = stage_w + (chunk_ctr & 1) * 4096;
+        ++chunk_ctr;
+        // the store that last read this chunk (two chunks ago) must have finished reading it
+        if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
+        __syncwarp();
+#pragma unroll 1
+        for (int c = 0; c < 8; ++c) {                  // 8 columns at a time
+          uint32_t ra[8], rb[8];
+          tmem_ld8x2(o_tmem + c * 8, o_tmem + D + c * 8, ra, rb);
+          uint32_t q[4];
+#pragma unroll
+          for (int e = 0; e < 4; ++e)
+            q[e] = pack_bf16x2(__uint_as_float(ra[2 * e]) * wa + __uint_as_float(rb[2 * e]) * wb,
+                               __uint_as_float(ra[2 * e + 1]) * wa + __uint_as_float(rb[2 * e + 1]) * wb);
+          st_shared_u4(dst + lane * 128 + (((uint32_t)c ^ (uint32_t)(lane & 7)) << 4), q);   // 128-byte swizzle
+        }
+        tc_fence_before();
+        mbar_arrive(smem_u32(&misc->o_free[i]));       // both accumulators have been read
+        fence_proxy_async_smem();
+        __syncwarp();
+        if (lane == 0) {                               // (rows past the end of the sequence are clipped by the tensor map)
+          tma_store_3d(&tm_o, dst, 0, w.q_row0 + i * kSub + wq * 32, w.bh);
+          tma_store_commit();
+        }
+      }
+      if (!ok) break;
+      tile = next_tile(seq, kRoleCorrection);
+    }
+    if (lane == 0) tma_store_wait_read();              // shared memory is read by the stores until here
+    __syncwarp();
+  } else if (warp < 24) {
+    // ============================== MMA issuer of one stream (the whole warp walks the loop, one lane issues)
+    setmaxnreg_dec<40>();
+    const int st = warp & 3, i = st >> 1, half = st & 1;
+    bool ok = run;
+    const uint32_t s_tmem = tmem_base + st * HKV, o_tmem = tmem_base + O_COL0 + st * D;
+    const uint32_t k_smem = ring_smem + half * (HKV * 128);       // this stream's keys in a ring item
+    uint32_t g = 0, done = 0, q_uses = 0;              // steps; finished tiles; Q loads that have been read
+    int pos = 0;                                       // ring position of the next item (K_0, V_0, K_1, V_1, ... of every tile)
+    uint32_t ph = 0;
+    auto wait = [&](uint64_t* bar, uint32_t parity, uint32_t id) __attribute__((always_inline)) -> bool {
+      if (!wait_quiet_warp(smem_u32(bar), parity, abort_flag, wait_info(kRoleMma, id, 0x100 * st + (g & 0xFF)))) { ok = false; return false; }
+      return true;
+    };
+    auto advance = [&]() __attribute__((always_inline)) { if (++pos == p.stages) { pos = 0; ph ^= 1u; } };
+    // (one lane) Scores of the keys at ring position k; last: no later step of the tile reads this Q.
+    auto issue_scores = [&](int k, bool last) __attribute__((always_inline)) {
+      const int b = (q_uses - 1) & 1;
+      issue_qk<D, HKV>(s_tmem, smem_base + (b * 2 + i) * SM::kSubBytes, k_smem + k * SM::kStageBytes);
+      umma_commit(smem_u32(&misc->s_full[st]));
+      umma_commit(smem_u32(&misc->kv_empty[k]));
+      if (last) umma_commit(smem_u32(&misc->q_empty[i][b]));
+    };
+    // Key steps that this stream's sub-tile does not run: their ring items are passed on as soon as they have arrived.
+    auto skip = [&](int steps) __attribute__((always_inline)) {
+#pragma unroll 1
+      for (int x = 0; x < 2 * steps; ++x) {
+        if (!wait(&misc->kv_full[pos], ph, kBarKvFull)) return;
+        if (lane == 0) mbar_arrive(smem_u32(&misc->kv_empty[pos]));
+        advance();
+      }
+    };
+    // A tile's first scores.
+    auto start = [&](int steps) __attribute__((always_inline)) {
+      if (!wait(&misc->q_full[i][q_uses & 1], (q_uses >> 1) & 1, kBarQ) || !wait(&misc->kv_full[pos], ph, kBarKvFull)) return;
+      ++q_uses;
+      tc_fence_after();
+      if (elect_one()) issue_scores(pos, steps == 1);
+      __syncwarp();
+      advance();
+    };
+    int tile = blockIdx.x;
+    for (int seq = 1; ok && tile >= 0; ++seq) {
+      const TileWork w = narrow_work<CAUSAL>(tile, p);
+      const int n = w.steps(i);
+      if (n > 0) start(n);
+      for (int j = 0; ok && j < n; ++j, ++g) {
+        const int v = pos;
+        if (!wait(&misc->kv_full[v], ph, kBarKvFull)) break;
+        advance();
+        const int k = pos;
+        const bool more = j + 1 < n;
+        if (more) {
+          if (!wait(&misc->kv_full[k], ph, kBarKvFull)) break;
+          advance();
+        }
+        // the tile before has left the accumulator
+        if (j == 0 && done > 0 && !wait(&misc->o_free[i], (done - 1) & 1, kBarOFull)) break;
+        if (!wait(&misc->p_full[st], g & 1, kBarPFull)) break;
+        tc_fence_after();
+        if (elect_one()) {
+          issue_pv<D, HKV>(o_tmem, s_tmem, k_smem + v * SM::kStageBytes, j > 0, TKV * 128, 1024);
+          umma_commit(smem_u32(&misc->kv_empty[v]));
+          if (more) issue_scores(k, j + 2 == n);
+          else umma_commit(smem_u32(&misc->o_full[i]));
+        }
+        __syncwarp();
+      }
+      if (!ok) break;
+      done += n > 0 ? 1u : 0u;
+      if (CAUSAL || n == 0) skip(w.steps() - n);
+      if (!ok) break;
+      tile = next_tile(seq, kRoleMma);
+    }
+  } else if (warp == 24) {
+    // ================================================== TMA producer, and the requests for the next tile
+    setmaxnreg_dec<40>();
+    bool ok = run;
+    int stage = 0, issued = 0, asked = 0;              // asked: requests made
+    uint32_t phase = 0;
+    uint32_t q_loads0 = 0, q_loads1 = 0;
+    // (the waits are taken by the whole warp, the copies issued by one lane)
+    auto load_kv = [&](const CUtensorMap* tm, int kv_row, int bh) __attribute__((always_inline)) -> bool {
+      if (!wait_quiet_warp(smem_u32(&misc->kv_empty[stage]), phase ^ 1u, abort_flag, wait_info(kRoleLoad, kBarKvEmpty, issued))) return false;
+      if (elect_one()) {
+        const uint32_t bar = smem_u32(&misc->kv_full[stage]);
+        mbar_arrive_expect_tx(bar, SM::kStageBytes);
+        tma_load_3d(ring_smem + stage * SM::kStageBytes, tm, 0, kv_row, bh, bar);
+      }
+      __syncwarp();
+      ++issued;
+      if (++stage == p.stages) { stage = 0; phase ^= 1u; }
+      return true;
+    };
+    auto load_q = [&](int i, const TileWork& w) __attribute__((always_inline)) -> bool {
+      const uint32_t u = i ? q_loads1 : q_loads0, b = u & 1;
+      if (u >= 2 && !wait_quiet_warp(smem_u32(&misc->q_empty[i][b]), (u / 2 - 1) & 1, abort_flag, wait_info(kRoleLoad, kBarQ, u))) return false;
+      if (elect_one()) {
+        const uint32_t bar = smem_u32(&misc->q_full[i][b]);
+        mbar_arrive_expect_tx(bar, SM::kSubBytes);
+        tma_load_3d(smem_base + (b * 2 + i) * SM::kSubBytes, &tm_q, 0, w.q_row0 + i * kSub, w.bh, bar);
+      }
+      __syncwarp();
+      if (i) ++q_loads1; else ++q_loads0;
+      return true;
+    };
+    int tile = blockIdx.x;
+    for (int seq = 1; ok && tile >= 0; ++seq) {
+      const TileWork w = narrow_work<CAUSAL>(tile, p);
+      const int n = w.steps();
+      // the first product needs K_0 and Q of sub-tile 0; the first tile's Q buffer is free at once
+      if (seq == 1) ok = load_q(0, w);
+      if (ok) ok = load_kv(&tm_k, 0, w.bh);
+      if (ok && seq > 1) ok = load_q(0, w);
+      if (ok && w.n1 > 0) ok = load_q(1, w);
+      for (int j = 0; ok && j < n; ++j) {
+        if (j > 0) ok = load_kv(&tm_k, j * TKV, w.bh);
+        if (ok && j == n - 1) {
+          // Ask for the tile after this one, into the slot that held the tile before this one -- as late as the answer is
+          // sure to be back in time (a ring's depth ahead of the MMA warp): a tile asked for early would be tied to this
+          // CTA while others run dry.
+          if (seq >= 3)
+            ok = wait_quiet_warp(smem_u32(&misc->sched_empty[seq & 1]), ((seq - 3) >> 1) & 1, abort_flag, wait_info(kRoleLoad, kBarSync, seq));
+          if (!ok) break;
+          if (elect_one()) {
+            mbar_arrive_expect_tx(smem_u32(&misc->sched_full[seq & 1]), 16);
+            clc_try_cancel(smem_u32(&misc->sched[seq & 1]), smem_u32(&misc->sched_full[seq & 1]));
+          }
+          __syncwarp();
+          asked = seq;
+        }
+        if (ok) ok = load_kv(&tm_v, j * TKV, w.bh);
+      }
+      if (!ok) break;
+      tile = next_tile(seq, kRoleLoad);
+    }
+    if (tile == -2) ok = false;
+    if (!ok && lane == 0) {
+      // Drain: every copy started here must land before the CTA may exit, and so must an answer still on its way.
+      for (int t = issued > p.stages ? issued - p.stages : 0; t < issued; ++t)
+        drain_bar(smem_u32(&misc->kv_full[t % p.stages]), (uint32_t)(t / p.stages) & 1u);
+      for (int i = 0; i < 2; ++i)
+        for (uint32_t q = i ? q_loads1 : q_loads0, u = q > 2u ? q - 2u : 0; u < q; ++u) drain_bar(smem_u32(&misc->q_full[i][u & 1]), (u / 2) & 1);
+      if (asked > 0) drain_bar(smem_u32(&misc->sched_full[asked & 1]), ((asked - 1) >> 1) & 1);
+    }
+  } else {
+    setmaxnreg_dec<40>();
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 25) {
+    tc_fence_after();
+    tmem_dealloc(tmem_base, 512);
+  }
+  if (threadIdx.x == 0) report_abort(&misc->abort);
+}
+
+}  // namespace attn

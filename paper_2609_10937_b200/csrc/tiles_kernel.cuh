@@ -1,5 +1,5 @@
-// attn_causal_tiles_kernel: the fused attention step loop of attn_kernels.cuh for causal grids in which every Q tile is worked on
-// by one CTA from its first key to its last (nothing to merge).
+// attn_causal_tiles_kernel: the fused attention step loop of attn_kernels.cuh at d = 128 for causal grids in which every Q tile is
+// worked on by one CTA from its first key to its last (nothing to merge).  (d = 64: narrow_kernel.cuh.)
 //
 // What it has over attn_fwd_kernel is a pipeline that does not stop between tiles.  There, the softmax warps finish a tile
 // themselves: they wait for its last product, normalise and store, and only then start on the next tile's scores -- about
@@ -29,33 +29,28 @@ struct TilesParams {
   unsigned int* status;    // as in FwdParams
 };
 
-template <int D>
 struct TilesSmem {
-  static constexpr int kQBufs = D == 64 ? 2 : 1;                 // Q tiles in shared memory
-  static constexpr int kSubBytes = kSub * D * 2;
-  static constexpr int kQBytes = kQBufs * 2 * kSubBytes;
-  static constexpr int kStageBytes = 128 * D * 2;
+  static constexpr int kSubBytes = kSub * 128 * 2;
+  static constexpr int kQBytes = 2 * kSubBytes;
+  static constexpr int kStageBytes = 128 * 128 * 2;
   static constexpr int kOutBytes = 8 * 4096;                     // two [32 rows][64 columns] bf16 chunks per correction warp
-  static constexpr int kMiscBytes = D == 64 ? 4096 : 3072;
+  static constexpr int kMiscBytes = 3072;
   __host__ __device__ static constexpr int total(int stages) { return kQBytes + stages * kStageBytes + kOutBytes + kMiscBytes; }
 };
 
 constexpr int kSchedReaders = 14;          // warps that read a tile's index: 8 softmax, 4 correction, MMA, TMA
-template <int D>
 struct TilesMisc {
-  // d = 64 stores a step's factor before it knows that the factor of the step before has been read
-  static constexpr int kAlphaBufs = D == 64 ? 2 : 1;
-  float alpha[2][kAlphaBufs][kSub];        // [sub-tile][step mod kAlphaBufs][row] rescale factor
+  float alpha[2][kSub];                    // [sub-tile][row] rescale factor
   float inv[2][kSub];                      // [sub-tile][row] 1 / denominator of a finished tile
   uint4 sched[2];              // answers of try_cancel (16 bytes each)
   uint64_t sched_full[2], sched_empty[2];
-  uint64_t q_full[2][2], q_empty[2][2];    // [sub-tile][buffer]
+  uint64_t q_full[2], q_empty[2];          // per sub-tile
   uint64_t kv_full[kMaxStages], kv_empty[kMaxStages];
-  uint64_t s_full[2], s_free[2], p_full[2], p_half[2], o_full[2], alpha_full[2], fin_full[2];
+  uint64_t s_full[2], p_full[2], p_half[2], o_full[2], alpha_full[2], fin_full[2];
   AbortCell abort;
   uint32_t tmem_slot;
 };
-static_assert(sizeof(TilesMisc<64>) <= TilesSmem<64>::kMiscBytes && sizeof(TilesMisc<128>) <= TilesSmem<128>::kMiscBytes, "misc region too large");
+static_assert(sizeof(TilesMisc) <= TilesSmem::kMiscBytes, "misc region too large");
 
 // Asks for the index of a CTA of this grid that has not been started; the 16-byte answer is counted on `bar`.
 __device__ __forceinline__ void clc_try_cancel(uint32_t answer_smem, uint32_t bar) {
@@ -97,23 +92,19 @@ __device__ __forceinline__ TileWork tile_work(int index, const TilesParams& p) {
   return w;
 }
 
-template <int D>
 __global__ void __launch_bounds__(512, 1)
 attn_causal_tiles_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                   const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_o, const TilesParams p) {
-  constexpr int TKV = 128, NCH = TKV / 32, KCH = D / 64;
-  constexpr bool kSplitP = D == 64;                   // P in tensor-memory columns of its own (see attn_fwd_kernel)
-  constexpr int O_COL0 = 2 * TKV, P_COL0 = 2 * (TKV + D);
+  constexpr int D = 128, TKV = 128, NCH = TKV / 32, KCH = D / 64;
+  constexpr int O_COL0 = 2 * TKV;
   constexpr int kPoly = kPolyPairsPer8;
-  using SM = TilesSmem<D>;
-  constexpr int QB = SM::kQBufs;
+  using SM = TilesSmem;
 
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   const uint32_t smem_base = smem_u32(smem_raw);
   const uint32_t ring_smem = smem_base + SM::kQBytes;
   const uint32_t out_smem = ring_smem + p.stages * SM::kStageBytes;
-  using Misc = TilesMisc<D>;
-  Misc* const misc = reinterpret_cast<Misc*>(smem_raw + SM::kQBytes + p.stages * SM::kStageBytes + SM::kOutBytes);
+  TilesMisc* const misc = reinterpret_cast<TilesMisc*>(smem_raw + SM::kQBytes + p.stages * SM::kStageBytes + SM::kOutBytes);
   volatile int* abort_flag = &misc->abort.flag;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
@@ -129,12 +120,9 @@ attn_causal_tiles_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
     for (int i = 0; i < 2; ++i) {
       mbar_init(smem_u32(&misc->sched_full[i]), 1);
       mbar_init(smem_u32(&misc->sched_empty[i]), kSchedReaders);
-      for (int b = 0; b < 2; ++b) {
-        mbar_init(smem_u32(&misc->q_full[i][b]), 1);
-        mbar_init(smem_u32(&misc->q_empty[i][b]), 1);
-      }
+      mbar_init(smem_u32(&misc->q_full[i]), 1);
+      mbar_init(smem_u32(&misc->q_empty[i]), 1);
       mbar_init(smem_u32(&misc->s_full[i]), 1);
-      mbar_init(smem_u32(&misc->s_free[i]), kSub);
       mbar_init(smem_u32(&misc->p_full[i]), 2 * kSub);          // softmax rows + correction rows
       mbar_init(smem_u32(&misc->p_half[i]), kSub);
       mbar_init(smem_u32(&misc->o_full[i]), 1);
@@ -176,7 +164,7 @@ attn_causal_tiles_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
     const int row = (warp & 3) * 32 + lane;
     const uint32_t lane_base = tmem_base + ((uint32_t)((warp & 3) * 32) << 16);
     const uint32_t s_tmem = lane_base + i * TKV;
-    const uint32_t p_tmem = kSplitP ? lane_base + P_COL0 + i * (TKV / 2) : s_tmem;   // else P aliases the front of S
+    const uint32_t p_tmem = s_tmem;                    // P overwrites the front of S
     const uint32_t bar_s = smem_u32(&misc->s_full[i]);
     const uint32_t bar_p = smem_u32(&misc->p_full[i]);
     const uint32_t bar_h = smem_u32(&misc->p_half[i]);
@@ -191,7 +179,6 @@ attn_causal_tiles_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
       const int n = w.steps(i);
       if (n > 0) {
         float m_run = -INFINITY, delta = 0.f;
-        const uint32_t g_seg0 = g;                     // this tile's first step
         // One key step.  The masked variant (the causal diagonal) is compiled separately so that
         // the common step pays nothing for it; `lim` is the last key column the thread's row may attend to.
         auto softmax_step = [&](auto mask_tag, int lim) __attribute__((always_inline)) -> bool {
@@ -216,10 +203,6 @@ attn_causal_tiles_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
                                    fmaxf(chain_max<TKV / 4, 3 * TKV / 8>(s), chain_max<3 * TKV / 8, TKV / 2>(s)));
 #pragma unroll
           for (int c = NCH / 2; c < NCH; ++c) tmem_ld_fence(*reinterpret_cast<uint32_t(*)[32]>(&s[c * 32]));
-          if constexpr (kSplitP) {
-            tc_fence_before();
-            mbar_arrive(smem_u32(&misc->s_free[i]));   // the scores are in registers: the buffer may be overwritten
-          }
           if constexpr (kMasked) {
 #pragma unroll
             for (int k = TKV / 2; k < TKV; ++k)
@@ -235,15 +218,7 @@ attn_causal_tiles_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
           const bool move = (gap > kRescaleThreshold) || (gap > 0.f && kDominanceFactor > delta * shrink);
           const float m_new = move ? m_cand : m_run;
           const float alpha = move ? shrink : 1.0f;
-          misc->alpha[i][g % Misc::kAlphaBufs][row] = alpha;
-          if constexpr (kSplitP) {
-            // P's columns must have been read by the previous step's P V, and every arrival of this step must come after
-            // it (attn_fwd_kernel says why); a tile's first step is covered by the wait at the end of the tile before
-            if (g != g_seg0) {
-              if (!wait_quiet_warp(smem_u32(&misc->o_full[i]), (g - 1) & 1, abort_flag, wait_info(kRoleSoftmax, kBarOFull, 0x4000 | g))) return false;
-              tc_fence_after();
-            }
-          }
+          misc->alpha[i][row] = alpha;
           mbar_arrive(bar_a);
           const uint64_t neg_m2 = pack_f32x2(-m_new, -m_new);
           uint64_t sum_a = 0ull, sum_b = 0ull;         // packed (0.f, 0.f)
@@ -284,8 +259,8 @@ attn_causal_tiles_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
         if (!ok) break;
         // The denominators go to the correction warpgroup, which finishes the tile.  Its arrival on p_full of a tile's first
         // step says that it has read those of the tile before; from two steps on, the second step's scores come after it.  A
-        // tile of one step waits for its only product instead, and so does d = 64 always (see softmax_step).
-        if (kSplitP || n == 1) {
+        // tile of one step waits for its only product instead.
+        if (n == 1) {
           ok = wait_quiet_warp(smem_u32(&misc->o_full[i]), (g - 1) & 1, abort_flag, wait_info(kRoleSoftmax, kBarOFull, g));
           if (!ok) break;
           tc_fence_after();
@@ -351,7 +326,7 @@ attn_causal_tiles_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
           if (j >= (i ? w.n1 : w.n0)) continue;
           const uint32_t gi = i ? g1 : g0;
           if (!wait_quiet_warp(smem_u32(&misc->alpha_full[i]), gi & 1, abort_flag, wait_info(kRoleCorrection, kBarAlpha, j))) { ok = false; break; }
-          const float a = misc->alpha[i][gi % Misc::kAlphaBufs][row];
+          const float a = misc->alpha[i][row];
           if (j > 0) {                                 // a tile's first step starts O afresh
             const bool need = __any_sync(0xffffffffu, a != 1.0f);
             if (need) {
@@ -401,34 +376,33 @@ attn_causal_tiles_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
       return true;
     };
     // A product S_i = Q_i K^T that is ready to be issued: its operands have arrived.
-    struct Scores { int st, b; bool go, last, release; };
+    struct Scores { int st; bool go, last, release; };
     // Waits for the operands: the K tile at ring position st and, for the first product of a tile, its Q.  last: no later
     // step reads this Q; release: no other sub-tile reads this K tile any more.
     auto ready = [&](int i, int st, uint32_t ph, bool first, bool last, bool release) __attribute__((always_inline)) -> Scores {
-      Scores sc = {st, 0, false, last, release};
+      Scores sc = {st, false, last, release};
       if (!wait(&misc->kv_full[st], ph, kBarKvFull, i)) return sc;
       if (first) {
         const uint32_t u = uses >> (8 * i);
-        if (!wait(&misc->q_full[i][QB == 2 ? u & 1 : 0], QB == 2 ? (u >> 1) & 1 : u & 1, kBarQ, i)) return sc;
+        if (!wait(&misc->q_full[i], u & 1, kBarQ, i)) return sc;
         uses = (uses & ~(3u << (8 * i))) | (((u + 1) & 3u) << (8 * i));
       }
-      sc.b = QB == 2 ? ((uses >> (8 * i)) + 1) & 1 : 0;           // the buffer of the load read last
       sc.go = true;
       return sc;
     };
     // (one lane)
     auto issue_scores = [&](int i, const Scores& sc) __attribute__((always_inline)) {
-      issue_qk<D, TKV>(tmem_base + i * TKV, smem_base + (sc.b * 2 + i) * SM::kSubBytes, ring_smem + sc.st * SM::kStageBytes);
+      issue_qk<D, TKV>(tmem_base + i * TKV, smem_base + i * SM::kSubBytes, ring_smem + sc.st * SM::kStageBytes);
       umma_commit(smem_u32(&misc->s_full[i]));
       if (sc.release) umma_commit(smem_u32(&misc->kv_empty[sc.st]));
-      if (sc.last) umma_commit(smem_u32(&misc->q_empty[i][sc.b]));
+      if (sc.last) umma_commit(smem_u32(&misc->q_empty[i]));
     };
     auto scores = [&](int i, const Scores& sc) __attribute__((always_inline)) {
       if (sc.go && elect_one()) issue_scores(i, sc);
       __syncwarp();
     };
     auto p_times_v = [&](int i, int j, bool second) __attribute__((always_inline)) {       // (one lane)
-      const uint32_t o = tmem_base + O_COL0 + i * D, pt = kSplitP ? tmem_base + P_COL0 + i * (TKV / 2) : tmem_base + i * TKV;
+      const uint32_t o = tmem_base + O_COL0 + i * D, pt = tmem_base + i * TKV;
       const uint32_t v = ring_smem + vs * SM::kStageBytes;
       if (!second) issue_pv<D, TKV>(o, pt, v, j > 0, TKV * 128, 1024, 0, TKV / 32);
       else {
@@ -444,18 +418,15 @@ attn_causal_tiles_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
       n1 = w.n1;
     }
     if (ok) {
-      // the first tile's first scores; at d = 64 sub-tile 1's follow half a step later (below), which sets up the offset
-      // between the two softmax warpgroups that the rest of the walk keeps
       scores(0, ready(0, 0, 0, true, n0 == 1, n1 == 0));
-      if (ok && !kSplitP && n1 > 0) scores(1, ready(1, 0, 0, true, n1 == 1, true));
+      if (ok && n1 > 0) scores(1, ready(1, 0, 0, true, n1 == 1, true));
     }
-    bool defer = kSplitP && n1 > 0;                    // (d = 64) sub-tile 1's first scores are still to come
     for (int seq = 1; ok && tile >= 0; ++seq) {
       const int n = n1 > n0 ? n1 : n0;
       int next = -3;                                   // not asked yet
       // The product that follows step j of sub-tile i: its next step, or its first step of the next tile.
       auto next_scores = [&](int i, int j) __attribute__((always_inline)) -> Scores {
-        const Scores none = {0, 0, false, false, false};
+        const Scores none = {0, false, false, false};
         const int ni = i ? n1 : n0;
         int items = 1, left = ni - j - 1, other = n1;  // ring items from V_j to the K tile; steps left with this Q; (release)
         const bool first = left <= 0;
@@ -481,62 +452,25 @@ attn_causal_tiles_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
         return ready(i, st, ph, first, left == 1, i == 1 || other == 0);
       };
       for (int j = 0; ok && j < n; ++j) {
-        if constexpr (kSplitP) {
-          // Nothing ties the two sub-tiles to each other here, and left alone their softmax warpgroups end up in the same
-          // phase of the step (both at the exponentials, then neither).  So sub-tile 1's scores are issued behind the first
-          // half of sub-tile 0's P of the step: half a step behind.
-          if (j < n0) {
-            if (!wait(&misc->s_free[0], gp & 1, kBarPFull, 0x100)) break;
-            scores(0, next_scores(0, j));
-            if (!ok || !wait(&misc->kv_full[vs], vph, kBarKvFull, 0x102) || !wait(&misc->p_full[0], gp & 1, kBarPFull, 0x103)) break;
-            if (elect_one()) p_times_v(0, j, false);
-            __syncwarp();
-          }
-          if (defer) {
-            defer = false;
-            scores(1, ready(1, 0, 0, true, n1 == 1, true));
+        if (!wait(&misc->kv_full[vs], vph, kBarKvFull, 0x10A)) break;
+#pragma unroll 1
+        for (int i = 0; i < 2; ++i) {
+          const int ni = i ? n1 : n0;
+          {
+            if (j < ni) {
+              if (!wait(&misc->p_full[i], (gp >> i) & 1, kBarPFull, i)) break;
+              if (elect_one()) p_times_v(i, j, false);
+              __syncwarp();
+              if (!wait(&misc->p_half[i], (gp >> i) & 1, kBarPFull, 0x8000 | i)) break;
+              if (elect_one()) p_times_v(i, j, true);
+              __syncwarp();
+              gp ^= 1u << i;
+            }
+            scores(i, next_scores(i, j));
             if (!ok) break;
           }
-          if (j < n1 && !wait(&misc->s_free[1], (gp >> 1) & 1, kBarPFull, 0x105)) break;
-          scores(1, next_scores(1, j));
-          if (!ok) break;
-          if (j < n0) {
-            if (!wait(&misc->p_half[0], gp & 1, kBarPFull, 0x106)) break;
-            if (elect_one()) p_times_v(0, j, true);
-            __syncwarp();
-            gp ^= 1u;
-          }
-          if (j < n1) {
-            if (j >= n0 && !wait(&misc->kv_full[vs], vph, kBarKvFull, 0x107)) break;
-            if (!wait(&misc->p_full[1], (gp >> 1) & 1, kBarPFull, 0x108)) break;
-            if (elect_one()) p_times_v(1, j, false);
-            __syncwarp();
-            if (!wait(&misc->p_half[1], (gp >> 1) & 1, kBarPFull, 0x109)) break;
-            if (elect_one()) p_times_v(1, j, true);
-            __syncwarp();
-            gp ^= 2u;
-          }
-        } else {
-          if (!wait(&misc->kv_full[vs], vph, kBarKvFull, 0x10A)) break;
-#pragma unroll 1
-          for (int i = 0; i < 2; ++i) {
-            const int ni = i ? n1 : n0;
-            {
-              if (j < ni) {
-                if (!wait(&misc->p_full[i], (gp >> i) & 1, kBarPFull, i)) break;
-                if (elect_one()) p_times_v(i, j, false);
-                __syncwarp();
-                if (!wait(&misc->p_half[i], (gp >> i) & 1, kBarPFull, 0x8000 | i)) break;
-                if (elect_one()) p_times_v(i, j, true);
-                __syncwarp();
-                gp ^= 1u << i;
-              }
-              scores(i, next_scores(i, j));
-              if (!ok) break;
-            }
-          }
-          if (!ok) break;
         }
+        if (!ok) break;
         if (elect_one()) umma_commit(smem_u32(&misc->kv_empty[vs]));
         __syncwarp();
         vs += 2;
@@ -569,10 +503,10 @@ attn_causal_tiles_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
       return true;
     };
     auto load_q = [&](int i, const TileWork& w) __attribute__((always_inline)) -> bool {
-      const uint32_t u = i ? q_loads1 : q_loads0, b = u % QB;
-      if (u >= QB && !wait_quiet_warp(smem_u32(&misc->q_empty[i][b]), (u / QB - 1) & 1, abort_flag, wait_info(kRoleLoad, kBarQ, u))) return false;
+      const uint32_t u = i ? q_loads1 : q_loads0;
+      if (u >= 1 && !wait_quiet_warp(smem_u32(&misc->q_empty[i]), (u - 1) & 1, abort_flag, wait_info(kRoleLoad, kBarQ, u))) return false;
       if (elect_one()) {
-        const uint32_t bar = smem_u32(&misc->q_full[i][b]), dst = smem_base + (b * 2 + i) * SM::kSubBytes;
+        const uint32_t bar = smem_u32(&misc->q_full[i]), dst = smem_base + i * SM::kSubBytes;
         mbar_arrive_expect_tx(bar, SM::kSubBytes);
 #pragma unroll
         for (int c = 0; c < KCH; ++c) tma_load_3d(dst + c * (kSub * 128), &tm_q, c * 64, w.q_row0 + i * kSub, w.bh, bar);
@@ -621,7 +555,7 @@ attn_causal_tiles_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
       for (int t = issued > p.stages ? issued - p.stages : 0; t < issued; ++t)
         drain(&misc->kv_full[t % p.stages], (uint32_t)(t / p.stages) & 1u);
       for (int i = 0; i < 2; ++i)
-        for (uint32_t q = i ? q_loads1 : q_loads0, u = q > (uint32_t)QB ? q - QB : 0; u < q; ++u) drain(&misc->q_full[i][u % QB], (u / QB) & 1);
+        if (const uint32_t q = i ? q_loads1 : q_loads0) drain(&misc->q_full[i], (q - 1) & 1);
       if (asked > 0) drain(&misc->sched_full[asked & 1], ((asked - 1) >> 1) & 1);
     }
   } else {

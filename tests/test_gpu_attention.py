@@ -1018,3 +1018,28 @@ def test_causal_whole_tiles_match_the_reference(env, B, H, L, d):
     for _ in range(3):
         again = binding.forward(*dev, causal=True)
         assert torch.equal(again.view(torch.int16), out.view(torch.int16))
+
+
+@pytest.mark.parametrize("H,Lq,Lk", [(444, 129, 129), (444, 200, 200), (444, 256, 256), (222, 257, 257), (222, 385, 385), (148, 700, 700),
+                                     (444, 200, 1), (444, 129, 63), (444, 256, 64), (222, 300, 65), (222, 512, 128), (222, 400, 129), (148, 641, 1100)])
+def test_narrow_whole_tiles_match_the_reference(env, H, Lq, Lk):
+    """d = 64, whole waves of tiles: sub-tiles that are absent, of one row and full; key tiles whose second half is absent, of one
+    key and full; tiles of one and of several key steps.  NaN-filled output, every element against fp64, the same bits again.
+    The bound per element is that of test_causal_whole_tiles_match_the_reference."""
+    torch, orc, binding = env
+    rng = np.random.default_rng([H, Lq, Lk, 6])
+    q, k, v = (to_cuda_bf16(synth.f32_to_bf16_bits((rng.standard_normal((H, n, 64)) * 1.5).astype(np.float32))).view(1, H, n, 64)
+               for n in (Lq, Lk, Lk))
+    out = torch.full((1, H, Lq, 64), float("nan"), dtype=torch.bfloat16, device="cuda")
+    binding.forward_qk(q, k, v, out)
+    torch.cuda.synchronize()
+    assert binding.last_device_status()[0] == 0
+    assert (binding.last_kernel(), binding.last_grid()) == (binding.KERNEL_NARROW_TILES, H * -(-Lq // 256))
+    for h in range(0, H, 37):
+        s = q[0, h:h + 37].double() @ k[0, h:h + 37].double().transpose(1, 2) / 8.0
+        p, vd, got = torch.softmax(s, dim=-1), v[0, h:h + 37].double(), out[0, h:h + 37].double()
+        ref, spread = p @ vd, p @ vd.abs()
+        assert ((got - ref).abs() <= (2.0 ** -8 + 2.0 ** -13) * spread + 2.0 ** -8 * ref.abs() + 1e-6).all(), h
+        assert float((got - ref).norm() / ref.norm()) <= 5e-3, h
+    for _ in range(3):
+        assert torch.equal(binding.forward_qk(q, k, v).view(torch.int16), out.view(torch.int16))
