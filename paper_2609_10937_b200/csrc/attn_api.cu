@@ -141,6 +141,28 @@ int allow_smem(const void* kern, int bytes) {
     if (rc__ != ATTN_OK) return rc__;                                                \
   } while (0)
 
+// Launches a kernel whose CTAs may start while the grid in front of it on the stream is still finishing (its set-up then runs under
+// that grid's last CTAs; every kernel here waits for the grids in front before it touches memory, ptx_sm100.cuh).  cluster: CTAs
+// of a thread-block cluster, 0 or 1 for none.
+template <class... P, class... A>
+cudaError_t launch_kernel(void (*kern)(P...), long long grid, int block, int smem, int cluster, cudaStream_t stream, const A&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3((unsigned)block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = (unsigned)cluster;
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = cluster > 1 ? 2 : 1;
+  return cudaLaunchKernelEx(&cfg, kern, args...);
+}
+
 bool overlaps(const void* a, size_t na, const void* b, size_t nb) {
   const uintptr_t a0 = (uintptr_t)a, b0 = (uintptr_t)b;
   return a0 < b0 + nb && b0 < a0 + na;
@@ -211,7 +233,7 @@ int launch_fwd(const void* q, const void* k, const void* v, void* o, int B, int 
   const bool wait_roles_ok = !may_overlap;
   auto launch = [&](auto kern) -> int {
     ATTN_ALLOW_SMEM(kern, smem);
-    kern<<<grid, 512, smem, stream>>>(tq, tk, tv, to, p);
+    ATTN_CUDA_TRY(launch_kernel(kern, grid, 512, smem, 0, stream, tq, tk, tv, to, p));
     return ATTN_OK;
   };
   // Uniform key split with few parts: the k CTAs of a tile are launched as one thread-block cluster and exchange
@@ -252,7 +274,7 @@ int launch_fwd(const void* q, const void* k, const void* v, void* o, int B, int 
       if ((long long)n_res * kk >= grid) {
         attn::FwdParams pc = p;
         pc.cluster_k = kk;
-        if (cudaLaunchKernelEx(&cfg, kern_cluster, tq, tk, tv, to, pc) == cudaSuccess) {
+        if (launch_kernel(kern_cluster, grid, 512, smem, kk, stream, tq, tk, tv, to, pc) == cudaSuccess) {
           t_cluster_size = kk;
           return ATTN_OK;
         }
@@ -260,7 +282,7 @@ int launch_fwd(const void* q, const void* k, const void* v, void* o, int B, int 
       }
     }
     if (!wait_roles_ok) return ATTN_ERR_BAD_TILES;        // (marker: the caller launches the last-finisher instantiation)
-    kern<<<grid, 512, smem, stream>>>(tq, tk, tv, to, p);
+    ATTN_CUDA_TRY(launch_kernel(kern, grid, 512, smem, 0, stream, tq, tk, tv, to, p));
     return ATTN_OK;
   };
   const int ck = (t.tiles > 0 && t.ctas % t.tiles == 0) ? t.ctas / t.tiles : 0;
@@ -295,7 +317,7 @@ int launch_fwd(const void* q, const void* k, const void* v, void* o, int B, int 
       }
       n_res = st->resident[1][ck] - 1;
     }
-    if ((long long)n_res * ck >= grid && cudaLaunchKernelEx(&cfg, kern, tq, tk, tv, to, pc) == cudaSuccess) {
+    if ((long long)n_res * ck >= grid && launch_kernel(kern, grid, 512, smem, ck, stream, tq, tk, tv, to, pc) == cudaSuccess) {
       t_cluster_size = ck;
       rc = ATTN_OK;
     } else {
@@ -335,19 +357,7 @@ int launch_decode(const void* q, const void* k, const void* v, void* o, int BH, 
   constexpr int smem = attn::decode_smem_total<MT>();
   ATTN_ALLOW_SMEM(kern, smem);
   if (cluster_k > 8) ATTN_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(BH * cluster_k));
-  cfg.blockDim = dim3(32 * attn::kDecodeWarps);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = cluster_k;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  ATTN_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, tk, tv, p));
+  ATTN_CUDA_TRY(launch_kernel(kern, (long long)BH * cluster_k, 32 * attn::kDecodeWarps, smem, cluster_k, stream, tk, tv, p));
   t_cluster_size = cluster_k > 1 ? cluster_k : 0;
   t_launch_count = 1;
   launched(ATTN_KERNEL_FEW_ROWS, (long long)BH * cluster_k);
@@ -450,8 +460,7 @@ int launch_causal_tiles(const void* q, const void* k, const void* v, void* o, in
   const int smem = SM::total(p.stages);
   auto kern = attn::attn_causal_tiles_kernel;
   ATTN_ALLOW_SMEM(kern, smem);
-  kern<<<(unsigned)(BH * p.q_tiles), 512, smem, stream>>>(tq, tk, tv, to, p);
-  ATTN_CUDA_TRY(cudaGetLastError());
+  ATTN_CUDA_TRY(launch_kernel(kern, (long long)BH * p.q_tiles, 512, smem, 0, stream, tq, tk, tv, to, p));
   t_cluster_size = 0;
   t_launch_count = 1;
   launched(ATTN_KERNEL_CAUSAL_TILES, (long long)BH * p.q_tiles);
@@ -485,8 +494,7 @@ int launch_narrow(const void* q, const void* k, const void* v, void* o, int BH, 
   const int smem = SM::total(p.stages);
   auto kern = attn::attn_narrow_kernel<CAUSAL>;
   ATTN_ALLOW_SMEM(kern, smem);
-  kern<<<(unsigned)(BH * p.q_tiles), attn::kNarrowThreads, smem, stream>>>(tq, tk, tv, to, p);
-  ATTN_CUDA_TRY(cudaGetLastError());
+  ATTN_CUDA_TRY(launch_kernel(kern, (long long)BH * p.q_tiles, attn::kNarrowThreads, smem, 0, stream, tq, tk, tv, to, p));
   t_cluster_size = 0;
   t_launch_count = 1;
   launched(CAUSAL ? ATTN_KERNEL_CAUSAL_TILES : ATTN_KERNEL_NARROW_TILES, (long long)BH * p.q_tiles);
@@ -1154,7 +1162,7 @@ int gemm_launch(const void* a, const void* b, void* c, int batch, int M, int N, 
     const int tiles = batch * p.m_tiles * p.n_tiles, smem = gemm::small_smem_total(p.stages);
     auto launch_small = [&](auto kernel) -> int {
       ATTN_ALLOW_SMEM(kernel, smem);
-      kernel<<<tiles, gemm::kThreads, smem, stream>>>(ta, tb, static_cast<__nv_bfloat16*>(c), p);
+      ATTN_CUDA_TRY(launch_kernel(kernel, tiles, gemm::kThreads, smem, 0, stream, ta, tb, static_cast<__nv_bfloat16*>(c), p));
       return ATTN_OK;
     };
     rc = b_layout == 0 ? launch_small(gemm::gemm_small_kernel<true>) : launch_small(gemm::gemm_small_kernel<false>);
@@ -1196,19 +1204,7 @@ int gemm_launch(const void* a, const void* b, void* c, int batch, int M, int N, 
     const int smem = gemm::pair_smem_total(t.stages, t.tile_n);
     auto launch_pair = [&](auto kernel) -> int {
       ATTN_ALLOW_SMEM(kernel, smem);
-      cudaLaunchConfig_t cfg = {};
-      cfg.gridDim = dim3((unsigned)t.ctas);
-      cfg.blockDim = dim3(gemm::kPairThreads);
-      cfg.dynamicSmemBytes = smem;
-      cfg.stream = stream;
-      cudaLaunchAttribute attr[1];
-      attr[0].id = cudaLaunchAttributeClusterDimension;
-      attr[0].val.clusterDim.x = 2;
-      attr[0].val.clusterDim.y = 1;
-      attr[0].val.clusterDim.z = 1;
-      cfg.attrs = attr;
-      cfg.numAttrs = 1;
-      ATTN_CUDA_TRY(cudaLaunchKernelEx(&cfg, kernel, ta, tb, tc, p));
+      ATTN_CUDA_TRY(launch_kernel(kernel, t.ctas, gemm::kPairThreads, smem, 2, stream, ta, tb, tc, p));
       return ATTN_OK;
     };
     if (t.tile_n == 256) rc = (b_layout == 0) ? launch_pair(gemm::gemm_pair_kernel<true, 256>) : launch_pair(gemm::gemm_pair_kernel<false, 256>);
@@ -1217,7 +1213,7 @@ int gemm_launch(const void* a, const void* b, void* c, int batch, int M, int N, 
     const int smem = gemm::smem_total(t.stages, t.tile_n);
     auto launch = [&](auto kernel) -> int {
       ATTN_ALLOW_SMEM(kernel, smem);
-      kernel<<<t.ctas, gemm::kThreads, smem, stream>>>(ta, tb, tc, p);
+      ATTN_CUDA_TRY(launch_kernel(kernel, t.ctas, gemm::kThreads, smem, 0, stream, ta, tb, tc, p));
       return ATTN_OK;
     };
     if (t.tile_n == 256) rc = (b_layout == 0) ? launch(gemm::gemm_kernel<true, 256>) : launch(gemm::gemm_kernel<false, 256>);
@@ -1248,17 +1244,18 @@ int softmax_launch(const void* s, void* pout, long long rows, int cols, float sc
   // (65536 x 1024: 43.2 us, 8 CTAs 47.9; one CTA per row is slower at every width up to here).
   auto launch_warp = [&](auto kern, int rows_per_warp) {
     ctas = std::min((rows + 4 * rows_per_warp - 1) / (4 * rows_per_warp), 16LL * sms);
-    kern<<<(unsigned)ctas, 128, 0, stream>>>(sp, pp, rows, cols, scale_log2);
+    return launch_kernel(kern, ctas, 128, 0, 0, stream, sp, pp, rows, cols, scale_log2);
   };
   // Longer rows: a CTA per row, as few warps as hold it at VPT vectors a thread (5000 columns on 160 threads: 16.9 us for
   // 5000 rows; a kernel with 256 threads for every row of 4104 to 8192 columns took 24.6).
-  auto launch_row = [&](auto kern, int threads) { kern<<<(unsigned)rows, threads, 0, stream>>>(sp, pp, cols, scale_log2); };
-#define SOFTMAX_ROW_CASE(VPT_, THREADS_) else if (nvec <= VPT_ * THREADS_) launch_row(gemm::softmax_rows_kernel<VPT_, THREADS_>, THREADS_)
-  if (nvec <= 16) launch_warp(gemm::softmax_rows_warp_kernel<1, 16>, 2);
-  else if (nvec <= 32) launch_warp(gemm::softmax_rows_warp_kernel<1, 32>, 1);
-  else if (nvec <= 64) launch_warp(gemm::softmax_rows_warp_kernel<2, 32>, 1);
-  else if (nvec <= 96) launch_warp(gemm::softmax_rows_warp_kernel<3, 32>, 1);
-  else if (nvec <= 128) launch_warp(gemm::softmax_rows_warp_kernel<4, 32>, 1);
+  auto launch_row = [&](auto kern, int threads) { return launch_kernel(kern, rows, threads, 0, 0, stream, sp, pp, cols, scale_log2); };
+#define SOFTMAX_ROW_CASE(VPT_, THREADS_) else if (nvec <= VPT_ * THREADS_) e = launch_row(gemm::softmax_rows_kernel<VPT_, THREADS_>, THREADS_)
+  cudaError_t e = cudaSuccess;
+  if (nvec <= 16) e = launch_warp(gemm::softmax_rows_warp_kernel<1, 16>, 2);
+  else if (nvec <= 32) e = launch_warp(gemm::softmax_rows_warp_kernel<1, 32>, 1);
+  else if (nvec <= 64) e = launch_warp(gemm::softmax_rows_warp_kernel<2, 32>, 1);
+  else if (nvec <= 96) e = launch_warp(gemm::softmax_rows_warp_kernel<3, 32>, 1);
+  else if (nvec <= 128) e = launch_warp(gemm::softmax_rows_warp_kernel<4, 32>, 1);
   SOFTMAX_ROW_CASE(2, 96);
   SOFTMAX_ROW_CASE(2, 128);
   SOFTMAX_ROW_CASE(4, 96);
@@ -1275,10 +1272,10 @@ int softmax_launch(const void* s, void* pout, long long rows, int cols, float sc
     // wider than the registers of one block hold: the row is staged in shared memory (2 bytes per column)
     auto kern = gemm::softmax_rows_staged_kernel<256>;
     ATTN_ALLOW_SMEM(kern, 65536);
-    kern<<<(unsigned)rows, 256, cols * 2, stream>>>(sp, pp, cols, scale_log2);
+    e = launch_kernel(kern, rows, 256, cols * 2, 0, stream, sp, pp, cols, scale_log2);
   }
 #undef SOFTMAX_ROW_CASE
-  ATTN_CUDA_TRY(cudaGetLastError());
+  ATTN_CUDA_TRY(e);
   ++t_launch_count;
   launched(ATTN_KERNEL_SOFTMAX, ctas);
   return ATTN_OK;

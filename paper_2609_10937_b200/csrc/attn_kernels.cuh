@@ -534,6 +534,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  grid_wait();
   // every CTA's barriers must exist before a peer touches them: arrive here, wait where the first peer access is
   bool cluster_waited = false;                           // this thread has completed the wait of that barrier
   (void)cluster_waited;
@@ -1339,6 +1340,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
         if (!ok) break;
         }
     }
+      grid_release();
       if (!ok) {
         // Drain: every copy this thread started must land before the CTA may exit.
         const int first = issued > p.stages ? issued - p.stages : 0;

@@ -104,6 +104,7 @@ attn_decode_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_consta
     prefetch_tmap(&tm_v);
   }
   __syncthreads();
+  grid_wait();
 
   // this CTA's slabs of the head's keys, every fourth of them this warp's
   const int slabs = (p.Lk + kSlab - 1) / kSlab;
@@ -247,6 +248,7 @@ attn_decode_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_consta
   }
   if (it < n && lane == 0)                                      // a wait gave up
     for (int u = it; u < decode_started(it, n); ++u) drain_bar(smem_u32(&misc->full[warp][u % kDecodeStages]), (uint32_t)(u / kDecodeStages) & 1u);
+  grid_release();
   __syncthreads();                                              // the rings are dead: they hold the partial results now
 
   float* part = reinterpret_cast<float*>(smem_raw);             // [warp][row][D], then the CTA's own [row][D]

@@ -115,6 +115,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CU
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  grid_wait();
   const uint32_t tmem_base = misc->tmem_slot;
   const long long tiles = (long long)p.batch * p.m_tiles * p.n_tiles;
   const int tile_m = p.n_sub * kSub;
@@ -146,6 +147,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CU
           if (++stage == p.stages) { stage = 0; phase ^= 1u; }
         }
       }
+      grid_release();
       if (!ok) {
         // Drain: every copy this thread started must land before the CTA may exit.
         const int first = issued > p.stages ? issued - p.stages : 0;
@@ -327,6 +329,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant
   cluster_arrive();
   cluster_wait();
   tc_fence_after();
+  grid_wait();
   const uint32_t tmem_base = misc->tmem_slot;
   const long long tiles = (long long)p.batch * p.m_tiles * p.n_tiles;
   const bool run = (*abort_flag == 0);
@@ -373,6 +376,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant
           if (++stage == p.stages) { stage = 0; phase ^= 1u; }
         }
       }
+      grid_release();
       if (!ok) {
         // Drain: a copy this thread started must land before the CTA may exit.  The bytes are counted on the even
         // CTA's barrier; the odd CTA cannot poll it, so it waits out the time a copy can take instead.
@@ -540,6 +544,7 @@ gemm_small_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constan
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  grid_wait();
   const uint32_t tmem_base = misc->tmem_slot;
   const bool run = (*abort_flag == 0);
   if (warp == 0) {
@@ -564,6 +569,7 @@ gemm_small_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constan
         ++issued;
         if (++stage == p.stages) { stage = 0; phase ^= 1u; }
       }
+      grid_release();
       if (!ok) {
         // Drain: every copy this thread started must land before the CTA may exit.
         for (int t = issued > p.stages ? issued - p.stages : 0; t < issued; ++t) {
@@ -698,7 +704,9 @@ softmax_rows_warp_kernel(const __nv_bfloat16* s, __nv_bfloat16* pout, long long 
   };
   const uint64_t scale2 = pack_f32x2(scale_log2, scale_log2);
   uint4 w[VPT];
+  grid_wait();
   load(w, row);
+  grid_release();
   // (the bound is the same for a warp's lanes: its first row)
   for (long long lead = row - (threadIdx.x & 31) / LANES; lead < rows; lead += stride, row += stride) {
     uint4 next[VPT];
@@ -753,12 +761,14 @@ softmax_rows_kernel(const __nv_bfloat16* s, __nv_bfloat16* pout, int cols, float
   uint4* dst = reinterpret_cast<uint4*>(pout + row * (size_t)cols);
   const int nvec = cols / 8;
   uint4 w[VPT];
+  grid_wait();
 #pragma unroll
   for (int v = 0; v < VPT; ++v) {
     const int idx = v * THREADS + threadIdx.x;
     w[v] = make_uint4(kNegInfPair, kNegInfPair, kNegInfPair, kNegInfPair);
     if (idx < nvec) w[v] = src[idx];
   }
+  grid_release();
   uint32_t mx2 = kNegInfPair;
 #pragma unroll
   for (int v = 0; v < VPT; ++v) mx2 = max_of(w[v], mx2);
@@ -819,12 +829,14 @@ softmax_rows_staged_kernel(const __nv_bfloat16* s, __nv_bfloat16* pout, int cols
   uint4* stage = reinterpret_cast<uint4*>(smem_row);
   const int nvec = cols / 8;
   uint32_t mx2 = 0xFF80FF80u;                               // (-inf, -inf) in bf16
+  grid_wait();
 #pragma unroll 4
   for (int idx = threadIdx.x; idx < nvec; idx += THREADS) {
     const uint4 q = src[idx];
     stage[idx] = q;                                         // (each thread re-reads only what it wrote: no barrier)
     mx2 = max_bf16x2(max_bf16x2(mx2, q.x), max_bf16x2(max_bf16x2(q.y, q.z), q.w));
   }
+  grid_release();
   float m = fmaxf(__uint_as_float(mx2 << 16), __uint_as_float(mx2 & 0xFFFF0000u)) * scale_log2;
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));

@@ -142,6 +142,7 @@ attn_causal_tiles_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  grid_wait();
   const uint32_t tmem_base = misc->tmem_slot;
   const bool run = *const_cast<volatile int*>(&misc->abort.flag) == 0;
 
@@ -545,6 +546,7 @@ attn_causal_tiles_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
       if (!ok) break;
       tile = next_tile(seq, kRoleLoad);
     }
+    grid_release();
     if (tile == -2) ok = false;
     if (!ok && lane == 0) {
       // Drain: every copy started here must land before the CTA may exit, and so must an answer still on its way.

@@ -1043,3 +1043,64 @@ def test_narrow_whole_tiles_match_the_reference(env, H, Lq, Lk):
         assert float((got - ref).norm() / ref.norm()) <= 5e-3, h
     for _ in range(3):
         assert torch.equal(binding.forward_qk(q, k, v).view(torch.int16), out.view(torch.int16))
+
+
+
+def _chain(binding, x, w, few, a, b, s, p, rounds):
+    """Calls of every kind on one stream, each reading what the one before wrote and overwriting what the one before it read."""
+    L = x.shape[2]
+    for it in range(rounds):
+        binding.forward(a, a, x, b)
+        binding.forward(b, x, b, a, causal=True)
+        binding.gemm(a[0], b[0], s, b_layout="nk")
+        binding.softmax_rows(s, 0.125, p)
+        binding.gemm(p, a[0], b[0])
+        binding.forward_qk(few, b, a, few_out := few.new_empty(few.shape))
+        binding.gemm(b.view(4 * L, 64), w, a.view(4 * L, 64), b_layout="nk")
+    return few_out
+
+
+@pytest.mark.parametrize("L", [256, 1000])
+def test_calls_that_follow_one_another_wait_for_what_they_read(env, L):
+    """A kernel's CTAs may start while the one in front of it on the stream is finishing: a chain of calls in which every one
+    reads the last one's output and overwrites its input gives the bits of the same chain with a synchronisation after every
+    call -- launched one by one, and replayed from a graph."""
+    torch, _, binding = env
+    gen = torch.Generator(device="cuda").manual_seed(L)
+    x = torch.randn(1, 4, L, 64, device="cuda", generator=gen).to(torch.bfloat16)
+    w = (torch.randn(64, 64, device="cuda", generator=gen) / 2).to(torch.bfloat16)
+    few = torch.randn(1, 4, 5, 64, device="cuda", generator=gen).to(torch.bfloat16)
+
+    class Synced:                                            # the binding with a synchronisation after every call
+        def __getattr__(self, name):
+            def call(*args, **kw):
+                out = getattr(binding, name)(*args, **kw)
+                torch.cuda.synchronize()
+                return out
+            return call
+
+    def buffers():
+        return x.clone(), torch.empty_like(x), *(torch.empty(4, L, L, dtype=x.dtype, device="cuda") for _ in range(2))
+
+    want = buffers()
+    want_few = _chain(Synced(), x, w, few, *want, 20)
+    got = buffers()
+    torch.cuda.synchronize()
+    got_few = _chain(binding, x, w, few, *got, 20)
+    torch.cuda.synchronize()
+    assert binding.last_device_status()[0] == 0
+    for g, r in zip((*got, got_few), (*want, want_few)):
+        assert torch.equal(g.view(torch.int16), r.view(torch.int16))
+
+    held = buffers()
+    graph, stream = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+    stream.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.graph(graph, stream=stream):
+        held_few = _chain(binding, x, w, few, *held, 20)
+    for _ in range(3):
+        held[0].copy_(x)
+        graph.replay()
+    torch.cuda.synchronize()
+    assert binding.last_device_status()[0] == 0
+    for g, r in zip((*held, held_few), (*want, want_few)):
+        assert torch.equal(g.view(torch.int16), r.view(torch.int16))
