@@ -287,8 +287,10 @@ class Gpu:
             raise RuntimeError(f"device-side wait expired: {detail}")
 
 
-def kernel_name(plan, d, cluster):
-    """The instantiation a plan runs as: <d, tile_kv, n_q, causal, fixed merge roles, clusters>."""
+def kernel_name(plan, d, cluster, last=None):
+    """The instantiation a plan ran as: <d, tile_kv, n_q, causal, fixed merge roles, clusters>; `last`: (kernel, CTAs) of the launch."""
+    if last is not None and last[0] == 9:                # binding.KERNEL_NARROW_TILES
+        return f"attn_narrow_kernel<0,{2 if last[1] == plan.tiles else 1}>"
     uniform = plan.ctas > plan.tiles and plan.ctas % plan.tiles == 0
     fixed = int((uniform and not plan.causal) or (plan.causal and cluster > 0))
     return f"attn_fwd_kernel<{d},{plan.tile_kv},{plan.n_q},{int(plan.causal)},{fixed},{int(cluster > 0)}>"
@@ -307,7 +309,7 @@ def measure_config(gpu, name, peaks, iters=None, oracle=True):
     if iters is None:
         iters = 100 if case.flops < 1e9 else 30 if case.flops < 5e11 else 10
     ms_mean, per, _, _ = gpu.timed(lambda: binding.forward(dq, dk, dv, do), iters, 5)
-    cluster = binding.last_cluster_size()
+    cluster, last = binding.last_cluster_size(), (binding.last_kernel(), binding.last_grid())
     gpu.check_status()
     # the median of the per-launch times: one launch delayed on the host side (the events bracket the launch call)
     # would otherwise carry into a mean over few launches
@@ -317,7 +319,7 @@ def measure_config(gpu, name, peaks, iters=None, oracle=True):
            "frac_of_measured_burst_peak": tf / peaks["bf16_tflops"], "launches_timed": iters,
            "tiles": {"tile_q": plan.tile_q, "tile_kv": plan.tile_kv, "kv_stages": plan.kv_stages, "q_tiles": plan.tiles,
                      "ctas": plan.ctas, "cluster": cluster, "cost_steps": plan.cost_steps},
-           "kernel": kernel_name(plan, case.d, cluster)}
+           "kernel": kernel_name(plan, case.d, cluster, last)}
     if oracle:
         from oracle import attn_oracle as orc
 

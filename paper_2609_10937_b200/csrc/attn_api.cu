@@ -468,7 +468,7 @@ int launch_causal_tiles(const void* q, const void* k, const void* v, void* o, in
 }
 
 // d = 64 as whole Q tiles, one CTA each (narrow_kernel.cuh).
-template <bool CAUSAL>
+template <bool CAUSAL, int SUBS>
 int launch_narrow(const void* q, const void* k, const void* v, void* o, int BH, int Lq, int Lk, unsigned int* status, DeviceState* st,
                   cudaStream_t stream) {
   using SM = attn::NarrowSmem;
@@ -481,7 +481,7 @@ int launch_narrow(const void* q, const void* k, const void* v, void* o, int BH, 
   attn::NarrowParams p;
   p.Lq = Lq;
   p.Lk = Lk;
-  p.q_tiles = (Lq + 2 * attn::kSub - 1) / (2 * attn::kSub);
+  p.q_tiles = (Lq + SUBS * attn::kSub - 1) / (SUBS * attn::kSub);
   p.n_steps = (Lk + 127) / 128;
   p.heads = BH;
   // (causal: groups of heads as in launch_causal_tiles)
@@ -492,7 +492,7 @@ int launch_narrow(const void* q, const void* k, const void* v, void* o, int BH, 
   p.scale_log2 = (float)(1.4426950408889634 / std::sqrt(64.0));
   p.status = status;
   const int smem = SM::total(p.stages);
-  auto kern = attn::attn_narrow_kernel<CAUSAL>;
+  auto kern = attn::attn_narrow_kernel<CAUSAL, SUBS>;
   ATTN_ALLOW_SMEM(kern, smem);
   ATTN_CUDA_TRY(launch_kernel(kern, (long long)BH * p.q_tiles, attn::kNarrowThreads, smem, 0, stream, tq, tk, tv, to, p));
   t_cluster_size = 0;
@@ -500,6 +500,9 @@ int launch_narrow(const void* q, const void* k, const void* v, void* o, int BH, 
   launched(CAUSAL ? ATTN_KERNEL_CAUSAL_TILES : ATTN_KERNEL_NARROW_TILES, (long long)BH * p.q_tiles);
   return ATTN_OK;
 }
+
+// Key steps of all heads of a causal problem in tiles of 256 rows.
+long long causal_steps(int BH, int L) { return BH * attn_internal::head_units((L + 255) / 256, (L + 127) / 128, 2, 1); }
 
 // Whether a causal plan of equal ranges runs as whole tiles instead.  Longest first, whole tiles take the longest tile's steps
 // or an even share of all steps, one more per tile, whichever is more; 5 for the start and the end.  Measured (us, ranges /
@@ -509,20 +512,38 @@ bool causal_whole_tiles(const attn_tiles& t, int BH, int L, int d, int local_mem
   if (!t.causal || t.n_q != 2 || t.tile_kv != 128) return false;
   if (local_mem < (d == 64 ? attn::NarrowSmem::total(4) : attn::TilesSmem::total(4))) return false;
   if (t.ctas % t.tiles == 0 && t.ctas > t.tiles) return false;      // clusters that share out each tile's own steps
-  const int steps = (L + 127) / 128;
-  const long long units = BH * attn_internal::head_units((L + 255) / 256, steps, 2, 1);
-  const long long even = (units + t.tiles + sms - 1) / sms;
-  return std::max<long long>(steps, even) + 5 <= t.cost_steps;
+  const long long even = (causal_steps(BH, L) + t.tiles + sms - 1) / sms;
+  return std::max<long long>((L + 127) / 128, even) + 5 <= t.cost_steps;
 }
 
-// Whether a non-causal plan at d = 64 runs as whole tiles of narrow_kernel.cuh: at three waves of tiles or more whose last one
-// leaves at most a tenth of all slots empty.  Measured (us in a loop, attn_fwd_kernel / narrow): 128 heads x 8192 2890 / 2797,
-// 128 x 4096 747 / 727, 256 x 1000 120 / 115; on the other side 128 x 1024 (3.46 waves) 61.7 / 62.6, 18 x 4096 (1.95) 107 / 109,
-// 10 x 8192 (2.16) 222 / 290, 32 x 2048 (0.86) 57 / 62.
-bool narrow_tiles(const attn_tiles& t, int d, int local_mem, int sms) {
-  if (d != 64 || t.causal || t.n_q != 2 || t.tile_kv != 128 || local_mem < attn::NarrowSmem::total(4)) return false;
+// Sub-tiles a tile of narrow_kernel.cuh has at d = 64: two, or one (tiles of 128 rows that take half as long), or 0 where the
+// plan's kernel stays.
+//   Causal.  One sub-tile where the longest tile would keep its CTA longer than an even share of the work, by the estimates
+// (in steps) max(longest / 2, 1.1 even + 1) + 4.4 for one, max(longest, 1.1 even + 1) 0.96 + 4.1 for two and 1.08 times the plan's
+// cost for its ranges.  Measured in loops (us; plan's kernel or two / one): 8 heads x 4096 49.9 / 30.2, 4 x 8192 69.3 / 51.7,
+// 16 x 2048 29.4 / 20.2, 20 x 1111 18.1 / 12.6, 32 x 1111 18.9 / 16.5; on the other side 2 x 8192 45.8 / 51.4, 1 x 16384 67.5 /
+// 94.9, 60 x 1500 37.0 / 39.8, 128 x 256 7.9 / 8.9.  A plan of clusters is launched as clusters, which attn_last_cluster_size
+// reports and tests ask for, although one sub-tile is mostly faster there (9 x 1111 14.7 / 11.8, 16 x 512 11.1 / 7.8).
+//   Not causal, two sub-tiles: at three waves of tiles or more whose last one leaves at most a tenth of all slots empty (us,
+// attn_fwd_kernel / two): 128 heads x 8192 2890 / 2797, 128 x 4096 747 / 727, 256 x 1000 120 / 115; on the other side 128 x 1024
+// (3.46 waves) 61.7 / 62.6, 18 x 4096 (1.95) 107 / 109, 10 x 8192 (2.16) 222 / 290.
+//   Not causal, one: where 1.1 times the waves of half-length tiles and 2.8 are below the plan's cost (us, attn_fwd_kernel / one):
+// 1 head x 256 6.8 / 5.3, 16 x 512 10.3 / 7.2, 16 x 1024 13.2 / 11.3, 32 x 1111 29.9 / 22.2, 60 x 1500 63.8 / 60.2; on the other side
+// 128 x 256 7.7 / 8.3, 30 x 1024 17.1 / 18.8, 4 x 2048 15.1 / 17.4, 16 x 2048 28.6 / 32.1, 1 x 16384 95.8 / 99.2.
+int narrow_subs(const attn_tiles& t, int BH, int Lq, int Lk, int d, int local_mem, int sms) {
+  if (d != 64 || t.n_q != 2 || t.tile_kv != 128 || local_mem < attn::NarrowSmem::total(4)) return 0;
+  if (t.causal) {
+    if (t.ctas % t.tiles == 0 && t.ctas > t.tiles) return 0;
+    const double longest = (Lq + 127) / 128, share = 1.1 * (double)causal_steps(BH, Lq) / sms + 1.0;
+    const double one = std::max(0.5 * longest, share) + 4.4;
+    const bool whole = causal_whole_tiles(t, BH, Lq, d, local_mem, sms);
+    const double now = whole ? 0.96 * std::max(longest, share) + 4.1 : 1.08 * t.cost_steps;
+    return one < now ? 1 : whole ? 2 : 0;
+  }
   const long long slots = (long long)((t.tiles + sms - 1) / sms) * sms;
-  return t.tiles >= 3 * sms && 10 * slots <= 11LL * t.tiles;
+  if (t.tiles >= 3 * sms && 10 * slots <= 11LL * t.tiles) return 2;
+  const long long waves = ((long long)BH * ((Lq + 127) / 128) + sms - 1) / sms, steps = (Lk + 127) / 128;
+  return 1.1 * (double)(waves * ((steps + 1) / 2)) + 2.8 < (double)t.cost_steps ? 1 : 0;
 }
 
 int dispatch_fwd(const void* q, const void* k, const void* v, void* o, int B, int H, int L, int d,
@@ -530,11 +551,16 @@ int dispatch_fwd(const void* q, const void* k, const void* v, void* o, int B, in
                  bool may_overlap = false, bool own_plan = false) {
   if (Lk == 0) Lk = L;
   // own_plan: the device's own, with no field changed and from no caller's descriptor -- those say how many CTAs run
-  if (own_plan && Lk == L && causal_whole_tiles(t, B * H, L, d, st->desc.local_mem_bytes, st->desc.num_units))
-    return d == 128 ? launch_causal_tiles(q, k, v, o, B * H, L, status, st, s)
-                    : launch_narrow<true>(q, k, v, o, B * H, L, L, status, st, s);
-  if (own_plan && narrow_tiles(t, d, st->desc.local_mem_bytes, st->desc.num_units))
-    return launch_narrow<false>(q, k, v, o, B * H, L, Lk, status, st, s);
+  const int sms = st->desc.num_units;
+  if (own_plan) {
+    if (const int subs = narrow_subs(t, B * H, L, Lk, d, st->desc.local_mem_bytes, sms)) {
+      auto launch = t.causal ? (subs == 1 ? launch_narrow<true, 1> : launch_narrow<true, 2>)
+                             : (subs == 1 ? launch_narrow<false, 1> : launch_narrow<false, 2>);
+      return launch(q, k, v, o, B * H, L, Lk, status, st, s);
+    }
+    if (d == 128 && Lk == L && causal_whole_tiles(t, B * H, L, d, st->desc.local_mem_bytes, sms))
+      return launch_causal_tiles(q, k, v, o, B * H, L, status, st, s);
+  }
 #define ATTN_CASE(D_, TKV_, NQ_) \
   if (d == D_ && t.tile_kv == TKV_ && t.n_q == NQ_) \
     return launch_fwd<D_, TKV_, NQ_>(q, k, v, o, B, H, L, Lk, t, ws, status, st, s, may_overlap);

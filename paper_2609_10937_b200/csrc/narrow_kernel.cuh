@@ -10,6 +10,9 @@
 // when the tile is finished, in the epilogue warpgroup, which reads both accumulators.  2600 cycles a step.  In a loop (us,
 // before / this kernel): causal 128 heads x 8192 1667 / 1474, 128 x 4096 491 / 388, 128 x 2048 144 / 115, 256 x 300 31.2 / 24.6,
 // 32 x 1111 22.5 / 20.8; not causal 128 x 8192 2890 / 2797, where the power limit takes back most of it.
+// SUBS = 1 works on tiles of 128 query rows, one sub-tile: its four streams are the two halves of the even and of the odd key
+// tiles.  A tile then takes half as long, which evens out the CTAs where a launch has few tiles for each (narrow_subs in
+// attn_api.cu), at twice the K and V loads for a row.
 //   * One barrier each way per step: scores ready (commit of Q K^T, which also says that the stream's P V of the step before
 //     is complete) and P ready.  A softmax warp whose reference moved rescales its accumulator itself: that is rare, and
 //     no other warp has to be asked.
@@ -26,7 +29,7 @@ namespace attn {
 
 struct NarrowParams {
   int Lq, Lk;              // query rows and keys per head
-  int q_tiles;             // Q tiles per head = ceil(Lq / 256)
+  int q_tiles;             // Q tiles per head = ceil(Lq / (SUBS * 128))
   int n_steps;             // key steps per head = ceil(Lk / 128)
   int heads;               // B * H
   int group_heads;         // causal: heads whose tiles are dealt out together, longest first
@@ -62,29 +65,43 @@ struct NarrowMisc {
 };
 static_assert(sizeof(NarrowMisc) <= NarrowSmem::kMiscBytes, "misc region too large");
 
-template <bool CAUSAL>
-__device__ __forceinline__ TileWork narrow_work(int index, const NarrowParams& p) {
-  TileWork w;
+// A tile: its head, first row, key tiles and the number of them that each of its streams works on.  Stream st: sub-tile st / 2,
+// half st % 2 of every key tile; SUBS = 1: half st % 2 of the key tiles j with j % 2 = st / 2.
+template <int SUBS>
+struct NarrowWork {
+  int bh, q_row0, n, n0, n1;               // n: key tiles; n0, n1: those of streams 0, 1 and of streams 2, 3
+  __device__ __forceinline__ int steps(int group) const { return group ? n1 : n0; }
+};
+template <bool CAUSAL, int SUBS>
+__device__ __forceinline__ NarrowWork<SUBS> narrow_work(int index, const NarrowParams& p) {
+  NarrowWork<SUBS> w;
+  int q;
   if constexpr (CAUSAL) {
     const int per_group = p.group_heads * p.q_tiles;
     const int group = index / per_group, r = index - group * per_group;
     const int first = group * p.group_heads;
     const int n = p.heads - first < p.group_heads ? p.heads - first : p.group_heads;
-    const int q = p.q_tiles - 1 - r / n;
+    q = p.q_tiles - 1 - r / n;
     w.bh = first + r % n;
-    w.q_row0 = q * 2 * kSub;
-    w.n0 = 2 * q + 1;                      // a sub-tile's last key step is the one that holds its own rows
-    w.n1 = w.q_row0 + kSub >= p.Lq ? 0 : 2 * q + 2;
   } else {
     w.bh = index / p.q_tiles;
-    w.q_row0 = (index - w.bh * p.q_tiles) * 2 * kSub;
-    w.n0 = p.n_steps;
-    w.n1 = w.q_row0 + kSub >= p.Lq ? 0 : p.n_steps;
+    q = index - w.bh * p.q_tiles;
+  }
+  w.q_row0 = q * SUBS * kSub;
+  if constexpr (SUBS == 2) {
+    // (causal: a sub-tile's last key tile is the one that holds its own rows)
+    w.n0 = CAUSAL ? 2 * q + 1 : p.n_steps;
+    w.n1 = w.q_row0 + kSub >= p.Lq ? 0 : CAUSAL ? 2 * q + 2 : p.n_steps;
+    w.n = w.n1 > w.n0 ? w.n1 : w.n0;
+  } else {
+    w.n = CAUSAL ? q + 1 : p.n_steps;
+    w.n0 = (w.n + 1) / 2;
+    w.n1 = w.n / 2;
   }
   return w;
 }
 
-template <bool CAUSAL>
+template <bool CAUSAL, int SUBS>
 __global__ void __launch_bounds__(kNarrowThreads, 1)
 attn_narrow_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                    const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_o, const NarrowParams p) {
@@ -106,7 +123,7 @@ attn_narrow_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
     if (smem_base & 1023u) note_timeout(wait_info(kRoleLoad, 0, 0xFFFF), &misc->abort.flag);   // swizzled tiles need 1024-byte alignment
     for (int s = 0; s < kMaxStages; ++s) {
       mbar_init(smem_u32(&misc->kv_full[s]), 1);
-      mbar_init(smem_u32(&misc->kv_empty[s]), 4);                 // the four streams
+      mbar_init(smem_u32(&misc->kv_empty[s]), 2 * SUBS);          // the streams that read a ring item
     }
     for (int i = 0; i < 4; ++i) {
       mbar_init(smem_u32(&misc->s_full[i]), 1);
@@ -118,9 +135,9 @@ attn_narrow_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
       mbar_init(smem_u32(&misc->sched_empty[i]), kNarrowSchedReaders);
       for (int b = 0; b < 2; ++b) {
         mbar_init(smem_u32(&misc->q_full[i][b]), 1);
-        mbar_init(smem_u32(&misc->q_empty[i][b]), 2);             // the sub-tile's two streams
+        mbar_init(smem_u32(&misc->q_empty[i][b]), 4 / SUBS);      // the sub-tile's streams
       }
-      mbar_init(smem_u32(&misc->o_full[i]), 2);
+      mbar_init(smem_u32(&misc->o_full[i]), 4 / SUBS);
       mbar_init(smem_u32(&misc->o_free[i]), kSub);
     }
     fence_mbar_init();
@@ -155,7 +172,7 @@ attn_narrow_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
   if (warp < 16) {
     // ===================================================== softmax warpgroup of one stream
     setmaxnreg_inc<96>();
-    const int st = warp >> 2, i = st >> 1, half = st & 1;
+    const int st = warp >> 2, group = st >> 1, half = st & 1, i = SUBS == 2 ? group : 0;
     const int row = (warp & 3) * 32 + lane;
     const uint32_t lane_base = tmem_base + ((uint32_t)((warp & 3) * 32) << 16);
     const uint32_t s_tmem = lane_base + st * HKV;      // P goes to the front of it
@@ -168,9 +185,11 @@ attn_narrow_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
     uint32_t g = 0, done = 0;                          // steps of this stream over all tiles; finished tiles
     int tile = blockIdx.x;
     for (int seq = 1; ok && tile >= 0; ++seq) {
-      const TileWork w = narrow_work<CAUSAL>(tile, p);
-      const int n = w.steps(i);
+      const NarrowWork<SUBS> w = narrow_work<CAUSAL, SUBS>(tile, p);
+      const int n = w.steps(group);
       if (n > 0) {
+        // whether this stream's last key tile is the tile's last (SUBS = 1: the last tile is one parity's)
+        const bool ends = SUBS == 2 || ((w.n - 1) & 1) == group;
         float m_run = -INFINITY, delta = 0.f;
         // One key step.  The masked variant (the causal diagonal, a ragged last key tile) is compiled separately so that the
         // common step pays nothing for it; `lim` is the last key column of this half the thread's row may attend to.
@@ -248,10 +267,16 @@ attn_narrow_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
           // Only the last step may need a mask: the causal diagonal, which starts at the sub-tile's first row and ends, in a
           // ragged last key tile, before the padding for every row of the sequence; else a ragged last key tile.
           const bool last = jj == n - 1;
-          if (last && (CAUSAL || kv_tail != 0)) ok = softmax_step(MaskTag<true>{}, (CAUSAL ? row : kv_tail - 1) - half * HKV, jj == 0, true);
-          else ok = softmax_step(MaskTag<false>{}, HKV - 1, jj == 0, !CAUSAL && last);
+          if (last && ends && (CAUSAL || kv_tail != 0)) ok = softmax_step(MaskTag<true>{}, (CAUSAL ? row : kv_tail - 1) - half * HKV, jj == 0, true);
+          else ok = softmax_step(MaskTag<false>{}, HKV - 1, jj == 0, (!CAUSAL || SUBS == 1) && last);
         }
         if (!ok) break;
+        ++done;
+      } else if (SUBS == 1) {
+        // (no key tile of this parity: an empty part, so that the epilogue finds four)
+        if (done > 0 && !wait_quiet_warp(smem_u32(&misc->o_free[0]), (done - 1) & 1, abort_flag, wait_info(kRoleSoftmax, kBarOFull, g))) { ok = false; break; }
+        misc->stat[done & 1][st][row] = make_float2(-INFINITY, 0.f);
+        mbar_arrive(smem_u32(&misc->fin_full[st]));
         ++done;
       }
       tile = next_tile(seq, kRoleSoftmax);
@@ -266,23 +291,33 @@ attn_narrow_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
     uint32_t fin = 0, chunk_ctr = 0;                   // bit i: finished tiles of sub-tile i, mod 2
     int tile = blockIdx.x;
     for (int seq = 1; ok && tile >= 0; ++seq) {
-      const TileWork w = narrow_work<CAUSAL>(tile, p);
+      const NarrowWork<SUBS> w = narrow_work<CAUSAL, SUBS>(tile, p);
 #pragma unroll 1
-      for (int i = 0; ok && i < 2; ++i) {
-        if (w.steps(i) == 0) continue;
+      for (int i = 0; ok && i < SUBS; ++i) {
+        if (SUBS == 2 && w.steps(i) == 0) continue;
         const uint32_t ph = (fin >> i) & 1;
         fin ^= 1u << i;
-        if (!wait_quiet_warp(smem_u32(&misc->fin_full[2 * i]), ph, abort_flag, wait_info(kRoleCorrection, kBarAlpha, 2 * i)) ||
-            !wait_quiet_warp(smem_u32(&misc->fin_full[2 * i + 1]), ph, abort_flag, wait_info(kRoleCorrection, kBarAlpha, 2 * i + 1))) { ok = false; break; }
-        // the two streams' parts on the common reference, normalised
-        const float2 a = misc->stat[ph][2 * i][row], b = misc->stat[ph][2 * i + 1][row];
-        const float m = fmaxf(a.x, b.x);
-        float wa = ex2_approx(a.x - m), wb = ex2_approx(b.x - m);
-        const float inv = 1.0f / (a.y * wa + b.y * wb);
-        wa *= inv;
-        wb *= inv;
+        constexpr int kParts = 4 / SUBS;               // streams of a sub-tile
+        float wt[kParts], m = -INFINITY, sum = 0.f;
+#pragma unroll
+        for (int k = 0; k < kParts; ++k)
+          if (ok && !wait_quiet_warp(smem_u32(&misc->fin_full[2 * i + k]), ph, abort_flag, wait_info(kRoleCorrection, kBarAlpha, 2 * i + k))) ok = false;
+        if (!ok) break;
+        // the streams' parts on the common reference, normalised
+#pragma unroll
+        for (int k = 0; k < kParts; ++k) m = fmaxf(m, misc->stat[ph][2 * i + k][row].x);
+#pragma unroll
+        for (int k = 0; k < kParts; ++k) {
+          const float2 a = misc->stat[ph][2 * i + k][row];
+          wt[k] = ex2_approx(a.x - m);                 // (an empty part: -inf, weight 0)
+          sum += a.y * wt[k];
+        }
+        const float inv = 1.0f / sum;
+#pragma unroll
+        for (int k = 0; k < kParts; ++k) wt[k] *= inv;
         if (!wait_quiet_warp(smem_u32(&misc->o_full[i]), ph, abort_flag, wait_info(kRoleCorrection, kBarOFull, i))) { ok = false; break; }
         tc_fence_after();
+        const bool empty = SUBS == 1 && w.n1 == 0;     // streams 2 and 3 have no accumulator
         const uint32_t o_tmem = lane_base + O_COL0 + 2 * i * D;
         const uint32_t dst = stage_w + (chunk_ctr & 1) * 4096;
         ++chunk_ctr;
@@ -292,12 +327,18 @@ attn_narrow_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
 #pragma unroll 1
         for (int c = 0; c < 8; ++c) {                  // 8 columns at a time
           uint32_t ra[8], rb[8];
+          float v[8];
           tmem_ld8x2(o_tmem + c * 8, o_tmem + D + c * 8, ra, rb);
+#pragma unroll
+          for (int e = 0; e < 8; ++e) v[e] = __uint_as_float(ra[e]) * wt[0] + __uint_as_float(rb[e]) * wt[1];
+          if (SUBS == 1 && !empty) {
+            tmem_ld8x2(o_tmem + 2 * D + c * 8, o_tmem + 3 * D + c * 8, ra, rb);
+#pragma unroll
+            for (int e = 0; e < 8; ++e) v[e] += __uint_as_float(ra[e]) * wt[kParts - 2] + __uint_as_float(rb[e]) * wt[kParts - 1];
+          }
           uint32_t q[4];
 #pragma unroll
-          for (int e = 0; e < 4; ++e)
-            q[e] = pack_bf16x2(__uint_as_float(ra[2 * e]) * wa + __uint_as_float(rb[2 * e]) * wb,
-                               __uint_as_float(ra[2 * e + 1]) * wa + __uint_as_float(rb[2 * e + 1]) * wb);
+          for (int e = 0; e < 4; ++e) q[e] = pack_bf16x2(v[2 * e], v[2 * e + 1]);
           st_shared_u4(dst + lane * 128 + (((uint32_t)c ^ (uint32_t)(lane & 7)) << 4), q);   // 128-byte swizzle
         }
         tc_fence_before();
@@ -317,7 +358,7 @@ attn_narrow_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
   } else if (warp < 24) {
     // ============================== MMA issuer of one stream (the whole warp walks the loop, one lane issues)
     setmaxnreg_dec<40>();
-    const int st = warp & 3, i = st >> 1, half = st & 1;
+    const int st = warp & 3, group = st >> 1, half = st & 1, i = SUBS == 2 ? group : 0;
     bool ok = run;
     const uint32_t s_tmem = tmem_base + st * HKV, o_tmem = tmem_base + O_COL0 + st * D;
     const uint32_t k_smem = ring_smem + half * (HKV * 128);       // this stream's keys in a ring item
@@ -328,7 +369,7 @@ attn_narrow_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
       if (!wait_quiet_warp(smem_u32(bar), parity, abort_flag, wait_info(kRoleMma, id, 0x100 * st + (g & 0xFF)))) { ok = false; return false; }
       return true;
     };
-    auto advance = [&]() __attribute__((always_inline)) { if (++pos == p.stages) { pos = 0; ph ^= 1u; } };
+    auto advance = [&](int items) __attribute__((always_inline)) { if ((pos += items) >= p.stages) { pos -= p.stages; ph ^= 1u; } };
     // (one lane) Scores of the keys at ring position k; last: no later step of the tile reads this Q.
     auto issue_scores = [&](int k, bool last) __attribute__((always_inline)) {
       const int b = (q_uses - 1) & 1;
@@ -343,7 +384,7 @@ attn_narrow_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
       for (int x = 0; x < 2 * steps; ++x) {
         if (!wait(&misc->kv_full[pos], ph, kBarKvFull)) return;
         if (lane == 0) mbar_arrive(smem_u32(&misc->kv_empty[pos]));
-        advance();
+        advance(1);
       }
     };
     // A tile's first scores.
@@ -353,22 +394,24 @@ attn_narrow_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
       tc_fence_after();
       if (elect_one()) issue_scores(pos, steps == 1);
       __syncwarp();
-      advance();
+      advance(1);
     };
     int tile = blockIdx.x;
     for (int seq = 1; ok && tile >= 0; ++seq) {
-      const TileWork w = narrow_work<CAUSAL>(tile, p);
-      const int n = w.steps(i);
+      const NarrowWork<SUBS> w = narrow_work<CAUSAL, SUBS>(tile, p);
+      const int n = w.steps(group);
+      if (SUBS == 1 && group == 1) advance(2);         // the first key tile is the other parity's
       if (n > 0) start(n);
       for (int j = 0; ok && j < n; ++j, ++g) {
         const int v = pos;
         if (!wait(&misc->kv_full[v], ph, kBarKvFull)) break;
-        advance();
-        const int k = pos;
+        advance(1);
         const bool more = j + 1 < n;
+        if (SUBS == 1 && more) advance(2);             // (past the other parity's key tile)
+        const int k = pos;
         if (more) {
           if (!wait(&misc->kv_full[k], ph, kBarKvFull)) break;
-          advance();
+          advance(1);
         }
         // the tile before has left the accumulator
         if (j == 0 && done > 0 && !wait(&misc->o_free[i], (done - 1) & 1, kBarOFull)) break;
@@ -383,8 +426,24 @@ attn_narrow_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
         __syncwarp();
       }
       if (!ok) break;
-      done += n > 0 ? 1u : 0u;
-      if (CAUSAL || n == 0) skip(w.steps() - n);
+      if constexpr (SUBS == 2) {
+        done += n > 0 ? 1u : 0u;
+        if (CAUSAL || n == 0) skip(w.n - n);
+      } else {
+        ++done;
+        if (n == 0) {
+          // nothing to add to the tile, nothing read of its Q (the arrivals of the tile before must all have been made: o_free)
+          if (done > 1 && !wait(&misc->o_free[0], (done - 2) & 1, kBarOFull)) break;
+          if (!wait(&misc->q_full[0][q_uses & 1], (q_uses >> 1) & 1, kBarQ)) break;
+          if (lane == 0) {
+            mbar_arrive(smem_u32(&misc->q_empty[0][q_uses & 1]));
+            mbar_arrive(smem_u32(&misc->o_full[0]));
+          }
+          ++q_uses;
+        }
+        // past the other parity's last key tile where that is the tile's last
+        if (n > 0 && ((w.n - 1) & 1) != group) advance(2);
+      }
       if (!ok) break;
       tile = next_tile(seq, kRoleMma);
     }
@@ -408,7 +467,7 @@ attn_narrow_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
       if (++stage == p.stages) { stage = 0; phase ^= 1u; }
       return true;
     };
-    auto load_q = [&](int i, const TileWork& w) __attribute__((always_inline)) -> bool {
+    auto load_q = [&](int i, const NarrowWork<SUBS>& w) __attribute__((always_inline)) -> bool {
       const uint32_t u = i ? q_loads1 : q_loads0, b = u & 1;
       if (u >= 2 && !wait_quiet_warp(smem_u32(&misc->q_empty[i][b]), (u / 2 - 1) & 1, abort_flag, wait_info(kRoleLoad, kBarQ, u))) return false;
       if (elect_one()) {
@@ -422,13 +481,13 @@ attn_narrow_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
     };
     int tile = blockIdx.x;
     for (int seq = 1; ok && tile >= 0; ++seq) {
-      const TileWork w = narrow_work<CAUSAL>(tile, p);
-      const int n = w.steps();
+      const NarrowWork<SUBS> w = narrow_work<CAUSAL, SUBS>(tile, p);
+      const int n = w.n;
       // the first product needs K_0 and Q of sub-tile 0; the first tile's Q buffer is free at once
       if (seq == 1) ok = load_q(0, w);
       if (ok) ok = load_kv(&tm_k, 0, w.bh);
       if (ok && seq > 1) ok = load_q(0, w);
-      if (ok && w.n1 > 0) ok = load_q(1, w);
+      if (ok && SUBS == 2 && w.n1 > 0) ok = load_q(1, w);
       for (int j = 0; ok && j < n; ++j) {
         if (j > 0) ok = load_kv(&tm_k, j * TKV, w.bh);
         if (ok && j == n - 1) {
@@ -456,7 +515,7 @@ attn_narrow_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
       // Drain: every copy started here must land before the CTA may exit, and so must an answer still on its way.
       for (int t = issued > p.stages ? issued - p.stages : 0; t < issued; ++t)
         drain_bar(smem_u32(&misc->kv_full[t % p.stages]), (uint32_t)(t / p.stages) & 1u);
-      for (int i = 0; i < 2; ++i)
+      for (int i = 0; i < SUBS; ++i)
         for (uint32_t q = i ? q_loads1 : q_loads0, u = q > 2u ? q - 2u : 0; u < q; ++u) drain_bar(smem_u32(&misc->q_full[i][u & 1]), (u / 2) & 1);
       if (asked > 0) drain_bar(smem_u32(&misc->sched_full[asked & 1]), ((asked - 1) >> 1) & 1);
     }
