@@ -97,7 +97,6 @@ attn_causal_tiles_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
                   const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_o, const TilesParams p) {
   constexpr int D = 128, TKV = 128, NCH = TKV / 32, KCH = D / 64;
   constexpr int O_COL0 = 2 * TKV;
-  constexpr int kPoly = kPolyPairsPer8;
   using SM = TilesSmem;
 
   extern __shared__ __align__(1024) uint8_t smem_raw[];
@@ -184,6 +183,12 @@ attn_causal_tiles_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
         // the common step pays nothing for it; `lim` is the last key column the thread's row may attend to.
         auto softmax_step = [&](auto mask_tag, int lim) __attribute__((always_inline)) -> bool {
           constexpr bool kMasked = decltype(mask_tag)::value;
+          // The common step takes no exponential by polynomial (attn_fwd_kernel takes two pairs of eight): a pair costs 14 more
+          // issue slots than on the exponential unit, which is not what bounds this kernel.  In loops, two pairs / none (us): 128
+          // heads x 4096 580 / 566, 256 x 2048 355 / 340, 64 x 2048 94.1 / 88.5, 200 x 1000 91.9 / 87.9, 16 x 8192 267 / 269.  (Not
+          // causal, 128 x 4096 in attn_fwd_kernel: 977 / 1005.)  The diagonal, one step of a tile, keeps them, and with them the
+          // bits of the rows that see only a few keys.
+          constexpr int kPoly = kMasked ? kPolyPairsPer8 : 0;
           if (!wait_quiet_warp(bar_s, g & 1, abort_flag, wait_info(kRoleSoftmax, kBarSFull, g))) return false;
           tc_fence_after();
           uint32_t s[TKV];
