@@ -25,6 +25,24 @@
 extern "C" {
 #endif
 
+/* gemm_forward and softmax_rows_forward with the arguments in memory, as attn_forward_call. */
+typedef struct gemm_call {
+  const void *a, *b;
+  void *c;
+  void *cuda_stream;
+  int32_t batch, M, N, K, b_layout;
+} gemm_call;
+typedef struct softmax_call {
+  const void *s;
+  void *p;
+  void *cuda_stream;
+  int64_t rows;
+  int32_t cols;
+  double scale;         /* rounded to float, as a float argument would be */
+} softmax_call;
+int gemm_forward_call(const gemm_call *call);
+int softmax_rows_forward_call(const softmax_call *call);
+
 /* Result of the closed-form tile derivation for the matrix product. */
 typedef struct gemm_tiles {
   int32_t tile_m;       /* rows of C per CTA = n_sub * atom_m                                   */

@@ -9,6 +9,7 @@ from __future__ import annotations
 
 import ctypes
 import math
+import struct
 from pathlib import Path
 
 _PKG = Path(__file__).resolve().parent
@@ -24,11 +25,13 @@ BIND_NAMES = ("none", "smem", "tmem", "reg", "atom", "shape")
 
 EXPORTED_SYMBOLS = (
     "attn_hw_desc_b200", "attn_hw_desc_query", "attn_plan", "attn_plan_ex", "attn_workspace_bytes",
-    "attn_set_workspace", "attn_workspace_init", "attn_forward_ws", "attn_status_read", "attn_forward", "attn_forward_causal", "attn_forward_tiles", "attn_forward_simple", "attn_forward_host", "attn_forward_host_workspace_bytes", "attn_forward_static_scratch", "attn_forward_desc", "attn_plan_qk", "attn_forward_qk",
+    "attn_set_workspace", "attn_workspace_init", "attn_forward_ws", "attn_status_read", "attn_forward", "attn_forward_causal", "attn_forward_tiles", "attn_forward_simple", "attn_forward_host", "attn_forward_host_workspace_bytes", "attn_forward_static_scratch", "attn_forward_desc", "attn_plan_qk", "attn_forward_qk", "attn_forward_call",
     "attn_last_device_status", "attn_selftest_wait_expiry", "attn_selftest_wait_expiry_to", "attn_selftest_quiet_expiry_to",
     "attn_last_launch_count", "attn_last_cluster_size", "attn_last_kernel", "attn_last_grid", "attn_status_string", "attn_last_cuda_error",
-    "gemm_plan", "gemm_forward", "gemm_forward_tiles", "softmax_rows_forward", "attn_forward_unfused",
+    "gemm_plan", "gemm_forward", "gemm_forward_tiles", "softmax_rows_forward", "attn_forward_unfused", "gemm_forward_call", "softmax_rows_forward_call",
 )
+# attn_call, gemm_call, softmax_call (native alignment; the trailing 0q pads to the struct's size)
+_ATTN_CALL, _GEMM_CALL, _SOFTMAX_CALL = (struct.Struct(f).pack for f in ("@5P6i0q", "@4P5i0q", "@3Pqid"))
 
 
 class AttnHwDesc(ctypes.Structure):
@@ -75,6 +78,19 @@ class AttnError(RuntimeError):
 _lib = None
 
 
+class _LazyTorch:
+    """torch, imported with the first use; every call used to pay 0.2 us for each of its three import statements."""
+
+    def __getattr__(self, name):
+        global _torch
+        import torch as _torch
+
+        return getattr(_torch, name)
+
+
+_torch = _LazyTorch()
+
+
 def lib() -> ctypes.CDLL:
     """The loaded shared library; raises if it has not been built."""
     global _lib
@@ -98,6 +114,7 @@ def lib() -> ctypes.CDLL:
         L.attn_forward_ws.argtypes = [vp, vp, vp, vp, i32, i32, i32, i32, i32, vp, ctypes.c_size_t, vp, vp]
         L.attn_status_read.argtypes = [vp, vp, vp, ctypes.POINTER(ctypes.c_uint32)]
         L.attn_plan_qk.argtypes = [ctypes.POINTER(AttnHwDesc), i32, i32, i32, i32, i32, ctypes.POINTER(AttnTiles)]
+        L.attn_forward_call.argtypes = L.gemm_forward_call.argtypes = L.softmax_rows_forward_call.argtypes = [ctypes.c_char_p]
         L.attn_forward_qk.argtypes = [vp, vp, vp, vp, i32, i32, i32, i32, i32, vp]
         L.attn_forward_tiles.argtypes = [vp, vp, vp, vp, i32, i32, i32, i32, ctypes.POINTER(AttnTiles), vp]
         L.attn_forward_simple.argtypes = [vp, vp, vp, vp, i32, i32, i32, i32, i32, vp, vp]
@@ -193,10 +210,8 @@ def ensure_workspace(device_index: int, nbytes: int) -> None:
 def _call(dev, where, fn, *args, workspace=None):
     """One library call with device `dev` current.  `workspace()` gives the bytes that the call's plan asks for; it is
     asked only when the library says that what is registered is too small, so that the usual call derives its plan once."""
-    import torch
-
-    if torch.cuda.current_device() != dev:
-        with torch.cuda.device(dev):
+    if _torch._C._cuda_getDevice() != dev:               # (a tensor on a device is in hand: CUDA is initialised)
+        with _torch.cuda.device(dev):
             return _call(dev, where, fn, *args, workspace=workspace)
     rc = fn(*args)
     if rc == ERR_NEED_WORKSPACE and workspace is not None:
@@ -208,14 +223,11 @@ def _call(dev, where, fn, *args, workspace=None):
 
 def _stream(dev: int) -> int:
     """Handle of the current stream of a device."""
-    import torch
-
-    return torch._C._cuda_getCurrentRawStream(dev)
+    return _torch._C._cuda_getCurrentRawStream(dev)
 
 
 def _prep(q, k, v, o):
-    import torch
-
+    torch = _torch
     bf16 = torch.bfloat16
     if q.dtype != bf16 or k.dtype != bf16 or v.dtype != bf16:
         raise TypeError("q, k, v must be torch.bfloat16")
@@ -240,8 +252,8 @@ def forward(q, k, v, o=None, causal=False):
 
     causal=True: row i attends to keys 0..i only."""
     o, B, H, L, d, dev, stream = _prep(q, k, v, o)
-    fn, where = (lib().attn_forward_causal, "attn_forward_causal") if causal else (lib().attn_forward, "attn_forward")
-    _call(dev, where, fn, q.data_ptr(), k.data_ptr(), v.data_ptr(), o.data_ptr(), B, H, L, d, stream,
+    _call(dev, "attn_forward_causal" if causal else "attn_forward", lib().attn_forward_call,
+          _ATTN_CALL(q.data_ptr(), k.data_ptr(), v.data_ptr(), o.data_ptr(), stream, B, H, L, L, d, 1 if causal else 0),
           workspace=lambda: workspace_bytes(plan(_device_desc(dev), B, H, L, d, causal), B, H, L, d))
     return o
 
@@ -322,8 +334,7 @@ def plan_qk(desc: AttnHwDesc, B: int, H: int, Lq: int, Lk: int, d: int) -> AttnT
 
 def forward_qk(q, k, v, o=None):
     """O = softmax(Q K^T / sqrt(d)) V for q [B, H, Lq, d] and k, v [B, H, Lk, d] (contiguous CUDA bf16)."""
-    import torch
-
+    torch = _torch
     for name, x in (("q", q), ("k", k), ("v", v)):
         if x.dtype != torch.bfloat16 or not x.is_cuda or not x.is_contiguous() or x.dim() != 4:
             raise ValueError(f"{name} must be a contiguous CUDA bfloat16 tensor [B, H, L, d]")
@@ -334,8 +345,8 @@ def forward_qk(q, k, v, o=None):
     if o is None:
         o = torch.empty_like(q)
     dev = q.get_device()
-    _call(dev, "attn_forward_qk", lib().attn_forward_qk, q.data_ptr(), k.data_ptr(), v.data_ptr(), o.data_ptr(),
-          B, H, Lq, Lk, d, _stream(dev),
+    _call(dev, "attn_forward_qk", lib().attn_forward_call,
+          _ATTN_CALL(q.data_ptr(), k.data_ptr(), v.data_ptr(), o.data_ptr(), _stream(dev), B, H, Lq, Lk, d, 0),
           workspace=lambda: workspace_bytes(plan_qk(_device_desc(dev), B, H, Lq, Lk, d), B, H, Lq, d))
     return o
 
@@ -441,8 +452,7 @@ def gemm_plan(desc: AttnHwDesc, batch: int, M: int, N: int, K: int) -> GemmTiles
 
 def _mat(x, name):
     """(batch, rows, columns) of a matrix operand."""
-    import torch
-
+    torch = _torch
     if x.dtype != torch.bfloat16 or not x.is_cuda or not x.is_contiguous() or x.dim() not in (2, 3):
         raise ValueError(f"{name} must be a contiguous CUDA bfloat16 tensor of 2 or 3 dimensions")
     return x.shape if x.dim() == 3 else (1, *x.shape)
@@ -453,8 +463,7 @@ def gemm(a, b, c=None, *, b_layout="kn", cta_pair=0, tile_n=0, tail_split=0):
 
     cta_pair (1 | 2), tile_n (128 | 256) and tail_split (-1: whole tiles in the last wave) override the closed-form
     tiles (tile sweep only; 0 keeps them)."""
-    import torch
-
+    torch = _torch
     batch, M, K = _mat(a, "a")
     b_batch, rows, cols = _mat(b, "b")
     if b_layout == "kn":
@@ -477,15 +486,14 @@ def gemm(a, b, c=None, *, b_layout="kn", cta_pair=0, tile_n=0, tail_split=0):
         _call(dev, "gemm_forward_tiles", lib().gemm_forward_tiles, a.data_ptr(), b.data_ptr(), c.data_ptr(), batch, M, N, K,
               layout, ctypes.byref(ov), _stream(dev))
     else:
-        _call(dev, "gemm_forward", lib().gemm_forward, a.data_ptr(), b.data_ptr(), c.data_ptr(), batch, M, N, K, layout,
-              _stream(dev))
+        _call(dev, "gemm_forward", lib().gemm_forward_call,
+              _GEMM_CALL(a.data_ptr(), b.data_ptr(), c.data_ptr(), _stream(dev), batch, M, N, K, layout))
     return c
 
 
 def softmax_rows(s, scale: float, out=None):
     """Row softmax of scale * s over the last dimension (bf16, CUDA, contiguous); out may be s."""
-    import torch
-
+    torch = _torch
     if s.dtype != torch.bfloat16 or not s.is_cuda or not s.is_contiguous():
         raise ValueError("s must be a contiguous CUDA bfloat16 tensor")
     if out is None:
@@ -495,8 +503,8 @@ def softmax_rows(s, scale: float, out=None):
     cols = int(s.shape[-1])
     rows = s.numel() // cols
     dev = s.get_device()
-    _call(dev, "softmax_rows_forward", lib().softmax_rows_forward, s.data_ptr(), out.data_ptr(), rows, cols, float(scale),
-          _stream(dev))
+    _call(dev, "softmax_rows_forward", lib().softmax_rows_forward_call,
+          _SOFTMAX_CALL(s.data_ptr(), out.data_ptr(), _stream(dev), rows, cols, float(scale)))
     return out
 
 

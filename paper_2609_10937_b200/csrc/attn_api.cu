@@ -806,6 +806,11 @@ extern "C" int attn_forward_causal(const void* q, const void* k, const void* v, 
   return forward_impl(q, k, v, o, B, H, L, d, 1, nullptr, cuda_stream);
 }
 
+extern "C" int attn_forward_call(const attn_call* c) {
+  if (!c || c->Lk <= 0) return ATTN_ERR_INVALID_ARG;
+  return forward_impl(c->q, c->k, c->v, c->o, c->B, c->H, c->Lq, c->d, c->causal ? 1 : 0, nullptr, c->cuda_stream, nullptr, c->Lk);
+}
+
 extern "C" int attn_forward_desc(const attn_hw_desc* desc, const void* q, const void* k, const void* v, void* o, int B, int H,
                                  int L, int d, int causal, void* cuda_stream) {
   if (!desc) return ATTN_ERR_INVALID_ARG;
@@ -1313,6 +1318,16 @@ extern "C" int gemm_forward(const void* a, const void* b, void* c, int batch, in
                             void* cuda_stream) {
   t_launch_count = 0;
   return gemm_launch(a, b, c, batch, M, N, K, b_layout, static_cast<cudaStream_t>(cuda_stream));
+}
+
+extern "C" int gemm_forward_call(const gemm_call* g) {
+  if (!g) return ATTN_ERR_INVALID_ARG;
+  return gemm_forward(g->a, g->b, g->c, g->batch, g->M, g->N, g->K, g->b_layout, g->cuda_stream);
+}
+
+extern "C" int softmax_rows_forward_call(const softmax_call* c) {
+  if (!c) return ATTN_ERR_INVALID_ARG;
+  return softmax_rows_forward(c->s, c->p, c->rows, c->cols, (float)c->scale, c->cuda_stream);
 }
 
 extern "C" int gemm_forward_tiles(const void* a, const void* b, void* c, int batch, int M, int N, int K, int b_layout,

@@ -302,3 +302,17 @@ def test_traffic_model_matches_the_paper_figures():
     assert round(traffic.unfused_bytes(1, 1, L, 128, 4, 4) / traffic.fused_bytes(1, 1, L, 128, 4)) == g["ratio"][1]
     assert round(traffic.unfused_bytes(1, 1, g["unfused_gb"][0], 128, 4, 4) / 1e9) == g["unfused_gb"][1]
     assert traffic.unfused_bytes(1, 1, L, 128, 4, 4) == po.traffic_unfused(1, 1, L, 128, 4, 4)
+
+
+def test_calls_with_their_arguments_in_memory_refuse_what_the_plain_calls_refuse(binding):
+    L = binding.lib()
+    assert L.attn_forward_call(None) == L.gemm_forward_call(None) == L.softmax_rows_forward_call(None) == binding.ERR_INVALID_ARG
+    at = 1 << 20
+    attn = lambda *sizes: L.attn_forward_call(binding._ATTN_CALL(at, 2 * at, 3 * at, 4 * at, 0, *sizes))
+    assert attn(0, 1, 128, 128, 64, 0) == attn(1, 1, 128, 0, 64, 0) == attn(1, 1, 128, 128, -1, 0) == binding.ERR_INVALID_ARG
+    assert attn(1, 1, 128, 128, 96, 0) == binding.ERR_UNSUPPORTED_SHAPE
+    assert L.attn_forward_call(binding._ATTN_CALL(at + 8, 2 * at, 3 * at, 4 * at, 0, 1, 1, 128, 128, 64, 0)) == binding.ERR_MISALIGNED
+    assert L.gemm_forward_call(binding._GEMM_CALL(at, 2 * at, 3 * at, 0, 1, 0, 64, 64, 0)) == binding.ERR_INVALID_ARG
+    rows = lambda n, cols, scale: L.softmax_rows_forward_call(binding._SOFTMAX_CALL(at, 2 * at, 0, n, cols, scale))
+    assert rows(0, 64, 1.0) == rows(4, 64, 1e300) == rows(4, 64, float("nan")) == rows(4, 64, -1.0) == binding.ERR_INVALID_ARG
+    assert rows(4, 60, 1.0) == rows(1 << 40, 64, 1.0) == binding.ERR_UNSUPPORTED_SHAPE
