@@ -422,7 +422,7 @@ enum attn_kernel {
   ATTN_KERNEL_GEMM_PAIR = 6,     /* matrix product, CTA pairs                                    */
   ATTN_KERNEL_GEMM_SMALL = 7,    /* matrix product, one 128 x 128 tile per CTA                   */
   ATTN_KERNEL_SOFTMAX = 8,       /* row softmax                                                  */
-  ATTN_KERNEL_NARROW_TILES = 9   /* d = 64, not causal, one CTA per Q tile                       */
+  ATTN_KERNEL_NARROW_TILES = 9   /* not causal, one CTA per Q tile (of 256 or 128 rows)          */
 };
 int attn_last_kernel(void);
 int attn_last_grid(void);

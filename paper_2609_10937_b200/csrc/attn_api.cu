@@ -467,17 +467,17 @@ int launch_causal_tiles(const void* q, const void* k, const void* v, void* o, in
   return ATTN_OK;
 }
 
-// d = 64 as whole Q tiles, one CTA each (narrow_kernel.cuh).
-template <bool CAUSAL, int SUBS>
+// Whole Q tiles, one CTA each, a few softmax streams per tile (narrow_kernel.cuh).
+template <int D, bool CAUSAL, int SUBS>
 int launch_narrow(const void* q, const void* k, const void* v, void* o, int BH, int Lq, int Lk, unsigned int* status, DeviceState* st,
                   cudaStream_t stream) {
-  using SM = attn::NarrowSmem;
+  using SM = attn::NarrowSmem<D>;
   CUtensorMap tq, tk, tv, to;
   int rc;
-  if ((rc = make_tmap(&tq, q, BH, Lq, 64, attn::kSub)) != ATTN_OK) return rc;
-  if ((rc = make_tmap(&tk, k, BH, Lk, 64, 128)) != ATTN_OK) return rc;
-  if ((rc = make_tmap(&tv, v, BH, Lk, 64, 128)) != ATTN_OK) return rc;
-  if ((rc = make_tmap(&to, o, BH, Lq, 64, 32)) != ATTN_OK) return rc;    // every warp stores its own 32 rows
+  if ((rc = make_tmap(&tq, q, BH, Lq, D, attn::kSub)) != ATTN_OK) return rc;
+  if ((rc = make_tmap(&tk, k, BH, Lk, D, 128)) != ATTN_OK) return rc;
+  if ((rc = make_tmap(&tv, v, BH, Lk, D, 128)) != ATTN_OK) return rc;
+  if ((rc = make_tmap(&to, o, BH, Lq, D, 32)) != ATTN_OK) return rc;    // every warp stores its own 32 rows
   attn::NarrowParams p;
   p.Lq = Lq;
   p.Lk = Lk;
@@ -485,16 +485,16 @@ int launch_narrow(const void* q, const void* k, const void* v, void* o, int BH, 
   p.n_steps = (Lk + 127) / 128;
   p.heads = BH;
   // (causal: groups of heads as in launch_causal_tiles)
-  const long long at_most = std::max(1LL, st->desc.cache_bytes / (3 * 4LL * Lk * 64));
+  const long long at_most = std::max(1LL, st->desc.cache_bytes / (3 * 4LL * Lk * D));
   const long long groups = (BH + at_most - 1) / at_most;
   p.group_heads = (int)((BH + groups - 1) / groups);
   p.stages = std::min(attn::kMaxStages, (st->desc.local_mem_bytes - SM::total(0)) / SM::kStageBytes);
-  p.scale_log2 = (float)(1.4426950408889634 / std::sqrt(64.0));
+  p.scale_log2 = (float)(1.4426950408889634 / std::sqrt((double)D));
   p.status = status;
   const int smem = SM::total(p.stages);
-  auto kern = attn::attn_narrow_kernel<CAUSAL, SUBS>;
+  auto kern = attn::attn_narrow_kernel<D, CAUSAL, SUBS>;
   ATTN_ALLOW_SMEM(kern, smem);
-  ATTN_CUDA_TRY(launch_kernel(kern, (long long)BH * p.q_tiles, attn::kNarrowThreads, smem, 0, stream, tq, tk, tv, to, p));
+  ATTN_CUDA_TRY(launch_kernel(kern, (long long)BH * p.q_tiles, attn::NarrowShape<D>::kThreads, smem, 0, stream, tq, tk, tv, to, p));
   t_cluster_size = 0;
   t_launch_count = 1;
   launched(CAUSAL ? ATTN_KERNEL_CAUSAL_TILES : ATTN_KERNEL_NARROW_TILES, (long long)BH * p.q_tiles);
@@ -510,14 +510,15 @@ long long causal_steps(int BH, int L) { return BH * attn_internal::head_units((L
 // tile decides, ranges stay: 8 x 4096 55 / (33 steps of 2) 66.  (Four ring stages: the MMA warp looks that far ahead.)
 bool causal_whole_tiles(const attn_tiles& t, int BH, int L, int d, int local_mem, int sms) {
   if (!t.causal || t.n_q != 2 || t.tile_kv != 128) return false;
-  if (local_mem < (d == 64 ? attn::NarrowSmem::total(4) : attn::TilesSmem::total(4))) return false;
+  if (local_mem < (d == 64 ? attn::NarrowSmem<64>::total(4) : attn::TilesSmem::total(4))) return false;
   if (t.ctas % t.tiles == 0 && t.ctas > t.tiles) return false;      // clusters that share out each tile's own steps
   const long long even = (causal_steps(BH, L) + t.tiles + sms - 1) / sms;
   return std::max<long long>((L + 127) / 128, even) + 5 <= t.cost_steps;
 }
 
-// Sub-tiles a tile of narrow_kernel.cuh has at d = 64: two, or one (tiles of 128 rows that take half as long), or 0 where the
-// plan's kernel stays.
+// Sub-tiles a tile of narrow_kernel.cuh has: two, or one (tiles of 128 rows that take half as long), or 0 where the plan's kernel
+// stays.  Estimates in units of about 1.4 us at d = 64, in us at d = 128 (where a step of this kernel is slower than one of
+// attn_fwd_kernel, 2.1 us against 1.75: its rows need every key tile for themselves).
 //   Causal.  One sub-tile where the longest tile would keep its CTA longer than an even share of the work, by the estimates
 // (in steps) max(longest / 2, 1.1 even + 1) + 4.4 for one, max(longest, 1.1 even + 1) 0.96 + 4.1 for two and 1.08 times the plan's
 // cost for its ranges.  Measured in loops (us; plan's kernel or two / one): 8 heads x 4096 49.9 / 30.2, 4 x 8192 69.3 / 51.7,
@@ -530,10 +531,24 @@ bool causal_whole_tiles(const attn_tiles& t, int BH, int L, int d, int local_mem
 //   Not causal, one: where 1.1 times the waves of half-length tiles and 2.8 are below the plan's cost (us, attn_fwd_kernel / one):
 // 1 head x 256 6.8 / 5.3, 16 x 512 10.3 / 7.2, 16 x 1024 13.2 / 11.3, 32 x 1111 29.9 / 22.2, 60 x 1500 63.8 / 60.2; on the other side
 // 128 x 256 7.7 / 8.3, 30 x 1024 17.1 / 18.8, 4 x 2048 15.1 / 17.4, 16 x 2048 28.6 / 32.1, 1 x 16384 95.8 / 99.2.
+//   d = 128, by the same reasoning.  Causal (us; plan's kernel / one): 8 heads x 4096 54.7 / 40.7, 16 x 2048 35.1 / 28.2, 20 x 1111
+// 21.6 / 16.3, 1 x 256 12.7 / 9.4; on the other side 32 x 1111 22.9 / 24.0, 24 x 2048 35.7 / 40.5, 2 x 8192 55.3 / 73.3, 128 x 256
+// 12.4 / 13.8.  Not causal: 1 x 256 8.1 / 5.8, 16 x 512 11.4 / 8.9, 32 x 1111 35.4 / 30.4; on the other side 30 x 1024 19.0 / 23.2,
+// 128 x 256 9.2 / 9.9, 16 x 2048 32.9 / 42.5, 1 x 16384 122 / 166.  Clusters stay here too (16 x 1024 15.2 / 13.9).
 int narrow_subs(const attn_tiles& t, int BH, int Lq, int Lk, int d, int local_mem, int sms) {
-  if (d != 64 || t.n_q != 2 || t.tile_kv != 128 || local_mem < attn::NarrowSmem::total(4)) return 0;
+  if (t.n_q != 2 || t.tile_kv != 128 || local_mem < (d == 64 ? attn::NarrowSmem<64>::total(4) : attn::NarrowSmem<128>::total(4))) return 0;
+  const bool clusters = t.ctas % t.tiles == 0 && t.ctas > t.tiles;
+  const long long waves = ((long long)BH * ((Lq + 127) / 128) + sms - 1) / sms, steps = (Lk + 127) / 128;
+  if (d == 128) {
+    if (clusters) return 0;
+    if (!t.causal) return 1.35 * (double)(waves * ((steps + 1) / 2)) + 2.3 < (double)t.cost_steps ? 1 : 0;
+    const double even = (double)causal_steps(BH, Lq) / sms;
+    const double one = 5.5 + 2.1 * std::max(0.5 * (double)steps, 1.2 * even + 1.5);
+    const double now = causal_whole_tiles(t, BH, Lq, d, local_mem, sms) ? 7.0 + 1.72 * std::max((double)steps, 1.1 * even + 1.0) : 1.7 * t.cost_steps;
+    return one < now ? 1 : 0;
+  }
   if (t.causal) {
-    if (t.ctas % t.tiles == 0 && t.ctas > t.tiles) return 0;
+    if (clusters) return 0;
     const double longest = (Lq + 127) / 128, share = 1.1 * (double)causal_steps(BH, Lq) / sms + 1.0;
     const double one = std::max(0.5 * longest, share) + 4.4;
     const bool whole = causal_whole_tiles(t, BH, Lq, d, local_mem, sms);
@@ -542,7 +557,6 @@ int narrow_subs(const attn_tiles& t, int BH, int Lq, int Lk, int d, int local_me
   }
   const long long slots = (long long)((t.tiles + sms - 1) / sms) * sms;
   if (t.tiles >= 3 * sms && 10 * slots <= 11LL * t.tiles) return 2;
-  const long long waves = ((long long)BH * ((Lq + 127) / 128) + sms - 1) / sms, steps = (Lk + 127) / 128;
   return 1.1 * (double)(waves * ((steps + 1) / 2)) + 2.8 < (double)t.cost_steps ? 1 : 0;
 }
 
@@ -554,8 +568,9 @@ int dispatch_fwd(const void* q, const void* k, const void* v, void* o, int B, in
   const int sms = st->desc.num_units;
   if (own_plan) {
     if (const int subs = narrow_subs(t, B * H, L, Lk, d, st->desc.local_mem_bytes, sms)) {
-      auto launch = t.causal ? (subs == 1 ? launch_narrow<true, 1> : launch_narrow<true, 2>)
-                             : (subs == 1 ? launch_narrow<false, 1> : launch_narrow<false, 2>);
+      auto launch = d == 128 ? (t.causal ? launch_narrow<128, true, 1> : launch_narrow<128, false, 1>)
+                    : t.causal ? (subs == 1 ? launch_narrow<64, true, 1> : launch_narrow<64, true, 2>)
+                               : (subs == 1 ? launch_narrow<64, false, 1> : launch_narrow<64, false, 2>);
       return launch(q, k, v, o, B * H, L, Lk, status, st, s);
     }
     if (d == 128 && Lk == L && causal_whole_tiles(t, B * H, L, d, st->desc.local_mem_bytes, sms))

@@ -1,5 +1,5 @@
-// attn_narrow_kernel: fused attention for d = 64 in which every Q tile is worked on by one CTA from its first key to its last
-// (nothing to merge between CTAs), causal or not.
+// attn_narrow_kernel: fused attention in which every Q tile is worked on by one CTA from its first key to its last (nothing to
+// merge between CTAs) by several softmax streams, causal or not: d = 64, and at d = 128 tiles of 128 rows.
 //
 // At d = 64 the step is bound by the softmax warps' instructions: 256 x 128 exponentials, maxima, conversions and sums take a
 // scheduler partition about 1930 cycles however they are written (2040 beside the matrix products), the products 1300.
@@ -12,7 +12,8 @@
 // 32 x 1111 22.5 / 20.8; not causal 128 x 8192 2890 / 2797, where the power limit takes back most of it.
 // SUBS = 1 works on tiles of 128 query rows, one sub-tile: its four streams are the two halves of the even and of the odd key
 // tiles.  A tile then takes half as long, which evens out the CTAs where a launch has few tiles for each (narrow_subs in
-// attn_api.cu), at twice the K and V loads for a row.
+// attn_api.cu), at twice the K and V loads for a row.  At d = 128, where a stream needs 256 columns of tensor memory, two
+// streams take the even and the odd key tiles, in that form only.
 //   * One barrier each way per step: scores ready (commit of Q K^T, which also says that the stream's P V of the step before
 //     is complete) and P ready.  A softmax warp whose reference moved rescales its accumulator itself: that is rare, and
 //     no other warp has to be asked.
@@ -38,18 +39,30 @@ struct NarrowParams {
   unsigned int* status;    // as in FwdParams
 };
 
+// d = 64: four streams, the halves of a key tile; d = 128: two, whole key tiles (SUBS = 1 only).
+template <int D>
+struct NarrowShape {
+  static constexpr int kHalves = D == 64 ? 2 : 1;                // streams that share a key tile
+  static constexpr int kStreams = 2 * kHalves;
+  static constexpr int kKeys = 128 / kHalves;                    // keys of a stream's step
+  static constexpr int kEpiWarp = 4 * kStreams, kMmaWarp = kEpiWarp + 4, kLoadWarp = kMmaWarp + kStreams, kAllocWarp = kLoadWarp + 1;
+  // d = 64: 16 softmax warps, 4 epilogue, 4 MMA, TMA, tensor-memory allocation, 2 idle; registers 896 x 72 at launch, then 512 x 96
+  // and 384 x 40.  d = 128: 8, 4, 2, 1, 1; 512 x 128 at launch, then 256 x 192 and 256 x 64.
+  static constexpr int kThreads = D == 64 ? 896 : 512;
+  static constexpr int kSoftmaxRegs = D == 64 ? 96 : 192, kOtherRegs = D == 64 ? 40 : 64;
+  static constexpr int kSchedReaders = kLoadWarp + 1;            // warps that read a tile's index
+};
+template <int D>
 struct NarrowSmem {
-  static constexpr int kSubBytes = kSub * 128;                   // one sub-tile of Q
-  static constexpr int kQBytes = 2 * 2 * kSubBytes;              // two tiles
-  static constexpr int kStageBytes = 128 * 128;
-  static constexpr int kOutBytes = 8 * 4096;                     // two [32 rows][64 columns] bf16 chunks per epilogue warp
+  static constexpr int kSubs = D == 64 ? 2 : 1;                  // sub-tiles of Q there is room for
+  static constexpr int kSubBytes = kSub * D * 2;                 // one sub-tile of Q
+  static constexpr int kQBytes = 2 * kSubs * kSubBytes;          // two tiles
+  static constexpr int kStageBytes = 128 * D * 2;
+  static constexpr int kChunks = D == 64 ? 2 : 1;                // [32 rows][64 columns] bf16 output chunks per epilogue warp
+  static constexpr int kOutBytes = 4 * kChunks * 4096;
   static constexpr int kMiscBytes = 9216;
   __host__ __device__ static constexpr int total(int stages) { return kQBytes + stages * kStageBytes + kOutBytes + kMiscBytes; }
 };
-// 16 softmax warps, 4 epilogue, 4 MMA, TMA, tensor-memory allocation, 2 idle.  Registers: 896 x 72 at launch, then 512 x 96 and
-// 384 x 40.
-constexpr int kNarrowThreads = 896;
-constexpr int kNarrowSchedReaders = 25;    // warps that read a tile's index: all but the last three
 
 struct NarrowMisc {
   float2 stat[2][4][kSub];                 // [the sub-tile's tiles mod 2][stream][row] reference and denominator of a finished tile
@@ -63,7 +76,7 @@ struct NarrowMisc {
   AbortCell abort;
   uint32_t tmem_slot;
 };
-static_assert(sizeof(NarrowMisc) <= NarrowSmem::kMiscBytes, "misc region too large");
+static_assert(sizeof(NarrowMisc) <= NarrowSmem<64>::kMiscBytes, "misc region too large");
 
 // A tile: its head, first row, key tiles and the number of them that each of its streams works on.  Stream st: sub-tile st / 2,
 // half st % 2 of every key tile; SUBS = 1: half st % 2 of the key tiles j with j % 2 = st / 2.
@@ -101,14 +114,17 @@ __device__ __forceinline__ NarrowWork<SUBS> narrow_work(int index, const NarrowP
   return w;
 }
 
-template <bool CAUSAL, int SUBS>
-__global__ void __launch_bounds__(kNarrowThreads, 1)
+template <int D, bool CAUSAL, int SUBS>
+__global__ void __launch_bounds__(NarrowShape<D>::kThreads, 1)
 attn_narrow_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                    const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_o, const NarrowParams p) {
-  constexpr int D = 64, TKV = 128, HKV = TKV / 2;     // a stream takes one half of every key tile
-  constexpr int O_COL0 = 4 * HKV;
+  using SH = NarrowShape<D>;
+  using SM = NarrowSmem<D>;
+  constexpr int TKV = 128, HKV = SH::kKeys, KCH = D / 64, NCH = HKV / 32, HALVES = SH::kHalves;
+  constexpr int O_COL0 = SH::kStreams * HKV;
   constexpr int kPoly = kPolyPairsPer8;
-  using SM = NarrowSmem;
+  constexpr int kParts = SH::kStreams / SUBS;         // streams of a sub-tile
+  static_assert(SUBS <= SM::kSubs, "no room for the second sub-tile");
 
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   const uint32_t smem_base = smem_u32(smem_raw);
@@ -123,7 +139,7 @@ attn_narrow_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
     if (smem_base & 1023u) note_timeout(wait_info(kRoleLoad, 0, 0xFFFF), &misc->abort.flag);   // swizzled tiles need 1024-byte alignment
     for (int s = 0; s < kMaxStages; ++s) {
       mbar_init(smem_u32(&misc->kv_full[s]), 1);
-      mbar_init(smem_u32(&misc->kv_empty[s]), 2 * SUBS);          // the streams that read a ring item
+      mbar_init(smem_u32(&misc->kv_empty[s]), HALVES * SUBS);     // the streams that read a ring item
     }
     for (int i = 0; i < 4; ++i) {
       mbar_init(smem_u32(&misc->s_full[i]), 1);
@@ -132,12 +148,12 @@ attn_narrow_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
     }
     for (int i = 0; i < 2; ++i) {
       mbar_init(smem_u32(&misc->sched_full[i]), 1);
-      mbar_init(smem_u32(&misc->sched_empty[i]), kNarrowSchedReaders);
+      mbar_init(smem_u32(&misc->sched_empty[i]), SH::kSchedReaders);
       for (int b = 0; b < 2; ++b) {
         mbar_init(smem_u32(&misc->q_full[i][b]), 1);
-        mbar_init(smem_u32(&misc->q_empty[i][b]), 4 / SUBS);      // the sub-tile's streams
+        mbar_init(smem_u32(&misc->q_empty[i][b]), kParts);        // the sub-tile's streams
       }
-      mbar_init(smem_u32(&misc->o_full[i]), 4 / SUBS);
+      mbar_init(smem_u32(&misc->o_full[i]), kParts);
       mbar_init(smem_u32(&misc->o_free[i]), kSub);
     }
     fence_mbar_init();
@@ -146,7 +162,7 @@ attn_narrow_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
     prefetch_tmap(&tm_v);
     prefetch_tmap(&tm_o);
   }
-  if (warp == 25) {
+  if (warp == SH::kAllocWarp) {
     tmem_alloc(smem_u32(&misc->tmem_slot), 512);
     tmem_relinquish();
   }
@@ -169,10 +185,10 @@ attn_narrow_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
     return x;
   };
 
-  if (warp < 16) {
+  if (warp < SH::kEpiWarp) {
     // ===================================================== softmax warpgroup of one stream
-    setmaxnreg_inc<96>();
-    const int st = warp >> 2, group = st >> 1, half = st & 1, i = SUBS == 2 ? group : 0;
+    setmaxnreg_inc<SH::kSoftmaxRegs>();
+    const int st = warp >> 2, group = st / HALVES, half = st % HALVES, i = SUBS == 2 ? group : 0;
     const int row = (warp & 3) * 32 + lane;
     const uint32_t lane_base = tmem_base + ((uint32_t)((warp & 3) * 32) << 16);
     const uint32_t s_tmem = lane_base + st * HKV;      // P goes to the front of it
@@ -199,9 +215,12 @@ attn_narrow_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
           tc_fence_after();
           uint32_t s[HKV];
           // load the row in two halves: the maximum of the first half is taken while the second is in flight
-          tmem_ld32_nowait(s_tmem, *reinterpret_cast<uint32_t(*)[32]>(&s[0]));
-          tmem_ld_fence(*reinterpret_cast<uint32_t(*)[32]>(&s[0]));
-          tmem_ld32_nowait(s_tmem + 32, *reinterpret_cast<uint32_t(*)[32]>(&s[32]));
+#pragma unroll
+          for (int c = 0; c < NCH / 2; ++c) tmem_ld32_nowait(s_tmem + c * 32, *reinterpret_cast<uint32_t(*)[32]>(&s[c * 32]));
+#pragma unroll
+          for (int c = 0; c < NCH / 2; ++c) tmem_ld_fence(*reinterpret_cast<uint32_t(*)[32]>(&s[c * 32]));
+#pragma unroll
+          for (int c = NCH / 2; c < NCH; ++c) tmem_ld32_nowait(s_tmem + c * 32, *reinterpret_cast<uint32_t(*)[32]>(&s[c * 32]));
           // keys past the end or after the query's position: score -inf, never zero
           if constexpr (kMasked) {
 #pragma unroll
@@ -209,7 +228,8 @@ attn_narrow_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
               if (k > lim) s[k] = 0xFF800000u;
           }
           const float mx_a = fmaxf(chain_max<0, HKV / 4>(s), chain_max<HKV / 4, HKV / 2>(s));
-          tmem_ld_fence(*reinterpret_cast<uint32_t(*)[32]>(&s[32]));
+#pragma unroll
+          for (int c = NCH / 2; c < NCH; ++c) tmem_ld_fence(*reinterpret_cast<uint32_t(*)[32]>(&s[c * 32]));
           if constexpr (kMasked) {
 #pragma unroll
             for (int k = HKV / 2; k < HKV; ++k)
@@ -238,12 +258,12 @@ attn_narrow_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
           }
           const uint64_t neg_m2 = pack_f32x2(-m_run, -m_run);
           uint64_t sum2 = 0ull;                        // packed (0.f, 0.f)
-          uint32_t pk[16];
-          exp_chunk<kPoly>(&s[0], ek, neg_m2, sum2, pk);
-          tmem_st16(s_tmem, pk);
-          uint32_t pk2[16];
-          exp_chunk<kPoly>(&s[32], ek, neg_m2, sum2, pk2);
-          tmem_st16(s_tmem + 16, pk2);
+#pragma unroll
+          for (int c = 0; c < NCH; ++c) {
+            uint32_t pk[16];
+            exp_chunk<kPoly>(&s[c * 32], ek, neg_m2, sum2, pk);
+            tmem_st16(s_tmem + c * 16, pk);
+          }
           float sum0, sum1;
           unpack_f32x2(sum2, sum0, sum1);
           delta = delta * alpha + (sum0 + sum1);
@@ -281,14 +301,14 @@ attn_narrow_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
       }
       tile = next_tile(seq, kRoleSoftmax);
     }
-  } else if (warp < 20) {
+  } else if (warp < SH::kMmaWarp) {
     // ================================================== epilogue warpgroup
-    setmaxnreg_dec<40>();
+    setmaxnreg_dec<SH::kOtherRegs>();
     const int wq = warp & 3, row = wq * 32 + lane;
     const uint32_t lane_base = tmem_base + ((uint32_t)(wq * 32) << 16);
-    const uint32_t stage_w = out_smem + wq * 8192;     // this warp's two staging chunks
+    const uint32_t stage_w = out_smem + wq * (SM::kChunks * 4096);     // this warp's staging chunks
     bool ok = run;
-    uint32_t fin = 0, chunk_ctr = 0;                   // bit i: finished tiles of sub-tile i, mod 2
+    uint32_t fin = 0, chunk = 0;                       // bit i: finished tiles of sub-tile i, mod 2; next staging chunk
     int tile = blockIdx.x;
     for (int seq = 1; ok && tile >= 0; ++seq) {
       const NarrowWork<SUBS> w = narrow_work<CAUSAL, SUBS>(tile, p);
@@ -297,18 +317,17 @@ attn_narrow_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
         if (SUBS == 2 && w.steps(i) == 0) continue;
         const uint32_t ph = (fin >> i) & 1;
         fin ^= 1u << i;
-        constexpr int kParts = 4 / SUBS;               // streams of a sub-tile
         float wt[kParts], m = -INFINITY, sum = 0.f;
 #pragma unroll
         for (int k = 0; k < kParts; ++k)
-          if (ok && !wait_quiet_warp(smem_u32(&misc->fin_full[2 * i + k]), ph, abort_flag, wait_info(kRoleCorrection, kBarAlpha, 2 * i + k))) ok = false;
+          if (ok && !wait_quiet_warp(smem_u32(&misc->fin_full[HALVES * i + k]), ph, abort_flag, wait_info(kRoleCorrection, kBarAlpha, HALVES * i + k))) ok = false;
         if (!ok) break;
         // the streams' parts on the common reference, normalised
 #pragma unroll
-        for (int k = 0; k < kParts; ++k) m = fmaxf(m, misc->stat[ph][2 * i + k][row].x);
+        for (int k = 0; k < kParts; ++k) m = fmaxf(m, misc->stat[ph][HALVES * i + k][row].x);
 #pragma unroll
         for (int k = 0; k < kParts; ++k) {
-          const float2 a = misc->stat[ph][2 * i + k][row];
+          const float2 a = misc->stat[ph][HALVES * i + k][row];
           wt[k] = ex2_approx(a.x - m);                 // (an empty part: -inf, weight 0)
           sum += a.y * wt[k];
         }
@@ -317,37 +336,49 @@ attn_narrow_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
         for (int k = 0; k < kParts; ++k) wt[k] *= inv;
         if (!wait_quiet_warp(smem_u32(&misc->o_full[i]), ph, abort_flag, wait_info(kRoleCorrection, kBarOFull, i))) { ok = false; break; }
         tc_fence_after();
-        const bool empty = SUBS == 1 && w.n1 == 0;     // streams 2 and 3 have no accumulator
-        const uint32_t o_tmem = lane_base + O_COL0 + 2 * i * D;
-        const uint32_t dst = stage_w + (chunk_ctr & 1) * 4096;
-        ++chunk_ctr;
-        // the store that last read this chunk (two chunks ago) must have finished reading it
-        if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
-        __syncwarp();
+        const bool empty = SUBS == 1 && w.n1 == 0;     // the streams of the odd key tiles have no accumulator
+        const uint32_t o_tmem = lane_base + O_COL0 + HALVES * i * D;
 #pragma unroll 1
-        for (int c = 0; c < 8; ++c) {                  // 8 columns at a time
-          uint32_t ra[8], rb[8];
-          float v[8];
-          tmem_ld8x2(o_tmem + c * 8, o_tmem + D + c * 8, ra, rb);
-#pragma unroll
-          for (int e = 0; e < 8; ++e) v[e] = __uint_as_float(ra[e]) * wt[0] + __uint_as_float(rb[e]) * wt[1];
-          if (SUBS == 1 && !empty) {
-            tmem_ld8x2(o_tmem + 2 * D + c * 8, o_tmem + 3 * D + c * 8, ra, rb);
-#pragma unroll
-            for (int e = 0; e < 8; ++e) v[e] += __uint_as_float(ra[e]) * wt[kParts - 2] + __uint_as_float(rb[e]) * wt[kParts - 1];
+        for (int h = 0; h < KCH; ++h) {
+          const uint32_t dst = stage_w + chunk * 4096;
+          chunk = chunk + 1 < SM::kChunks ? chunk + 1 : 0;
+          // the store that last read this chunk must have finished reading it
+          if (lane == 0) {
+            if (SM::kChunks == 2) asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
+            else tma_store_wait_read();
           }
-          uint32_t q[4];
+          __syncwarp();
+#pragma unroll 1
+          for (int c = 0; c < 8; ++c) {                // 8 columns at a time
+            const uint32_t col = o_tmem + h * 64 + c * 8;
+            uint32_t ra[8], rb[8];
+            float v[8];
+            tmem_ld8x2(col, col + D, ra, rb);
 #pragma unroll
-          for (int e = 0; e < 4; ++e) q[e] = pack_bf16x2(v[2 * e], v[2 * e + 1]);
-          st_shared_u4(dst + lane * 128 + (((uint32_t)c ^ (uint32_t)(lane & 7)) << 4), q);   // 128-byte swizzle
-        }
-        tc_fence_before();
-        mbar_arrive(smem_u32(&misc->o_free[i]));       // both accumulators have been read
-        fence_proxy_async_smem();
-        __syncwarp();
-        if (lane == 0) {                               // (rows past the end of the sequence are clipped by the tensor map)
-          tma_store_3d(&tm_o, dst, 0, w.q_row0 + i * kSub + wq * 32, w.bh);
-          tma_store_commit();
+            for (int e = 0; e < 8; ++e) {
+              v[e] = __uint_as_float(ra[e]) * wt[0];
+              if (HALVES == 2 || !empty) v[e] += __uint_as_float(rb[e]) * wt[1];
+            }
+            if (kParts == 4 && !empty) {
+              tmem_ld8x2(col + 2 * D, col + 3 * D, ra, rb);
+#pragma unroll
+              for (int e = 0; e < 8; ++e) v[e] += __uint_as_float(ra[e]) * wt[kParts - 2] + __uint_as_float(rb[e]) * wt[kParts - 1];
+            }
+            uint32_t q[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) q[e] = pack_bf16x2(v[2 * e], v[2 * e + 1]);
+            st_shared_u4(dst + lane * 128 + (((uint32_t)c ^ (uint32_t)(lane & 7)) << 4), q);   // 128-byte swizzle
+          }
+          if (h == KCH - 1) {
+            tc_fence_before();
+            mbar_arrive(smem_u32(&misc->o_free[i]));   // every accumulator has been read
+          }
+          fence_proxy_async_smem();
+          __syncwarp();
+          if (lane == 0) {                             // (rows past the end of the sequence are clipped by the tensor map)
+            tma_store_3d(&tm_o, dst, h * 64, w.q_row0 + i * kSub + wq * 32, w.bh);
+            tma_store_commit();
+          }
         }
       }
       if (!ok) break;
@@ -355,10 +386,10 @@ attn_narrow_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
     }
     if (lane == 0) tma_store_wait_read();              // shared memory is read by the stores until here
     __syncwarp();
-  } else if (warp < 24) {
+  } else if (warp < SH::kLoadWarp) {
     // ============================== MMA issuer of one stream (the whole warp walks the loop, one lane issues)
-    setmaxnreg_dec<40>();
-    const int st = warp & 3, group = st >> 1, half = st & 1, i = SUBS == 2 ? group : 0;
+    setmaxnreg_dec<SH::kOtherRegs>();
+    const int st = warp - SH::kMmaWarp, group = st / HALVES, half = st % HALVES, i = SUBS == 2 ? group : 0;
     bool ok = run;
     const uint32_t s_tmem = tmem_base + st * HKV, o_tmem = tmem_base + O_COL0 + st * D;
     const uint32_t k_smem = ring_smem + half * (HKV * 128);       // this stream's keys in a ring item
@@ -373,7 +404,7 @@ attn_narrow_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
     // (one lane) Scores of the keys at ring position k; last: no later step of the tile reads this Q.
     auto issue_scores = [&](int k, bool last) __attribute__((always_inline)) {
       const int b = (q_uses - 1) & 1;
-      issue_qk<D, HKV>(s_tmem, smem_base + (b * 2 + i) * SM::kSubBytes, k_smem + k * SM::kStageBytes);
+      issue_qk<D, HKV>(s_tmem, smem_base + (b * SM::kSubs + i) * SM::kSubBytes, k_smem + k * SM::kStageBytes);
       umma_commit(smem_u32(&misc->s_full[st]));
       umma_commit(smem_u32(&misc->kv_empty[k]));
       if (last) umma_commit(smem_u32(&misc->q_empty[i][b]));
@@ -447,9 +478,9 @@ attn_narrow_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
       if (!ok) break;
       tile = next_tile(seq, kRoleMma);
     }
-  } else if (warp == 24) {
+  } else if (warp == SH::kLoadWarp) {
     // ================================================== TMA producer, and the requests for the next tile
-    setmaxnreg_dec<40>();
+    setmaxnreg_dec<SH::kOtherRegs>();
     bool ok = run;
     int stage = 0, issued = 0, asked = 0;              // asked: requests made
     uint32_t phase = 0;
@@ -460,7 +491,8 @@ attn_narrow_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
       if (elect_one()) {
         const uint32_t bar = smem_u32(&misc->kv_full[stage]);
         mbar_arrive_expect_tx(bar, SM::kStageBytes);
-        tma_load_3d(ring_smem + stage * SM::kStageBytes, tm, 0, kv_row, bh, bar);
+#pragma unroll
+        for (int c = 0; c < KCH; ++c) tma_load_3d(ring_smem + stage * SM::kStageBytes + c * (TKV * 128), tm, c * 64, kv_row, bh, bar);
       }
       __syncwarp();
       ++issued;
@@ -473,7 +505,9 @@ attn_narrow_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
       if (elect_one()) {
         const uint32_t bar = smem_u32(&misc->q_full[i][b]);
         mbar_arrive_expect_tx(bar, SM::kSubBytes);
-        tma_load_3d(smem_base + (b * 2 + i) * SM::kSubBytes, &tm_q, 0, w.q_row0 + i * kSub, w.bh, bar);
+#pragma unroll
+        for (int c = 0; c < KCH; ++c)
+          tma_load_3d(smem_base + (b * SM::kSubs + i) * SM::kSubBytes + c * (kSub * 128), &tm_q, c * 64, w.q_row0 + i * kSub, w.bh, bar);
       }
       __syncwarp();
       if (i) ++q_loads1; else ++q_loads0;
@@ -520,11 +554,11 @@ attn_narrow_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
       if (asked > 0) drain_bar(smem_u32(&misc->sched_full[asked & 1]), ((asked - 1) >> 1) & 1);
     }
   } else {
-    setmaxnreg_dec<40>();
+    setmaxnreg_dec<SH::kOtherRegs>();
   }
   tc_fence_before();
   __syncthreads();
-  if (warp == 25) {
+  if (warp == SH::kAllocWarp) {
     tc_fence_after();
     tmem_dealloc(tmem_base, 512);
   }

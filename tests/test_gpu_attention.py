@@ -1047,22 +1047,24 @@ def test_narrow_whole_tiles_match_the_reference(env, H, Lq, Lk):
 
 
 
-@pytest.mark.parametrize("H,Lq,Lk,causal", [
+@pytest.mark.parametrize("d,H,Lq,Lk,causal", [(128, *c) for c in (
+    (1, 129, 129, True), (3, 256, 256, True), (40, 385, 385, True), (20, 1111, 1111, True), (16, 2048, 2048, True), (8, 4096, 4096, True),
+    (1, 256, 256, False), (16, 300, 129, False), (16, 512, 512, False), (32, 1111, 1111, False), (32, 1100, 1025, False))] + [(64, *c) for c in (
     (1, 129, 129, True), (3, 256, 256, True), (40, 385, 385, True), (50, 512, 512, True), (20, 1111, 1111, True), (32, 1111, 1111, True),
     (16, 2048, 2048, True), (12, 4096, 4096, True), (1, 256, 256, False), (16, 300, 129, False),
     (16, 257, 193, False), (16, 512, 512, False), (32, 1111, 1111, False), (70, 640, 640, False), (128, 384, 384, False),
-    (60, 1500, 1500, False), (16, 1000, 833, False)])
-def test_narrow_tiles_of_one_sub_tile_match_the_reference(env, H, Lq, Lk, causal):
-    """d = 64, tiles of 128 rows whose streams share out the key tiles: odd and even numbers of them, one (half of the streams
+    (60, 1500, 1500, False), (16, 1000, 833, False))])
+def test_narrow_tiles_of_one_sub_tile_match_the_reference(env, d, H, Lq, Lk, causal):
+    """Tiles of 128 rows whose streams share out the key tiles: odd and even numbers of them, one (half of the streams
     then have none), a last one of one key, of half a tile and full; one and several tiles per CTA.  NaN-filled output, every
     element against fp64, the same bits again.  The bound per element is that of
     test_causal_whole_tiles_match_the_reference."""
     torch, orc, binding = env
-    rng = np.random.default_rng([H, Lq, Lk, 7])
-    q, k, v = (to_cuda_bf16(synth.f32_to_bf16_bits((rng.standard_normal((H, n, 64)) * 1.5).astype(np.float32))).view(1, H, n, 64)
+    rng = np.random.default_rng([H, Lq, Lk, d, 7])
+    q, k, v = (to_cuda_bf16(synth.f32_to_bf16_bits((rng.standard_normal((H, n, d)) * 1.5).astype(np.float32))).view(1, H, n, d)
                for n in (Lq, Lk, Lk))
     call = lambda *o: binding.forward(q, k, v, *o, causal=True) if causal else binding.forward_qk(q, k, v, *o)
-    out = torch.full((1, H, Lq, 64), float("nan"), dtype=torch.bfloat16, device="cuda")
+    out = torch.full((1, H, Lq, d), float("nan"), dtype=torch.bfloat16, device="cuda")
     call(out)
     torch.cuda.synchronize()
     assert binding.last_device_status()[0] == 0
@@ -1070,7 +1072,7 @@ def test_narrow_tiles_of_one_sub_tile_match_the_reference(env, H, Lq, Lk, causal
     assert binding.last_grid() == H * -(-Lq // 128)
     keep = torch.ones((Lq, Lk), dtype=torch.bool, device="cuda").tril() if causal else None
     for h in range(0, H, 8):
-        s = q[0, h:h + 8].double() @ k[0, h:h + 8].double().transpose(1, 2) / 8.0
+        s = q[0, h:h + 8].double() @ k[0, h:h + 8].double().transpose(1, 2) / d ** 0.5
         if causal:
             s = s.masked_fill(~keep, -math.inf)
         p, vd, got = torch.softmax(s, dim=-1), v[0, h:h + 8].double(), out[0, h:h + 8].double()
