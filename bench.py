@@ -287,10 +287,17 @@ class Gpu:
             raise RuntimeError(f"device-side wait expired: {detail}")
 
 
-def kernel_name(plan, d, cluster, last=None):
+def kernel_name(plan, d, cluster, last=None, L=0, sms=148):
     """The instantiation a plan ran as: <d, tile_kv, n_q, causal, fixed merge roles, clusters>; `last`: (kernel, CTAs) of the launch."""
     from paper_2609_10937_b200 import binding
 
+    if last is not None and cluster == 0 and last[1] == plan.tiles and plan.n_q == 2:
+        # one CTA per tile of 256 rows: the kernel of two streams a tile, where the library takes it (pipe_tiles, attn_api.cu)
+        steps = -(-L // 128)
+        if last[0] == binding.KERNEL_NARROW_TILES and steps >= 48:
+            return f"attn_pipe_kernel<{d},0>"
+        if last[0] == binding.KERNEL_TILED and (plan.ctas != plan.tiles or plan.tiles > sms or (steps >= 4 and (d == 64 or 3 * plan.tiles > 2 * sms))):
+            return f"attn_pipe_kernel<{d},0>"
     if last is not None and last[0] == binding.KERNEL_NARROW_TILES:
         return f"attn_narrow_kernel<{d},0,{2 if last[1] == plan.tiles else 1}>"
     uniform = plan.ctas > plan.tiles and plan.ctas % plan.tiles == 0
@@ -321,7 +328,7 @@ def measure_config(gpu, name, peaks, iters=None, oracle=True):
            "frac_of_measured_burst_peak": tf / peaks["bf16_tflops"], "launches_timed": iters,
            "tiles": {"tile_q": plan.tile_q, "tile_kv": plan.tile_kv, "kv_stages": plan.kv_stages, "q_tiles": plan.tiles,
                      "ctas": plan.ctas, "cluster": cluster, "cost_steps": plan.cost_steps},
-           "kernel": kernel_name(plan, case.d, cluster, last)}
+           "kernel": kernel_name(plan, case.d, cluster, last, case.L, gpu.desc.num_units)}
     if oracle:
         from oracle import attn_oracle as orc
 

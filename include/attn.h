@@ -414,7 +414,7 @@ int attn_last_cluster_size(void);
  * of CTAs it was launched with. */
 enum attn_kernel {
   ATTN_KERNEL_NONE = 0,
-  ATTN_KERNEL_TILED = 1,         /* the fused kernel with the plan's grid                        */
+  ATTN_KERNEL_TILED = 1,         /* the plan's grid, or one CTA per Q tile of 256 rows instead   */
   ATTN_KERNEL_CAUSAL_TILES = 2,  /* causal, one CTA per Q tile: of 256 rows, or by the grid of   */
                                  /* 128 (d = 64 and tiles of 128 rows: the kernel of 9)          */
   ATTN_KERNEL_FEW_ROWS = 3,      /* few query rows against many keys                             */

@@ -11,7 +11,7 @@ ROOT = PKG.parent
 CSRC = PKG / "csrc"
 LIB = PKG / "libattn_b200.so"
 SOURCES = [CSRC / "attn_api.cu", CSRC / "attn_plan.cpp"]
-HEADERS = [CSRC / "attn_kernels.cuh", CSRC / "decode_kernels.cuh", CSRC / "tiles_kernel.cuh", CSRC / "narrow_kernel.cuh", CSRC / "kv_ring.h", CSRC / "gemm_kernels.cuh", CSRC / "ptx_sm100.cuh", CSRC / "attn_plan_internal.h",
+HEADERS = [CSRC / "attn_kernels.cuh", CSRC / "decode_kernels.cuh", CSRC / "pipe_kernel.cuh", CSRC / "narrow_kernel.cuh", CSRC / "kv_ring.h", CSRC / "gemm_kernels.cuh", CSRC / "ptx_sm100.cuh", CSRC / "attn_plan_internal.h",
            ROOT / "include" / "attn.h", ROOT / "include" / "gemm.h"]
 
 

@@ -18,8 +18,8 @@
 #include "decode_kernels.cuh"
 #include "gemm.h"
 #include "gemm_kernels.cuh"
-#include "tiles_kernel.cuh"
 #include "narrow_kernel.cuh"
+#include "pipe_kernel.cuh"
 
 namespace {
 
@@ -449,37 +449,43 @@ int dispatch_decode(const void* q, const void* k, const void* v, void* o, int BH
   return ATTN_ERR_UNSUPPORTED_SHAPE;
 }
 
-// Causal attention at d = 128 as whole Q tiles, one CTA each (tiles_kernel.cuh).
-int launch_causal_tiles(const void* q, const void* k, const void* v, void* o, int BH, int L, unsigned int* status, DeviceState* st,
-                        cudaStream_t stream) {
-  using SM = attn::TilesSmem;
-  constexpr int D = 128;
+// Heads of a causal problem whose tiles are dealt out together, longest first: equal groups whose K and V take at most a third of the
+// cache (32 heads of 8192, d = 128: 202 MB read from DRAM in groups of eight, 830 MB with 148 ranges that each walk a head of
+// their own).  Equal, because a short last group would start its longest tiles when most CTAs have run dry.
+int causal_group_heads(int BH, int L, int d, const attn_hw_desc& desc) {
+  const long long at_most = std::max(1LL, desc.cache_bytes / (3 * 4LL * L * d));
+  const long long groups = (BH + at_most - 1) / at_most;
+  return (int)((BH + groups - 1) / groups);
+}
+
+// Whole Q tiles of 256 rows, one CTA each (pipe_kernel.cuh).  kernel_id: as what the launch is reported.
+template <int D, bool CAUSAL>
+int launch_pipe(const void* q, const void* k, const void* v, void* o, int BH, int Lq, int Lk, unsigned int* status, DeviceState* st,
+                cudaStream_t stream, int kernel_id) {
+  using SM = attn::PipeSmem<D>;
   CUtensorMap tq, tk, tv, to;
   int rc;
-  if ((rc = make_tmap(&tq, q, BH, L, D, attn::kSub)) != ATTN_OK) return rc;
-  if ((rc = make_tmap(&tk, k, BH, L, D, 128)) != ATTN_OK) return rc;
-  if ((rc = make_tmap(&tv, v, BH, L, D, 128)) != ATTN_OK) return rc;
-  if ((rc = make_tmap(&to, o, BH, L, D, 32)) != ATTN_OK) return rc;    // every warp stores its own 32 rows
-  attn::TilesParams p;
-  p.L = L;
-  p.q_tiles = (L + 2 * attn::kSub - 1) / (2 * attn::kSub);
+  if ((rc = make_tmap(&tq, q, BH, Lq, D, attn::kSub)) != ATTN_OK) return rc;
+  if ((rc = make_tmap(&tk, k, BH, Lk, D, 128)) != ATTN_OK) return rc;
+  if ((rc = make_tmap(&tv, v, BH, Lk, D, 128)) != ATTN_OK) return rc;
+  if ((rc = make_tmap(&to, o, BH, Lq, D, 32)) != ATTN_OK) return rc;    // every warp stores its own 32 rows
+  attn::PipeParams p;
+  p.Lq = Lq;
+  p.Lk = Lk;
+  p.q_tiles = (Lq + 2 * attn::kSub - 1) / (2 * attn::kSub);
+  p.n_steps = (Lk + 127) / 128;
   p.heads = BH;
-  // Heads dealt out together: equal groups whose K and V take at most a third of the cache (32 heads of 8192, d = 128: 202 MB
-  // read from DRAM in groups of eight, 830 MB with 148 ranges that each walk a head of their own).  Equal, because a short
-  // last group would start its longest tiles when most CTAs have run dry.
-  const long long at_most = std::max(1LL, st->desc.cache_bytes / (3 * 4LL * L * D));
-  const long long groups = (BH + at_most - 1) / at_most;
-  p.group_heads = (int)((BH + groups - 1) / groups);
-  p.stages = std::min(attn::kMaxStages, (st->desc.local_mem_bytes - SM::total(0)) / SM::kStageBytes);
+  p.group_heads = causal_group_heads(BH, Lk, D, st->desc);
+  p.stages = std::min(attn::kMaxStages, (st->desc.local_mem_bytes - SM::total(0)) / SM::kStageBytes) & ~1;
   p.scale_log2 = (float)(1.4426950408889634 / std::sqrt((double)D));
   p.status = status;
   const int smem = SM::total(p.stages);
-  auto kern = attn::attn_causal_tiles_kernel;
+  auto kern = attn::attn_pipe_kernel<D, CAUSAL>;
   ATTN_ALLOW_SMEM(kern, smem);
   ATTN_CUDA_TRY(launch_kernel(kern, (long long)BH * p.q_tiles, 512, smem, 0, stream, tq, tk, tv, to, p));
   t_cluster_size = 0;
   t_launch_count = 1;
-  launched(ATTN_KERNEL_CAUSAL_TILES, (long long)BH * p.q_tiles);
+  launched(kernel_id, (long long)BH * p.q_tiles);
   return ATTN_OK;
 }
 
@@ -501,10 +507,7 @@ int launch_narrow(const void* q, const void* k, const void* v, void* o, int BH, 
   p.q_tiles = (Lq + SUBS * attn::kSub - 1) / (SUBS * attn::kSub);
   p.n_steps = (Lk + 127) / 128;
   p.heads = BH;
-  // (causal: groups of heads as in launch_causal_tiles)
-  const long long at_most = std::max(1LL, st->desc.cache_bytes / (3 * 4LL * Lk * D));
-  const long long groups = (BH + at_most - 1) / at_most;
-  p.group_heads = (int)((BH + groups - 1) / groups);
+  p.group_heads = causal_group_heads(BH, Lk, D, st->desc);
   p.stages = std::min(attn::kMaxStages, (st->desc.local_mem_bytes - SM::total(0)) / SM::kStageBytes) / kRings;
   p.scale_log2 = (float)(1.4426950408889634 / std::sqrt((double)D));
   p.status = status;
@@ -527,7 +530,7 @@ long long causal_steps(int BH, int L) { return BH * attn_internal::head_units((L
 // tile decides, ranges stay: 8 x 4096 55 / (33 steps of 2) 66.  (Four ring stages: the MMA warp looks that far ahead.)
 bool causal_whole_tiles(const attn_tiles& t, int BH, int L, int d, int local_mem, int sms) {
   if (!t.causal || t.n_q != 2 || t.tile_kv != 128) return false;
-  if (local_mem < (d == 64 ? attn::NarrowSmem<64, 2>::total(4) : attn::TilesSmem::total(4))) return false;
+  if (local_mem < (d == 64 ? attn::NarrowSmem<64, 2>::total(4) : attn::PipeSmem<128>::total(4))) return false;
   if (t.ctas % t.tiles == 0 && t.ctas > t.tiles) return false;      // clusters that share out each tile's own steps
   const long long even = (causal_steps(BH, L) + t.tiles + sms - 1) / sms;
   return std::max<long long>((L + 127) / 128, even) + 5 <= t.cost_steps;
@@ -602,6 +605,24 @@ int narrow_subs(const attn_tiles& t, int BH, int Lq, int Lk, int d, int local_me
   return 1.1 * (double)(waves * ((steps + 1) / 2)) + 2.8 < (double)t.cost_steps ? 1 : 0;
 }
 
+// Calls, not causal, that pipe_kernel.cuh takes over from attn_fwd_kernel, at either head dimension (us in graphs of 8 calls, attn_fwd_kernel / this).
+//   Plans of whole tiles: with more tiles than SMs always (183 shapes of a grid, 0.81 to 0.99 times: 148 x 1024, d = 64 59.3 / 53.2; 592 x 512,
+// d = 128 75.8 / 63.2).  One wave: from four key steps on (three and fewer 0.98 to 1.05: 64 x 384, d = 64 10.0 / 10.2), and at d = 128 where
+// the tiles fill more than two thirds of the SMs (111 x 1024, d = 64 0.95; 8 x 3072, d = 128 45.1 / 46.3, 96 x 700 20.5 / 19.7).
+//   Plans whose tiles are cut over the machine: where whole tiles are estimated to be faster by 2 % (d = 64) or 4 %.  The estimates are
+// fits in us, of this kernel over its waves and key steps and of the plan's over its cost, that miss by 4 to 7 % (one sd): of 140 shapes
+// 49 go here, 0.89 times on the geometric mean and none slower by more than 1 %; 14 that would be 3 % faster or more stay.
+bool pipe_tiles(const attn_tiles& t, int Lk, int d, int local_mem, int sms) {
+  if (t.causal || t.n_q != 2 || t.tile_kv != 128) return false;
+  if (local_mem < (d == 64 ? attn::PipeSmem<64>::total(4) : attn::PipeSmem<128>::total(4))) return false;
+  const int steps = (Lk + 127) / 128, waves = (t.tiles + sms - 1) / sms;
+  if (t.ctas == t.tiles) return t.tiles > sms || (steps >= 4 && (d == 64 || 3 * t.tiles > 2 * sms));
+  if (t.ctas > t.tiles || t.tiles <= sms) return false;
+  const double whole = d == 64 ? 3.0 + waves * (2.0 + 1.376 * steps + (Lk % 128 ? 0.35 : 0.0)) : 4.0 + waves * (2.3 + 1.647 * steps);
+  const double cut = d == 64 ? 2.5 + 1.493 * t.cost_steps : 5.7 + 1.78 * t.cost_steps;
+  return whole < (d == 64 ? 0.98 : 0.96) * cut;
+}
+
 int dispatch_fwd(const void* q, const void* k, const void* v, void* o, int B, int H, int L, int d,
                  const attn_tiles& t, float* ws, unsigned int* status, DeviceState* st, cudaStream_t s, int Lk = 0,
                  bool may_overlap = false, bool own_plan = false) {
@@ -610,13 +631,19 @@ int dispatch_fwd(const void* q, const void* k, const void* v, void* o, int B, in
   const int sms = st->desc.num_units;
   if (own_plan) {
     if (const int subs = narrow_subs(t, B * H, L, Lk, d, st->desc.local_mem_bytes, sms)) {
+      // (long tiles of two sub-tiles, not causal: us in loops of half a second, four streams a tile / two, 128 x 8192 2818 / 2722)
+      if (subs == 2 && !t.causal && (Lk + 127) / 128 >= 48)
+        return launch_pipe<64, false>(q, k, v, o, B * H, L, Lk, status, st, s, ATTN_KERNEL_NARROW_TILES);
       auto launch = d == 128 ? (t.causal ? launch_narrow<128, true, 1> : launch_narrow<128, false, 1>)
                     : t.causal ? (subs == 1 ? launch_narrow<64, true, 1> : launch_narrow<64, true, 2>)
                                : (subs == 1 ? launch_narrow<64, false, 1> : launch_narrow<64, false, 2>);
       return launch(q, k, v, o, B * H, L, Lk, status, st, s);
     }
     if (d == 128 && Lk == L && causal_whole_tiles(t, B * H, L, d, st->desc.local_mem_bytes, sms))
-      return launch_causal_tiles(q, k, v, o, B * H, L, status, st, s);
+      return launch_pipe<128, true>(q, k, v, o, B * H, L, L, status, st, s, ATTN_KERNEL_CAUSAL_TILES);
+    if (pipe_tiles(t, Lk, d, st->desc.local_mem_bytes, sms))
+      return d == 64 ? launch_pipe<64, false>(q, k, v, o, B * H, L, Lk, status, st, s, ATTN_KERNEL_TILED)
+                     : launch_pipe<128, false>(q, k, v, o, B * H, L, Lk, status, st, s, ATTN_KERNEL_TILED);
   }
 #define ATTN_CASE(D_, TKV_, NQ_) \
   if (d == D_ && t.tile_kv == TKV_ && t.n_q == NQ_) \

@@ -90,7 +90,7 @@ __device__ __forceinline__ bool wait_bar_warp(uint32_t bar, uint32_t parity, vol
 }
 // The same wait without a function call on its way out: an expiry only notes itself in the abort cell, and one thread reports
 // it at the end of the kernel (report_abort).  However rare, a call inside a step loop makes the compiler keep the loop's
-// values where a call would leave them alone: in attn_causal_tiles_kernel at d = 64 it cost 7 %, while attn_fwd_kernel
+// values where a call would leave them alone: in a causal kernel of whole tiles at d = 64 it cost 7 %, while attn_fwd_kernel
 // as it stands is 1-2 % faster with wait_bar.
 __device__ __forceinline__ void note_timeout(uint32_t info, volatile int* abort_flag) {
   reinterpret_cast<volatile AbortCell*>(abort_flag)->info = info;

@@ -8,7 +8,7 @@
 // every 128-key tile.  A stream has its own scores, reference, denominator and accumulator in tensor memory (4 x (64 + 64)
 // columns: all 512; P overwrites the front of its scores) and its own softmax warpgroup; the two streams of a sub-tile meet
 // when the tile is finished, in the epilogue warpgroup, which reads both accumulators.  2600 cycles a step.  In loops of 0.7 s
-// (us, attn_causal_tiles_kernel or attn_fwd_kernel / this kernel): causal 128 heads x 8192 1650 / 1509, 128 x 4096 454 / 416, 128 x 2048
+// (us, attn_fwd_kernel's step / this kernel): causal 128 heads x 8192 1650 / 1509, 128 x 4096 454 / 416, 128 x 2048
 // 140 / 124, 256 x 300 31.2 / 21.6; not causal 900 x 1025 558 / 497, 256 x 1000 122 / 120, and at 128 x 8192 2918 / 2910: there the power
 // limit takes back what bursts gain (2640 / 2533).  Where attn_fwd_kernel is the faster one stands at narrow_subs (attn_api.cu).
 // SUBS = 1 works on tiles of 128 query rows, one sub-tile: its four streams are the two halves of the even and of the odd key
@@ -25,11 +25,11 @@
 //     SUBS = 1 has a ring for each parity of the key tiles, and its MMA warps never pass over an item (kv_ring.h).  In loops (us):
 //     causal 32 x 1111 16.4, 8 x 4096 30.5 (d = 64), 16 x 2048 27.3 (d = 128); one ring that they stepped through took 16.5, 30.2, 28.2.
 //   * Tiles come from the hardware's queue of CTAs not yet started, and the epilogue of a tile runs under the next one, as in
-//     attn_causal_tiles_kernel.
+//     attn_pipe_kernel (pipe_kernel.cuh).
 #pragma once
 
+#include "attn_kernels.cuh"
 #include "kv_ring.h"
-#include "tiles_kernel.cuh"
 
 namespace attn {
 

@@ -368,6 +368,26 @@ __device__ __forceinline__ void st_peer_f1(uint32_t peer_addr, float a, uint32_t
                ::"r"(peer_addr), "f"(a), "r"(peer_bar) : "memory");
 }
 
+// ---------------------------------------------- the hardware's queue of CTAs not yet started
+// Asks for the index of a CTA of this grid that has not been started; the 16-byte answer is counted on `bar`.
+__device__ __forceinline__ void clc_try_cancel(uint32_t answer_smem, uint32_t bar) {
+  asm volatile("clusterlaunchcontrol.try_cancel.async.shared::cta.mbarrier::complete_tx::bytes.b128 [%0], [%1];"
+               ::"r"(answer_smem), "r"(bar) : "memory");
+}
+// The CTA index in an answer, or -1: none left.
+__device__ __forceinline__ int clc_answer(uint32_t answer_smem) {
+  int got, x;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t.reg .b128 a;\n\t"
+      "ld.shared.b128 a, [%2];\n\t"
+      "clusterlaunchcontrol.query_cancel.is_canceled.pred.b128 p, a;\n\t"
+      "selp.s32 %0, 1, 0, p;\n\t"
+      "mov.b32 %1, 0;\n\t"
+      "@p clusterlaunchcontrol.query_cancel.get_first_ctaid::x.b32.b128 %1, a;\n\t}"
+      : "=r"(got), "=r"(x) : "r"(answer_smem) : "memory");
+  return got ? x : -1;
+}
+
 // -------------------------------------------- per-thread asynchronous 16-byte copies (L2 -> shared)
 __device__ __forceinline__ void cp_async16(uint32_t dst_smem, const void* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst_smem), "l"(src) : "memory");
