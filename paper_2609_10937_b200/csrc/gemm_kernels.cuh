@@ -160,40 +160,64 @@ gemm_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CU
     }
   } else if (warp == 1) {
     // ============================================================ MMA issuer
-    bool ok = run;
+    // One sub-tile: one lane walks the loop (see gemm_small_kernel; 128 x 128 x 8192 33.6 us with the whole warp).  Two sub-tiles: the
+    // whole warp does, one lane issues: their eight instructions a step cover its waits.
     int stage = 0;
     uint32_t phase = 0, tile_ctr = 0;
     constexpr uint32_t idesc = make_idesc_bf16(kSub, kTileN, B_KN);
     constexpr uint32_t hi_k = attn::desc_hi_sw128(1024);
-    for (long long t = blockIdx.x; ok && t < tiles; t += gridDim.x, ++tile_ctr) {
-      if (tile_ctr > 0) {
-        ok = attn::wait_bar_warp(smem_u32(&misc->acc_empty), (tile_ctr - 1) & 1, abort_flag, attn::wait_info(kRoleGemmMma, 2, tile_ctr));
-        if (!ok) break;
-        tc_fence_after();
+    // (one lane) The products of sub-tile `sub` with the stage's K step.
+    auto issue = [&](int sub, int ks) __attribute__((always_inline)) {
+      const uint32_t a_smem = smem_base + stage * kStageBytes, b_smem = a_smem + kStageA;
+      const uint32_t a_lo = attn::desc_lo(a_smem + sub * (kSub * 128), 16);
+      const uint32_t b_lo = B_KN ? attn::desc_lo(b_smem, kTileK * 128) : attn::desc_lo(b_smem, 16);
+#pragma unroll
+      for (int k16 = 0; k16 < kTileK / 16; ++k16) {
+        const uint64_t a = attn::desc_from_words(a_lo + ((k16 * 32) >> 4), hi_k);
+        // K-major B: 16 columns further along the swizzle row; MN-major B: 16 key rows = 2048 bytes further
+        const uint64_t b = attn::desc_from_words(b_lo + ((B_KN ? k16 * 2048 : k16 * 32) >> 4), hi_k);
+        umma_ss(tmem_base + sub * kTileN, a, b, idesc, (ks > 0 || k16 > 0) ? 1u : 0u);
       }
-      for (int ks = 0; ok && ks < p.k_steps; ++ks) {
-        if (!attn::wait_bar_warp(smem_u32(&misc->full[stage]), phase, abort_flag, attn::wait_info(kRoleGemmMma, 1, ks))) { ok = false; break; }
-        tc_fence_after();
-        if (elect_one()) {
-          const uint32_t a_smem = smem_base + stage * kStageBytes, b_smem = a_smem + kStageA;
-          const uint32_t b_lo = B_KN ? attn::desc_lo(b_smem, kTileK * 128) : attn::desc_lo(b_smem, 16);
-#pragma unroll
-          for (int sub = 0; sub < 2; ++sub) {
-            if (sub >= p.n_sub) break;
-            const uint32_t a_lo = attn::desc_lo(a_smem + sub * (kSub * 128), 16);
-#pragma unroll
-            for (int k16 = 0; k16 < kTileK / 16; ++k16) {
-              const uint64_t a = attn::desc_from_words(a_lo + ((k16 * 32) >> 4), hi_k);
-              // K-major B: 16 columns further along the swizzle row; MN-major B: 16 key rows = 2048 bytes further
-              const uint64_t b = attn::desc_from_words(b_lo + ((B_KN ? k16 * 2048 : k16 * 32) >> 4), hi_k);
-              umma_ss(tmem_base + sub * kTileN, a, b, idesc, (ks > 0 || k16 > 0) ? 1u : 0u);
-            }
+    };
+    if (p.n_sub == 1) {
+      if (run && elect_one()) {
+        bool ok = true;
+        for (long long t = blockIdx.x; ok && t < tiles; t += gridDim.x, ++tile_ctr) {
+          if (tile_ctr > 0) {
+            if (!attn::wait_bar(smem_u32(&misc->acc_empty), (tile_ctr - 1) & 1, abort_flag, attn::wait_info(kRoleGemmMma, 2, tile_ctr))) break;
+            tc_fence_after();
           }
-          umma_commit(smem_u32(&misc->empty[stage]));
-          if (ks == p.k_steps - 1) umma_commit(smem_u32(&misc->acc_full));
+          for (int ks = 0; ks < p.k_steps; ++ks) {
+            if (!attn::wait_bar(smem_u32(&misc->full[stage]), phase, abort_flag, attn::wait_info(kRoleGemmMma, 1, ks))) { ok = false; break; }
+            tc_fence_after();
+            issue(0, ks);
+            umma_commit(smem_u32(&misc->empty[stage]));
+            if (ks == p.k_steps - 1) umma_commit(smem_u32(&misc->acc_full));
+            if (++stage == p.stages) { stage = 0; phase ^= 1u; }
+          }
         }
-        __syncwarp();
-        if (++stage == p.stages) { stage = 0; phase ^= 1u; }
+      }
+      __syncwarp();
+    } else {
+      bool ok = run;
+      for (long long t = blockIdx.x; ok && t < tiles; t += gridDim.x, ++tile_ctr) {
+        if (tile_ctr > 0) {
+          ok = attn::wait_bar_warp(smem_u32(&misc->acc_empty), (tile_ctr - 1) & 1, abort_flag, attn::wait_info(kRoleGemmMma, 2, tile_ctr));
+          if (!ok) break;
+          tc_fence_after();
+        }
+        for (int ks = 0; ok && ks < p.k_steps; ++ks) {
+          if (!attn::wait_bar_warp(smem_u32(&misc->full[stage]), phase, abort_flag, attn::wait_info(kRoleGemmMma, 1, ks))) { ok = false; break; }
+          tc_fence_after();
+          if (elect_one()) {
+            issue(0, ks);
+            issue(1, ks);
+            umma_commit(smem_u32(&misc->empty[stage]));
+            if (ks == p.k_steps - 1) umma_commit(smem_u32(&misc->acc_full));
+          }
+          __syncwarp();
+          if (++stage == p.stages) { stage = 0; phase ^= 1u; }
+        }
       }
     }
   } else {
@@ -581,14 +605,17 @@ gemm_small_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constan
     }
   } else if (warp == 1) {
     // ============================================================ MMA issuer
-    int stage = 0;
-    uint32_t phase = 0;
-    constexpr uint32_t idesc = make_idesc_bf16(kSub, kSmallTile, B_KN);
-    constexpr uint32_t hi_k = attn::desc_hi_sw128(1024);
-    for (int ks = 0; run && ks < p.k_steps; ++ks) {
-      if (!attn::wait_bar_warp(smem_u32(&misc->full[stage]), phase, abort_flag, attn::wait_info(kRoleGemmMma, 1, ks))) break;
-      tc_fence_after();
-      if (elect_one()) {
+    // One lane walks the loop.  With the whole warp in it a K step took 490 cycles, the vote and the reconvergence after its wait among
+    // them, where the four instructions take 256: 300 x 520 x 8192 35.6 us, one lane 21.9.  (gemm_pair_kernel's longer instructions cover
+    // that, and there one lane is slower: 4096^3 93.4 / 102.4.)
+    if (run && elect_one()) {
+      int stage = 0;
+      uint32_t phase = 0;
+      constexpr uint32_t idesc = make_idesc_bf16(kSub, kSmallTile, B_KN);
+      constexpr uint32_t hi_k = attn::desc_hi_sw128(1024);
+      for (int ks = 0; ks < p.k_steps; ++ks) {
+        if (!attn::wait_bar(smem_u32(&misc->full[stage]), phase, abort_flag, attn::wait_info(kRoleGemmMma, 1, ks))) break;
+        tc_fence_after();
         const uint32_t a_smem = smem_base + stage * kSmallStageBytes, b_smem = a_smem + kSmallTile * kTileK * 2;
         const uint32_t a_lo = attn::desc_lo(a_smem, 16);
         const uint32_t b_lo = B_KN ? attn::desc_lo(b_smem, kTileK * 128) : attn::desc_lo(b_smem, 16);
@@ -600,10 +627,10 @@ gemm_small_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constan
         }
         umma_commit(smem_u32(&misc->empty[stage]));
         if (ks == p.k_steps - 1) umma_commit(smem_u32(&misc->acc_full));
+        if (++stage == p.stages) { stage = 0; phase ^= 1u; }
       }
-      __syncwarp();
-      if (++stage == p.stages) { stage = 0; phase ^= 1u; }
     }
+    __syncwarp();
   } else {
     // ===================================== accumulator -> fp32 [128][128] at the front of the ring (four lane quarters x two halves)
     // 16-byte unit u of row r lies at position u ^ (r mod 32): a warp's rows then spread over the banks
