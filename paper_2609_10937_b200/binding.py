@@ -1,5 +1,8 @@
 """ctypes binding of libattn_b200.so: argument marshalling only.
 
+The four calls of every program (forward, forward_qk, gemm, softmax_rows) go through csrc/py_fast.cpp first, which does the same
+for plain contiguous tensors on the current device without the interpreter; everything else is handled here.
+
 Every step of the attention path runs inside the library's CUDA kernels; this
 module turns torch tensors into device pointers, keeps the caller-owned
 workspace alive and raises on error codes.  There is no CPU fallback: if the
@@ -14,6 +17,7 @@ from pathlib import Path
 
 _PKG = Path(__file__).resolve().parent
 LIB_PATH = _PKG / "libattn_b200.so"
+_FAST_PATH = _PKG / "_fast.so"
 
 ATTN_OK = 0
 ERR_INVALID_ARG, ERR_UNSUPPORTED_SHAPE, ERR_MISALIGNED, ERR_ALIASING = -1, -2, -3, -4
@@ -146,6 +150,40 @@ def lib() -> ctypes.CDLL:
     return _lib
 
 
+class _NoFast:
+    """Stands in for csrc/py_fast.cpp where it has not been built: no call is the usual one."""
+
+    @staticmethod
+    def attn(*args):
+        return None
+
+    gemm = softmax = attn
+
+
+class _LazyFast:
+    """csrc/py_fast.cpp, loaded with the first call."""
+
+    def __getattr__(self, name):
+        global _fast
+        handle = lib()
+        if _FAST_PATH.exists():
+            import torch  # noqa: F401  (whose libraries the module needs)
+            from importlib import machinery, util
+
+            loader = machinery.ExtensionFileLoader(__package__ + "._fast", str(_FAST_PATH))
+            module = util.module_from_spec(util.spec_from_loader(loader.name, loader))
+            loader.exec_module(module)
+            module.bind(*(ctypes.cast(f, ctypes.c_void_p).value for f in (
+                handle.attn_forward_call, handle.gemm_forward_call, handle.softmax_rows_forward_call)))
+            _fast = module
+        else:
+            _fast = _NoFast
+        return getattr(_fast, name)
+
+
+_fast = _LazyFast()
+
+
 def status_string(code: int) -> str:
     return lib().attn_status_string(int(code)).decode()
 
@@ -251,6 +289,9 @@ def forward(q, k, v, o=None, causal=False):
     """O = softmax(Q K^T / sqrt(d)) V with the closed-form default tiles (asynchronous).
 
     causal=True: row i attends to keys 0..i only."""
+    done = _fast.attn(q, k, v, o, causal, False)
+    if done is not None:
+        return done
     o, B, H, L, d, dev, stream = _prep(q, k, v, o)
     _call(dev, "attn_forward_causal" if causal else "attn_forward", lib().attn_forward_call,
           _ATTN_CALL(q.data_ptr(), k.data_ptr(), v.data_ptr(), o.data_ptr(), stream, B, H, L, L, d, 1 if causal else 0),
@@ -334,6 +375,9 @@ def plan_qk(desc: AttnHwDesc, B: int, H: int, Lq: int, Lk: int, d: int) -> AttnT
 
 def forward_qk(q, k, v, o=None):
     """O = softmax(Q K^T / sqrt(d)) V for q [B, H, Lq, d] and k, v [B, H, Lk, d] (contiguous CUDA bf16)."""
+    done = _fast.attn(q, k, v, o, False, True)
+    if done is not None:
+        return done
     torch = _torch
     for name, x in (("q", q), ("k", k), ("v", v)):
         if x.dtype != torch.bfloat16 or not x.is_cuda or not x.is_contiguous() or x.dim() != 4:
@@ -463,6 +507,10 @@ def gemm(a, b, c=None, *, b_layout="kn", cta_pair=0, tile_n=0, tail_split=0):
 
     cta_pair (1 | 2), tile_n (128 | 256) and tail_split (-1: whole tiles in the last wave) override the closed-form
     tiles (tile sweep only; 0 keeps them)."""
+    if not (cta_pair or tile_n or tail_split):
+        done = _fast.gemm(a, b, c, b_layout)
+        if done is not None:
+            return done
     torch = _torch
     batch, M, K = _mat(a, "a")
     b_batch, rows, cols = _mat(b, "b")
@@ -493,6 +541,9 @@ def gemm(a, b, c=None, *, b_layout="kn", cta_pair=0, tile_n=0, tail_split=0):
 
 def softmax_rows(s, scale: float, out=None):
     """Row softmax of scale * s over the last dimension (bf16, CUDA, contiguous); out may be s."""
+    done = _fast.softmax(s, scale, out)
+    if done is not None:
+        return done
     torch = _torch
     if s.dtype != torch.bfloat16 or not s.is_cuda or not s.is_contiguous():
         raise ValueError("s must be a contiguous CUDA bfloat16 tensor")
