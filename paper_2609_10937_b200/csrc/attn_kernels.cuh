@@ -337,6 +337,7 @@ struct FwdMisc {               // lives in the last 3072 bytes of dynamic shared
   uint64_t q_empty;            // every product that reads the Q tile of a segment has finished
   uint64_t o_free[2];          // the epilogue of a segment has read its O accumulator
   uint64_t s_free[2];          // d = 64: the softmax warpgroup holds the step's scores in registers
+  uint64_t turn[2];            // d = 128: the sub-tile's MMA warp may issue its step
   uint64_t peers_ready;        // cluster: every other CTA of the tile has finished with its K/V ring
   uint64_t data_ready[8][2];   // cluster: the other CTAs' parts of softmax warp w's rows have landed ([1]: columns 64..)
   AbortCell abort;
@@ -421,6 +422,67 @@ __device__ __forceinline__ void exp_chunk(const uint32_t* s, const ExpConsts& k,
     pk[j] = pack_bf16x2(e0, e1);
   }
 }
+__device__ __forceinline__ float lg2_approx(float x) {
+  float y;
+  asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+__device__ __forceinline__ uint64_t pair_of(const uint32_t* s) { return pack_f32x2(__uint_as_float(s[0]), __uint_as_float(s[1])); }
+// The operations of exp_chunk_in_place: volatile, so that they reach the assembler in the order in which they stand there.
+__device__ __forceinline__ float ex2_in_order(float x) {
+  float y;
+  asm volatile("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+__device__ __forceinline__ uint64_t fma2_in_order(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t d;
+  asm volatile("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+__device__ __forceinline__ uint64_t add2_in_order(uint64_t a, uint64_t b) {
+  uint64_t d;
+  asm volatile("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ uint32_t pack_in_order(const uint32_t* e) {
+  uint32_t d;
+  asm volatile("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(d) : "r"(e[1]), "r"(e[0]));
+  return d;
+}
+// Which of eight pairs take the polynomial.
+template <int kPolyPairs>
+__host__ __device__ constexpr bool poly_pair(int j) {
+  return kPolyPairs == 1 ? (j & 7) == 7 : kPolyPairs == 3 && ((j & 7) == 2 || (j & 7) == 5 || (j & 7) == 7);
+}
+// exp2(s * scale - m) of 32 scores in place and as bf16 pairs in pk; beside them, with kSum, the 32 exponentials at `done` are
+// added to the partial sums.  A pair's argument is computed three pairs ahead, its bf16 two pairs later.
+template <int kPolyPairs, bool kSum>
+__device__ __forceinline__ void exp_chunk_in_place(uint32_t* s, const uint32_t* done, uint64_t (&sum)[2], const ExpConsts& k, uint64_t neg_m2,
+                                                   uint32_t (&pk)[16]) {
+  constexpr int kAhead = 3;
+  uint64_t x[16];
+#pragma unroll
+  for (int j = 0; j < kAhead; ++j) x[j] = fma2_in_order(pair_of(s + 2 * j), k.scale2, neg_m2);
+#pragma unroll
+  for (int j = 0; j < 18; ++j) {
+    if (j < 16) {
+      float a, b;
+      if (poly_pair<kPolyPairs>(j)) {
+        exp2_poly_pair(x[j], k, a, b);
+      } else {
+        unpack_f32x2(x[j], a, b);
+        a = ex2_in_order(a);
+      }
+      if (j + kAhead < 16) x[j + kAhead] = fma2_in_order(pair_of(s + 2 * (j + kAhead)), k.scale2, neg_m2);
+      if (!poly_pair<kPolyPairs>(j)) b = ex2_in_order(b);
+      s[2 * j] = __float_as_uint(a);
+      s[2 * j + 1] = __float_as_uint(b);
+      if (kSum) sum[j & 1] = add2_in_order(sum[j & 1], pair_of(done + 2 * j));
+    }
+    if (j >= 2) pk[j - 2] = pack_in_order(s + 2 * (j - 2));
+  }
+}
+
 // 32 fp32 values of one output row -> bf16, written into a 128-byte-swizzled [128][64] staging chunk.
 __device__ __forceinline__ void stage_row_chunk(uint32_t stage_out, int c, int row, const float (&val)[32]) {
   const uint32_t chunk_base = stage_out + (c >> 1) * (kSub * 128) + row * 128;
@@ -451,6 +513,11 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
   // warpgroup has read it into registers, and the next step's Q K^T runs during this step's exponentials instead
   // of after this step's P V.  (d = 128 fills tensor memory: P overwrites the front of the score buffer.)
   constexpr bool kSplitP = (D == 64) && NQ == 2 && (NQ * (S_COLS + D) + NQ * (TKV / 2) <= 512);
+  // Causal, d = 128: an MMA warp for each sub-tile, in turns, and the softmax step of attn_pipe_kernel (pipe_kernel.cuh).  us in graphs of 8
+  // calls, one MMA warp and the step below / this: clusters 5 x 640 15.7 / 15.3, 16 x 1024 19.8 / 18.6, ranges 3 x 8192 64.5 / 59.9; of 203 shapes on a
+  // grid none slower, 0.957 times.  Not causal it is no gain: clusters 0.995 times with 23 of 121 shapes up to 3 % slower (1 x 2048 16.1 /
+  // 16.6), cut tiles 1.008.
+  constexpr bool kTwoMma = CAUSAL && NQ == 2 && !kSplitP;
   constexpr int P_COL0 = NQ * (S_COLS + D);           // kSplitP: bf16 P, TKV / 2 columns per sub-tile
   constexpr uint32_t kPartBytes = 32 * D * 4 + 256;   // cluster: one warp's part -- O of 32 rows, then m and delta
   constexpr int kTmemUsed = NQ * (S_COLS + D) + (kSplitP ? NQ * (TKV / 2) : 0);
@@ -497,9 +564,10 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     mbar_init(smem_u32(&misc->q_full[1]), 1);
     for (int s = 0; s < kMaxStages; ++s) {
       mbar_init(smem_u32(&misc->kv_full[s]), 1);
-      mbar_init(smem_u32(&misc->kv_empty[s]), 1);
+      mbar_init(smem_u32(&misc->kv_empty[s]), kTwoMma ? 2 : 1);
     }
     for (int i = 0; i < 2; ++i) {
+      mbar_init(smem_u32(&misc->turn[i]), 1);
       mbar_init(smem_u32(&misc->s_full[i]), 1);
       mbar_init(smem_u32(&misc->p_full[i]), 2 * kSub);   // softmax rows + correction rows
       mbar_init(smem_u32(&misc->p_half[i]), kSub);
@@ -508,7 +576,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
       mbar_init(smem_u32(&misc->o_free[i]), kSub);
       mbar_init(smem_u32(&misc->s_free[i]), kSub);
     }
-    mbar_init(smem_u32(&misc->q_empty), 1);
+    mbar_init(smem_u32(&misc->q_empty), kTwoMma ? 2 : 1);
     if constexpr (CLUSTER) {
       {
         // Partials travel through distributed shared memory (see the end of a segment).  The merging warps of
@@ -550,7 +618,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
   // segments of this CTA and gives the parity of the per-step barriers.
   if (warp < 4 * NQ) {
     // ===================================================== softmax warpgroup
-    setmaxnreg_inc<(NQ == 2) ? 192 : 232>();
+    setmaxnreg_inc<kTwoMma ? 200 : NQ == 2 ? 192 : 232>();
     const int i = warp >> 2;
     const int row = (warp & 3) * 32 + lane;
     const uint32_t lane_base = tmem_base + ((uint32_t)((warp & 3) * 32) << 16);
@@ -574,7 +642,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
       while (ok && next_segment<CAUSAL>(u, u_hi, seg_ctr, p.n_steps, p.q_tiles, p.ratio, p.head_units, NQ * kSub, sg, p.seg_skip)) {
         const int tile = sg.tile, j0 = sg.j0, j1 = sg.j1, n = sg.n, bh = sg.bh, q_row0 = sg.q_row0, seg = sg.seg;
         (void)tile; (void)j0; (void)j1; (void)bh; (void)q_row0; (void)seg;
-      float m_run = -INFINITY, delta = 0.f;
+      float m_run = -INFINITY, delta = 0.f, lim_move = 0.f;
       const uint32_t g_seg0 = g;                         // first step of this segment
       (void)g_seg0;
       // One KV step of this sub-tile.  The masked variant (a ragged last KV tile, or a causal step that
@@ -625,6 +693,45 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
         // Otherwise the reference stays stale, which changes nothing in exact arithmetic because
         // delta and O carry the same factor.  First step: m_run = -inf, gap = +inf, alpha = 0.
         // (masked steps can leave a row with no admissible key yet: keep the reference finite)
+        if constexpr (kTwoMma) {
+          // (as in attn_pipe_kernel; a masked step can leave a row that has had no admissible key yet: its reference stays finite)
+          const float m_cand = kMasked ? fmaxf(mx * scale, kEmptyReference) : mx * scale;
+          const float gap = m_cand - m_run;
+          const bool move = gap > lim_move;
+          m_run = move ? m_cand : m_run;
+          const uint64_t neg_m2 = pack_f32x2(-m_run, -m_run);
+          const float alpha = move ? ex2_approx(-gap) : 1.0f;
+          misc->alpha[i][g & 1][row] = alpha;
+          mbar_arrive(bar_a);
+          delta *= alpha;
+          uint64_t sum[2] = {0ull, 0ull};
+          uint32_t pk[16], pk2[16];
+          exp_chunk_in_place<1, false>(&s[0], s, sum, ek, neg_m2, pk2);
+          tmem_st16(p_tmem, pk2);
+          if constexpr (TKV == 128) {
+            exp_chunk_in_place<1, true>(&s[32], &s[0], sum, ek, neg_m2, pk);
+            tmem_st16(p_tmem + 16, pk);
+          }
+          exp_chunk_in_place<1, true>(&s[TKV / 2], &s[TKV / 2 - 32], sum, ek, neg_m2, pk2);
+          tmem_wait_st();
+          tc_fence_before();
+          mbar_arrive(bar_p);
+          tmem_st16(p_tmem + TKV / 4, pk2);
+          if constexpr (TKV == 128) {
+            exp_chunk_in_place<1, true>(&s[96], &s[64], sum, ek, neg_m2, pk);
+            tmem_st16(p_tmem + 48, pk);
+          }
+          tmem_wait_st();
+          tc_fence_before();
+          mbar_arrive(bar_h);
+#pragma unroll
+          for (int j = 0; j < 16; ++j) sum[j & 1] = add_f32x2(sum[j & 1], pair_of(&s[TKV - 32 + 2 * j]));
+          float s0, s1;
+          unpack_f32x2(add_f32x2(sum[0], sum[1]), s0, s1);
+          delta += s0 + s1;
+          lim_move = fminf(fmaxf(lg2_approx(delta) - 4.0f, 0.f), kRescaleThreshold);
+          return true;
+        }
         const float m_cand = kMasked ? fmaxf(fmaxf(m_run, mx * scale), kEmptyReference) : fmaxf(m_run, mx * scale);
         const float gap = m_cand - m_run;
         const float shrink = ex2_approx(-gap);             // 2^-gap: the rescale factor if the reference moves
@@ -1142,14 +1249,82 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
       if (!ok) break;
       }
     }
-  } else if (warp == 12) {
+  } else if (kTwoMma && (warp == 12 || warp == 14)) {
+    // ============================================================ MMA issuer of one sub-tile
+    // The whole warp walks the loop and the waits (converged control flow keeps descriptors and counters in the uniform datapath);
+    // one elected lane issues.  Issue of a matrix instruction blocks until those in front of it have started, so one warp for both
+    // sub-tiles left the tensor pipe idle during its waits; the two take turns, a step's P V and Q K^T at a time, which also keeps
+    // the softmax warpgroups apart (see attn_pipe_kernel).  (setmaxnreg is warpgroup-aligned: warps 12-15 request the same count.)
+    setmaxnreg_dec<kTwoMma ? 48 : 64>();
+    const int i = warp == 14;
+    const uint32_t s_acc = tmem_base + i * S_COLS, o_acc = tmem_base + O_COL0 + i * D, q_sub = q_smem + i * (kSub * D * 2);
+    bool ok = run;
+    uint32_t g = 0;
+    int stage = 0;
+    uint32_t phase = 0;
+    auto advance = [&]() { if (++stage == p.stages) { stage = 0; phase ^= 1u; } };
+    auto wait = [&](uint64_t* bar, uint32_t parity, uint32_t id, uint32_t tag) __attribute__((always_inline)) -> bool {
+      ok = wait_bar_warp(smem_u32(bar), parity, abort_flag, wait_info(kRoleMma, id, tag));
+      return ok;
+    };
+    auto issue_scores = [&](int k, bool last) __attribute__((always_inline)) {
+      issue_qk<D, TKV>(s_acc, q_sub, ring_smem + k * SM::kStageBytes);
+      umma_commit(smem_u32(&misc->s_full[i]));
+      umma_commit(smem_u32(&misc->kv_empty[k]));
+      // The last product that reads this segment's Q tile is issued one step before the segment ends: the next segment's Q tile
+      // can be fetched while that last step runs.
+      if (last) umma_commit(smem_u32(&misc->q_empty));
+    };
+    if (ok) {
+      long long u = u_lo;
+      int seg_ctr = 0;
+      Segment sg;
+      while (ok && next_segment<CAUSAL>(u, u_hi, seg_ctr, p.n_steps, p.q_tiles, p.ratio, p.head_units, NQ * kSub, sg, p.seg_skip)) {
+        const int n = sg.n, seg = sg.seg;
+        if (!wait(&misc->q_full[i], seg & 1, kBarQ, 0x8000 * i + seg) || !wait(&misc->kv_full[stage], phase, kBarKvFull, g)) break;
+        tc_fence_after();
+        if (elect_one()) issue_scores(stage, n == 1);
+        __syncwarp();
+        advance();
+        for (int jj = 0; ok && jj < n; ++jj, ++g) {
+          const int v_stage = stage;
+          const uint32_t v_phase = phase;
+          advance();
+          const int k_stage = stage;
+          const uint32_t k_phase = phase;
+          const bool more = jj + 1 < n;
+          if (more) advance();
+          const uint32_t v_smem = ring_smem + v_stage * SM::kStageBytes;
+          if (!wait(&misc->kv_full[v_stage], v_phase, kBarKvFull, g)) break;
+          if (more && !wait(&misc->kv_full[k_stage], k_phase, kBarKvFull, g)) break;
+          // the previous segment's epilogue must have read O before the first product overwrites it
+          if (jj == 0 && seg > 0 && !wait(&misc->o_free[i], (seg - 1) & 1, kBarOFull, 0x8000 | seg)) break;
+          if (!wait(&misc->turn[i], (g + 1 + i) & 1, kBarSync, g)) break;                   // (sub-tile 0 begins)
+          if (!wait(&misc->p_full[i], g & 1, kBarPFull, g)) break;
+          tc_fence_after();
+          if (elect_one()) issue_pv<D, TKV>(o_acc, s_acc, v_smem, jj > 0, TKV * 128, 1024, 0, TKV / 32);
+          __syncwarp();
+          if (!wait(&misc->p_half[i], g & 1, kBarPFull, 0x8000 | g)) break;
+          tc_fence_after();
+          if (elect_one()) {
+            issue_pv<D, TKV>(o_acc, s_acc, v_smem, true, TKV * 128, 1024, TKV / 32, TKV / 16);
+            umma_commit(smem_u32(&misc->o_full[i]));
+            if (more) issue_scores(k_stage, jj + 2 == n);
+            mbar_arrive(smem_u32(&misc->turn[i ^ 1]));
+            umma_commit(smem_u32(&misc->kv_empty[v_stage]));
+          }
+          __syncwarp();
+        }
+      }
+    }
+  } else if (!kTwoMma && warp == 12) {
     // ============================================================ MMA issuer
     // The whole warp walks the loop and the waits (converged control flow keeps descriptors and
     // counters in the uniform datapath); one elected lane issues the matrix instructions and the
     // commits.  Sub-tiles are served strictly in turn: that order is what keeps the two softmax
     // warpgroups half a step apart, so that one computes exponentials while the tensor pipe works
     // for the other.  (setmaxnreg is warpgroup-aligned: warps 12-15 request the same count.)
-    setmaxnreg_dec<64>();
+    setmaxnreg_dec<kTwoMma ? 48 : 64>();
     bool ok = run;
     uint32_t g = 0;
     int stage = 0;
@@ -1302,7 +1477,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     }
   } else if (warp == 13) {
     // ========================================================== TMA producer
-    setmaxnreg_dec<64>();
+    setmaxnreg_dec<kTwoMma ? 48 : 64>();
     if (run && elect_one()) {
       int stage = 0;
       uint32_t phase = 0;
@@ -1365,7 +1540,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
       }
     }
   } else {
-    setmaxnreg_dec<64>();
+    setmaxnreg_dec<kTwoMma ? 48 : 64>();
   }
   tc_fence_before();
   __syncthreads();

@@ -122,67 +122,6 @@ __device__ __forceinline__ void wait_on(uint32_t bar, uint32_t parity, volatile 
 }
 __device__ __forceinline__ bool any_dead(bool dead) { return __any_sync(0xffffffffu, dead); }
 
-__device__ __forceinline__ float lg2_approx(float x) {
-  float y;
-  asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
-__device__ __forceinline__ uint64_t pair_of(const uint32_t* s) { return pack_f32x2(__uint_as_float(s[0]), __uint_as_float(s[1])); }
-// The operations of exp_chunk_in_place: volatile, so that they reach the assembler in the order in which they stand there.
-__device__ __forceinline__ float ex2_in_order(float x) {
-  float y;
-  asm volatile("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
-__device__ __forceinline__ uint64_t fma2_in_order(uint64_t a, uint64_t b, uint64_t c) {
-  uint64_t d;
-  asm volatile("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-  return d;
-}
-__device__ __forceinline__ uint64_t add2_in_order(uint64_t a, uint64_t b) {
-  uint64_t d;
-  asm volatile("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
-__device__ __forceinline__ uint32_t pack_in_order(const uint32_t* e) {
-  uint32_t d;
-  asm volatile("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(d) : "r"(e[1]), "r"(e[0]));
-  return d;
-}
-// Which of eight pairs take the polynomial.
-template <int kPolyPairs>
-__host__ __device__ constexpr bool poly_pair(int j) {
-  return kPolyPairs == 1 ? (j & 7) == 7 : kPolyPairs == 3 && ((j & 7) == 2 || (j & 7) == 5 || (j & 7) == 7);
-}
-// exp2(s * scale - m) of 32 scores in place and as bf16 pairs in pk; beside them, with kSum, the 32 exponentials at `done` are
-// added to the partial sums.  A pair's argument is computed three pairs ahead, its bf16 two pairs later.
-template <int kPolyPairs, bool kSum>
-__device__ __forceinline__ void exp_chunk_in_place(uint32_t* s, const uint32_t* done, uint64_t (&sum)[2], const ExpConsts& k, uint64_t neg_m2,
-                                                   uint32_t (&pk)[16]) {
-  constexpr int kAhead = 3;
-  uint64_t x[16];
-#pragma unroll
-  for (int j = 0; j < kAhead; ++j) x[j] = fma2_in_order(pair_of(s + 2 * j), k.scale2, neg_m2);
-#pragma unroll
-  for (int j = 0; j < 18; ++j) {
-    if (j < 16) {
-      float a, b;
-      if (poly_pair<kPolyPairs>(j)) {
-        exp2_poly_pair(x[j], k, a, b);
-      } else {
-        unpack_f32x2(x[j], a, b);
-        a = ex2_in_order(a);
-      }
-      if (j + kAhead < 16) x[j + kAhead] = fma2_in_order(pair_of(s + 2 * (j + kAhead)), k.scale2, neg_m2);
-      if (!poly_pair<kPolyPairs>(j)) b = ex2_in_order(b);
-      s[2 * j] = __float_as_uint(a);
-      s[2 * j + 1] = __float_as_uint(b);
-      if (kSum) sum[j & 1] = add2_in_order(sum[j & 1], pair_of(done + 2 * j));
-    }
-    if (j >= 2) pk[j - 2] = pack_in_order(s + 2 * (j - 2));
-  }
-}
-
 template <int D, bool CAUSAL>
 __global__ void __launch_bounds__(512, 1)
 attn_pipe_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
