@@ -296,7 +296,7 @@ def kernel_name(plan, d, cluster, last=None, L=0, sms=148):
         steps = -(-L // 128)
         if last[0] == binding.KERNEL_NARROW_TILES and steps >= 48:
             return f"attn_pipe_kernel<{d},0>"
-        if last[0] == binding.KERNEL_TILED and (plan.ctas != plan.tiles or plan.tiles > sms or (steps >= 4 and (d == 64 or 3 * plan.tiles > 2 * sms))):
+        if last[0] == binding.KERNEL_TILED and (plan.ctas != plan.tiles or plan.tiles > sms or (steps >= 4 and (d == 64 or 10 * plan.tiles > 7 * sms))):
             return f"attn_pipe_kernel<{d},0>"
     if last is not None and last[0] == binding.KERNEL_NARROW_TILES:
         return f"attn_narrow_kernel<{d},0,{2 if last[1] == plan.tiles else 1}>"

@@ -608,7 +608,7 @@ int narrow_subs(const attn_tiles& t, int BH, int Lq, int Lk, int d, int local_me
 // Calls, not causal, that pipe_kernel.cuh takes over from attn_fwd_kernel, at either head dimension (us in graphs of 8 calls, attn_fwd_kernel / this).
 //   Plans of whole tiles: with more tiles than SMs always (183 shapes of a grid, 0.81 to 0.99 times: 148 x 1024, d = 64 59.3 / 53.2; 592 x 512,
 // d = 128 75.8 / 63.2).  One wave: from four key steps on (three and fewer 0.98 to 1.05: 64 x 384, d = 64 10.0 / 10.2), and at d = 128 where
-// the tiles fill more than two thirds of the SMs (111 x 1024, d = 64 0.95; 8 x 3072, d = 128 45.1 / 46.3, 96 x 700 20.5 / 19.7).
+// the tiles fill more than seven tenths of the SMs (12 x 1536, d = 64 0.96; 10 x 2560, d = 128 38.7 / 39.7, 24 x 1300 23.8 / 22.7).
 //   Plans whose tiles are cut over the machine: where whole tiles are estimated to be faster by 2 % (d = 64) or 4 %.  The estimates are
 // fits in us, of this kernel over its waves and key steps and of the plan's over its cost, that miss by 4 to 7 % (one sd): of 140 shapes
 // 49 go here, 0.89 times on the geometric mean and none slower by more than 1 %; 14 that would be 3 % faster or more stay.
@@ -616,7 +616,7 @@ bool pipe_tiles(const attn_tiles& t, int Lk, int d, int local_mem, int sms) {
   if (t.causal || t.n_q != 2 || t.tile_kv != 128) return false;
   if (local_mem < (d == 64 ? attn::PipeSmem<64>::total(4) : attn::PipeSmem<128>::total(4))) return false;
   const int steps = (Lk + 127) / 128, waves = (t.tiles + sms - 1) / sms;
-  if (t.ctas == t.tiles) return t.tiles > sms || (steps >= 4 && (d == 64 || 3 * t.tiles > 2 * sms));
+  if (t.ctas == t.tiles) return t.tiles > sms || (steps >= 4 && (d == 64 || 10 * t.tiles > 7 * sms));
   if (t.ctas > t.tiles || t.tiles <= sms) return false;
   const double whole = d == 64 ? 3.0 + waves * (2.0 + 1.376 * steps + (Lk % 128 ? 0.35 : 0.0)) : 4.0 + waves * (2.3 + 1.647 * steps);
   const double cut = d == 64 ? 2.5 + 1.493 * t.cost_steps : 5.7 + 1.78 * t.cost_steps;

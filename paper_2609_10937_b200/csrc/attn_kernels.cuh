@@ -452,7 +452,7 @@ __device__ __forceinline__ uint32_t pack_in_order(const uint32_t* e) {
 // Which of eight pairs take the polynomial.
 template <int kPolyPairs>
 __host__ __device__ constexpr bool poly_pair(int j) {
-  return kPolyPairs == 1 ? (j & 7) == 7 : kPolyPairs == 3 && ((j & 7) == 2 || (j & 7) == 5 || (j & 7) == 7);
+  return kPolyPairs == 1 ? (j & 7) == 7 : kPolyPairs == 2 ? (j & 7) < 2 : (j & 7) == 2 || (j & 7) == 5 || (j & 7) == 7;
 }
 // exp2(s * scale - m) of 32 scores in place and as bf16 pairs in pk; beside them, with kSum, the 32 exponentials at `done` are
 // added to the partial sums.  A pair's argument is computed three pairs ahead, its bf16 two pairs later.
@@ -509,14 +509,15 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
   constexpr int O_COL0 = NQ * S_COLS;                 // O accumulators follow the score buffers
   constexpr int NCH = TKV / 32;                       // 32-column chunks of one score row
   constexpr int kPoly = kPolyPairsPer8;             // polynomial pairs per 8
-  // d = 64 leaves tensor memory for P next to S and O.  The score buffer is then free as soon as the softmax
+  // d = 64, not causal, leaves tensor memory for P next to S and O.  The score buffer is then free as soon as the softmax
   // warpgroup has read it into registers, and the next step's Q K^T runs during this step's exponentials instead
   // of after this step's P V.  (d = 128 fills tensor memory: P overwrites the front of the score buffer.)
-  constexpr bool kSplitP = (D == 64) && NQ == 2 && (NQ * (S_COLS + D) + NQ * (TKV / 2) <= 512);
-  // Causal, d = 128: an MMA warp for each sub-tile, in turns, and the softmax step of attn_pipe_kernel (pipe_kernel.cuh).  us in graphs of 8
-  // calls, one MMA warp and the step below / this: clusters 5 x 640 15.7 / 15.3, 16 x 1024 19.8 / 18.6, ranges 3 x 8192 64.5 / 59.9; of 203 shapes on a
-  // grid none slower, 0.957 times.  Not causal it is no gain: clusters 0.995 times with 23 of 121 shapes up to 3 % slower (1 x 2048 16.1 /
-  // 16.6), cut tiles 1.008.
+  constexpr bool kSplitP = (D == 64) && NQ == 2 && !CAUSAL && (NQ * (S_COLS + D) + NQ * (TKV / 2) <= 512);
+  // Causal: an MMA warp for each sub-tile, in turns, and the softmax step of attn_pipe_kernel (pipe_kernel.cuh), at either head dimension (at
+  // d = 64 too P overwrites the front of its scores then).  us in graphs of 8 calls, one MMA warp and the step below / this: d = 128 clusters 5
+  // x 640 15.7 / 15.3, 16 x 1024 19.8 / 18.6, ranges 3 x 8192 65.0 / 60.4; of 203 shapes on a grid none slower, 0.965 times; d = 64 ranges 2 x
+  // 8192 45.8 / 42.0, of 197 shapes none slower, 0.941 times.  Not causal it is no gain at d = 128: clusters 0.995 times with 23 of 121 shapes up to
+  // 3 % slower (1 x 2048 16.1 / 16.6), cut tiles 1.008.
   constexpr bool kTwoMma = CAUSAL && NQ == 2 && !kSplitP;
   constexpr int P_COL0 = NQ * (S_COLS + D);           // kSplitP: bf16 P, TKV / 2 columns per sub-tile
   constexpr uint32_t kPartBytes = 32 * D * 4 + 256;   // cluster: one warp's part -- O of 32 rows, then m and delta
@@ -695,6 +696,8 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
         // (masked steps can leave a row with no admissible key yet: keep the reference finite)
         if constexpr (kTwoMma) {
           // (as in attn_pipe_kernel; a masked step can leave a row that has had no admissible key yet: its reference stays finite)
+          // One pair of eight takes the polynomial, in a masked step two as in exp_chunk: those steps hold the rows that see few keys.
+          constexpr int kStepPoly = kMasked ? kPolyPairsPer8 : 1;
           const float m_cand = kMasked ? fmaxf(mx * scale, kEmptyReference) : mx * scale;
           const float gap = m_cand - m_run;
           const bool move = gap > lim_move;
@@ -706,19 +709,19 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
           delta *= alpha;
           uint64_t sum[2] = {0ull, 0ull};
           uint32_t pk[16], pk2[16];
-          exp_chunk_in_place<1, false>(&s[0], s, sum, ek, neg_m2, pk2);
+          exp_chunk_in_place<kStepPoly, false>(&s[0], s, sum, ek, neg_m2, pk2);
           tmem_st16(p_tmem, pk2);
           if constexpr (TKV == 128) {
-            exp_chunk_in_place<1, true>(&s[32], &s[0], sum, ek, neg_m2, pk);
+            exp_chunk_in_place<kStepPoly, true>(&s[32], &s[0], sum, ek, neg_m2, pk);
             tmem_st16(p_tmem + 16, pk);
           }
-          exp_chunk_in_place<1, true>(&s[TKV / 2], &s[TKV / 2 - 32], sum, ek, neg_m2, pk2);
+          exp_chunk_in_place<kStepPoly, true>(&s[TKV / 2], &s[TKV / 2 - 32], sum, ek, neg_m2, pk2);
           tmem_wait_st();
           tc_fence_before();
           mbar_arrive(bar_p);
           tmem_st16(p_tmem + TKV / 4, pk2);
           if constexpr (TKV == 128) {
-            exp_chunk_in_place<1, true>(&s[96], &s[64], sum, ek, neg_m2, pk);
+            exp_chunk_in_place<kStepPoly, true>(&s[96], &s[64], sum, ek, neg_m2, pk);
             tmem_st16(p_tmem + 48, pk);
           }
           tmem_wait_st();
