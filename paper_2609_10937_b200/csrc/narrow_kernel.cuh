@@ -18,6 +18,9 @@
 //   * One barrier each way per step: scores ready (commit of Q K^T, which also says that the stream's P V of the step before
 //     is complete) and P ready.  A softmax warp whose reference moved rescales its accumulator itself: that is rare, and
 //     no other warp has to be asked.
+//     Its waits, and the MMA warps', are those of attn_pipe_kernel, without a vote, and so is its decision to move the reference: with a vote
+//     at each wait, the factor computed in every step and the threshold compared after it, 24 shapes of two sub-tiles took 1.02 times as
+//     long, 244 of one 1.01 (d = 64), 119 1.02 (d = 128), causal ones 1.01 (us, before / now: 592 x 384 50.9 / 49.4, 1000 x 256 35.1 / 34.6, 32 x 1111, d = 128 31.7 / 31.0).
 //   * Every stream has an MMA warp of its own, which issues P V of a step and then Q K^T of the stream's next step: what is in
 //     flight for one stream runs under the exponentials of the other three.  One MMA warp that served the streams in turn took
 //     800 cycles a turn, waits and instruction issue together, and bound the step at 3200 cycles.
@@ -202,7 +205,7 @@ attn_narrow_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
     const float scale = p.scale_log2;
     const ExpConsts ek = make_exp_consts(scale);
     const int kv_tail = CAUSAL ? 0 : p.Lk & (TKV - 1);
-    bool ok = run;
+    bool ok = run, dead = false;
     uint32_t g = 0, done = 0;                          // steps of this stream over all tiles; finished tiles
     int tile = blockIdx.x;
     for (int seq = 1; ok && tile >= 0; ++seq) {
@@ -211,12 +214,12 @@ attn_narrow_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
       if (n > 0) {
         // whether this stream's last key tile is the tile's last (SUBS = 1: the last tile is one parity's)
         const bool ends = SUBS == 2 || ((w.n - 1) & 1) == group;
-        float m_run = -INFINITY, delta = 0.f;
+        float m_run = -INFINITY, delta = 0.f, lim_move = 0.f;   // lim_move: as in attn_pipe_kernel
         // One key step.  The masked variant (the causal diagonal, a ragged last key tile) is compiled separately so that the
         // common step pays nothing for it; `lim` is the last key column of this half the thread's row may attend to.
         auto softmax_step = [&](auto mask_tag, int lim, bool first, bool last) __attribute__((always_inline)) -> bool {
           constexpr bool kMasked = decltype(mask_tag)::value;
-          if (!wait_quiet_warp(bar_s, g & 1, abort_flag, wait_info(kRoleSoftmax, kBarSFull, g))) return false;
+          wait_on(bar_s, g & 1, abort_flag, wait_info(kRoleSoftmax, kBarSFull, g), dead);
           tc_fence_after();
           uint32_t s[HKV];
           // load the row in two halves: the maximum of the first half is taken while the second is in flight
@@ -243,22 +246,24 @@ attn_narrow_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
           const float mx = max3(mx_a, chain_max<HKV / 2, 3 * HKV / 4>(s), chain_max<3 * HKV / 4, HKV>(s));
           // Lazy rescale, as in attn_fwd_kernel.  The reference is finite from the first step on, also where a stream's
           // half of the keys holds none that the row may attend to.
-          const float m_cand = max3(m_run, mx * scale, kEmptyReference);
+          const float m_cand = fmaxf(mx * scale, kEmptyReference);
           const float gap = m_cand - m_run;
-          const float shrink = ex2_approx(-gap);
-          const bool move = (gap > kRescaleThreshold) || (gap > 0.f && kDominanceFactor > delta * shrink);
-          const float alpha = move ? shrink : 1.0f;
+          const bool move = gap > lim_move;
           m_run = move ? m_cand : m_run;
           // The step before is complete (see s_full), so the accumulator may be rescaled here; P V of this step waits for P.
-          if (!first && __any_sync(0xffffffffu, move)) {
-            const uint32_t o_tmem = lane_base + O_COL0 + st * D;
+          if (__any_sync(0xffffffffu, move)) {
+            const float alpha = move ? ex2_approx(-gap) : 1.0f;
+            delta *= alpha;
+            if (!first) {
+              const uint32_t o_tmem = lane_base + O_COL0 + st * D;
 #pragma unroll 1
-            for (int c = 0; c < D / 16; ++c) {
-              uint32_t r[16];
-              tmem_ld16(o_tmem + c * 16, r);
+              for (int c = 0; c < D / 16; ++c) {
+                uint32_t r[16];
+                tmem_ld16(o_tmem + c * 16, r);
 #pragma unroll
-              for (int k = 0; k < 16; ++k) r[k] = __float_as_uint(__uint_as_float(r[k]) * alpha);
-              tmem_st16(o_tmem + c * 16, r);
+                for (int k = 0; k < 16; ++k) r[k] = __float_as_uint(__uint_as_float(r[k]) * alpha);
+                tmem_st16(o_tmem + c * 16, r);
+              }
             }
           }
           const uint64_t neg_m2 = pack_f32x2(-m_run, -m_run);
@@ -271,7 +276,7 @@ attn_narrow_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
           }
           float sum0, sum1;
           unpack_f32x2(sum2, sum0, sum1);
-          delta = delta * alpha + (sum0 + sum1);
+          delta += sum0 + sum1;
           if (last) {
             // The epilogue warpgroup finishes the tile.  It has read what stood here two tiles ago: this tile's first scores
             // came after the first P V of the tile before, which waited for that (o_free).  The arrival stands before the one
@@ -286,7 +291,8 @@ attn_narrow_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
           tmem_wait_st();
           tc_fence_before();
           mbar_arrive(bar_p);
-          return true;
+          lim_move = fminf(fmaxf(lg2_approx(delta) - 4.0f, 0.f), kRescaleThreshold);
+          return !any_dead(dead);
         };
         for (int jj = 0; ok && jj < n; ++jj, ++g) {
           // Only the last step may need a mask: the causal diagonal, which starts at the sub-tile's first row and ends, in a
@@ -395,20 +401,19 @@ attn_narrow_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
     // ============================== MMA issuer of one stream (the whole warp walks the loop, one lane issues)
     setmaxnreg_dec<SH::kOtherRegs>();
     const int st = warp - SH::kMmaWarp, group = st / HALVES, half = st % HALVES, i = SUBS == 2 ? group : 0;
-    bool ok = run;
+    bool ok = run, dead = false;
     const uint32_t s_tmem = tmem_base + st * HKV, o_tmem = tmem_base + O_COL0 + st * D;
     const uint32_t k_smem = ring_smem + half * (HKV * 128);       // this stream's keys in a ring item
     uint32_t g = 0, done = 0, q_uses = 0;              // steps; finished tiles; Q loads that have been read
     const int first_stage = RINGS::of_group(group) * p.stages;
     KvRing ring = {first_stage, 0u};                   // K and V of this stream's key tiles, one after another, over all tiles
-    auto wait = [&](uint64_t* bar, uint32_t parity, uint32_t id) __attribute__((always_inline)) -> bool {
-      if (!wait_quiet_warp(smem_u32(bar), parity, abort_flag, wait_info(kRoleMma, id, 0x100 * st + (g & 0xFF)))) { ok = false; return false; }
-      return true;
+    auto wait = [&](uint64_t* bar, uint32_t parity, uint32_t id) __attribute__((always_inline)) {
+      wait_on(smem_u32(bar), parity, abort_flag, wait_info(kRoleMma, id, 0x100 * st + (g & 0xFF)), dead);
     };
-    // Waits for the ring's next item and passes it; its stage, or -1 if the wait expired.
+    // Waits for the ring's next item and passes it; its stage.
     auto take = [&]() __attribute__((always_inline)) -> int {
       const int stage = ring.pos;
-      if (!wait(&misc->kv_full[stage], ring.phase, kBarKvFull)) return -1;
+      wait(&misc->kv_full[stage], ring.phase, kBarKvFull);
       ring.advance(first_stage, p.stages);
       return stage;
     };
@@ -425,15 +430,13 @@ attn_narrow_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
 #pragma unroll 1
       for (int x = 0; x < 2 * steps; ++x) {
         const int stage = take();
-        if (stage < 0) return;
         if (lane == 0) mbar_arrive(smem_u32(&misc->kv_empty[stage]));
       }
     };
     // A tile's first scores.
     auto start = [&](int steps) __attribute__((always_inline)) {
-      if (!wait(&misc->q_full[i][q_uses & 1], (q_uses >> 1) & 1, kBarQ)) return;
+      wait(&misc->q_full[i][q_uses & 1], (q_uses >> 1) & 1, kBarQ);
       const int k = take();
-      if (k < 0) return;
       ++q_uses;
       tc_fence_after();
       if (elect_one()) issue_scores(k, steps == 1);
@@ -446,13 +449,11 @@ attn_narrow_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
       if (n > 0) start(n);
       for (int j = 0; ok && j < n; ++j, ++g) {
         const int v = take();
-        if (v < 0) break;
         const bool more = j + 1 < n;
         const int k = more ? take() : 0;
-        if (k < 0) break;
         // the tile before has left the accumulator
-        if (j == 0 && done > 0 && !wait(&misc->o_free[i], (done - 1) & 1, kBarOFull)) break;
-        if (!wait(&misc->p_full[st], g & 1, kBarPFull)) break;
+        if (j == 0 && done > 0) wait(&misc->o_free[i], (done - 1) & 1, kBarOFull);
+        wait(&misc->p_full[st], g & 1, kBarPFull);
         tc_fence_after();
         if (elect_one()) {
           issue_pv<D, HKV>(o_tmem, s_tmem, k_smem + v * SM::kStageBytes, j > 0, TKV * 128, 1024);
@@ -461,6 +462,7 @@ attn_narrow_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
           else umma_commit(smem_u32(&misc->o_full[i]));
         }
         __syncwarp();
+        if (any_dead(dead)) ok = false;
       }
       if (!ok) break;
       if constexpr (SUBS == 2) {
@@ -470,8 +472,8 @@ attn_narrow_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
         ++done;
         if (n == 0) {
           // nothing to add to the tile, nothing read of its Q (the arrivals of the tile before must all have been made: o_free)
-          if (done > 1 && !wait(&misc->o_free[0], (done - 2) & 1, kBarOFull)) break;
-          if (!wait(&misc->q_full[0][q_uses & 1], (q_uses >> 1) & 1, kBarQ)) break;
+          if (done > 1) wait(&misc->o_free[0], (done - 2) & 1, kBarOFull);
+          wait(&misc->q_full[0][q_uses & 1], (q_uses >> 1) & 1, kBarQ);
           if (lane == 0) {
             mbar_arrive(smem_u32(&misc->q_empty[0][q_uses & 1]));
             mbar_arrive(smem_u32(&misc->o_full[0]));
@@ -479,7 +481,7 @@ attn_narrow_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
           ++q_uses;
         }
       }
-      if (!ok) break;
+      if (any_dead(dead)) break;
       tile = next_tile(seq, kRoleMma);
     }
   } else if (warp == SH::kLoadWarp) {

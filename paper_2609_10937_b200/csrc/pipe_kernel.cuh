@@ -100,28 +100,6 @@ __device__ __forceinline__ PipeWork pipe_work(int index, const PipeParams& p) {
   return w;
 }
 
-// Waits for a phase.  An expiry, here or elsewhere in the CTA, sets `dead`: the caller goes on, for at most a step, until it looks.
-// No warp waits for ever: those that follow an expired one find the abort flag.
-__device__ __forceinline__ void wait_on(uint32_t bar, uint32_t parity, volatile int* abort_flag, uint32_t info, bool& dead) {
-  if (mbar_try_wait(bar, parity)) return;
-  const uint32_t t0 = (uint32_t)clock64();
-  uint32_t it = 0;
-  while (!mbar_try_wait(bar, parity)) {
-    if ((++it & 63u) == 0u) {
-      if (*abort_flag) {
-        dead = true;
-        return;
-      }
-      if ((uint32_t)clock64() - t0 > (uint32_t)kWaitLimitCycles) {
-        note_timeout(info, abort_flag);
-        dead = true;
-        return;
-      }
-    }
-  }
-}
-__device__ __forceinline__ bool any_dead(bool dead) { return __any_sync(0xffffffffu, dead); }
-
 template <int D, bool CAUSAL>
 __global__ void __launch_bounds__(512, 1)
 attn_pipe_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
