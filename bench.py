@@ -294,8 +294,6 @@ def kernel_name(plan, d, cluster, last=None, L=0, sms=148):
     if last is not None and cluster == 0 and last[1] == plan.tiles and plan.n_q == 2:
         # one CTA per tile of 256 rows: the kernel of two streams a tile, where the library takes it (pipe_tiles, attn_api.cu)
         steps = -(-L // 128)
-        if last[0] == binding.KERNEL_NARROW_TILES and steps >= 48:
-            return f"attn_pipe_kernel<{d},0>"
         if last[0] == binding.KERNEL_TILED and (plan.ctas != plan.tiles or plan.tiles > sms or (steps >= 4 and (d == 64 or 10 * plan.tiles > 7 * sms))):
             return f"attn_pipe_kernel<{d},0>"
     if last is not None and last[0] == binding.KERNEL_NARROW_TILES:

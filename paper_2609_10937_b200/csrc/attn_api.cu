@@ -606,9 +606,15 @@ int narrow_subs(const attn_tiles& t, int BH, int Lq, int Lk, int d, int local_me
 }
 
 // Calls, not causal, that pipe_kernel.cuh takes over from attn_fwd_kernel, at either head dimension (us in graphs of 8 calls, attn_fwd_kernel / this).
-//   Plans of whole tiles: with more tiles than SMs always (183 shapes of a grid, 0.81 to 0.99 times: 148 x 1024, d = 64 59.3 / 53.2; 592 x 512,
-// d = 128 75.8 / 63.2).  One wave: from four key steps on (three and fewer 0.98 to 1.05: 64 x 384, d = 64 10.0 / 10.2), and at d = 128 where
-// the tiles fill more than seven tenths of the SMs (12 x 1536, d = 64 0.96; 10 x 2560, d = 128 38.7 / 39.7, 24 x 1300 23.8 / 22.7).
+//   Plans of whole tiles, d = 128: with more tiles than SMs always (95 shapes, 0.91 times on the geometric mean: 592 x 512 75.8 / 63.2).  One wave: from four
+// key steps on (three and fewer 0.98 to 1.05) where the tiles fill more than seven tenths of the SMs (10 x 2560 38.7 / 39.7, 24 x 1300 23.8 /
+// 22.7).
+//   d = 64: its step takes one cubic and two quartics of eight pairs where attn_fwd_kernel takes two cubics, which costs 2 % of a step and leaves
+// long tiles to that kernel.  One wave from 4 key steps (3: 64 x 384 10.0 / 10.2) to 15 (148 x (256 x 1280) 20.7 / 20.2, 80 x (256 x 2048)
+// 29.4 / 29.4, 120 x (256 x 4096) 53.3 / 55.0); two waves to 15, three to 21, four to 27 (32 x 2304 59.4 / 60.2, 24 x 3000 77.6 / 78.9, 37 x 4000
+// 205 / 208), more to 31, where the last wave is full to 23 (60 x 3000 203 / 195, 111 x 3000 352 / 352, 74 x 4096 408 / 414).  An odd
+// number of steps without a masked one is a good one for attn_fwd_kernel: 5 (148 x 640 31.5 / 33.0), and from 7 on where the last wave is full
+// (148 x 896 52.2 / 54.0, but 128 x 896 0.90 times; 148 x 1152 79.1 / 80.9).  425 shapes on two grids go here, 0.958 times, three of them slower by 1 to 1.6 %.
 //   Plans whose tiles are cut over the machine: where whole tiles are estimated to be faster by 2 % (d = 64) or 4 %.  The estimates are
 // fits in us, of this kernel over its waves and key steps and of the plan's over its cost, that miss by 4 to 7 % (one sd): of 140 shapes
 // 49 go here, 0.89 times on the geometric mean and none slower by more than 1 %; 14 that would be 3 % faster or more stay.
@@ -616,6 +622,11 @@ bool pipe_tiles(const attn_tiles& t, int Lk, int d, int local_mem, int sms) {
   if (t.causal || t.n_q != 2 || t.tile_kv != 128) return false;
   if (local_mem < (d == 64 ? attn::PipeSmem<64>::total(4) : attn::PipeSmem<128>::total(4))) return false;
   const int steps = (Lk + 127) / 128, waves = (t.tiles + sms - 1) / sms;
+  if (d == 64) {
+    const bool full = 100LL * t.tiles >= 98LL * waves * sms;       // the last wave
+    if (steps >= 32 || steps >= std::max(16, 4 + 6 * waves) || (full && steps >= 24)) return false;
+    if (waves > 1 && Lk % 128 == 0 && steps % 2 == 1 && (steps == 5 || (steps >= 7 && full))) return false;
+  }
   if (t.ctas == t.tiles) return t.tiles > sms || (steps >= 4 && (d == 64 || 10 * t.tiles > 7 * sms));
   if (t.ctas > t.tiles || t.tiles <= sms) return false;
   const double whole = d == 64 ? 3.0 + waves * (2.0 + 1.376 * steps + (Lk % 128 ? 0.35 : 0.0)) : 4.0 + waves * (2.3 + 1.647 * steps);
@@ -631,9 +642,6 @@ int dispatch_fwd(const void* q, const void* k, const void* v, void* o, int B, in
   const int sms = st->desc.num_units;
   if (own_plan) {
     if (const int subs = narrow_subs(t, B * H, L, Lk, d, st->desc.local_mem_bytes, sms)) {
-      // (long tiles of two sub-tiles, not causal: us in loops of half a second, four streams a tile / two, 128 x 8192 2818 / 2722)
-      if (subs == 2 && !t.causal && (Lk + 127) / 128 >= 48)
-        return launch_pipe<64, false>(q, k, v, o, B * H, L, Lk, status, st, s, ATTN_KERNEL_NARROW_TILES);
       auto launch = d == 128 ? (t.causal ? launch_narrow<128, true, 1> : launch_narrow<128, false, 1>)
                     : t.causal ? (subs == 1 ? launch_narrow<64, true, 1> : launch_narrow<64, true, 2>)
                                : (subs == 1 ? launch_narrow<64, false, 1> : launch_narrow<64, false, 2>);

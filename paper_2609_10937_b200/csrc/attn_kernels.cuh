@@ -385,7 +385,10 @@ __device__ __forceinline__ float chain_max(const uint32_t* s) {
 }
 // Constants of the exponential evaluation, packed once per thread.
 struct ExpConsts {
-  uint64_t scale2, magic2, c3, c2, c1, c0;
+  uint64_t scale2, magic2;
+  uint64_t c3, c2, c1, c0;               // cubic, quartic and quintic for 2^f
+  uint64_t f4, f3, f2, f1, f0;
+  uint64_t g5, g4, g3, g2, g1, g0;
 };
 __device__ __forceinline__ ExpConsts make_exp_consts(float scale) {
   ExpConsts k;
@@ -396,10 +399,24 @@ __device__ __forceinline__ ExpConsts make_exp_consts(float scale) {
   k.c2 = pack_f32x2(0.24260213971138f, 0.24260213971138f);
   k.c1 = pack_f32x2(0.6932607889175415f, 0.6932607889175415f);
   k.c0 = pack_f32x2(0.9999286532402039f, 0.9999286532402039f);
+  // quartic, relative error 2.6e-6 (as the cubic and the quintic: a linear programme over a grid of f, then rounded to fp32)
+  k.f4 = pack_f32x2(0.00957053154706955f, 0.00957053154706955f);
+  k.f3 = pack_f32x2(0.05591866374015808f, 0.05591866374015808f);
+  k.f2 = pack_f32x2(0.24024735391139984f, 0.24024735391139984f);
+  k.f1 = pack_f32x2(0.6931216716766357f, 0.6931216716766357f);
+  k.f0 = pack_f32x2(0.9999992847442627f, 0.9999992847442627f);
+  // quintic, relative error 2.1e-7 in fp32 arithmetic
+  k.g5 = pack_f32x2(0.0013291396899148822f, 0.0013291396899148822f);
+  k.g4 = pack_f32x2(0.009675704874098301f, 0.009675704874098301f);
+  k.g3 = pack_f32x2(0.05550655350089073f, 0.05550655350089073f);
+  k.g2 = pack_f32x2(0.24022117257118225f, 0.24022117257118225f);
+  k.g1 = pack_f32x2(0.6931470036506653f, 0.6931470036506653f);
+  k.g0 = pack_f32x2(1.0000001192092896f, 1.0000001192092896f);
   return k;
 }
 // exp2 of a packed pair on the FMA/ALU pipes (no MUFU): x = n + f with n integer, f in [-0.5, 0.5];
-// 2^f by the cubic, 2^n by adding n to the exponent field.  x is clamped at -126 (result ~1e-38).
+// 2^f by the polynomial, 2^n by adding n to the exponent field.  x is clamped at -126 (result ~1e-38).
+template <int kDegree = 3>
 __device__ __forceinline__ void exp2_poly_pair(uint64_t x2, const ExpConsts& k, float& e0, float& e1) {
   float x0, x1;
   unpack_f32x2(x2, x0, x1);
@@ -409,9 +426,24 @@ __device__ __forceinline__ void exp2_poly_pair(uint64_t x2, const ExpConsts& k, 
   const uint64_t r2 = add_f32x2(xc, k.magic2);
   const uint64_t n2 = sub_f32x2(r2, k.magic2);
   const uint64_t f2 = sub_f32x2(xc, n2);
-  uint64_t p2 = fma_f32x2(f2, k.c3, k.c2);
-  p2 = fma_f32x2(p2, f2, k.c1);
-  p2 = fma_f32x2(p2, f2, k.c0);
+  static_assert(kDegree >= 3 && kDegree <= 5, "no such polynomial");
+  uint64_t p2;
+  if constexpr (kDegree == 5) {
+    p2 = fma_f32x2(f2, k.g5, k.g4);
+    p2 = fma_f32x2(p2, f2, k.g3);
+    p2 = fma_f32x2(p2, f2, k.g2);
+    p2 = fma_f32x2(p2, f2, k.g1);
+    p2 = fma_f32x2(p2, f2, k.g0);
+  } else if constexpr (kDegree == 4) {
+    p2 = fma_f32x2(f2, k.f4, k.f3);
+    p2 = fma_f32x2(p2, f2, k.f2);
+    p2 = fma_f32x2(p2, f2, k.f1);
+    p2 = fma_f32x2(p2, f2, k.f0);
+  } else {
+    p2 = fma_f32x2(f2, k.c3, k.c2);
+    p2 = fma_f32x2(p2, f2, k.c1);
+    p2 = fma_f32x2(p2, f2, k.c0);
+  }
   float p0, p1, r0, r1;
   unpack_f32x2(p2, p0, p1);
   unpack_f32x2(r2, r0, r1);
@@ -470,14 +502,22 @@ __device__ __forceinline__ uint32_t pack_in_order(const uint32_t* e) {
   asm volatile("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(d) : "r"(e[1]), "r"(e[0]));
   return d;
 }
-// Which of eight pairs take the polynomial.
-template <int kPolyPairs>
-__host__ __device__ constexpr bool poly_pair(int j) {
-  return kPolyPairs == 1 ? (j & 7) == 7 : kPolyPairs == 2 ? (j & 7) < 2 : (j & 7) == 2 || (j & 7) == 5 || (j & 7) == 7;
+// Which of eight pairs take the polynomial, and of which degree (0: the exponential unit).  A weight that the cubic gives is off by up to
+// 7.6e-5 and the denominators are sums of weights, so its share is nowhere larger than the two of eight of exp_chunk, and none where the
+// unit alone does as well: three of eight are one cubic and two quartics (0.7 times the error of two cubics), and the one pair of
+// kMixUnit a quintic, which is as close as the unit (2.4e-7).
+enum ExpMix { kMixOne, kMixTwo, kMixThree, kMixUnit };
+template <int kMix>
+__host__ __device__ constexpr int poly_degree(int j) {
+  const int e = j & 7;
+  return kMix == kMixOne   ? (e == 7 ? 3 : 0)
+         : kMix == kMixTwo ? (e < 2 ? 3 : 0)
+         : kMix == kMixThree ? (e == 1 ? 3 : e == 4 || e == 6 ? 4 : 0)
+                             : (e == 7 ? 5 : 0);
 }
 // exp2(s * scale - m) of 32 scores in place and as bf16 pairs in pk; beside them, with kSum, the 32 exponentials at `done` are
 // added to the partial sums.  A pair's argument is computed three pairs ahead, its bf16 two pairs later.
-template <int kPolyPairs, bool kSum>
+template <int kMix, bool kSum>
 __device__ __forceinline__ void exp_chunk_in_place(uint32_t* s, const uint32_t* done, uint64_t (&sum)[2], const ExpConsts& k, uint64_t neg_m2,
                                                    uint32_t (&pk)[16]) {
   constexpr int kAhead = 3;
@@ -488,14 +528,16 @@ __device__ __forceinline__ void exp_chunk_in_place(uint32_t* s, const uint32_t* 
   for (int j = 0; j < 18; ++j) {
     if (j < 16) {
       float a, b;
-      if (poly_pair<kPolyPairs>(j)) {
-        exp2_poly_pair(x[j], k, a, b);
+      if (poly_degree<kMix>(j) != 0) {
+        if (poly_degree<kMix>(j) == 5) exp2_poly_pair<5>(x[j], k, a, b);
+        else if (poly_degree<kMix>(j) == 4) exp2_poly_pair<4>(x[j], k, a, b);
+        else exp2_poly_pair<3>(x[j], k, a, b);
       } else {
         unpack_f32x2(x[j], a, b);
         a = ex2_in_order(a);
       }
       if (j + kAhead < 16) x[j + kAhead] = fma2_in_order(pair_of(s + 2 * (j + kAhead)), k.scale2, neg_m2);
-      if (!poly_pair<kPolyPairs>(j)) b = ex2_in_order(b);
+      if (poly_degree<kMix>(j) == 0) b = ex2_in_order(b);
       s[2 * j] = __float_as_uint(a);
       s[2 * j + 1] = __float_as_uint(b);
       if (kSum) sum[j & 1] = add2_in_order(sum[j & 1], pair_of(done + 2 * j));
@@ -718,7 +760,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
         if constexpr (kTwoMma) {
           // (as in attn_pipe_kernel; a masked step can leave a row that has had no admissible key yet: its reference stays finite)
           // One pair of eight takes the polynomial, in a masked step two as in exp_chunk: those steps hold the rows that see few keys.
-          constexpr int kStepPoly = kMasked ? kPolyPairsPer8 : 1;
+          constexpr int kStepPoly = kMasked ? kMixTwo : kMixOne;
           const float m_cand = kMasked ? fmaxf(mx * scale, kEmptyReference) : mx * scale;
           const float gap = m_cand - m_run;
           const bool move = gap > lim_move;

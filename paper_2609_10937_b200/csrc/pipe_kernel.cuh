@@ -17,16 +17,19 @@
 //     (Exponentials of the first chunk ahead of the maximum, on the old reference, were 2 % faster on flat scores and slower
 //     wherever references move; the code that mends them costs moves in every step.)
 //   * At d = 128 one pair of eight takes the polynomial instead of two (a pair costs eight issue slots more than on the exponential
-//     unit; none: 0-1 % slower not causal, the same causal).  At d = 64 there is no chain: P has columns of its own, the next
-//     scores are produced under this step's exponentials, both warpgroups work all the time, and three pairs of eight are fastest (2: 867,
-//     3: 829, 4: 887 us at 148 x 4096).
+//     unit; none: 0-1 % slower).  Causal, where the kernel before took none in the common step, it is the quintic, which is as exact as
+//     the unit (128 x 4096 in loops: cubic 547, quintic 549, none 551 us).  At d = 64 there is no chain: P has columns of its own, the
+//     next scores are produced under this step's exponentials, both warpgroups work all the time, and three pairs of eight are
+//     fastest (2: 867, 3: 829, 4: 887 us at 148 x 4096); one of them is a cubic and two are quartics, so that a weight is nowhere
+//     less exact than with two cubics (three cubics: 824, as it is 855, three quartics 865; 148 x 1024 55.6 / 57.1 / 57.3).
 // As before it: the epilogue of a tile runs under the next one (the correction warpgroup normalises and stores it), a sub-tile runs
 // only its own steps, tiles come from the hardware's queue of CTAs not yet started (clusterlaunchcontrol.try_cancel), causal ones
 // longest first within groups of heads whose K and V stay in L2.
 // Measured (us, the kernels before / this one, calls back to back): d = 128 causal 128 x 4096 549 / 516, 600 x 512 87.5 / 76.4, 213 shapes in
 // whole tiles 0.84 times on the geometric mean; not causal 148 x 4096 1080 / 1053, 148 x 2048 with variance 3 303 / 294, 95 shapes
-// in waves of whole tiles 0.91 times; d = 64 148 x 4096 820 / 794, 128 x 8192 2818 / 2722, 88 shapes 0.93 times.  Long calls run into the power limit (990 W) and keep less:
-// in loops of seconds 4 x 32 x 4096, d = 128, takes 1000 / 982, causal 582 / 549, 4 x 32 x 8192, d = 64, 2928 / 2898.
+// in waves of whole tiles 0.91 times; d = 64 (tiles that are not long, pipe_tiles in attn_api.cu) 148 x 1024 58.9 / 57.1, 128 x 2000 195 / 178, 425
+// shapes 0.958 times.  Long calls run into the power limit (990 W) and keep less: in loops of seconds 4 x 32 x 4096, d = 128, takes 1000 /
+// 982, causal 582 / 549.
 #pragma once
 
 #include "attn_kernels.cuh"
@@ -108,7 +111,7 @@ attn_pipe_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
   constexpr int TKV = 128, KCH = D / 64, O_COL0 = 2 * TKV;
   constexpr bool kSplit = D == 64;                      // P has columns of its own (else it overwrites the front of its scores)
   constexpr int P_COL0 = O_COL0 + 2 * D;
-  constexpr int kPoly = D == 64 ? 3 : 1;
+  constexpr int kPoly = D == 64 ? kMixThree : CAUSAL ? kMixUnit : kMixOne;
   constexpr int kFirstK = D == 64 ? 6 : 4;              // 16-key steps of P V that the first hand-over of P allows
 
   extern __shared__ __align__(1024) uint8_t smem_raw[];
