@@ -343,6 +343,11 @@ constexpr float kDominanceFactor = 16.0f;   // a new maximum heavier than delta/
 // Reference of a row that has seen no admissible key yet: finite, so that -inf less it is -inf, and -FLT_MAX, because no finite
 // score times a scale below 1 lies under it (a higher one would take such a row's weights to zero and its result to NaN).
 constexpr float kEmptyReference = -3.402823466e38f;
+// 1 / denominator of a finished row.  NaN if its reference is no number or infinite (the polynomial's weights would be finite), or if no key
+// that it may attend to has a finite score (a denominator of weights that the polynomial clamps, of masked keys too).
+__device__ __forceinline__ float row_inverse(float delta, float m) {
+  return 1.0f / (m == kEmptyReference ? __int_as_float(0x7FFFFFFF) : delta + (m - m));
+}
 constexpr int kCounterBytes = 65536;   // head of the workspace: 16384 arrival counters
 
 struct FwdMisc {               // lives in the last 3072 bytes of dynamic shared memory
@@ -374,13 +379,25 @@ __device__ __forceinline__ float max3(float a, float b, float c) {
   asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
   return d;
 }
-// max of s[B..E) as one dependency chain of 3-input maxima
+// The same, NaN where an operand is: the row maximum of attention carries a NaN score to its row's result.  (The polynomial of
+// exp2_poly_pair would turn the score itself into a weight of 1e-38, and the row into a mean over the other keys.)
+__device__ __forceinline__ float max3_nan(float a, float b, float c) {
+  float d;
+  asm("max.NaN.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+  return d;
+}
+__device__ __forceinline__ float max_nan(float a, float b) {
+  float d;
+  asm("max.NaN.f32 %0, %1, %2;" : "=f"(d) : "f"(a), "f"(b));
+  return d;
+}
+// max of s[B..E) as one dependency chain of 3-input maxima; NaN where one of them is
 template <int B, int E>
 __device__ __forceinline__ float chain_max(const uint32_t* s) {
   float m = __uint_as_float(s[B]);
 #pragma unroll
-  for (int k = B + 1; k + 1 < E; k += 2) m = max3(m, __uint_as_float(s[k]), __uint_as_float(s[k + 1]));
-  if (((E - B - 1) & 1) != 0) m = fmaxf(m, __uint_as_float(s[E - 1]));
+  for (int k = B + 1; k + 1 < E; k += 2) m = max3_nan(m, __uint_as_float(s[k]), __uint_as_float(s[k + 1]));
+  if (((E - B - 1) & 1) != 0) m = max_nan(m, __uint_as_float(s[E - 1]));
   return m;
 }
 // Constants of the exponential evaluation, packed once per thread.
@@ -731,8 +748,8 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
           for (int k = 0; k < TKV / 2; ++k)
             if (k > lim) s[k] = 0xFF800000u;
         }
-        const float mx_a = fmaxf(fmaxf(chain_max<0, TKV / 8>(s), chain_max<TKV / 8, TKV / 4>(s)),
-                                 fmaxf(chain_max<TKV / 4, 3 * TKV / 8>(s), chain_max<3 * TKV / 8, TKV / 2>(s)));
+        const float mx_a = max_nan(max_nan(chain_max<0, TKV / 8>(s), chain_max<TKV / 8, TKV / 4>(s)),
+                                   max_nan(chain_max<TKV / 4, 3 * TKV / 8>(s), chain_max<3 * TKV / 8, TKV / 2>(s)));
 #pragma unroll
         for (int c = NCH / 2; c < NCH; ++c) tmem_ld_fence(*reinterpret_cast<uint32_t(*)[32]>(&s[c * 32]));
         if constexpr (kSplitP) {
@@ -744,9 +761,9 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
           for (int k = TKV / 2; k < TKV; ++k)
             if (k > lim) s[k] = 0xFF800000u;
         }
-        const float mx_b = fmaxf(fmaxf(chain_max<TKV / 2, 5 * TKV / 8>(s), chain_max<5 * TKV / 8, 3 * TKV / 4>(s)),
-                                 fmaxf(chain_max<3 * TKV / 4, 7 * TKV / 8>(s), chain_max<7 * TKV / 8, TKV>(s)));
-        const float mx = fmaxf(mx_a, mx_b);
+        const float mx_b = max_nan(max_nan(chain_max<TKV / 2, 5 * TKV / 8>(s), chain_max<5 * TKV / 8, 3 * TKV / 4>(s)),
+                                   max_nan(chain_max<3 * TKV / 4, 7 * TKV / 8>(s), chain_max<7 * TKV / 8, TKV>(s)));
+        const float mx = max_nan(mx_a, mx_b);
         // Lazy rescale.  The reference maximum m_run moves (and O, delta are rescaled by alpha) only
         //  (a) when the row maximum grew by more than kRescaleThreshold (log2 units), which bounds
         //      P = exp2(s - m_run) by 2^threshold, or
@@ -761,9 +778,9 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
           // (as in attn_pipe_kernel; a masked step can leave a row that has had no admissible key yet: its reference stays finite)
           // One pair of eight takes the polynomial, in a masked step two as in exp_chunk: those steps hold the rows that see few keys.
           constexpr int kStepPoly = kMasked ? kMixTwo : kMixOne;
-          const float m_cand = kMasked ? fmaxf(mx * scale, kEmptyReference) : mx * scale;
+          const float m_cand = kMasked ? max_nan(mx * scale, kEmptyReference) : mx * scale;
           const float gap = m_cand - m_run;
-          const bool move = gap > lim_move;
+          const bool move = !(gap <= lim_move);            // (a NaN moves it)
           m_run = move ? m_cand : m_run;
           const uint64_t neg_m2 = pack_f32x2(-m_run, -m_run);
           const float alpha = move ? ex2_approx(-gap) : 1.0f;
@@ -798,10 +815,10 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
           lim_move = fminf(fmaxf(lg2_approx(delta) - 4.0f, 0.f), kRescaleThreshold);
           return true;
         }
-        const float m_cand = kMasked ? fmaxf(fmaxf(m_run, mx * scale), kEmptyReference) : fmaxf(m_run, mx * scale);
+        const float m_cand = kMasked ? max3_nan(m_run, mx * scale, kEmptyReference) : max_nan(m_run, mx * scale);
         const float gap = m_cand - m_run;
         const float shrink = ex2_approx(-gap);             // 2^-gap: the rescale factor if the reference moves
-        const bool move = (gap > kRescaleThreshold) || (gap > 0.f && kDominanceFactor > delta * shrink);
+        const bool move = !(gap <= kRescaleThreshold) || (gap > 0.f && kDominanceFactor > delta * shrink);   // (a NaN moves it)
         const float m_new = move ? m_cand : m_run;
         const float alpha = move ? shrink : 1.0f;
         if constexpr (kSplitP) {
@@ -926,7 +943,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
       };
       if (sg.full) {
         // The whole Q tile was processed here: normalise and store.
-        const float inv = 1.0f / delta;
+        const float inv = row_inverse(delta, m_run);
 #pragma unroll 1
         for (int h = 0; h < KCH; ++h) {
           uint32_t r0[32], r1[32];
@@ -1017,7 +1034,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                 const float d_q = (q == mine) ? delta : stat(q)[32 + lane];
                 d_all += d_q * exp2f(m_q - m_all);
               }
-              const float inv = 1.0f / d_all;
+              const float inv = row_inverse(d_all, m_all);
 #pragma unroll 1
               for (int h = 0; h < KCH; ++h) {
                 if (h == 1 &&
@@ -1167,7 +1184,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
               ww[sp] = (sp < parts) ? exp2f(mm[sp] - m_all) : 0.f;
               if (sp < parts) d_all += dd[sp] * ww[sp];
             }
-            const float inv = 1.0f / d_all;
+            const float inv = row_inverse(d_all, m_all);
             int k = 0;
 #pragma unroll 1
             for (int h = 0; h < KCH; ++h) {
@@ -1222,7 +1239,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
             const float d_sp = (sp == mine) ? delta : __ldcg(b + (size_t)kSub * D + kSub + row);
             d_all += d_sp * exp2f(m_sp - m_all);
           }
-          const float inv = 1.0f / d_all;
+          const float inv = row_inverse(d_all, m_all);
 #pragma unroll 1
           for (int h = 0; h < KCH; ++h) {
             float val[64];

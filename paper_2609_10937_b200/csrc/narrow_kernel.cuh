@@ -235,7 +235,7 @@ attn_narrow_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
             for (int k = 0; k < HKV / 2; ++k)
               if (k > lim) s[k] = 0xFF800000u;
           }
-          const float mx_a = fmaxf(chain_max<0, HKV / 4>(s), chain_max<HKV / 4, HKV / 2>(s));
+          const float mx_a = max_nan(chain_max<0, HKV / 4>(s), chain_max<HKV / 4, HKV / 2>(s));
 #pragma unroll
           for (int c = NCH / 2; c < NCH; ++c) tmem_ld_fence(*reinterpret_cast<uint32_t(*)[32]>(&s[c * 32]));
           if constexpr (kMasked) {
@@ -243,12 +243,12 @@ attn_narrow_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
             for (int k = HKV / 2; k < HKV; ++k)
               if (k > lim) s[k] = 0xFF800000u;
           }
-          const float mx = max3(mx_a, chain_max<HKV / 2, 3 * HKV / 4>(s), chain_max<3 * HKV / 4, HKV>(s));
+          const float mx = max3_nan(mx_a, chain_max<HKV / 2, 3 * HKV / 4>(s), chain_max<3 * HKV / 4, HKV>(s));
           // Lazy rescale, as in attn_fwd_kernel.  The reference is finite from the first step on, also where a stream's
           // half of the keys holds none that the row may attend to.
-          const float m_cand = fmaxf(mx * scale, kEmptyReference);
+          const float m_cand = max_nan(mx * scale, kEmptyReference);
           const float gap = m_cand - m_run;
-          const bool move = gap > lim_move;
+          const bool move = !(gap <= lim_move);        // (a NaN moves it)
           m_run = move ? m_cand : m_run;
           // The step before is complete (see s_full), so the accumulator may be rescaled here; P V of this step waits for P.
           if (__any_sync(0xffffffffu, move)) {
@@ -342,7 +342,7 @@ attn_narrow_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
           wt[k] = ex2_approx(a.x - m);                 // (an empty part: -inf, weight 0)
           sum += a.y * wt[k];
         }
-        const float inv = 1.0f / sum;
+        const float inv = row_inverse(sum, m);
 #pragma unroll
         for (int k = 0; k < kParts; ++k) wt[k] *= inv;
         if (!wait_quiet_warp(smem_u32(&misc->o_full[i]), ph, abort_flag, wait_info(kRoleCorrection, kBarOFull, i))) { ok = false; break; }

@@ -220,7 +220,7 @@ attn_pipe_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
 #pragma unroll
           for (int c = 2; c < 4; ++c) tmem_ld32_nowait(s_tmem + c * 32, chunk(c));
           if (masked) mask(0);
-          const float mx_a = fmaxf(fmaxf(chain_max<0, 16>(s), chain_max<16, 32>(s)), fmaxf(chain_max<32, 48>(s), chain_max<48, 64>(s)));
+          const float mx_a = max_nan(max_nan(chain_max<0, 16>(s), chain_max<16, 32>(s)), max_nan(chain_max<32, 48>(s), chain_max<48, 64>(s)));
 #pragma unroll
           for (int c = 2; c < 4; ++c) tmem_ld_fence(chunk(c));
           if constexpr (kSplit) {
@@ -228,12 +228,12 @@ attn_pipe_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
             mbar_arrive(smem_u32(&misc->s_free[i]));   // the scores are in registers: the buffer may be overwritten
           }
           if (masked) mask(TKV / 2);
-          const float mx_b = fmaxf(fmaxf(chain_max<64, 80>(s), chain_max<80, 96>(s)), fmaxf(chain_max<96, 112>(s), chain_max<112, 128>(s)));
+          const float mx_b = max_nan(max_nan(chain_max<64, 80>(s), chain_max<80, 96>(s)), max_nan(chain_max<96, 112>(s), chain_max<112, 128>(s)));
           // Lazy rescale, as in attn_fwd_kernel: the reference moves to the row maximum if that lies above it by more than
           // kRescaleThreshold, or by anything that gives the new maximum's key more than 1 / kDominanceFactor of the denominator.
-          const float m_cand = fmaxf(mx_a, mx_b) * scale;
+          const float m_cand = max_nan(mx_a, mx_b) * scale;
           const float gap = m_cand - m_run;
-          const bool move = gap > lim;
+          const bool move = !(gap <= lim);             // (a NaN moves it)
           m_run = move ? m_cand : m_run;
           const uint64_t neg_m2 = pack_f32x2(-m_run, -m_run);
           const float alpha = move ? ex2_approx(-gap) : 1.0f;
@@ -280,7 +280,7 @@ attn_pipe_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
           wait_on(smem_u32(&misc->o_full[i]), (kSplit ? g - 1 : done) & 1, abort_flag, wait_info(kRoleSoftmax, kBarOFull, g), dead);
           tc_fence_after();
         }
-        misc->inv[i][row] = 1.0f / delta;
+        misc->inv[i][row] = row_inverse(delta, m_run);
         mbar_arrive(smem_u32(&misc->fin_full[i]));
         ++done;
       }
