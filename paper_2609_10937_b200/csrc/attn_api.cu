@@ -611,10 +611,10 @@ int narrow_subs(const attn_tiles& t, int BH, int Lq, int Lk, int d, int local_me
 // 22.7).
 //   d = 64: its step takes one cubic and two quartics of eight pairs where attn_fwd_kernel takes two cubics, which costs 2 % of a step and leaves
 // long tiles to that kernel.  One wave from 4 key steps (3: 64 x 384 10.0 / 10.2) to 15 (148 x (256 x 1280) 20.7 / 20.2, 80 x (256 x 2048)
-// 29.4 / 29.4, 120 x (256 x 4096) 53.3 / 55.0); two waves to 15, three to 21, four to 27 (32 x 2304 59.4 / 60.2, 24 x 3000 77.6 / 78.9, 37 x 4000
+// 29.4 / 29.4, 120 x (256 x 4096) 53.3 / 55.0); two waves to 17, three to 23, four to 29 (32 x 2048 54.0 / 53.5, 32 x 2304 59.4 / 60.2, 24 x 3000 77.6 / 78.9, 37 x 4000
 // 205 / 208), more to 31, where the last wave is full to 23 (60 x 3000 203 / 195, 111 x 3000 352 / 352, 74 x 4096 408 / 414).  An odd
 // number of steps without a masked one is a good one for attn_fwd_kernel: 5 (148 x 640 31.5 / 33.0), and from 7 on where the last wave is full
-// (148 x 896 52.2 / 54.0, but 128 x 896 0.90 times; 148 x 1152 79.1 / 80.9).  425 shapes on two grids go here, 0.958 times, three of them slower by 1 to 1.6 %.
+// (148 x 896 52.2 / 54.0, but 128 x 896 0.90 times; 148 x 1152 79.1 / 80.9).  436 shapes on two grids go here, 0.958 times, four of them slower by 1 to 1.6 %.
 //   Plans whose tiles are cut over the machine: where whole tiles are estimated to be faster by 2 % (d = 64) or 4 %.  The estimates are
 // fits in us, of this kernel over its waves and key steps and of the plan's over its cost, that miss by 4 to 7 % (one sd): of 140 shapes
 // 49 go here, 0.89 times on the geometric mean and none slower by more than 1 %; 14 that would be 3 % faster or more stay.
@@ -624,7 +624,7 @@ bool pipe_tiles(const attn_tiles& t, int Lk, int d, int local_mem, int sms) {
   const int steps = (Lk + 127) / 128, waves = (t.tiles + sms - 1) / sms;
   if (d == 64) {
     const bool full = 100LL * t.tiles >= 98LL * waves * sms;       // the last wave
-    if (steps >= 32 || steps >= std::max(16, 4 + 6 * waves) || (full && steps >= 24)) return false;
+    if (steps >= 32 || steps >= (waves == 1 ? 16 : 6 + 6 * waves) || (full && steps >= 24)) return false;
     if (waves > 1 && Lk % 128 == 0 && steps % 2 == 1 && (steps == 5 || (steps >= 7 && full))) return false;
   }
   if (t.ctas == t.tiles) return t.tiles > sms || (steps >= 4 && (d == 64 || 10 * t.tiles > 7 * sms));
