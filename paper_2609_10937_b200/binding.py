@@ -30,7 +30,7 @@ BIND_NAMES = ("none", "smem", "tmem", "reg", "atom", "shape")
 EXPORTED_SYMBOLS = (
     "attn_hw_desc_b200", "attn_hw_desc_query", "attn_plan", "attn_plan_ex", "attn_workspace_bytes",
     "attn_set_workspace", "attn_workspace_init", "attn_forward_ws", "attn_status_read", "attn_forward", "attn_forward_causal", "attn_forward_tiles", "attn_forward_simple", "attn_forward_host", "attn_forward_host_workspace_bytes", "attn_forward_static_scratch", "attn_forward_desc", "attn_plan_qk", "attn_forward_qk", "attn_forward_call",
-    "attn_last_device_status", "attn_selftest_wait_expiry", "attn_selftest_wait_expiry_to", "attn_selftest_quiet_expiry_to",
+    "attn_last_device_status", "attn_selftest_wait_expiry", "attn_selftest_wait_expiry_to", "attn_selftest_quiet_expiry_to", "attn_selftest_issue_expiry_to",
     "attn_last_launch_count", "attn_last_cluster_size", "attn_last_kernel", "attn_last_grid", "attn_status_string", "attn_last_cuda_error",
     "gemm_plan", "gemm_forward", "gemm_forward_tiles", "softmax_rows_forward", "attn_forward_unfused", "gemm_forward_call", "softmax_rows_forward_call",
 )
@@ -131,6 +131,7 @@ def lib() -> ctypes.CDLL:
         L.attn_selftest_wait_expiry.argtypes = [vp]
         L.attn_selftest_wait_expiry_to.argtypes = [vp, vp]
         L.attn_selftest_quiet_expiry_to.argtypes = [vp, vp]
+        L.attn_selftest_issue_expiry_to.argtypes = [vp, vp]
         L.attn_last_launch_count.argtypes = []
         L.attn_last_cluster_size.argtypes = []
         L.attn_last_kernel.argtypes = []

@@ -1144,16 +1144,49 @@ __global__ void quiet_expiry_selftest_kernel(unsigned int* status) {
   __syncthreads();
   if (threadIdx.x == 0) attn::report_abort(&abort_cell);
 }
+
+// The way out of wait_on, as a warp that issues products takes it: a phase that nothing completes runs out, the wait after it ends at once,
+// no lane may issue or pass anything on, and the warp finds out when it looks.  A second warp whose phase has completed may issue, by
+// one lane.  The reported step is ATTN_SELFTEST_STEP only if all of that was so.
+__global__ void issue_expiry_selftest_kernel(unsigned int* status) {
+  __shared__ uint64_t bar, done_bar;
+  __shared__ attn::AbortCell abort_cell;
+  __shared__ int issued[2], seen;
+  const int warp = threadIdx.x >> 5;
+  if (threadIdx.x == 0) {
+    attn::abort_cell_init(&abort_cell, status);
+    sm100::mbar_init(sm100::smem_u32(&bar), 1);
+    sm100::mbar_init(sm100::smem_u32(&done_bar), 1);
+    sm100::fence_mbar_init();
+    sm100::mbar_arrive(sm100::smem_u32(&done_bar));
+    issued[0] = issued[1] = seen = 0;
+  }
+  __syncthreads();
+  const uint32_t info = attn::wait_info(attn::kRoleSimple, attn::kBarSync, ATTN_SELFTEST_STEP);
+  bool dead = false;
+  attn::wait_on(sm100::smem_u32(warp == 0 ? &bar : &done_bar), 0, &abort_cell.flag, info, dead);
+  const long long t0 = clock64();
+  if (warp == 0) attn::wait_on(sm100::smem_u32(&bar), 0, &abort_cell.flag, info, dead);
+  const bool quick = clock64() - t0 < attn::kWaitLimitCycles / 16;
+  if (attn::may_issue(dead)) atomicAdd(&issued[warp], 1);
+  __syncwarp();
+  if (attn::any_dead(dead) && dead && quick) atomicAdd(&seen, 1);
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    if (issued[0] != 0 || issued[1] != 1 || seen != 32) abort_cell.info = attn::wait_info(attn::kRoleSimple, attn::kBarSync, 0);
+    attn::report_abort(&abort_cell);
+  }
+}
 }  // namespace
 
 namespace {
 template <class Kernel>
-int launch_selftest(Kernel kern, uint32_t* status_dev, void* cuda_stream) {
+int launch_selftest(Kernel kern, uint32_t* status_dev, void* cuda_stream, int threads = 32) {
   if (status_dev && ((uintptr_t)status_dev & 15u)) return ATTN_ERR_MISALIGNED;
   DeviceState* st = nullptr;
   int rc = device_state(&st);
   if (rc != ATTN_OK) return rc;
-  kern<<<1, 32, 0, static_cast<cudaStream_t>(cuda_stream)>>>(status_dev);
+  kern<<<1, threads, 0, static_cast<cudaStream_t>(cuda_stream)>>>(status_dev);
   ATTN_CUDA_TRY(cudaGetLastError());
   return ATTN_OK;
 }
@@ -1165,6 +1198,10 @@ extern "C" int attn_selftest_wait_expiry_to(uint32_t* status_dev, void* cuda_str
 
 extern "C" int attn_selftest_quiet_expiry_to(uint32_t* status_dev, void* cuda_stream) {
   return launch_selftest(quiet_expiry_selftest_kernel, status_dev, cuda_stream);
+}
+
+extern "C" int attn_selftest_issue_expiry_to(uint32_t* status_dev, void* cuda_stream) {
+  return launch_selftest(issue_expiry_selftest_kernel, status_dev, cuda_stream, 64);
 }
 
 extern "C" int attn_selftest_wait_expiry(void* cuda_stream) { return attn_selftest_wait_expiry_to(nullptr, cuda_stream); }

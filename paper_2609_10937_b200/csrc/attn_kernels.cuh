@@ -114,8 +114,9 @@ __device__ __forceinline__ bool wait_quiet(uint32_t bar, uint32_t parity, volati
 __device__ __forceinline__ bool wait_quiet_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag, uint32_t info) {
   return __all_sync(0xffffffffu, wait_quiet(bar, parity, abort_flag, info) ? 1 : 0) != 0;
 }
-// Waits for a phase.  An expiry, here or elsewhere in the CTA, sets `dead`: the caller goes on, for at most a step, until it looks.
-// No warp waits for ever: those that follow an expired one find the abort flag.
+// Waits for a phase.  An expiry, here or elsewhere in the CTA, sets `dead`: the caller goes on, for at most a step, until it looks, on
+// registers and tensor memory of its own; it issues no product and passes on no buffer (may_issue).  No warp waits for ever: those that
+// follow an expired one find the abort flag.
 __device__ __forceinline__ void wait_on(uint32_t bar, uint32_t parity, volatile int* abort_flag, uint32_t info, bool& dead) {
   if (mbar_try_wait(bar, parity)) return;
   const uint32_t t0 = (uint32_t)clock64();
@@ -135,6 +136,9 @@ __device__ __forceinline__ void wait_on(uint32_t bar, uint32_t parity, volatile 
   }
 }
 __device__ __forceinline__ bool any_dead(bool dead) { return __any_sync(0xffffffffu, dead); }
+// The lane that issues a warp's products and their commits, if each of its waits has ended with the phase: what it issues reads operands that
+// have landed, and a buffer that it passes on has been filled.
+__device__ __forceinline__ bool may_issue(bool dead) { return elect_one() && !dead; }
 // On the way out of an expired wait: a copy that is under way must land before its memory is used again or the CTA exits.
 // Bounded like the waits; false if it has not landed.
 __device__ __forceinline__ bool drain_bar(uint32_t bar, uint32_t parity) {

@@ -430,7 +430,7 @@ attn_narrow_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
 #pragma unroll 1
       for (int x = 0; x < 2 * steps; ++x) {
         const int stage = take();
-        if (lane == 0) mbar_arrive(smem_u32(&misc->kv_empty[stage]));
+        if (lane == 0 && !dead) mbar_arrive(smem_u32(&misc->kv_empty[stage]));
       }
     };
     // A tile's first scores.
@@ -439,7 +439,7 @@ attn_narrow_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
       const int k = take();
       ++q_uses;
       tc_fence_after();
-      if (elect_one()) issue_scores(k, steps == 1);
+      if (may_issue(dead)) issue_scores(k, steps == 1);
       __syncwarp();
     };
     int tile = blockIdx.x;
@@ -455,7 +455,7 @@ attn_narrow_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
         if (j == 0 && done > 0) wait(&misc->o_free[i], (done - 1) & 1, kBarOFull);
         wait(&misc->p_full[st], g & 1, kBarPFull);
         tc_fence_after();
-        if (elect_one()) {
+        if (may_issue(dead)) {
           issue_pv<D, HKV>(o_tmem, s_tmem, k_smem + v * SM::kStageBytes, j > 0, TKV * 128, 1024);
           umma_commit(smem_u32(&misc->kv_empty[v]));
           if (more) issue_scores(k, j + 2 == n);
@@ -474,7 +474,7 @@ attn_narrow_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
           // nothing to add to the tile, nothing read of its Q (the arrivals of the tile before must all have been made: o_free)
           if (done > 1) wait(&misc->o_free[0], (done - 2) & 1, kBarOFull);
           wait(&misc->q_full[0][q_uses & 1], (q_uses >> 1) & 1, kBarQ);
-          if (lane == 0) {
+          if (lane == 0 && !dead) {
             mbar_arrive(smem_u32(&misc->q_empty[0][q_uses & 1]));
             mbar_arrive(smem_u32(&misc->o_full[0]));
           }

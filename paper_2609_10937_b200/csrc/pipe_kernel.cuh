@@ -303,6 +303,7 @@ attn_pipe_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
       const float inv = misc->inv[i][row];
       wait_on(smem_u32(&misc->o_full[i]), kSplit ? ((i ? g1 : g0) - 1) & 1 : (fin >> i) & 1, abort_flag, wait_info(kRoleCorrection, kBarOFull, 0x8000), dead);
       fin ^= 1u << i;
+      if (any_dead(dead)) return;                      // (nothing to store)
       tc_fence_after();
       const uint32_t o_tmem = lane_base + O_COL0 + i * D;
 #pragma unroll 1
@@ -423,8 +424,8 @@ attn_pipe_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
         if (kSplit && qk > 0) wait(&misc->s_free[i], (qk - 1) & 1, kBarSFull);
         ++qk;
         tc_fence_after();
-        if (elect_one()) issue_scores(k0, ni == 1);
-      } else if (lane == 0) {
+        if (may_issue(dead)) issue_scores(k0, ni == 1);
+      } else if (lane == 0 && !dead) {
         mbar_arrive(smem_u32(&misc->kv_empty[k0]));
       }
       __syncwarp();
@@ -438,7 +439,7 @@ attn_pipe_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
               wait(&misc->s_free[i], (qk - 1) & 1, kBarSFull);
               ++qk;
               tc_fence_after();
-              if (elect_one()) issue_scores(ks, j + 2 == ni);
+              if (may_issue(dead)) issue_scores(ks, j + 2 == ni);
               __syncwarp();
             }
           } else {
@@ -446,11 +447,11 @@ attn_pipe_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
           }
           wait(&misc->p_full[i], g & 1, kBarPFull);
           tc_fence_after();
-          if (elect_one()) issue_pv<D, TKV>(o_tmem, p_tmem, v, j > 0, TKV * 128, 1024, 0, kFirstK);
+          if (may_issue(dead)) issue_pv<D, TKV>(o_tmem, p_tmem, v, j > 0, TKV * 128, 1024, 0, kFirstK);
           __syncwarp();
           wait(&misc->p_half[i], g & 1, kBarPFull);
           tc_fence_after();
-          if (elect_one()) {
+          if (may_issue(dead)) {
             issue_pv<D, TKV>(o_tmem, p_tmem, v, true, TKV * 128, 1024, kFirstK, 8);
             if (!kSplit && j + 1 < ni) issue_scores(ks, j + 2 == ni);
             else umma_commit(smem_u32(&misc->o_full[i]));
@@ -463,7 +464,7 @@ attn_pipe_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
         } else {
           // a step that only the other sub-tile has
           if (!kSplit) wait(&misc->turn[i], (slot + 1 + i) & 1, kBarSync);
-          if (lane == 0) {
+          if (lane == 0 && !dead) {
             if (!kSplit) mbar_arrive(smem_u32(&misc->turn[i ^ 1]));
             mbar_arrive(smem_u32(&misc->kv_empty[vs]));
             if (j + 1 < n) mbar_arrive(smem_u32(&misc->kv_empty[ks]));
