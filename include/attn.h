@@ -402,7 +402,8 @@ int attn_selftest_wait_expiry_to(uint32_t *status_dev, void *cuda_stream);
  * a second. */
 int attn_selftest_quiet_expiry_to(uint32_t *status_dev, void *cuda_stream);
 /* The same for the wait that lets its warp go on for up to a step (softmax and product-issuing warps of the kernels of whole tiles):
- * detail[1] as above if no lane of the expired warp could issue a product or pass a buffer on, step 0 in it if one could. */
+ * detail[1] as above if no lane of the expired warp could issue a product or pass a buffer on, and a product that another warp had
+ * under way was complete when its drain ended; step 0 in it if not. */
 int attn_selftest_issue_expiry_to(uint32_t *status_dev, void *cuda_stream);
 
 /* Number of kernels the last attn_forward* call on this thread launched. */

@@ -1146,12 +1146,15 @@ __global__ void quiet_expiry_selftest_kernel(unsigned int* status) {
 }
 
 // The way out of wait_on, as a warp that issues products takes it: a phase that nothing completes runs out, the wait after it ends at once,
-// no lane may issue or pass anything on, and the warp finds out when it looks.  A second warp whose phase has completed may issue, by
-// one lane.  The reported step is ATTN_SELFTEST_STEP only if all of that was so.
+// no lane may issue or pass anything on, and the warp finds out when it looks.  A second warp whose phase has completed issues a product,
+// by one lane, and drains it: its accumulator, 128 x 128 sums of 64 ones, is complete then.  The reported step is ATTN_SELFTEST_STEP only
+// if all of that was so.
 __global__ void issue_expiry_selftest_kernel(unsigned int* status) {
-  __shared__ uint64_t bar, done_bar;
+  __shared__ __align__(1024) uint32_t ones[2][128 * 32];           // two tiles of [128][64] bf16
+  __shared__ uint64_t bar, done_bar, drained;
   __shared__ attn::AbortCell abort_cell;
-  __shared__ int issued[2], seen;
+  __shared__ int issued[2], seen, wrong;
+  __shared__ uint32_t tmem_slot;
   const int warp = threadIdx.x >> 5;
   if (threadIdx.x == 0) {
     attn::abort_cell_init(&abort_cell, status);
@@ -1159,21 +1162,47 @@ __global__ void issue_expiry_selftest_kernel(unsigned int* status) {
     sm100::mbar_init(sm100::smem_u32(&done_bar), 1);
     sm100::fence_mbar_init();
     sm100::mbar_arrive(sm100::smem_u32(&done_bar));
-    issued[0] = issued[1] = seen = 0;
+    issued[0] = issued[1] = seen = wrong = 0;
   }
+  for (int i = threadIdx.x; i < 2 * 128 * 32; i += blockDim.x) (&ones[0][0])[i] = 0x3F803F80u;
+  sm100::fence_proxy_async_smem();
+  if (warp == 1) {
+    sm100::tmem_alloc(sm100::smem_u32(&tmem_slot), 128);
+    sm100::tmem_relinquish();
+  }
+  sm100::tc_fence_before();
   __syncthreads();
+  sm100::tc_fence_after();
   const uint32_t info = attn::wait_info(attn::kRoleSimple, attn::kBarSync, ATTN_SELFTEST_STEP);
   bool dead = false;
   attn::wait_on(sm100::smem_u32(warp == 0 ? &bar : &done_bar), 0, &abort_cell.flag, info, dead);
   const long long t0 = clock64();
   if (warp == 0) attn::wait_on(sm100::smem_u32(&bar), 0, &abort_cell.flag, info, dead);
   const bool quick = clock64() - t0 < attn::kWaitLimitCycles / 16;
-  if (attn::may_issue(dead)) atomicAdd(&issued[warp], 1);
+  if (attn::may_issue(dead)) {
+    atomicAdd(&issued[warp], 1);
+    if (warp == 1) {
+      attn::issue_qk<64, 128>(tmem_slot, sm100::smem_u32(ones[0]), sm100::smem_u32(ones[1]));
+      if (!attn::drain_products(sm100::smem_u32(&drained))) atomicAdd(&wrong, 1);
+    }
+  }
   __syncwarp();
+  if (warp == 1) {
+    sm100::tc_fence_after();
+    for (int c = 0; c < 4; ++c) {
+      uint32_t r[32];
+      sm100::tmem_ld32(tmem_slot + (32u << 16) + c * 32, r);       // (rows 32 to 63: warp 1's)
+      for (int k = 0; k < 32; ++k)
+        if (r[k] != __float_as_uint(64.0f)) atomicAdd(&wrong, 1);
+    }
+    sm100::tc_fence_before();
+    __syncwarp();
+    sm100::tmem_dealloc(tmem_slot, 128);
+  }
   if (attn::any_dead(dead) && dead && quick) atomicAdd(&seen, 1);
   __syncthreads();
   if (threadIdx.x == 0) {
-    if (issued[0] != 0 || issued[1] != 1 || seen != 32) abort_cell.info = attn::wait_info(attn::kRoleSimple, attn::kBarSync, 0);
+    if (issued[0] != 0 || issued[1] != 1 || seen != 32 || wrong != 0) abort_cell.info = attn::wait_info(attn::kRoleSimple, attn::kBarSync, 0);
     attn::report_abort(&abort_cell);
   }
 }

@@ -147,6 +147,25 @@ __device__ __forceinline__ bool drain_bar(uint32_t bar, uint32_t parity) {
     if (clock64() - t0 > kWaitLimitCycles) return false;
   return true;
 }
+// The same for products, by the lane that issued a warp's: they must have finished before tensor memory is freed or the CTA exits.  (On the
+// usual way out the warp waits for the commit behind the last of them instead, while others do the same.)  `bar` is memory for a
+// barrier that nothing else uses.  kPair: the products of a pair of CTAs, by the even one's lane.  For the matrix products.
+template <bool kPair = false>
+__device__ __forceinline__ bool drain_products(uint32_t bar) {
+  mbar_init(bar, 1);
+  fence_mbar_init();
+  if constexpr (kPair) umma_commit_pair(bar, 1);
+  else umma_commit(bar);
+  return drain_bar(bar, 0);
+}
+// The same in the attention kernels, by the warp that frees tensor memory, behind the CTA's last barrier and an expired wait.  An instruction
+// is issued when those in front of it have started, so that two or three of up to 256 cycles each may be under way, with nothing but
+// on-chip operands: this is a thousand times as long, and covers the products of every warp, whichever wait ran out.  (drain_products
+// in their MMA warps and at their ends: more spills, 1 to 3 % on short plans; 24 heads x 512 causal, d = 64 11.1 / 11.4 us.)
+__device__ __forceinline__ void products_end() {
+  const long long t0 = clock64();
+  while (clock64() - t0 < 1000000LL) {}
+}
 // By one thread, when every thread of the CTA is past its last wait.
 __device__ __forceinline__ void report_abort(const AbortCell* c) {
   if (c->flag == 0) return;
@@ -1638,6 +1657,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
   }
   if (warp == 15) {
     tc_fence_after();
+    if (*abort_flag) products_end();
     tmem_dealloc(tmem_base, TMEM_COLS);
   }
 }

@@ -68,6 +68,7 @@ struct GemmMisc {
   uint64_t acc_full;      // all products of a tile have finished
   uint64_t acc_empty;     // the epilogue has read the accumulators of a tile
   uint64_t epi_sync[2];   // rendezvous of the four epilogue warps of a sub-tile
+  uint64_t drained;       // for drain_products
   attn::AbortCell abort;
   uint32_t tmem_slot;
 };
@@ -184,7 +185,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CU
         bool ok = true;
         for (long long t = blockIdx.x; ok && t < tiles; t += gridDim.x, ++tile_ctr) {
           if (tile_ctr > 0) {
-            if (!attn::wait_bar(smem_u32(&misc->acc_empty), (tile_ctr - 1) & 1, abort_flag, attn::wait_info(kRoleGemmMma, 2, tile_ctr))) break;
+            if (!attn::wait_bar(smem_u32(&misc->acc_empty), (tile_ctr - 1) & 1, abort_flag, attn::wait_info(kRoleGemmMma, 2, tile_ctr))) { ok = false; break; }
             tc_fence_after();
           }
           for (int ks = 0; ks < p.k_steps; ++ks) {
@@ -196,6 +197,9 @@ gemm_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CU
             if (++stage == p.stages) { stage = 0; phase ^= 1u; }
           }
         }
+        // no product is under way when this warp leaves
+        if (ok && tile_ctr > 0) ok = attn::wait_bar(smem_u32(&misc->acc_full), (tile_ctr - 1) & 1, abort_flag, attn::wait_info(kRoleGemmMma, 3, tile_ctr));
+        if (!ok) attn::drain_products(smem_u32(&misc->drained));
       }
       __syncwarp();
     } else {
@@ -219,6 +223,9 @@ gemm_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CU
           if (++stage == p.stages) { stage = 0; phase ^= 1u; }
         }
       }
+      if (ok && tile_ctr > 0) ok = attn::wait_bar_warp(smem_u32(&misc->acc_full), (tile_ctr - 1) & 1, abort_flag, attn::wait_info(kRoleGemmMma, 3, tile_ctr));
+      if (!ok && elect_one()) attn::drain_products(smem_u32(&misc->drained));
+      __syncwarp();
     }
   } else {
     // ============================================================== epilogue
@@ -301,6 +308,7 @@ struct GemmPairMisc {
   uint64_t empty[kMaxStages];
   uint64_t acc_full[4];
   uint64_t acc_empty[4];
+  uint64_t drained;       // for drain_products (even CTA)
   attn::AbortCell abort;
   uint32_t tmem_slot;
 };
@@ -453,6 +461,11 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant
         if (++stage == p.stages) { stage = 0; phase ^= 1u; }
       }
     }
+    // no product of the pair is under way when this warp leaves
+    if (ok && tile_ctr > 0)
+      ok = attn::wait_bar_warp(smem_u32(&misc->acc_full[(tile_ctr - 1) % kBufs]), ((tile_ctr - 1) / kBufs) & 1, abort_flag, attn::wait_info(kRoleGemmMma, 3, tile_ctr));
+    if (!ok && rank == 0 && elect_one()) attn::drain_products<true>(smem_u32(&misc->drained));
+    __syncwarp();
   } else {
     // ============================================================== epilogue (both CTAs, each its own 128 rows)
     // Eight warps, none of which meets another: warp w reads lanes 32 (w mod 4) .. + 31 (its rows) of one column
@@ -629,6 +642,8 @@ gemm_small_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constan
         if (ks == p.k_steps - 1) umma_commit(smem_u32(&misc->acc_full));
         if (++stage == p.stages) { stage = 0; phase ^= 1u; }
       }
+      // no product is under way when this warp leaves
+      if (!attn::wait_bar(smem_u32(&misc->acc_full), 0, abort_flag, attn::wait_info(kRoleGemmMma, 3, 0))) attn::drain_products(smem_u32(&misc->drained));
     }
     __syncwarp();
   } else {

@@ -569,6 +569,7 @@ attn_narrow_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
   __syncthreads();
   if (warp == SH::kAllocWarp) {
     tc_fence_after();
+    if (*abort_flag) products_end();
     tmem_dealloc(tmem_base, 512);
   }
   if (threadIdx.x == 0) report_abort(&misc->abort);

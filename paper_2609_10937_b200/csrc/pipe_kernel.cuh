@@ -576,6 +576,7 @@ attn_pipe_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
   __syncthreads();
   if (warp == 15) {
     tc_fence_after();
+    if (*abort_flag) products_end();
     tmem_dealloc(tmem_base, 512);
   }
   if (threadIdx.x == 0) report_abort(&misc->abort);

@@ -8,7 +8,7 @@ pytestmark = pytest.mark.gpu
 def test_a_warp_whose_wait_expired_issues_nothing(own_status):
     """A warp of the library's self-test waits, as the warps that issue products do, on a barrier nothing arrives at (half a second).
     None of its lanes may issue afterwards, its next wait ends at once, and the expiry is reported in the caller's status words or in the
-    device-wide record; a warp whose phase had completed may issue.  The kernels that wait this way then compute as before."""
+    device-wide record; a warp whose phase had completed issues a product, whose drain leaves it complete.  The kernels that wait this way then compute as before."""
     torch = pytest.importorskip("torch")
     from paper_2609_10937_b200 import binding
 
