@@ -277,6 +277,8 @@ def _prep(q, k, v, o):
         raise ValueError("q, k, v must be CUDA tensors (there is no CPU path)")
     if not (q.is_contiguous() and k.is_contiguous() and v.is_contiguous()):
         raise ValueError("q, k, v must be contiguous [B][H][L][d]")
+    if k.device != q.device or v.device != q.device:
+        raise ValueError("q, k, v must be on one device")
     if o is None:
         o = torch.empty_like(q)
     elif o.shape != q.shape or o.dtype != torch.bfloat16 or not o.is_contiguous() or o.device != q.device:
@@ -375,7 +377,7 @@ def plan_qk(desc: AttnHwDesc, B: int, H: int, Lq: int, Lk: int, d: int) -> AttnT
 
 
 def forward_qk(q, k, v, o=None):
-    """O = softmax(Q K^T / sqrt(d)) V for q [B, H, Lq, d] and k, v [B, H, Lk, d] (contiguous CUDA bf16)."""
+    """O = softmax(Q K^T / sqrt(d)) V for q [B, H, Lq, d] and k, v [B, H, Lk, d] (contiguous CUDA bf16); o: B*H*Lq*d elements in a row."""
     done = _fast.attn(q, k, v, o, False, True)
     if done is not None:
         return done
@@ -387,8 +389,12 @@ def forward_qk(q, k, v, o=None):
     Lk = k.shape[2]
     if k.shape != (B, H, Lk, d) or v.shape != (B, H, Lk, d):
         raise ValueError("k and v must be [B, H, Lk, d] with q's B, H and d")
+    if k.device != q.device or v.device != q.device:
+        raise ValueError("q, k, v must be on one device")
     if o is None:
         o = torch.empty_like(q)
+    elif o.dtype != torch.bfloat16 or not o.is_contiguous() or o.numel() != q.numel() or o.device != q.device:
+        raise ValueError("o must be a contiguous bfloat16 tensor of B*H*Lq*d elements on q's device")
     dev = q.get_device()
     _call(dev, "attn_forward_qk", lib().attn_forward_call,
           _ATTN_CALL(q.data_ptr(), k.data_ptr(), v.data_ptr(), o.data_ptr(), _stream(dev), B, H, Lq, Lk, d, 0),
@@ -523,6 +529,8 @@ def gemm(a, b, c=None, *, b_layout="kn", cta_pair=0, tile_n=0, tail_split=0):
         raise ValueError("b_layout is 'kn' or 'nk'")
     if kb != K or b_batch != batch:
         raise ValueError("a and b do not agree in batch or K")
+    if b.device != a.device:
+        raise ValueError("a and b must be on one device")
     if c is None:
         c = torch.empty((batch, M, N) if a.dim() == 3 else (M, N), dtype=torch.bfloat16, device=a.device)
     elif c.dtype != torch.bfloat16 or not c.is_contiguous() or c.numel() != batch * M * N or c.device != a.device:
