@@ -175,7 +175,7 @@ class _LazyFast:
             module = util.module_from_spec(util.spec_from_loader(loader.name, loader))
             loader.exec_module(module)
             module.bind(*(ctypes.cast(f, ctypes.c_void_p).value for f in (
-                handle.attn_forward_call, handle.gemm_forward_call, handle.softmax_rows_forward_call)))
+                handle.attn_forward_call, handle.gemm_forward_call, handle.softmax_rows_forward_call)), _refused)
             _fast = module
         else:
             _fast = _NoFast
@@ -183,6 +183,10 @@ class _LazyFast:
 
 
 _fast = _LazyFast()
+
+
+def _refused(rc: int, where: str):
+    raise AttnError(rc, where)
 
 
 def status_string(code: int) -> str:

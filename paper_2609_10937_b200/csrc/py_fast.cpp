@@ -1,6 +1,7 @@
 // The usual call of binding.py in native code: tensors checked, the output allocated, the argument struct filled and the
-// library entered without the interpreter in between.  What is not the usual call returns None and goes through binding.py,
-// which checks, reports and provides a workspace; nothing has been launched then.
+// library entered without the interpreter in between.  What is not the usual call, or lacks a workspace, returns None and goes through
+// binding.py, which checks, reports and provides one; nothing has been launched then.  What the library refuses otherwise is
+// raised from here: entered again, a call could succeed and an error of CUDA's that the first entry took would be lost.
 //
 // A call of one head of 256 x 256 takes its kernel 4.9 us and took the host 7.1: the interpreter's part of that, attribute by attribute,
 // was 3.3 us and is under 1 here (loop of calls: 7.3 -> 5.3 us; small row softmax 5.3 -> 3.5).
@@ -26,6 +27,7 @@ namespace {
 int (*g_attn)(const attn_call*) = nullptr;
 int (*g_gemm)(const gemm_call*) = nullptr;
 int (*g_softmax)(const softmax_call*) = nullptr;
+PyObject* g_refused = nullptr;   // binding.py's: raises for (status, entry point)
 
 // Someone looks at or stands in for the operations of a call: those are binding.py's to make.
 bool watched() {
@@ -64,8 +66,13 @@ int enter(int (*fn)(const C*), const C& call) {
   Py_END_ALLOW_THREADS
   return rc;
 }
-PyObject* answer(int rc, PyObject* given, at::Tensor& made) {
-  if (rc != 0) Py_RETURN_NONE;
+PyObject* answer(int rc, const char* where, PyObject* given, at::Tensor& made) {
+  if (rc == ATTN_ERR_NEED_WORKSPACE) Py_RETURN_NONE;
+  if (rc != ATTN_OK) {
+    Py_XDECREF(PyObject_CallFunction(g_refused, "is", rc, where));
+    if (!PyErr_Occurred()) PyErr_SetString(PyExc_RuntimeError, where);
+    return nullptr;
+  }
   if (given != Py_None) return Py_NewRef(given);
   return THPVariable_Wrap(std::move(made));
 }
@@ -104,7 +111,7 @@ PyObject* py_attn(PyObject*, PyObject* const* args, Py_ssize_t n) {
   c.Lk = (int)ks[2];
   c.d = (int)qs[3];
   c.causal = causal;
-  return answer(enter(g_attn, c), args[3], made);
+  return answer(enter(g_attn, c), other_length ? "attn_forward_qk" : causal ? "attn_forward_causal" : "attn_forward", args[3], made);
   END_HANDLE_TH_ERRORS
 }
 
@@ -141,7 +148,7 @@ PyObject* py_gemm(PyObject*, PyObject* const* args, Py_ssize_t n) {
   g.N = (int)N;
   g.K = (int)K;
   g.b_layout = kn ? 0 : 1;
-  return answer(enter(g_gemm, g), args[2], made);
+  return answer(enter(g_gemm, g), "gemm_forward", args[2], made);
   END_HANDLE_TH_ERRORS
 }
 
@@ -169,14 +176,14 @@ PyObject* py_softmax(PyObject*, PyObject* const* args, Py_ssize_t n) {
   c.cols = (int)s->sizes().back();
   c.rows = s->numel() / c.cols;
   c.scale = PyFloat_AS_DOUBLE(args[1]);
-  return answer(enter(g_softmax, c), args[2], made);
+  return answer(enter(g_softmax, c), "softmax_rows_forward", args[2], made);
   END_HANDLE_TH_ERRORS
 }
 
-// bind(addresses of attn_forward_call, gemm_forward_call, softmax_rows_forward_call)
+// bind(addresses of attn_forward_call, gemm_forward_call, softmax_rows_forward_call, a callable that raises for a status and an entry point)
 PyObject* py_bind(PyObject*, PyObject* const* args, Py_ssize_t n) {
-  if (n != 3) {
-    PyErr_SetString(PyExc_TypeError, "bind takes three addresses");
+  if (n != 4 || !PyCallable_Check(args[3])) {
+    PyErr_SetString(PyExc_TypeError, "bind takes three addresses and a callable");
     return nullptr;
   }
   void* p[3];
@@ -190,6 +197,7 @@ PyObject* py_bind(PyObject*, PyObject* const* args, Py_ssize_t n) {
   g_attn = reinterpret_cast<decltype(g_attn)>(p[0]);
   g_gemm = reinterpret_cast<decltype(g_gemm)>(p[1]);
   g_softmax = reinterpret_cast<decltype(g_softmax)>(p[2]);
+  Py_XSETREF(g_refused, Py_NewRef(args[3]));
   Py_RETURN_NONE;
 }
 

@@ -82,3 +82,30 @@ def test_what_is_not_usual_is_left_to_binding(binding):
     assert seen == [None]
     assert fast.softmax(q, 1, None) is None and fast.gemm(q[0], q[0], None, 0) is None
     assert binding.last_kernel() == before and binding.last_device_status()[0] == 0
+
+
+@pytest.mark.gpu
+def test_a_refusal_is_raised_by_the_entry_that_met_it(binding):
+    """The library is entered once: a second entry could succeed where the first one met, and took, an error of CUDA's."""
+    import ctypes
+
+    torch = importlib.import_module("torch")
+    q, a = torch.zeros(1, 2, 64, 64, dtype=torch.bfloat16, device="cuda"), torch.zeros(64, 64, dtype=torch.bfloat16, device="cuda")
+    binding.forward(q, q, q)                                  # (loads the module)
+    handle, entered = binding.lib(), []
+    fail = ctypes.CFUNCTYPE(ctypes.c_int, ctypes.c_void_p)(lambda call: entered.append(call) or binding.ERR_CUDA)
+    address = lambda f: ctypes.cast(f, ctypes.c_void_p).value
+    binding._fast.bind(address(fail), address(fail), address(fail), binding._refused)
+    try:
+        before = binding.last_kernel(), binding.last_grid()
+        for call, where in ((lambda: binding.forward(q, q, q), "attn_forward"), (lambda: binding.forward(q, q, q, causal=True), "attn_forward_causal"),
+                            (lambda: binding.forward_qk(q, q, q), "attn_forward_qk"), (lambda: binding.gemm(a, a), "gemm_forward"),
+                            (lambda: binding.softmax_rows(a, 1.0), "softmax_rows_forward")):
+            entered.clear()
+            with pytest.raises(binding.AttnError) as err:
+                call()
+            assert err.value.code == binding.ERR_CUDA and where in str(err.value) and len(entered) == 1
+        assert before == (binding.last_kernel(), binding.last_grid())
+    finally:
+        binding._fast.bind(address(handle.attn_forward_call), address(handle.gemm_forward_call), address(handle.softmax_rows_forward_call), binding._refused)
+    assert binding.forward(q, q, q).shape == q.shape and binding.last_device_status()[0] == 0
