@@ -13,11 +13,11 @@ from __future__ import annotations
 import ctypes
 import math
 import struct
+import warnings
 from pathlib import Path
 
 _PKG = Path(__file__).resolve().parent
 LIB_PATH = _PKG / "libattn_b200.so"
-_FAST_PATH = _PKG / "_fast.so"
 
 ATTN_OK = 0
 ERR_INVALID_ARG, ERR_UNSUPPORTED_SHAPE, ERR_MISALIGNED, ERR_ALIASING = -1, -2, -3, -4
@@ -152,7 +152,7 @@ def lib() -> ctypes.CDLL:
 
 
 class _NoFast:
-    """Stands in for csrc/py_fast.cpp where it has not been built: no call is the usual one."""
+    """Stands in for csrc/py_fast.cpp where it has not been built, or not for this interpreter and torch: no call is the usual one."""
 
     @staticmethod
     def attn(*args):
@@ -161,24 +161,35 @@ class _NoFast:
     gemm = softmax = attn
 
 
+def _load_fast(handle):
+    """csrc/py_fast.cpp with the library's entry points, or _NoFast."""
+    import torch  # noqa: F401  (whose libraries the module needs)
+    from importlib import machinery, util
+
+    from .build import fast_path
+
+    path = fast_path()
+    if not path.exists():
+        return _NoFast
+    loader = machinery.ExtensionFileLoader(__package__ + "._fast", str(path))
+    try:
+        module = util.module_from_spec(util.spec_from_loader(loader.name, loader))
+        loader.exec_module(module)
+    except ImportError as e:
+        warnings.warn(f"{path.name} cannot be loaded ({e}): build it again (python -m {__package__}.build); calls go without it")
+        return _NoFast
+    module.bind(*(ctypes.cast(f, ctypes.c_void_p).value for f in (
+        handle.attn_forward_call, handle.gemm_forward_call, handle.softmax_rows_forward_call)), _refused)
+    return module
+
+
 class _LazyFast:
     """csrc/py_fast.cpp, loaded with the first call."""
 
     def __getattr__(self, name):
         global _fast
         handle = lib()
-        if _FAST_PATH.exists():
-            import torch  # noqa: F401  (whose libraries the module needs)
-            from importlib import machinery, util
-
-            loader = machinery.ExtensionFileLoader(__package__ + "._fast", str(_FAST_PATH))
-            module = util.module_from_spec(util.spec_from_loader(loader.name, loader))
-            loader.exec_module(module)
-            module.bind(*(ctypes.cast(f, ctypes.c_void_p).value for f in (
-                handle.attn_forward_call, handle.gemm_forward_call, handle.softmax_rows_forward_call)), _refused)
-            _fast = module
-        else:
-            _fast = _NoFast
+        _fast = _load_fast(handle)
         return getattr(_fast, name)
 
 
