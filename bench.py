@@ -287,22 +287,6 @@ class Gpu:
             raise RuntimeError(f"device-side wait expired: {detail}")
 
 
-def kernel_name(plan, d, cluster, last=None, L=0, sms=148):
-    """The instantiation a plan ran as: <d, tile_kv, n_q, causal, fixed merge roles, clusters>; `last`: (kernel, CTAs) of the launch."""
-    from paper_2609_10937_b200 import binding
-
-    if last is not None and cluster == 0 and last[1] == plan.tiles and plan.n_q == 2:
-        # one CTA per tile of 256 rows: the kernel of two streams a tile, where the library takes it (pipe_tiles, attn_api.cu)
-        steps = -(-L // 128)
-        if last[0] == binding.KERNEL_TILED and (plan.ctas != plan.tiles or plan.tiles > sms or (steps >= 4 and (d == 64 or 10 * plan.tiles > 7 * sms))):
-            return f"attn_pipe_kernel<{d},0>"
-    if last is not None and last[0] == binding.KERNEL_NARROW_TILES:
-        return f"attn_narrow_kernel<{d},0,{2 if last[1] == plan.tiles else 1}>"
-    uniform = plan.ctas > plan.tiles and plan.ctas % plan.tiles == 0
-    fixed = int((uniform and not plan.causal) or (plan.causal and cluster > 0))
-    return f"attn_fwd_kernel<{d},{plan.tile_kv},{plan.n_q},{int(plan.causal)},{fixed},{int(cluster > 0)}>"
-
-
 def measure_config(gpu, name, peaks, iters=None, oracle=True):
     """One benchmark configuration with the closed-form default tiles: time, TFLOP/s, error against the oracle."""
     from paper_2609_10937_b200 import synth
@@ -316,7 +300,7 @@ def measure_config(gpu, name, peaks, iters=None, oracle=True):
     if iters is None:
         iters = 100 if case.flops < 1e9 else 30 if case.flops < 5e11 else 10
     ms_mean, per, _, _ = gpu.timed(lambda: binding.forward(dq, dk, dv, do), iters, 5)
-    cluster, last = binding.last_cluster_size(), (binding.last_kernel(), binding.last_grid())
+    cluster, kernel = binding.last_cluster_size(), binding.last_kernel_name()
     gpu.check_status()
     # the median of the per-launch times: one launch delayed on the host side (the events bracket the launch call)
     # would otherwise carry into a mean over few launches
@@ -326,7 +310,7 @@ def measure_config(gpu, name, peaks, iters=None, oracle=True):
            "frac_of_measured_burst_peak": tf / peaks["bf16_tflops"], "launches_timed": iters,
            "tiles": {"tile_q": plan.tile_q, "tile_kv": plan.tile_kv, "kv_stages": plan.kv_stages, "q_tiles": plan.tiles,
                      "ctas": plan.ctas, "cluster": cluster, "cost_steps": plan.cost_steps},
-           "kernel": kernel_name(plan, case.d, cluster, last, case.L, gpu.desc.num_units)}
+           "kernel": kernel}
     if oracle:
         from oracle import attn_oracle as orc
 
@@ -419,7 +403,7 @@ def run_ours(args):
     ms, per, t0, t1 = gpu.timed(step, args.steps, args.warmup, barrier)
     ms = multirank.max_over_ranks(ms, dist, "cuda")      # the slowest rank sets the step time
     launches_per_step = binding.last_launch_count()
-    cluster = binding.last_cluster_size()
+    cluster, kernel = binding.last_cluster_size(), binding.last_kernel_name()
     clocks = sampler.window(t0, t1) if sampler else None
     gpu.check_status()
     e2e_steps = max(3, min(args.steps, 10))
@@ -462,7 +446,7 @@ def run_ours(args):
             "traffic_source": ({k_: capture.get(k_) for k_ in ("capture", "commit", "kernel")} if capture else None),
             "peak_source": f"{peaks['source']} cuBLAS bf16 burst (kernel timed alone)",
             "frac_of_nominal_2250": achieved / 2250.0,
-            "kernel": kernel_name(plan, case.d, cluster) + " (one launch per step; split-key partials are merged in the same kernel)",
+            "kernel": kernel + " (one launch per step; split-key partials are merged in the same kernel)",
             "algorithmic_flops_per_launch": flops,
             "unfused_traffic_bytes_bf16_scores": unfused_bytes(case.B, case.H, case.L, case.d, 2, 2),
             "compulsory_traffic_bytes": fused_bytes(case.B, case.H, case.L, case.d, 2),

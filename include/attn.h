@@ -431,6 +431,10 @@ enum attn_kernel {
 };
 int attn_last_kernel(void);
 int attn_last_grid(void);
+/* The same kernel by its name in the library's sources, attention and products with their template arguments as numbers
+ * ("attn_pipe_kernel<128,1>"); "" before the first launch.  attn_last_kernel groups calls by what is asked for, and several kernels
+ * answer to 1, 2 and 9; this tells them apart.  Valid until the thread asks again. */
+const char *attn_last_kernel_name(void);
 
 /* Static description of a status code; never NULL. */
 const char *attn_status_string(int status);

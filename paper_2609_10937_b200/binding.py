@@ -31,7 +31,7 @@ EXPORTED_SYMBOLS = (
     "attn_hw_desc_b200", "attn_hw_desc_query", "attn_plan", "attn_plan_ex", "attn_workspace_bytes",
     "attn_set_workspace", "attn_workspace_init", "attn_forward_ws", "attn_status_read", "attn_forward", "attn_forward_causal", "attn_forward_tiles", "attn_forward_simple", "attn_forward_host", "attn_forward_host_workspace_bytes", "attn_forward_static_scratch", "attn_forward_desc", "attn_plan_qk", "attn_forward_qk", "attn_forward_call",
     "attn_last_device_status", "attn_selftest_wait_expiry", "attn_selftest_wait_expiry_to", "attn_selftest_quiet_expiry_to", "attn_selftest_issue_expiry_to",
-    "attn_last_launch_count", "attn_last_cluster_size", "attn_last_kernel", "attn_last_grid", "attn_status_string", "attn_last_cuda_error",
+    "attn_last_launch_count", "attn_last_cluster_size", "attn_last_kernel", "attn_last_kernel_name", "attn_last_grid", "attn_status_string", "attn_last_cuda_error",
     "gemm_plan", "gemm_forward", "gemm_forward_tiles", "softmax_rows_forward", "attn_forward_unfused", "gemm_forward_call", "softmax_rows_forward_call",
 )
 # attn_call, gemm_call, softmax_call (native alignment; the trailing 0q pads to the struct's size)
@@ -140,6 +140,7 @@ def lib() -> ctypes.CDLL:
         L.attn_status_string.restype = ctypes.c_char_p
         L.attn_last_cuda_error.argtypes = []
         L.attn_last_cuda_error.restype = ctypes.c_char_p
+        L.attn_last_kernel_name.restype = ctypes.c_char_p
         L.gemm_plan.argtypes = [ctypes.POINTER(AttnHwDesc), i32, i32, i32, i32, ctypes.POINTER(GemmTiles)]
         L.gemm_forward.argtypes = [vp, vp, vp, i32, i32, i32, i32, i32, vp]
         L.gemm_forward_tiles.argtypes = [vp, vp, vp, i32, i32, i32, i32, i32, ctypes.POINTER(GemmTiles), vp]
@@ -502,6 +503,11 @@ def last_cluster_size() -> int:
 def last_kernel() -> int:
     """Kernel of the last launch on this thread (KERNEL_...)."""
     return int(lib().attn_last_kernel())
+
+
+def last_kernel_name() -> str:
+    """Its name and template arguments, as in "attn_pipe_kernel<128,1>" ("" before the first launch)."""
+    return lib().attn_last_kernel_name().decode()
 
 
 def last_grid() -> int:

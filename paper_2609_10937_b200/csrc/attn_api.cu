@@ -27,7 +27,13 @@ thread_local char t_cuda_error[256] = "";
 thread_local int t_launch_count = 0;
 thread_local int t_cluster_size = 0;   // CTAs per thread-block cluster of the last fused launch (0: no clusters)
 thread_local int t_kernel = ATTN_KERNEL_NONE, t_grid = 0;   // the last launch and its CTAs
-void launched(int kernel, long long ctas) { t_kernel = kernel; t_grid = (int)ctas; }
+// Name and template arguments of the last launch's kernel, put together where they are asked for.
+struct Instantiation {
+  const char* name = "";
+  int args = 0, arg[6] = {};
+};
+thread_local Instantiation t_instantiation;
+void launched(int kernel, long long ctas, const Instantiation& inst) { t_kernel = kernel; t_grid = (int)ctas; t_instantiation = inst; }
 
 int cuda_fail(cudaError_t e, const char* what) {
   (void)cudaGetLastError();              // reported here: the next call must not find it again
@@ -296,6 +302,7 @@ int launch_fwd(const void* q, const void* k, const void* v, void* o, int B, int 
     ATTN_CUDA_TRY(launch_kernel(kern, grid, 512, smem, 0, stream, tq, tk, tv, to, p));
     return ATTN_OK;
   };
+  bool fixed_roles = false;                              // of the instantiation that is launched
   const int ck = (t.tiles > 0 && t.ctas % t.tiles == 0) ? t.ctas / t.tiles : 0;
   const size_t c_landing = ck > 2 ? (size_t)((4 * NQ + ck - 1) / ck) * (ck - 1) * (32 * D * 4 + 256) : 0;
   if (p.causal && ck >= 2 && ck <= 4 && p.ratio >= 2 && c_landing <= (size_t)t.kv_stages * SM::kStageBytes) {
@@ -331,6 +338,7 @@ int launch_fwd(const void* q, const void* k, const void* v, void* o, int B, int 
     }
     if ((long long)n_res * ck >= grid && launch_kernel(kern, grid, 512, smem, ck, stream, tq, tk, tv, to, pc) == cudaSuccess) {
       t_cluster_size = ck;
+      fixed_roles = true;
       rc = ATTN_OK;
     } else {
       (void)cudaGetLastError();
@@ -339,12 +347,13 @@ int launch_fwd(const void* q, const void* k, const void* v, void* o, int B, int 
   } else if (p.causal) rc = launch(attn::attn_fwd_kernel<D, TKV, NQ, true, false>);
   else if (eager) {
     rc = launch_eager(attn::attn_fwd_kernel<D, TKV, NQ, false, true>, attn::attn_fwd_kernel<D, TKV, NQ, false, true, true>);
+    fixed_roles = rc == ATTN_OK;
     if (rc == ATTN_ERR_BAD_TILES && !wait_roles_ok) rc = launch(attn::attn_fwd_kernel<D, TKV, NQ, false, false>);
   } else rc = launch(attn::attn_fwd_kernel<D, TKV, NQ, false, false>);
   if (rc != ATTN_OK) return rc;
   ATTN_CUDA_TRY(cudaGetLastError());
   t_launch_count = 1;
-  launched(ATTN_KERNEL_TILED, grid);
+  launched(ATTN_KERNEL_TILED, grid, {"attn_fwd_kernel", 6, {D, TKV, NQ, p.causal, fixed_roles ? 1 : 0, t_cluster_size > 0 ? 1 : 0}});
   return ATTN_OK;
 }
 
@@ -376,7 +385,7 @@ int launch_decode(const void* q, const void* k, const void* v, void* o, int BH, 
   ATTN_CUDA_TRY(launch_kernel(kern, (long long)BH * cluster_k, 32 * attn::kDecodeWarps, smem, cluster_k, stream, tk, tv, p));
   t_cluster_size = cluster_k > 1 ? cluster_k : 0;
   t_launch_count = 1;
-  launched(ATTN_KERNEL_FEW_ROWS, (long long)BH * cluster_k);
+  launched(ATTN_KERNEL_FEW_ROWS, (long long)BH * cluster_k, {"attn_decode_kernel", 3, {D, MT, HALF ? 1 : 0}});
   return ATTN_OK;
 }
 
@@ -485,7 +494,7 @@ int launch_pipe(const void* q, const void* k, const void* v, void* o, int BH, in
   ATTN_CUDA_TRY(launch_kernel(kern, (long long)BH * p.q_tiles, 512, smem, 0, stream, tq, tk, tv, to, p));
   t_cluster_size = 0;
   t_launch_count = 1;
-  launched(kernel_id, (long long)BH * p.q_tiles);
+  launched(kernel_id, (long long)BH * p.q_tiles, {"attn_pipe_kernel", 2, {D, CAUSAL ? 1 : 0}});
   return ATTN_OK;
 }
 
@@ -517,7 +526,8 @@ int launch_narrow(const void* q, const void* k, const void* v, void* o, int BH, 
   ATTN_CUDA_TRY(launch_kernel(kern, (long long)BH * p.q_tiles, attn::NarrowShape<D>::kThreads, smem, 0, stream, tq, tk, tv, to, p));
   t_cluster_size = 0;
   t_launch_count = 1;
-  launched(CAUSAL ? ATTN_KERNEL_CAUSAL_TILES : ATTN_KERNEL_NARROW_TILES, (long long)BH * p.q_tiles);
+  launched(CAUSAL ? ATTN_KERNEL_CAUSAL_TILES : ATTN_KERNEL_NARROW_TILES, (long long)BH * p.q_tiles,
+           {"attn_narrow_kernel", 3, {D, CAUSAL ? 1 : 0, SUBS}});
   return ATTN_OK;
 }
 
@@ -779,7 +789,7 @@ int launch_simple(const void* q, const void* k, const void* v, void* o, int B, i
   kern<<<grid, 128, smem, stream>>>(tq, tk, tv, reinterpret_cast<__nv_bfloat16*>(o), L, scale_log2, scores_out);
   ATTN_CUDA_TRY(cudaGetLastError());
   t_launch_count = 1;
-  launched(ATTN_KERNEL_SIMPLE, (long long)grid.x * grid.y);
+  launched(ATTN_KERNEL_SIMPLE, (long long)grid.x * grid.y, {"attn_fwd_simple_kernel", 2, {D, TKV}});
   return ATTN_OK;
 }
 
@@ -1259,6 +1269,13 @@ extern "C" int attn_last_launch_count(void) { return t_launch_count; }
 extern "C" int attn_last_cluster_size(void) { return t_cluster_size; }
 extern "C" int attn_last_kernel(void) { return t_kernel; }
 extern "C" int attn_last_grid(void) { return t_grid; }
+extern "C" const char* attn_last_kernel_name(void) {
+  thread_local char text[96];
+  const Instantiation& x = t_instantiation;
+  int n = std::snprintf(text, sizeof text, "%s", x.name);
+  for (int i = 0; i < x.args; ++i) n += std::snprintf(text + n, sizeof text - n, "%c%d%s", i ? ',' : '<', x.arg[i], i + 1 == x.args ? ">" : "");
+  return text;
+}
 
 extern "C" const char* attn_last_cuda_error(void) { return t_cuda_error; }
 
@@ -1358,7 +1375,7 @@ int gemm_launch(const void* a, const void* b, void* c, int batch, int M, int N, 
     if (rc != ATTN_OK) return rc;
     ATTN_CUDA_TRY(cudaGetLastError());
     ++t_launch_count;
-    launched(ATTN_KERNEL_GEMM_SMALL, tiles);
+    launched(ATTN_KERNEL_GEMM_SMALL, tiles, {"gemm_small_kernel", 1, {b_layout == 0 ? 1 : 0}});
     return ATTN_OK;
   }
   CUtensorMap ta, tb, tc;
@@ -1411,7 +1428,7 @@ int gemm_launch(const void* a, const void* b, void* c, int batch, int M, int N, 
   if (rc != ATTN_OK) return rc;
   ATTN_CUDA_TRY(cudaGetLastError());
   ++t_launch_count;
-  launched(pair ? ATTN_KERNEL_GEMM_PAIR : ATTN_KERNEL_GEMM, t.ctas);
+  launched(pair ? ATTN_KERNEL_GEMM_PAIR : ATTN_KERNEL_GEMM, t.ctas, {pair ? "gemm_pair_kernel" : "gemm_kernel", 2, {b_layout == 0 ? 1 : 0, t.tile_n}});
   return ATTN_OK;
 }
 
@@ -1468,7 +1485,7 @@ int softmax_launch(const void* s, void* pout, long long rows, int cols, float sc
 #undef SOFTMAX_ROW_CASE
   ATTN_CUDA_TRY(e);
   ++t_launch_count;
-  launched(ATTN_KERNEL_SOFTMAX, ctas);
+  launched(ATTN_KERNEL_SOFTMAX, ctas, {"softmax_rows", 0, {}});
   return ATTN_OK;
 }
 
