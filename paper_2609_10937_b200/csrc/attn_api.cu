@@ -216,7 +216,8 @@ int launch_fwd(const void* q, const void* k, const void* v, void* o, int B, int 
   p.ws = ws ? ws + attn::kCounterBytes / sizeof(float) : nullptr;    // partial results follow
   int grid = t.ctas;
   p.seg_skip = 0;
-  // One CTA per tile with more tiles than SMs: a persistent grid of one CTA per SM runs them in the same order.
+  // One CTA per tile with more tiles than SMs: a persistent grid of one CTA per SM runs them in the same order.  (Of the device's own plans those
+  // at d = 64 that pipe_tiles leaves here; at d = 128 overrides and callers' descriptors only.)
   const int sms = st->desc.num_units;                      // of the device itself (the plan may be for a smaller machine)
   if (!p.causal && t.ctas == t.tiles) {
     if (sms > 0 && t.tiles > sms) {
@@ -535,9 +536,9 @@ int launch_narrow(const void* q, const void* k, const void* v, void* o, int BH, 
 long long causal_steps(int BH, int L) { return BH * attn_internal::head_units((L + 255) / 256, (L + 127) / 128, 2, 1); }
 
 // Whether a causal plan of equal ranges runs as whole tiles instead.  Longest first, whole tiles take the longest tile's steps
-// or an even share of all steps, one more per tile, whichever is more; 5 for the start and the end.  Measured (us, ranges /
-// whole tiles): 128 heads x 4096, d = 128 625 / 501; 32 x 1111, d = 64 36 / 20; 16 x 4096, d = 128 88 / 66; where the longest
-// tile decides, ranges stay: 8 x 4096 55 / (33 steps of 2) 66.  (Four ring stages: the MMA warp looks that far ahead.)
+// or an even share of all steps, one more per tile, whichever is more; 5 for the start and the end.  Measured (us in graphs, ranges /
+// whole tiles): 128 heads x 4096, d = 128 571 / 471; 32 x 1111, d = 64 28.3 / 19.1; 16 x 4096, d = 128 89.6 / 72.4; where the longest
+// tile decides, ranges stay: 8 x 4096 55.6 / (33 steps of 1.8) 61.4.  (Four ring stages: the MMA warps look that far ahead.)
 bool causal_whole_tiles(const attn_tiles& t, int BH, int L, int d, int local_mem, int sms) {
   if (!t.causal || t.n_q != 2 || t.tile_kv != 128) return false;
   if (local_mem < (d == 64 ? attn::NarrowSmem<64, 2>::total(4) : attn::PipeSmem<128>::total(4))) return false;
@@ -546,38 +547,42 @@ bool causal_whole_tiles(const attn_tiles& t, int BH, int L, int d, int local_mem
   return std::max<long long>((L + 127) / 128, even) + 5 <= t.cost_steps;
 }
 
-// Sub-tiles a tile of narrow_kernel.cuh has: two, or one (tiles of 128 rows that take half as long), or 0 where the plan's kernel
+// Sub-tiles a tile of narrow_kernel.cuh has: two, or one (tiles of 128 rows that take half as long), or 0 where another kernel
 // stays.  Estimates in units of about 1.4 us at d = 64, in us at d = 128 (where a step of this kernel is slower than one of
-// attn_fwd_kernel, 2.1 us against 1.75: its rows need every key tile for themselves).
+// attn_fwd_kernel, 2.1 us against 1.75: its rows need every key tile for themselves).  Figures: us in graphs of 12 calls.
 //   Causal.  One sub-tile where the longest tile would keep its CTA longer than an even share of the work, by the estimates
 // (in steps) max(longest / 2, 1.1 even + 1) + 4.4 for one, max(longest, 1.1 even + 1) 0.96 + 4.1 for two and 1.08 times the plan's
-// cost for its ranges.  Measured in loops (us; plan's kernel or two / one): 8 heads x 4096 49.9 / 30.2, 4 x 8192 69.3 / 51.7,
-// 16 x 2048 29.4 / 20.2, 20 x 1111 18.1 / 12.6, 32 x 1111 18.9 / 16.5; on the other side 2 x 8192 45.8 / 51.4, 1 x 16384 67.5 /
-// 94.9, 60 x 1500 37.0 / 39.8, 128 x 256 7.9 / 8.9.  A plan of clusters is launched as clusters, which attn_last_cluster_size
-// reports and tests ask for, although one sub-tile is mostly faster there (9 x 1111 14.7 / 11.8, 16 x 512 11.1 / 7.8).
-//   Not causal, one sub-tile: where 1.1 times the waves of half-length tiles and 2.8 are below the plan's cost (us, attn_fwd_kernel /
-// one): 1 head x 256 6.8 / 5.3, 16 x 512 10.3 / 7.2, 16 x 1024 13.2 / 11.3, 32 x 1111 29.9 / 22.2, 60 x 1500 63.8 / 60.2; on the other
-// side 128 x 256 7.7 / 8.3, 30 x 1024 17.1 / 18.8, 4 x 2048 15.1 / 17.4, 16 x 2048 28.6 / 32.1, 1 x 16384 95.8 / 99.2.  With more
-// tiles than SMs the cost leaves out what a change of tile and a masked step take, and the kind of plan decides as well (us, graphs
-// of 12 calls).  Whole tiles: only where half-length ones end in fewer than twice as many waves: 192 x 384 22.3 / 17.7, 111 x 512
-// 19.6 / 16.4; as many 296 x 256 13.1 / 13.7, 96 x 1024 44.8 / 48.2, 85 x 1280 53.4 / 59.3; a single key step 256 x (512 x 128) 15.2 /
-// 16.9, 61 x (3731 x 128) 25.6 / 28.0.  Tiles shared between CTAs, whose change and merge this kernel does not have: a masked last key tile 128 x 1000 71.5 / 60.1,
-// 128 x 1300 116 / 113, few steps 222 x 640 52.8 / 47.3, few waves 48 x 1024 30.5 / 26.6; else 111 x 1536 98.8 / 105, 160 x 1280 106 / 111.
+// cost for its ranges (plan's kernel or two / one): 8 heads x 4096 40.8 / 30.9, 4 x 8192 61.4 / 52.1, 16 x 2048 29.9 / 19.8,
+// 20 x 1111 18.6 / 12.6, 32 x 1111 19.1 / 16.4; on the other side 2 x 8192 41.8 / 50.9, 1 x 16384 62.6 / 95.9, 60 x 1500 37.5 / 39.8,
+// 128 x 256 8.0 / 9.2.  A plan of clusters is launched as clusters, which attn_last_cluster_size reports and tests ask for, although one
+// sub-tile is mostly faster there (9 x 1111 13.8 / 11.9, 16 x 512 10.2 / 8.0).
+//   Not causal, one sub-tile: where 1.1 times the waves of half-length tiles and 2.8 are below the plan's cost (attn_fwd_kernel / one):
+// 1 head x 256 7.2 / 5.5, 16 x 512 10.6 / 7.3, 16 x 1024 13.3 / 11.3, 32 x 1111 29.9 / 22.7, 60 x 1500 64.0 / 61.3; on the other
+// side 128 x 256 7.9 / 8.4, 30 x 1024 17.2 / 19.1, 4 x 2048 15.5 / 17.6, 16 x 2048 28.8 / 32.3, 1 x 16384 95.4 / 98.3.  With more
+// tiles than SMs the cost leaves out what a change of tile and a masked step take, and the kind of plan decides as well.  Whole tiles: only
+// where half-length ones end in fewer than twice as many waves: 192 x 384 22.2 / 17.4, 111 x 512 19.3 / 16.0; as many 296 x 256
+// 13.1 / 13.3, 96 x 1024 44.5 / 48.0, 85 x 1280 52.9 / 59.2; a single key step 256 x (512 x 128) 15.0 / 16.7, 61 x (3731 x 128) 24.4 /
+// 26.8.  Tiles shared between CTAs, whose change and merge this kernel does not have: a masked last key tile 128 x 1000 71.0 / 60.9,
+// 128 x 1300 116 / 113, few steps 222 x 640 51.9 / 47.5, few waves 48 x 1024 30.2 / 26.5; else 111 x 1536 98.0 / 104, 160 x 1280 105 / 109.
 //   Not causal, two: whole waves of tiles, three or more with at most a tenth of all slots empty.  There a step of this kernel is
-// 4 to 8 % slower than attn_fwd_kernel's until the power limit evens them out (us, attn_fwd_kernel / two: 148 x 1024 58.8 / 63.7, 74 x
-// 2048 105 / 112, 148 x 4096 for half a second 863 / 880, 128 x 8192 2640 / 2533 in short bursts and 2943 / 2914 for half a second),
-// a tile's end is cheaper: 48 key steps or more; shared tiles of up to 8 steps, 11 with a masked one (1000 x 256 44.7 / 35.1, 256 x 1000
-// 122 / 111, 192 x 1300 168 / 153; 192 x 1280 125 / 127); whole tiles, four waves, up to 5 steps with a masked one, or a single
-// step (296 x 450 39.4 / 38.1, 370 x (512 x 128) 18.5 / 17.5; three waves 444 x 256 17.6 / 17.9, 148 x 640 31.5 / 32.8).
-//   d = 128, by the same reasoning.  Causal (us; plan's kernel / one): 8 heads x 4096 54.7 / 40.7, 16 x 2048 35.1 / 28.2, 20 x 1111
-// 21.6 / 16.3, 1 x 256 12.7 / 9.4; on the other side 32 x 1111 22.9 / 24.0, 24 x 2048 35.7 / 40.5, 2 x 8192 55.3 / 73.3, 128 x 256
-// 12.4 / 13.8.  Not causal: 1 x 256 8.1 / 5.8, 16 x 512 11.4 / 8.9, 32 x 1111 35.4 / 30.4; on the other side 30 x 1024 19.0 / 23.2,
-// 128 x 256 9.2 / 9.9, 16 x 2048 32.9 / 42.5, 1 x 16384 122 / 166.  Clusters stay here too (16 x 1024 15.2 / 13.9).
-// A masked last key tile costs a tile of one sub-tile 2.4 us here (256 x 256 15.2, 256 x 200 25.0): with more tiles than SMs and whole
-// ones only up to two waves (96 x 300 20.5 / 17.4; three 192 x 200 16.7 / 19.9, 96 x 450 23.9 / 26.4), and not beside two steps on more
-// than half the SMs (48 x 130 8.7 / 9.2).  Else the waves may be half as many again as the plan's (192 x 384 26.9 / 22.7, 160 x 640 54.2 /
-// 48.1; 111 x 768 44.7 / 46.4), whole tiles of up to three steps less than twice as many (370 x 256 22.8 / 20.2; 256 x 512 44.1 / 47.4),
-// and a single step is not worth it (256 x (512 x 128) 19.5 / 22.4).
+// 4 to 8 % slower than attn_fwd_kernel's until the power limit evens them out (attn_fwd_kernel / two: 148 x 1024 60.2 / 64.5, 74 x
+// 2048 110 / 116, 148 x 4096 859 / 842, 128 x 8192 3009 / 2760), and a tile's end is cheaper: 48 key steps or more; shared tiles
+// of up to 8 steps, 11 with a masked one (1000 x 256 50.7 / 39.3, 256 x 1000 128 / 114, 192 x 1300 172 / 154; 192 x 1280 126 / 131);
+// whole tiles, four waves, up to 5 steps with a masked one, or a single step (296 x 450 41.0 / 38.9, 370 x (512 x 128) 18.8 / 17.6; three waves
+// 444 x 256 17.7 / 17.6, 148 x 640 31.2 / 32.6).
+//   The lines for calls that are not causal lie between this kernel and attn_fwd_kernel.  attn_pipe_kernel, which is asked after them, is
+// faster than this one at some calls on this side: d = 64 128 x 1000 60.8 / 55.8, 256 x 1000 114 / 102, 192 x 1300 154 / 152, 296 x 450
+// 39.1 / 36.5, d = 128 160 x 640 47.4 / 43.7.
+//   d = 128, by the same reasoning.  Causal (plan's kernel or whole tiles / one): 8 heads x 4096 55.6 / 42.3, 16 x 2048 34.5 / 28.5, 20 x 1111
+// 19.6 / 16.4, 1 x 256 8.9 / 7.3; on the other side 32 x 1111 20.3 / 22.9, 24 x 2048 33.3 / 39.3, 2 x 8192 51.0 / 71.5, 128 x 256
+// 9.9 / 12.8.  (The estimates for the other kernels are of slower ones that were there before them.)  Not causal: 1 x 256 8.7 / 6.5, 16 x 512
+// 12.3 / 9.6, 32 x 1111 36.5 / 30.0; on the other side 30 x 1024 19.8 / 23.4, 128 x 256 9.6 / 9.9, 16 x 2048 32.1 / 39.3, 1 x 16384
+// 113 / 143.  Clusters stay here too (16 x 1024 15.9 / 14.3).
+// A masked last key tile costs a tile of one sub-tile 2.4 us here (256 x 256 15.0, 256 x 200 23.9): with more tiles than SMs and whole
+// ones only up to two waves (96 x 300 19.8 / 17.1; three 192 x 200 16.4 / 19.1, 96 x 450 23.4 / 25.9), and not beside two steps on more
+// than half the SMs (48 x 130 8.7 / 8.9).  Else the waves may be half as many again as the plan's (192 x 384 26.1 / 21.8, 160 x 640 53.6 /
+// 47.3; 111 x 768 44.4 / 45.6), whole tiles of up to three steps less than twice as many (370 x 256 22.2 / 19.8; 256 x 512 43.7 / 46.9),
+// and a single step is not worth it (256 x (512 x 128) 21.2 / 23.2).
 int narrow_subs(const attn_tiles& t, int BH, int Lq, int Lk, int d, int local_mem, int sms) {
   if (t.n_q != 2 || t.tile_kv != 128 || local_mem < (d == 64 ? attn::NarrowSmem<64, 2>::total(4) : attn::NarrowSmem<128, 1>::total(4))) return 0;
   const bool clusters = t.ctas % t.tiles == 0 && t.ctas > t.tiles;

@@ -386,8 +386,8 @@ struct FwdMisc {               // lives in the last 3072 bytes of dynamic shared
   uint64_t alpha_full[2];
   uint64_t q_empty;            // every product that reads the Q tile of a segment has finished
   uint64_t o_free[2];          // the epilogue of a segment has read its O accumulator
-  uint64_t s_free[2];          // d = 64: the softmax warpgroup holds the step's scores in registers
-  uint64_t turn[2];            // d = 128: the sub-tile's MMA warp may issue its step
+  uint64_t s_free[2];          // d = 64, not causal: the softmax warpgroup holds the step's scores in registers
+  uint64_t turn[2];            // causal, two sub-tiles: the sub-tile's MMA warp may issue its step
   uint64_t peers_ready;        // cluster: every other CTA of the tile has finished with its K/V ring
   uint64_t data_ready[8][2];   // cluster: the other CTAs' parts of softmax warp w's rows have landed ([1]: columns 64..)
   AbortCell abort;
@@ -812,7 +812,8 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
           mbar_arrive(bar_a);
           delta *= alpha;
           uint64_t sum[2] = {0ull, 0ull};
-          uint32_t pk[16], pk2[16];
+          [[maybe_unused]] uint32_t pk[16];
+          uint32_t pk2[16];
           exp_chunk_in_place<kStepPoly, false>(&s[0], s, sum, ek, neg_m2, pk2);
           tmem_st16(p_tmem, pk2);
           if constexpr (TKV == 128) {

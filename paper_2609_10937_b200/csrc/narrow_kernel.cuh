@@ -7,10 +7,11 @@
 // 64 scores a row: a tile of 256 query rows is worked on as four streams, two sub-tiles of 128 rows times the two halves of
 // every 128-key tile.  A stream has its own scores, reference, denominator and accumulator in tensor memory (4 x (64 + 64)
 // columns: all 512; P overwrites the front of its scores) and its own softmax warpgroup; the two streams of a sub-tile meet
-// when the tile is finished, in the epilogue warpgroup, which reads both accumulators.  2600 cycles a step.  In loops of 0.7 s
-// (us, attn_fwd_kernel's step / this kernel): causal 128 heads x 8192 1650 / 1509, 128 x 4096 454 / 416, 128 x 2048
-// 140 / 124, 256 x 300 31.2 / 21.6; not causal 900 x 1025 558 / 497, 256 x 1000 122 / 120, and at 128 x 8192 2918 / 2910: there the power
-// limit takes back what bursts gain (2640 / 2533).  Where attn_fwd_kernel is the faster one stands at narrow_subs (attn_api.cu).
+// when the tile is finished, in the epilogue warpgroup, which reads both accumulators.  2600 cycles a step.  In loops of 0.8 s
+// (us, attn_fwd_kernel / this kernel): causal 128 heads x 8192 1708 / 1499, 128 x 4096 454 / 413; not causal 900 x 1025 544 / 490, 256 x 1000
+// 122 / 117, 128 x 8192 2898 / 2842 (attn_pipe_kernel 2886), 148 x 4096 855 / 864: the power limit takes back a part of what bursts gain (128 x 8192
+// 3009 / 2760 in graphs).  In graphs: causal 128 x 2048 141 / 114, 256 x 300 39.1 / 22.2.  Where another kernel is the faster one stands at
+// narrow_subs and pipe_tiles (attn_api.cu).
 // SUBS = 1 works on tiles of 128 query rows, one sub-tile: its four streams are the two halves of the even and of the odd key
 // tiles.  A tile then takes half as long, which evens out the CTAs where a launch has few tiles for each (narrow_subs in
 // attn_api.cu), at twice the K and V loads for a row.  At d = 128, where a stream needs 256 columns of tensor memory, two

@@ -20,16 +20,16 @@
 //     unit; none: 0-1 % slower).  Causal, where the kernel before took none in the common step, it is the quintic, which is as exact as
 //     the unit (128 x 4096 in loops: cubic 547, quintic 549, none 551 us).  At d = 64 there is no chain: P has columns of its own, the
 //     next scores are produced under this step's exponentials, both warpgroups work all the time, and three pairs of eight are
-//     fastest (2: 867, 3: 829, 4: 887 us at 148 x 4096); one of them is a cubic and two are quartics, so that a weight is nowhere
-//     less exact than with two cubics (three cubics: 824, as it is 855, three quartics 865; 148 x 1024 55.6 / 57.1 / 57.3).
+//     fastest (2: 867, 3: 829, 4: 887 us at 148 x 4096); one of them is a cubic and two are quartics, whose errors together are 0.7 times
+//     those of two cubics (three cubics: 824, as it is 855, three quartics 865; 148 x 1024 55.6 / 57.1 / 57.3).
 // As before it: the epilogue of a tile runs under the next one (the correction warpgroup normalises and stores it), a sub-tile runs
 // only its own steps, tiles come from the hardware's queue of CTAs not yet started (clusterlaunchcontrol.try_cancel), causal ones
 // longest first within groups of heads whose K and V stay in L2.
 // Measured (us, the kernels before / this one, calls back to back): d = 128 causal 128 x 4096 549 / 516, 600 x 512 87.5 / 76.4, 213 shapes in
 // whole tiles 0.84 times on the geometric mean; not causal 148 x 4096 1080 / 1053, 148 x 2048 with variance 3 303 / 294, 95 shapes
 // in waves of whole tiles 0.91 times; d = 64 (tiles that are not long, pipe_tiles in attn_api.cu) 148 x 1024 58.9 / 57.1, 128 x 2000 195 / 178, 436
-// shapes 0.958 times.  Long calls run into the power limit (990 W) and keep less: in loops of seconds 4 x 32 x 4096, d = 128, takes 1000 /
-// 982, causal 582 / 549.
+// shapes 0.958 times.  Long calls run into the power limit (990 W) and keep less: in loops of 0.8 s 4 x 32 x 4096, d = 128, takes 983 /
+// 967, causal 580 / 543.
 #pragma once
 
 #include "attn_kernels.cuh"
