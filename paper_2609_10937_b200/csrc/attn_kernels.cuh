@@ -368,9 +368,11 @@ constexpr float kDominanceFactor = 16.0f;   // a new maximum heavier than delta/
 // score times a scale below 1 lies under it (a higher one would take such a row's weights to zero and its result to NaN).
 constexpr float kEmptyReference = -3.402823466e38f;
 // 1 / denominator of a finished row.  NaN if its reference is no number or infinite (the polynomial's weights would be finite), or if no key
-// that it may attend to has a finite score (a denominator of weights that the polynomial clamps, of masked keys too).
+// that it may attend to has a finite score (kEmptyReference; a denominator of weights that the polynomial clamps, of masked keys too).  A
+// finite score times the scale, which is below 1/2, is finite when doubled.
 __device__ __forceinline__ float row_inverse(float delta, float m) {
-  return 1.0f / (m == kEmptyReference ? __int_as_float(0x7FFFFFFF) : delta + (m - m));
+  const float twice = m + m;
+  return 1.0f / (delta + (twice - twice));
 }
 constexpr int kCounterBytes = 65536;   // head of the workspace: 16384 arrival counters
 
