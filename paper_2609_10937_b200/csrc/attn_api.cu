@@ -620,30 +620,34 @@ int narrow_subs(const attn_tiles& t, int BH, int Lq, int Lk, int d, int local_me
   return 1.1 * (double)(waves * ((steps + 1) / 2)) + 2.8 < (double)t.cost_steps ? 1 : 0;
 }
 
-// Calls, not causal, that pipe_kernel.cuh takes over from attn_fwd_kernel, at either head dimension (us in graphs of 8 calls, attn_fwd_kernel / this).
+// Calls, not causal, that pipe_kernel.cuh takes over from attn_fwd_kernel, at either head dimension (us in graphs of 8 to 40 calls, attn_fwd_kernel / this).
 //   Plans of whole tiles, d = 128: with more tiles than SMs always (95 shapes, 0.91 times on the geometric mean: 592 x 512 75.8 / 63.2).  One wave: from four
-// key steps on (three and fewer 0.98 to 1.05) where the tiles fill more than seven tenths of the SMs (10 x 2560 38.7 / 39.7, 24 x 1300 23.8 /
-// 22.7).
+// key steps on (three and fewer 0.98 to 1.05) where the tiles fill three quarters of the SMs (128 x (256 x 1000) 0.97 times; 104 x (256 x
+// 1280) 22.6 / 24.8, 10 x 2560 38.7 / 39.7).  From a dozen steps on without a masked one this kernel is 1 to 2 % slower in a burst of some
+// milliseconds and as much faster in a loop of seconds, under the power limit (8 x 4096 66.5 / 65.9, 74 x (1000 x 2048) 79.5 / 78.9, 37 x (4096 x 2560)
+// 185 / 182): the line is drawn for loops.
 //   d = 64: its step takes one cubic and two quartics of eight pairs where attn_fwd_kernel takes two cubics, which costs 2 % of a step and leaves
-// long tiles to that kernel.  One wave from 4 key steps (3: 64 x 384 10.0 / 10.2) to 15 (148 x (256 x 1280) 20.7 / 20.2, 80 x (256 x 2048)
-// 29.4 / 29.4, 120 x (256 x 4096) 53.3 / 55.0); two waves to 17, three to 23, four to 29 (32 x 2048 54.0 / 53.5, 32 x 2304 59.4 / 60.2, 24 x 3000 77.6 / 78.9, 37 x 4000
-// 205 / 208), more to 31, where the last wave is full to 23 (60 x 3000 203 / 195, 111 x 3000 352 / 352, 74 x 4096 408 / 414).  An odd
-// number of steps without a masked one is a good one for attn_fwd_kernel: 5 (148 x 640 31.5 / 33.0), and from 7 on where the last wave is full
-// (148 x 896 52.2 / 54.0, but 128 x 896 0.90 times; 148 x 1152 79.1 / 80.9).  436 shapes on two grids go here, 0.958 times, four of them slower by 1 to 1.6 %.
+// long tiles to that kernel.  One wave from 4 key steps (3: 64 x 384 10.0 / 10.2) to 10 (148 x (256 x 1280) 20.7 / 20.2; 20 x (1700 x 1700)
+// 25.7 / 26.3); two waves to 17, three to 23, four to 29 (32 x 2048 54.0 / 53.5, 32 x 2304 59.4 / 60.2, 24 x 3000 77.6 / 78.9, 37 x 4000
+// 205 / 208), more to 31, where the last wave is full to 23 (60 x 3000 203 / 195, 111 x 3000 352 / 352, 74 x 4096 408 / 414).  A head whose last
+// tile has only one sub-tile gains nothing there: the sub-tile takes nearly as long alone.  In full waves of whole tiles such calls stay from 3 steps on, with a
+// masked one, which attn_fwd_kernel is slow at, from 8 (148 x 640 31.2 / 32.8, 148 x (1100 x 512) 1.056 times, 148 x (1280 x 512) 0.945).  Of 554
+// shapes on two grids 434 go here, 0.956 times, four of them slower by 1 to 1.6 %.
 //   Plans whose tiles are cut over the machine: where whole tiles are estimated to be faster by 2 % (d = 64) or 4 %.  The estimates are
 // fits in us, of this kernel over its waves and key steps and of the plan's over its cost, that miss by 4 to 7 % (one sd): of 140 shapes
 // 49 go here, 0.89 times on the geometric mean and none slower by more than 1 %; 14 that would be 3 % faster or more stay.
-bool pipe_tiles(const attn_tiles& t, int Lk, int d, int local_mem, int sms) {
+bool pipe_tiles(const attn_tiles& t, int Lq, int Lk, int d, int local_mem, int sms) {
   if (t.causal || t.n_q != 2 || t.tile_kv != 128) return false;
   if (local_mem < (d == 64 ? attn::PipeSmem<64>::total(4) : attn::PipeSmem<128>::total(4))) return false;
   const int steps = (Lk + 127) / 128, waves = (t.tiles + sms - 1) / sms;
+  const long long filled = 100LL * t.tiles / ((long long)waves * sms);       // per cent of the waves' slots
+  if (waves == 1) return t.ctas == t.tiles && steps >= 4 && (d == 64 ? steps <= 10 : 4 * t.tiles >= 3 * sms);
   if (d == 64) {
-    const bool full = 100LL * t.tiles >= 98LL * waves * sms;       // the last wave
-    if (steps >= 32 || steps >= (waves == 1 ? 16 : 6 + 6 * waves) || (full && steps >= 24)) return false;
-    if (waves > 1 && Lk % 128 == 0 && steps % 2 == 1 && (steps == 5 || (steps >= 7 && full))) return false;
+    if (steps >= 32 || steps >= 6 + 6 * waves || (filled >= 98 && steps >= 24)) return false;
+    if (t.ctas == t.tiles && filled >= 97 && (Lq - 1) % 256 < 128 && steps >= (Lk % 128 ? 8 : 3)) return false;
   }
-  if (t.ctas == t.tiles) return t.tiles > sms || (steps >= 4 && (d == 64 || 10 * t.tiles > 7 * sms));
-  if (t.ctas > t.tiles || t.tiles <= sms) return false;
+  if (t.ctas == t.tiles) return true;
+  if (t.ctas > t.tiles) return false;
   const double whole = d == 64 ? 3.0 + waves * (2.0 + 1.376 * steps + (Lk % 128 ? 0.35 : 0.0)) : 4.0 + waves * (2.3 + 1.647 * steps);
   const double cut = d == 64 ? 2.5 + 1.493 * t.cost_steps : 5.7 + 1.78 * t.cost_steps;
   return whole < (d == 64 ? 0.98 : 0.96) * cut;
@@ -664,7 +668,7 @@ int dispatch_fwd(const void* q, const void* k, const void* v, void* o, int B, in
     }
     if (d == 128 && Lk == L && causal_whole_tiles(t, B * H, L, d, st->desc.local_mem_bytes, sms))
       return launch_pipe<128, true>(q, k, v, o, B * H, L, L, status, st, s, ATTN_KERNEL_CAUSAL_TILES);
-    if (pipe_tiles(t, Lk, d, st->desc.local_mem_bytes, sms))
+    if (pipe_tiles(t, L, Lk, d, st->desc.local_mem_bytes, sms))
       return d == 64 ? launch_pipe<64, false>(q, k, v, o, B * H, L, Lk, status, st, s, ATTN_KERNEL_TILED)
                      : launch_pipe<128, false>(q, k, v, o, B * H, L, Lk, status, st, s, ATTN_KERNEL_TILED);
   }

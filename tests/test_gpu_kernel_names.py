@@ -22,16 +22,17 @@ PIPE, NARROW, FWD = "attn_pipe_kernel", "attn_narrow_kernel", "attn_fwd_kernel"
 
 
 @pytest.mark.parametrize("d,H,Lq,Lk,causal,name", [
-    # d = 128, not causal: waves of whole tiles; one wave from four key steps on more than seven tenths of 148 SMs; tiles the plan would cut
+    # d = 128, not causal: waves of whole tiles; one wave from four key steps on three quarters of 148 SMs; tiles the plan would cut
     (128, 300, 129, 129, False, f"{PIPE}<128,0>"), (128, 160, 257, 1, False, f"{PIPE}<128,0>"), (128, 150, 300, 128, False, f"{PIPE}<128,0>"),
-    (128, 152, 640, 640, False, f"{PIPE}<128,0>"), (128, 110, 200, 900, False, f"{PIPE}<128,0>"), (128, 104, 256, 900, False, f"{PIPE}<128,0>"),
-    (128, 100, 256, 900, False, f"{FWD}<128,128,2,0,0,0>"), (128, 110, 256, 384, False, f"{FWD}<128,128,2,0,0,0>"), (128, 222, 640, 640, False, f"{PIPE}<128,0>"),
+    (128, 152, 640, 640, False, f"{PIPE}<128,0>"), (128, 111, 200, 900, False, f"{PIPE}<128,0>"), (128, 111, 256, 512, False, f"{PIPE}<128,0>"),
+    (128, 110, 256, 900, False, f"{FWD}<128,128,2,0,0,0>"), (128, 111, 256, 384, False, f"{FWD}<128,128,2,0,0,0>"), (128, 222, 640, 640, False, f"{PIPE}<128,0>"),
     (128, 16, 512, 512, False, f"{NARROW}<128,0,1>"), (128, 4, 4096, 4096, False, f"{FWD}<128,128,2,0,1,1>"), (128, 1, 16384, 16384, False, f"{FWD}<128,128,2,0,0,0>"),
     # d = 64: the same up to the steps from which the plan's kernel is the faster one
     (64, 74, 900, 900, False, f"{PIPE}<64,0>"), (64, 148, 1024, 1024, False, f"{PIPE}<64,0>"), (64, 60, 300, 449, False, f"{PIPE}<64,0>"),
-    (64, 148, 256, 1920, False, f"{PIPE}<64,0>"), (64, 148, 256, 1921, False, f"{FWD}<64,128,2,0,0,0>"), (64, 74, 1024, 2100, False, f"{PIPE}<64,0>"),
+    (64, 148, 256, 1280, False, f"{PIPE}<64,0>"), (64, 148, 256, 1281, False, f"{FWD}<64,128,2,0,0,0>"), (64, 74, 1024, 2100, False, f"{PIPE}<64,0>"),
     (64, 74, 1024, 2304, False, f"{FWD}<64,128,2,0,0,0>"), (64, 160, 3500, 3500, False, f"{PIPE}<64,0>"), (64, 160, 3500, 4000, False, f"{FWD}<64,128,2,0,0,0>"),
-    (64, 148, 640, 640, False, f"{FWD}<64,128,2,0,0,0>"), (64, 148, 640, 600, False, f"{PIPE}<64,0>"), (64, 128, 896, 896, False, f"{PIPE}<64,0>"),
+    (64, 148, 640, 640, False, f"{FWD}<64,128,2,0,0,0>"), (64, 148, 640, 600, False, f"{PIPE}<64,0>"), (64, 148, 640, 256, False, f"{PIPE}<64,0>"),
+    (64, 148, 600, 1000, False, f"{FWD}<64,128,2,0,0,0>"), (64, 148, 641, 640, False, f"{PIPE}<64,0>"), (64, 128, 896, 896, False, f"{PIPE}<64,0>"),
     (64, 148, 896, 896, False, f"{FWD}<64,128,2,0,0,0>"), (64, 111, 1300, 1300, False, f"{PIPE}<64,0>"), (64, 37, 6144, 6144, False, f"{NARROW}<64,0,2>"),
     (64, 296, 300, 300, False, f"{NARROW}<64,0,2>"), (64, 16, 512, 512, False, f"{NARROW}<64,0,1>"), (64, 8, 1000, 1000, False, f"{FWD}<64,128,2,0,1,1>"),
     # causal
