@@ -631,8 +631,8 @@ int narrow_subs(const attn_tiles& t, int BH, int Lq, int Lk, int d, int local_me
 // 25.7 / 26.3); two waves to 17, three to 23, four to 29 (32 x 2048 54.0 / 53.5, 32 x 2304 59.4 / 60.2, 24 x 3000 77.6 / 78.9, 37 x 4000
 // 205 / 208), more to 31, where the last wave is full to 23 (60 x 3000 203 / 195, 111 x 3000 352 / 352, 74 x 4096 408 / 414).  A head whose last
 // tile has only one sub-tile gains nothing there: the sub-tile takes nearly as long alone.  In full waves of whole tiles such calls stay from 3 steps on, with a
-// masked one, which attn_fwd_kernel is slow at, from 8 (148 x 640 31.2 / 32.8, 148 x (1100 x 512) 1.056 times, 148 x (1280 x 512) 0.945).  Of 554
-// shapes on two grids 434 go here, 0.956 times, four of them slower by 1 to 1.6 %.
+// masked one, which attn_fwd_kernel is slow at, from 12 (148 x 640 31.2 / 32.8, 148 x (1100 x 512) 1.056 times, 148 x 1111 1.00; 148 x (1280 x 512) 0.945).  Of 554
+// shapes on two grids 442 go here, 0.959 times, six of them slower by 1 to 2.7 %.
 //   Plans whose tiles are cut over the machine: where whole tiles are estimated to be faster by 2 % (d = 64) or 4 %.  The estimates are
 // fits in us, of this kernel over its waves and key steps and of the plan's over its cost, that miss by 4 to 7 % (one sd): of 140 shapes
 // 49 go here, 0.89 times on the geometric mean and none slower by more than 1 %; 14 that would be 3 % faster or more stay.
@@ -644,7 +644,7 @@ bool pipe_tiles(const attn_tiles& t, int Lq, int Lk, int d, int local_mem, int s
   if (waves == 1) return t.ctas == t.tiles && steps >= 4 && (d == 64 ? steps <= 10 : 4 * t.tiles >= 3 * sms);
   if (d == 64) {
     if (steps >= 32 || steps >= 6 + 6 * waves || (filled >= 98 && steps >= 24)) return false;
-    if (t.ctas == t.tiles && filled >= 97 && (Lq - 1) % 256 < 128 && steps >= (Lk % 128 ? 8 : 3)) return false;
+    if (t.ctas == t.tiles && filled >= 97 && (Lq - 1) % 256 < 128 && steps >= (Lk % 128 ? 12 : 3)) return false;
   }
   if (t.ctas == t.tiles) return true;
   if (t.ctas > t.tiles) return false;

@@ -27,8 +27,8 @@
 // longest first within groups of heads whose K and V stay in L2.
 // Measured (us, the kernels before / this one, calls back to back): d = 128 causal 128 x 4096 549 / 516, 600 x 512 87.5 / 76.4, 213 shapes in
 // whole tiles 0.84 times on the geometric mean; not causal 148 x 4096 1080 / 1053, 148 x 2048 with variance 3 303 / 294, 95 shapes
-// in waves of whole tiles 0.91 times; d = 64 (tiles that are not long, pipe_tiles in attn_api.cu) 148 x 1024 58.9 / 57.1, 128 x 2000 195 / 178, 434
-// shapes 0.956 times.  Long calls run into the power limit (990 W) and keep less: in loops of 0.8 s 4 x 32 x 4096, d = 128, takes 983 /
+// in waves of whole tiles 0.91 times; d = 64 (tiles that are not long, pipe_tiles in attn_api.cu) 148 x 1024 58.9 / 57.1, 128 x 2000 195 / 178, 442
+// shapes 0.959 times.  Long calls run into the power limit (990 W) and keep less: in loops of 0.8 s 4 x 32 x 4096, d = 128, takes 983 /
 // 967, causal 580 / 543.
 #pragma once
 

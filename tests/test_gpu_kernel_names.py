@@ -32,7 +32,7 @@ PIPE, NARROW, FWD = "attn_pipe_kernel", "attn_narrow_kernel", "attn_fwd_kernel"
     (64, 148, 256, 1280, False, f"{PIPE}<64,0>"), (64, 148, 256, 1281, False, f"{FWD}<64,128,2,0,0,0>"), (64, 74, 1024, 2100, False, f"{PIPE}<64,0>"),
     (64, 74, 1024, 2304, False, f"{FWD}<64,128,2,0,0,0>"), (64, 160, 3500, 3500, False, f"{PIPE}<64,0>"), (64, 160, 3500, 4000, False, f"{FWD}<64,128,2,0,0,0>"),
     (64, 148, 640, 640, False, f"{FWD}<64,128,2,0,0,0>"), (64, 148, 640, 600, False, f"{PIPE}<64,0>"), (64, 148, 640, 256, False, f"{PIPE}<64,0>"),
-    (64, 148, 600, 1000, False, f"{FWD}<64,128,2,0,0,0>"), (64, 148, 641, 640, False, f"{PIPE}<64,0>"), (64, 128, 896, 896, False, f"{PIPE}<64,0>"),
+    (64, 148, 600, 1500, False, f"{FWD}<64,128,2,0,0,0>"), (64, 148, 600, 1300, False, f"{PIPE}<64,0>"), (64, 148, 641, 640, False, f"{PIPE}<64,0>"), (64, 128, 896, 896, False, f"{PIPE}<64,0>"),
     (64, 148, 896, 896, False, f"{FWD}<64,128,2,0,0,0>"), (64, 111, 1300, 1300, False, f"{PIPE}<64,0>"), (64, 37, 6144, 6144, False, f"{NARROW}<64,0,2>"),
     (64, 296, 300, 300, False, f"{NARROW}<64,0,2>"), (64, 16, 512, 512, False, f"{NARROW}<64,0,1>"), (64, 8, 1000, 1000, False, f"{FWD}<64,128,2,0,1,1>"),
     # causal
